@@ -123,7 +123,16 @@ typedef enum {
  *                extra FFT with weight 1.  Default (<= 0): an explicit
  *                taylor_order keeps the Taylor series; the automatic order
  *                takes the series with fewer FFTs for the precision's
- *                remainder bound (Taylor on a tie)
+ *                remainder bound (Taylor on a tie).  With the automatic
+ *                series and order, sub-FFT length included, the same
+ *                transform runs gridded where that applies (height * rho_max
+ *                <= 3.5 and a grid of at most half the contour's own period):
+ *                the nodes are spread onto a coarse grid in beta with complex
+ *                Gaussian weights that carry the contour factor, one FFT
+ *                follows, and no series is summed; and the spectra come from
+ *                tables in beta where the contour has at least four times
+ *                their nodes.  An explicit series (1 or 2), order or sub-FFT
+ *                length keeps the spectra at every node and the series of FFTs
  *   BP_KERNEL    interpolation kernel of the back-projection.  1: Lagrange
  *                polynomials on the transform grid g(s_k).  2: the ES
  *                kernel exp(beta (sqrt(1 - (2x/w)^2) - 1)) of width w = taps
@@ -266,10 +275,10 @@ cfft_status cfft_contour_series_order(double x, cfft_precision precision, int se
  * and rho_r = r * rho_max / (n_rho - 1), r = 0..n_rho-1:
  *   Z'_ab(rho, phi) = sum_q Z_ab,q(rho) exp(i q phi)               (Eq. 9)
  * computed by the C-FFT: MBF spectra along the contour (Eq. 11), the kernel
- * H = M_t . G . M_b^* (Eq. 10), azimuthal harmonics, the Taylor expansion of
- * the contour factor (Eq. 22), one zero-padded FFT per (pair, harmonic,
- * Taylor term) (Eq. 23-24) and a back-projection over the angle to the
- * uniform rho grid.  The back-projection's midpoint rule in the angle takes,
+ * H = M_t . G . M_b^* (Eq. 10), azimuthal harmonics, the contour factor
+ * (Eq. 22: in the weights of a gridded FFT, or as a series of zero-padded
+ * FFTs, Eq. 23-24; see CONTOUR_SERIES) and a back-projection over the angle
+ * to the uniform rho grid.  The back-projection's midpoint rule in the angle takes,
  * for the rows of each chunk up to rho, ceil((z + q_max)/2 + c z^(1/3) +
  * margin/2) + 1 nodes with z = |beta_c|max rho, margin = ALPHA_MARGIN (24)
  * and c = 4 in FP64, 2 in FP32-mixed: the first aliased angular harmonic
@@ -445,12 +454,13 @@ cfft_status cfft_fill_backward_residual(cfft_ctx* ctx, int n_elements, const dou
 /* Diagnostics of the last tabulation (host values): highest term index of
  * the contour-factor series used (taylor_order; contour_series 0: Taylor,
  * 1: Chebyshev; the FFTs per (pair, harmonic) are taylor_order + 1, or + 2
- * for Chebyshev),
+ * for Chebyshev; a gridded transform sums no series and reports the one the
+ * automatic choice would take),
  * n_alpha, sigma, FFT length, sub-FFT length, grid half-width K, back-
  * projection taps, fill taps, series count, the device time of each stage in
  * milliseconds (contour, integrand, fft, backproject; CUDA events on the
  * context stream), the number of kernels launched, and the work of each
- * stage: integrand points (nodes x angles), sub-FFTs run (each of length
+ * stage: integrand points (nodes, or spectral table nodes, x angles), sub-FFTs run (each of length
  * sub_len), and back-projection node evaluations (series x rows x angles).
  * spectra_tc: 1 when the MBF spectra ran on the tensor cores; bp_form: 0 the
  * gather form of the back-projection, 1 the matrix form, 2 the paired-

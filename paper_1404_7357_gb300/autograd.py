@@ -43,8 +43,26 @@ class FillProblem:
                                      el.width, el.q)
         self.ctx.build_contour(c.n, c.beta_max, c.beta_p, c.height, -1)
         self.ctx.set_option(cfft.OPT_DERIVATIVES, 1 if derivatives else 0)
-        self.ctx.tabulate_reactions(self.q_max, self.rho_max, self.n_rho, self.precision,
-                                    self.classes)
+        # The gradients are float64 sums over a float32 table, so they show that table's last
+        # bits (a relative 2e-6 between two equally accurate tables).  They are kept to what
+        # the direct pipeline gives: the automatic series, named explicitly, selects it
+        # (gridded tables would take the 2,000-element gradient from 51.6 to 32.5 ms on GB300).
+        # A series set by the caller on self.ctx stays as it is.
+        own = self.ctx._options.get(cfft.OPT_CONTOUR_SERIES, 0.0)
+        pin = 0
+        if self.precision == cfft.CFFT_FP32_MIXED and own <= 0:
+            try:
+                pin = 1 + cfft.contour_series_order(c.height * self.rho_max, self.precision)[0]
+            except cfft.CfftError:
+                pin = 0           # no order reaches the bound: the tabulation says so
+        if pin:
+            self.ctx.set_option(cfft.OPT_CONTOUR_SERIES, pin)
+        try:
+            self.ctx.tabulate_reactions(self.q_max, self.rho_max, self.n_rho, self.precision,
+                                        self.classes)
+        finally:
+            if pin:
+                self.ctx.set_option(cfft.OPT_CONTOUR_SERIES, own)
 
     @property
     def dtype(self):

@@ -182,6 +182,7 @@ class Context:
             stream = torch.cuda.current_stream(device)
         handle = stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
         self.device = device
+        self._options = {}
         self._h = ctypes.c_void_p()
         st = _lib.cfft_create(ctypes.byref(self._h), int(device), ctypes.c_void_p(handle))
         if st != 0:
@@ -231,6 +232,7 @@ class Context:
 
     def set_option(self, key, value):
         self._check(_lib.cfft_set_option(self._h, key, float(value)))
+        self._options[key] = float(value)
 
     def tabulate_reactions(self, q_max, rho_max, n_rho, precision, rotation_classes=1):
         self._table_desc = {"q_max": int(q_max), "rho_max": float(rho_max), "n_rho": int(n_rho),

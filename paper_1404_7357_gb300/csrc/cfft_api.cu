@@ -115,12 +115,12 @@ struct cfft_ctx {
   DevBuf beta_c, weight, bw, bi_rel, green_p, green_r, dp_eps, dr_eps, dp_h, dr_h;
   int channels = 1;  // 1: table; 3: table, d/d eps_r, d/d h
   DevBuf d_shapes, d_bx, d_by, d_q, d_y, d_grid, d_table, d_tw, d_cnodes, d_coff, d_cos, d_lag, d_prec,
-      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_gres;
+      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_gres, d_gtab, d_coarse, d_snodes, d_spec;
   int tw_len = 0, tw_prec = -1;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   // batched sweep: plan arrays, scratch, stream, captured graph, tuned shape
   DevBuf b_cargs, b_cdata, b_iargs, b_fargs, b_bargs, b_cmap, b_imap, b_ftask, b_btask, b_count,
-      b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag;
+      b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag, b_sargs, b_smap, b_gargs, b_gmap, b_coarse, b_gtab;
   cudaStream_t bstream = nullptr;
   cudaEvent_t bev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t bgraph = nullptr;
@@ -294,6 +294,43 @@ void set_extraction(const cfft_ctx* ctx, double eps_r, int* extract, double* eps
   *deps_eff = automatic ? 0.5 : 0.0;
 }
 
+// the gridding arguments of a transform whose tables live at `buf`: output factors
+// ([2K + 1], padded), then the real and the imaginary spreading weights
+template <class T>
+void fill_grid_args(GridArgs<T>* ga, const GridShape& g, int n, int series, int grid_half, int sigma, int64_t fft_len,
+                    T* buf) {
+  ga->n = n;
+  ga->series = series;
+  ga->grid_half = grid_half;
+  ga->sigma = sigma;
+  ga->fft_len = fft_len;
+  ga->m = g.m;
+  ga->hw = g.hw;
+  ga->kmax = g.kmax;
+  ga->n_cells = g.n_cells;
+  ga->act_cells = g.act_cells;
+  ga->nc = g.nc;
+  ga->a = g.a;
+  ga->y_scale = g.y_scale;
+  ga->inv_norm = std::sqrt(g.a / kPi);
+  ga->out_factor = reinterpret_cast<cpx<T>*>(buf);
+  ga->wre = buf + 2 * (2 * (size_t)grid_half + 2);
+  ga->wim = ga->wre + (size_t)2 * g.hw * g.kmax * g.n_cells;
+}
+
+// the transform task of a gridded transform: one term over the coarse samples, length m
+template <class T>
+void set_gridded_fft(FftArgs<T>* fa, const GridArgs<T>& ga) {
+  fa->n = ga.nc;
+  fa->fft_len = ga.m;
+  fa->taylor = 0;
+  fa->expansion = 0;
+  fa->n_active = 0;
+  fa->y = ga.coarse;
+  fa->prec = nullptr;
+  fa->out_factor = ga.out_factor;
+}
+
 // One tabulation into `dst` on n_rho points rho_r = r rho_max / (n_rho - 1).  primary: the
 // table of cfft_tabulate_reactions (its diagnostics go to ctx->info); otherwise the table
 // that the fill interpolates when the tabulated grid misses the fill's target.
@@ -365,13 +402,42 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   }
   int log2L = 0;
   while ((1 << log2L) < L) ++log2L;
-  const int D = (int)(P / L);
+  int D = (int)(P / L);
   // nodes with beta_I > 0 form a prefix of the contour
   int n_active = (int)std::min<double>(n, std::ceil(ctx->beta_p / step - 0.5));
   if (ctx->height <= 0) n_active = 0;
   if (n_active < 0) n_active = 0;
 
+  // an explicit order, series or sub-FFT length asks for the direct pipeline: the spectra at
+  // every node and the series of FFTs
+  const bool direct = ctx->taylor_req >= 0 || ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0 || l_req > 0;
+  GridShape gs{};
+  const bool gridded = !direct && grid_plan(fp64, n, P, n_active, K, ds, ctx->height, rho_max, 256, &gs);
+  if (gridded) {
+    L = std::min(gs.m, l_max);
+    while (L > 256 && (int64_t)series * (gs.m / L) < 2 * ctx->sm_count) L /= 2;
+    log2L = 0;
+    while ((1 << log2L) < L) ++log2L;
+    D = gs.m / L;
+  }
+  // the spectra from tables in beta (k_grid.cu) where those have far fewer nodes than the
+  // contour; short contours evaluate them at every node
+  int nc_spec = 0;
+  double spec_beta0 = 0, spec_d = 0;
+  spectral_table_shape(fp64, ctx->elem_radius, ctx->beta_max, &nc_spec, &spec_beta0, &spec_d);
+  const bool spec_tab = !direct && 4 * (int64_t)nc_spec <= n;
+
   // ---- buffers
+  if (gridded) {
+    const size_t nw = (size_t)2 * gs.hw * gs.kmax;
+    CFFT_CUDA(ctx->d_gtab.ensure(nw * (gs.n_cells + gs.act_cells) * sizeof(T) + (size_t)(2 * K + 2) * sizeof(cpx<T>)),
+              "alloc gridding");
+    CFFT_CUDA(ctx->d_coarse.ensure((size_t)series * gs.nc * sizeof(cpx<T>)), "alloc gridding");
+  }
+  if (spec_tab) {
+    CFFT_CUDA(ctx->d_snodes.ensure((size_t)8 * nc_spec * sizeof(double2)), "alloc spectra");
+    CFFT_CUDA(ctx->d_spec.ensure((size_t)series * 2 * nc_spec * sizeof(cpx<T>)), "alloc spectra");
+  }
   CFFT_CUDA(ctx->beta_c.ensure(n * sizeof(double2)), "alloc contour");
   CFFT_CUDA(ctx->weight.ensure(n * sizeof(double2)), "alloc contour");
   CFFT_CUDA(ctx->bw.ensure(n * sizeof(double2)), "alloc contour");
@@ -455,10 +521,14 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   double bp_nodes = 0, bp_macs = 0, bp_stencils = 0, tc_int_flops = 0, tc_bp_flops = 0;
   int bp_form_used = 0;
   bool in_tc = false, bp_tc = false;
+  const double2* gp_ch[3] = {ctx->green_p.as<double2>(), ctx->dp_eps.as<double2>(), ctx->dp_h.as<double2>()};
+  const double2* gr_ch[3] = {ctx->green_r.as<double2>(), ctx->dr_eps.as<double2>(), ctx->dr_h.as<double2>()};
   for (int ch = 0; ch < channels; ++ch) {
-  // ---- a2/a3: spectra, kernel, harmonics
+  // ---- a2/a3: spectra, kernel, harmonics: at every contour node, or (spec_tab) once on the
+  // tables' nodes and interpolated per channel (the tables do not depend on the substrate)
+  if (ch == 0 || !spec_tab) {
   IntegrandArgs<T> ia{};
-  ia.n = n;
+  ia.n = spec_tab ? 2 * nc_spec : n;
   ia.n_alpha = n_alpha;
   ia.q_max = ctx->q_max;
   ia.n_cls = cls_c;
@@ -471,11 +541,20 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   ia.q = ctx->d_q.as<cpx<T>>();
   ia.beta_c = ctx->beta_c.as<double2>();
   ia.bw = ctx->bw.as<double2>();
-  const double2* gp_ch[3] = {ctx->green_p.as<double2>(), ctx->dp_eps.as<double2>(), ctx->dp_h.as<double2>()};
-  const double2* gr_ch[3] = {ctx->green_r.as<double2>(), ctx->dr_eps.as<double2>(), ctx->dr_h.as<double2>()};
   ia.green_p = gp_ch[ch];
   ia.green_r = gr_ch[ch];
   ia.y = ctx->d_y.as<cpx<T>>();
+  if (spec_tab) {
+    double2* sn = ctx->d_snodes.as<double2>();
+    launch_spectral_nodes(nc_spec, spec_beta0, spec_d, sn, sn + 2 * nc_spec, sn + 4 * nc_spec, sn + 6 * nc_spec, st);
+    ++launches;
+    CFFT_CUDA(cudaGetLastError(), "spectral nodes kernel");
+    ia.beta_c = sn;
+    ia.bw = sn + 2 * nc_spec;
+    ia.green_p = sn + 4 * nc_spec;
+    ia.green_r = sn + 6 * nc_spec;
+    ia.y = ctx->d_spec.as<cpx<T>>();
+  }
   bool ran_tc = false;
   if constexpr (sizeof(T) == 4) {
     if (tc_spectra) {
@@ -492,13 +571,30 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
         // (padded) basis function x tc_ncol columns, three TF32 products
         const int jt = integrand_tc_nodes(n_alpha);
         const double nb_pad = (double)((ctx->n_basis + kTcBasis - 1) / kTcBasis * kTcBasis);
-        tc_int_flops += (double)((n + jt - 1) / jt) * 3.0 * 2.0 * 256.0 * 4.0 * nb_pad * ia.tc_ncol;
+        tc_int_flops += (double)((ia.n + jt - 1) / jt) * 3.0 * 2.0 * 256.0 * 4.0 * nb_pad * ia.tc_ncol;
       }
     }
   }
   if (!ran_tc) CFFT_CUDA(launch_integrand<T>(ia, ctx->n_mbf_pad, st), "integrand kernel");
   in_tc = in_tc || ran_tc;
   ++launches;
+  }
+  if (spec_tab) {
+    SpecInterpArgs<T> sa{};
+    sa.n = n;
+    sa.nc = nc_spec;
+    sa.series = series;
+    sa.beta0 = spec_beta0;
+    sa.inv_d = 1.0 / spec_d;
+    sa.tab = ctx->d_spec.as<cpx<T>>();
+    sa.beta_c = ctx->beta_c.as<double2>();
+    sa.bw = ctx->bw.as<double2>();
+    sa.green_p = gp_ch[ch];
+    sa.green_r = gr_ch[ch];
+    sa.y = ctx->d_y.as<cpx<T>>();
+    CFFT_CUDA(launch_spectral_interp<T>(sa, st), "spectral interpolation kernel");
+    ++launches;
+  }
   if (ch == 0) CFFT_CUDA(cudaEventRecord(ctx->ev[2], st), "event");
 
   // ---- a4: Taylor terms x pruned zero-padded FFTs
@@ -530,6 +626,21 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   fa.twiddle = ctx->d_tw.as<cpx<T>>();
   if constexpr (sizeof(T) == 4) fa.prec = bp_es ? ctx->d_prec.as<cpx<float>>() : nullptr;
   fa.grid = ctx->d_grid.as<cpx<T>>();
+  if (gridded) {
+    GridArgs<T> ga{};
+    fill_grid_args<T>(&ga, gs, n, series, K, sigma, P, ctx->d_gtab.as<T>());
+    ga.bi_rel = ctx->bi_rel.as<double>();
+    ga.prec = fa.prec;
+    ga.y = fa.y;
+    ga.coarse = ctx->d_coarse.as<cpx<T>>();
+    if (ch == 0) {
+      CFFT_CUDA(launch_grid_tables<T>(ga, st), "gridding tables kernel");
+      ++launches;
+    }
+    CFFT_CUDA(launch_spread<T>(ga, st), "spreading kernel");
+    ++launches;
+    set_gridded_fft<T>(&fa, ga);
+  }
   CFFT_CUDA(launch_fft<T>(fa, st), "fft kernel");
   ++launches;
   if (ch == 0) CFFT_CUDA(cudaEventRecord(ctx->ev[3], st), "event");
@@ -700,8 +811,8 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   in.ms_backproject = ms;
   in.launches = launches;
   in.n_basis = ctx->n_basis;
-  in.work_points = (double)n * n_alpha;
-  in.work_subffts = (double)series * D * n_terms;
+  in.work_points = (double)(spec_tab ? 2 * nc_spec : n) * n_alpha;
+  in.work_subffts = (double)series * D * (gridded ? 1 : n_terms);
   in.work_bp_nodes = bp_nodes;
   in.spectra_tc = in_tc ? 1 : 0;
   in.bp_form = bp_form_used;
@@ -1000,6 +1111,7 @@ struct BatchItemPlan {
   int na_need;   // angular samples the item's own spectra need (a power of two)
   int64_t P;
   double step, ds, beta_abs;
+  GridShape g;   // gridded transform (when every item of the batch takes it)
 };
 
 constexpr size_t kWaveScratch = size_t(24) << 30;  // Y + grid bytes per wave
@@ -1064,12 +1176,37 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   if (l_common < 1024) return fail(ctx, CFFT_ERR_ARG, "batch: sigma * n must be divisible by 1024");
   if (n_alpha % 4 != 0) return fail(ctx, CFFT_ERR_ARG, "n_alpha must be a multiple of 4");
 
+  // the gridded transform and the spectral tables (k_grid.cu), each when every item would
+  // take it in a tabulation of its own; the tables are shared by all items
+  bool gridded = !(ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0);
+  bool direct = !gridded;
+  double beta_top = 0;
+  bool spec_tab = true;   // every item as its single tabulation would choose
+  for (int i = 0; i < n_items; ++i) {
+    BatchItemPlan& p = ip[i];
+    direct = direct || items[i].taylor_order >= 0;
+    gridded = gridded && items[i].taylor_order < 0 &&
+              grid_plan(fp64, p.n, p.P, p.n_active, p.K, p.ds, items[i].height, rho_max, 1024, &p.g);
+    int nc = 0;
+    double b0 = 0, d = 0;
+    spectral_table_shape(fp64, ctx->elem_radius, items[i].beta_max, &nc, &b0, &d);
+    spec_tab = spec_tab && 4 * (int64_t)nc <= p.n;
+    beta_top = std::max(beta_top, items[i].beta_max);
+  }
+  spec_tab = spec_tab && !direct;
+  int nc_spec = 0;
+  double spec_beta0 = 0, spec_d = 0;
+  spectral_table_shape(fp64, ctx->elem_radius, beta_top, &nc_spec, &spec_beta0, &spec_d);
+  auto grid_scratch = [&](const BatchItemPlan& p) {   // spreading weights and output factors, elements of T
+    return ((size_t)2 * p.g.hw * p.g.kmax * (p.g.n_cells + p.g.act_cells) + 2 * (2 * (size_t)p.K + 2) + 3) / 4 * 4;
+  };
+
   // ---- signature (graph and tuning cache key)
   std::string sig = std::to_string(n_items) + ":" + std::to_string(q_max) + ":" + std::to_string(n_rho) +
                     ":" + std::to_string(rho_max) + ":" + std::to_string(sizeof(T)) + ":" +
                     std::to_string(n_alpha) + ":" + std::to_string((size_t)tables) + ":" +
                     std::to_string(ctx->n_basis) + ":" + std::to_string(M) + ":" + std::to_string(bp_taps) + ":" +
-                    std::to_string(bp_kern);
+                    std::to_string(bp_kern) + ":" + std::to_string(gridded) + std::to_string(spec_tab);
   for (int i = 0; i < n_items; ++i)
     sig += ":" + std::to_string(ip[i].n) + "/" + std::to_string(ip[i].taylor) + "/" + std::to_string(ip[i].series) +
            "/" + std::to_string(ip[i].na_need);
@@ -1097,18 +1234,24 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   // ---- waves: consecutive items whose harmonics + transform grids fit the wave scratch
   struct Wave { int i0, i1; };
   std::vector<Wave> waves;
-  size_t max_nodes_wave = 0, max_y = 0, max_grid = 0;
+  size_t max_nodes_wave = 0, max_y = 0, max_grid = 0, max_coarse = 0, max_gtab = 0;
   {
     int i0 = 0;
-    size_t nodes = 0, yb = 0, gb = 0;
+    size_t nodes = 0, yb = 0, gb = 0, cb = 0, tb = 0;
     for (int i = 0; i < n_items; ++i) {
       size_t yi = (size_t)series * ip[i].n * sizeof(cpx<T>);
       size_t gi = (size_t)series * (2 * ip[i].K + 1) * sizeof(cpx<T>);
-      if (i > i0 && yb + gb + yi + gi > kWaveScratch) {
+      const size_t ci = gridded ? (size_t)series * ip[i].g.nc * sizeof(cpx<T>) : 0;
+      const size_t ti = gridded ? grid_scratch(ip[i]) * sizeof(T) : 0;
+      if (i > i0 && yb + gb + cb + tb + yi + gi + ci + ti > kWaveScratch) {
         waves.push_back({i0, i});
         i0 = i;
-        nodes = yb = gb = 0;
+        nodes = yb = gb = cb = tb = 0;
       }
+      cb += ci;
+      tb += ti;
+      max_coarse = std::max(max_coarse, cb);
+      max_gtab = std::max(max_gtab, tb);
       nodes += ip[i].n;
       yb += yi;
       gb += gi;
@@ -1121,6 +1264,11 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   CFFT_CUDA(ctx->b_contour.ensure(max_nodes_wave * (4 * sizeof(double2) + sizeof(double) + sizeof(double2) + 64)), "alloc batch contour");
   CFFT_CUDA(ctx->b_y.ensure(max_y), "alloc batch harmonics");
   CFFT_CUDA(ctx->b_grid.ensure(max_grid), "alloc batch grid");
+  if (gridded) {
+    CFFT_CUDA(ctx->b_coarse.ensure(max_coarse), "alloc batch gridding");
+    CFFT_CUDA(ctx->b_gtab.ensure(max_gtab), "alloc batch gridding");
+  }
+  if (spec_tab) CFFT_CUDA(ctx->d_spec.ensure((size_t)series * 2 * nc_spec * sizeof(cpx<T>)), "alloc spectra");
 
   // contour buffers carved from b_contour: beta_c, weight, bw, green_p, green_r (double2), bi_rel (double)
   double2* c_beta = ctx->b_contour.as<double2>();
@@ -1184,20 +1332,29 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     std::vector<IntegrandArgs<T>> hia(n_items);
     std::vector<FftArgs<T>> hfa(n_items);
     std::vector<BackprojArgs<T>> hba(n_items);
-    std::vector<int2> cmap, imap;
+    std::vector<SpecInterpArgs<T>> hsa(n_items);
+    std::vector<GridArgs<T>> hga(n_items);
+    std::vector<int2> cmap, imap, smap, gmap;   // contour, integrand, interpolation, spreading blocks
     std::vector<int4> ftask, btask;
     std::vector<int> cnodes((size_t)n_items * n_chunks);
     std::vector<int64_t> coff((size_t)n_items * n_chunks);
     struct FftBucket { int log2L; size_t f0, f1; int max_nout; };
     // integrand blocks of a wave: [i0, im) at 128 angles when the counts are split, [im, i1)
     // at n_alpha
-    struct WaveRanges { size_t c0, c1, i0, im, i1, f0, f1, b0, b1; std::vector<FftBucket> fb; };
+    struct WaveRanges {
+      size_t c0, c1, i0, im, i1, f0, f1, b0, b1;
+      std::vector<FftBucket> fb;
+      size_t s0, s1, g0, g1;   // interpolation and spreading blocks
+      int it0, it1;            // items
+    };
     std::vector<WaveRanges> wr;
     int64_t cos_total = 0;
     int max_nodes = 0, max_seg = 0, max_nout = 0, max_active = 0, max_n_item = 0, zt_arrays = 1;
+    int max_hw = 0;
     for (int i = 0; i < n_items; ++i) {
-      max_active = std::max(max_active, ip[i].n_active);
-      max_n_item = std::max(max_n_item, ip[i].n);
+      if (gridded) max_hw = std::max(max_hw, ip[i].g.hw);
+      else max_active = std::max(max_active, ip[i].n_active);
+      max_n_item = std::max(max_n_item, gridded ? ip[i].g.nc : ip[i].n);
       if (ip[i].series == 1) zt_arrays = 2;   // the Chebyshev recurrence keeps two terms
     }
     for (int i = 0; i < n_items; ++i) {
@@ -1230,6 +1387,10 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     for (int i = 0; i < n_items; ++i) {
       const BatchItemPlan& p = ip[i];
       int l = 1;
+      if (gridded) {   // the coarse transform in as few sub-FFTs as the cap L allows
+        li[i] = std::min(L, p.g.m);
+        continue;
+      }
       while ((p.P % (2 * (int64_t)l)) == 0 && 2 * l <= L) l *= 2;
       while (l > 1024 && p.P / l < 4) l /= 2;
       auto smem_of = [&](int ll) {
@@ -1244,14 +1405,16 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       li[i] = l;
     }
     for (const Wave& w : waves) {
-      WaveRanges r{cmap.size(), 0, imap.size(), 0, 0, ftask.size(), 0, btask.size(), 0, {}};
+      WaveRanges r{cmap.size(), 0, imap.size(), 0, 0, ftask.size(), 0, btask.size(), 0, {}, smap.size(), 0,
+                   gmap.size(), 0, w.i0, w.i1};
+      size_t coarse_off = 0, gtab_off = 0;
       // the 128-angle items' integrand blocks first
       for (int i = w.i0; i < w.i1; ++i)
-        if (item_na[i] != n_alpha)
+        if (item_na[i] != n_alpha && !spec_tab)
           for (int j0 = 0; j0 < items[i].n; j0 += jt128) imap.push_back(make_int2(i, j0));
       r.im = imap.size();
       for (int i = w.i0; i < w.i1; ++i)
-        if (item_na[i] == n_alpha)
+        if (item_na[i] == n_alpha && !spec_tab)
           for (int j0 = 0; j0 < items[i].n; j0 += jt) imap.push_back(make_int2(i, j0));
       int64_t node_off = 0, grid_off = 0;
       for (int i = w.i0; i < w.i1; ++i) {
@@ -1293,10 +1456,16 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
           ia.tc_rmax = shape_args.tc_rmax;
           ia.err = ctx->b_flag.as<int>() + 1;
         }
+        if (spec_tab) {
+          SpecInterpArgs<T>& sa = hsa[i];
+          sa = SpecInterpArgs<T>{it.n, nc_spec, series, spec_beta0, 1.0 / spec_d, ctx->d_spec.as<cpx<T>>(),
+                                 ia.beta_c, ia.bw, ia.green_p, ia.green_r, ia.y};
+          for (int j0 = 0; j0 < it.n; j0 += spectral_interp_nodes<T>()) smap.push_back(make_int2(i, j0));
+        }
         const int Li = li[i];
         int log2Li = 0;
         while ((1 << log2Li) < Li) ++log2Li;
-        const int D = (int)(p.P / Li);
+        const int D = (int)((gridded ? (int64_t)p.g.m : p.P) / Li);
         FftArgs<T>& fa = hfa[i];
         fa = FftArgs<T>{};
         fa.series = series;
@@ -1317,10 +1486,23 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         fa.twiddle = ctx->d_tw.as<cpx<T>>();
         if constexpr (sizeof(T) == 4) fa.prec = bp_es ? reinterpret_cast<const cpx<float>*>(c_prec + node_off) : nullptr;
         fa.grid = ctx->b_grid.as<cpx<T>>() + grid_off;
+        if (gridded) {
+          GridArgs<T>& ga = hga[i];
+          ga = GridArgs<T>{};
+          fill_grid_args<T>(&ga, p.g, it.n, series, p.K, sigma, p.P, ctx->b_gtab.as<T>() + gtab_off);
+          ga.bi_rel = fa.bi_rel;
+          ga.prec = fa.prec;
+          ga.y = fa.y;
+          ga.coarse = ctx->b_coarse.as<cpx<T>>() + coarse_off;
+          set_gridded_fft<T>(&fa, ga);
+          for (int i0 = 0; i0 < p.g.nc; i0 += spread_samples()) gmap.push_back(make_int2(i, i0));
+          gtab_off += grid_scratch(p);
+          coarse_off += (size_t)series * p.g.nc;
+        }
         max_nout = std::max(max_nout, (2 * p.K + 1) / D + 2);
         for (int sr = 0; sr < series; ++sr)
           for (int k2 = 0; k2 < D; ++k2) ftask.push_back(make_int4(i, sr, k2, log2Li));
-        work_fft += (double)series * D * (p.taylor + (p.series == 1 ? 2 : 1));
+        work_fft += (double)series * D * (gridded ? 1 : p.taylor + (p.series == 1 ? 2 : 1));
         BackprojArgs<T>& ba = hba[i];
         ba = BackprojArgs<T>{};
         ba.series_per_q = pairs;
@@ -1361,6 +1543,8 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       r.i1 = imap.size();
       r.f1 = ftask.size();
       r.b1 = btask.size();
+      r.s1 = smap.size();
+      r.g1 = gmap.size();
       // FFT tasks of the wave grouped by sub-FFT length (one persistent launch per length),
       // the larger transforms first inside each group
       std::stable_sort(ftask.begin() + r.f0, ftask.end(),
@@ -1370,7 +1554,8 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         int mo = 0;
         while (u < r.f1 && ftask[u].w == ftask[t].w) {
           const int i = ftask[u].x;
-          mo = std::max(mo, (2 * ip[i].K + 1) / (int)(ip[i].P / li[i]) + 2);
+          // a gridded task keeps no outputs in shared memory
+          mo = gridded ? -2 : std::max(mo, (2 * ip[i].K + 1) / (int)(ip[i].P / li[i]) + 2);
           ++u;
         }
         r.fb.push_back(FftBucket{ftask[t].w, t, u, mo});
@@ -1398,6 +1583,24 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     CFFT_CUDA(up(ctx->b_imap, imap.data(), imap.size() * sizeof(int2)), "upload plan");
     CFFT_CUDA(up(ctx->b_ftask, ftask.data(), ftask.size() * sizeof(int4)), "upload plan");
     CFFT_CUDA(up(ctx->b_btask, btask.data(), btask.size() * sizeof(int4)), "upload plan");
+    if (spec_tab) {
+      // nodes of the spectral tables: D with (P, R beta^2) = (1, 0), E with (0, -1)
+      std::vector<double2> hn((size_t)8 * nc_spec);
+      for (int i = 0; i < 2 * nc_spec; ++i) {
+        const bool e = i >= nc_spec;
+        hn[i] = make_double2(spec_beta0 + (i - (e ? nc_spec : 0)) * spec_d, 0.0);
+        hn[2 * nc_spec + i] = make_double2(1.0, 0.0);
+        hn[4 * nc_spec + i] = make_double2(e ? 0.0 : 1.0, 0.0);
+        hn[6 * nc_spec + i] = make_double2(e ? -1.0 : 0.0, 0.0);
+      }
+      CFFT_CUDA(up(ctx->d_snodes, hn.data(), hn.size() * sizeof(double2)), "upload plan");
+      CFFT_CUDA(up(ctx->b_sargs, hsa.data(), hsa.size() * sizeof(SpecInterpArgs<T>)), "upload plan");
+      CFFT_CUDA(up(ctx->b_smap, smap.data(), smap.size() * sizeof(int2)), "upload plan");
+    }
+    if (gridded) {
+      CFFT_CUDA(up(ctx->b_gargs, hga.data(), hga.size() * sizeof(GridArgs<T>)), "upload plan");
+      CFFT_CUDA(up(ctx->b_gmap, gmap.data(), gmap.size() * sizeof(int2)), "upload plan");
+    }
     CFFT_CUDA(up(ctx->b_cnodes, cnodes.data(), cnodes.size() * sizeof(int)), "upload plan");
     CFFT_CUDA(up(ctx->b_coff, coff.data(), coff.size() * sizeof(int64_t)), "upload plan");
     CFFT_CUDA(ctx->b_count.ensure(8 * wr.size() * sizeof(int)), "alloc plan");
@@ -1421,16 +1624,19 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                         (long long)split_na,
                         (long long)n_chunks, (long long)max_nodes, (long long)max_seg, (long long)max_nout,
                         (long long)max_active, (long long)max_n_item, (long long)cos_total,
-                        (long long)zt_arrays})
+                        (long long)zt_arrays, (long long)gridded, (long long)spec_tab, (long long)max_hw,
+                        (long long)(spec_tab ? nc_spec : 0)})
       add(v);
     for (const void* ptr : {ctx->d_tw.p, ctx->b_cnodes.p, ctx->b_coff.p, ctx->b_cos.p, ctx->b_count.p,
                             ctx->b_cargs.p, ctx->b_cdata.p, ctx->b_iargs.p, ctx->b_fargs.p, ctx->b_bargs.p,
                             ctx->b_cmap.p, ctx->b_imap.p, ctx->b_ftask.p, ctx->b_btask.p, ctx->b_flag.p,
                             ctx->b_y.p, ctx->b_grid.p, ctx->b_contour.p, ctx->d_bx.p, ctx->d_by.p, ctx->d_q.p,
-                            ctx->d_shapes.p, ctx->tc_bx.p, ctx->tc_by.p, ctx->tc_bmat_mirror.p})
+                            ctx->d_shapes.p, ctx->tc_bx.p, ctx->tc_by.p, ctx->tc_bmat_mirror.p,
+                            ctx->d_spec.p, ctx->d_snodes.p, ctx->b_sargs.p, ctx->b_smap.p, ctx->b_gargs.p,
+                            ctx->b_gmap.p, ctx->b_coarse.p, ctx->b_gtab.p})
       add((long long)(uintptr_t)ptr);
     for (const WaveRanges& r : wr) {
-      for (size_t v : {r.c0, r.c1, r.i0, r.i1, r.f0, r.f1, r.b0, r.b1}) add((long long)v);
+      for (size_t v : {r.c0, r.c1, r.i0, r.i1, r.f0, r.f1, r.b0, r.b1, r.s0, r.s1, r.g0, r.g1}) add((long long)v);
       for (const FftBucket& fb : r.fb) {
         add(fb.log2L);
         add((long long)fb.f0);
@@ -1456,6 +1662,29 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       ++launches;
       e = cudaMemsetAsync(ctx->b_count.p, 0, 8 * wr.size() * sizeof(int), st);
       if (e != cudaSuccess) return e;
+      // the spectral tables, shared by every item
+      auto issue_tables = [&]() -> cudaError_t {
+        IntegrandArgs<T> ia = shape_args;
+        const double2* sn = ctx->d_snodes.as<double2>();
+        ia.n = 2 * nc_spec;
+        ia.q_max = q_max;
+        ia.n_cls = 1;
+        ia.n_shape = (int)ctx->shapes.size();
+        ia.shapes = ctx->d_shapes.as<ShapeClass>();
+        ia.bx = ctx->d_bx.as<T>();
+        ia.by = ctx->d_by.as<T>();
+        ia.q = ctx->d_q.as<cpx<T>>();
+        ia.beta_c = sn;
+        ia.bw = sn + 2 * nc_spec;
+        ia.green_p = sn + 4 * nc_spec;
+        ia.green_r = sn + 6 * nc_spec;
+        ia.y = ctx->d_spec.as<cpx<T>>();
+        ia.err = ctx->b_flag.as<int>() + 1;
+        ++launches;
+        if constexpr (sizeof(T) == 4)
+          if (tc_b) return launch_integrand_tc(ia, st);
+        return launch_integrand<T>(ia, ctx->n_mbf_pad, st);
+      };
       const size_t n_waves = mode == 3 ? 1 : wr.size();  // tuning times the first wave only
       for (size_t w = 0; w < n_waves; ++w) {
         const WaveRanges& r = wr[w];
@@ -1464,7 +1693,11 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         launch_contour_batch(ctx->b_cargs.as<ContourArgs>(), ctx->b_cdata.as<ContourData>(),
                              ctx->b_cmap.as<int2>() + r.c0, (int)(r.c1 - r.c0), st);
         ++launches;
-        if constexpr (sizeof(T) == 4) {
+        if (spec_tab) {
+          if (w == 0 && (e = issue_tables()) != cudaSuccess) return e;
+          e = launch_spectral_interp_batch<T>(ctx->b_sargs.as<SpecInterpArgs<T>>(), ctx->b_smap.as<int2>() + r.s0,
+                                              (int)(r.s1 - r.s0), series, st);
+        } else if constexpr (sizeof(T) == 4) {
           if (tc_b) {
             e = cudaSuccess;
             if (r.im > r.i0) {
@@ -1489,6 +1722,14 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         if (e != cudaSuccess) return e;
         ++launches;
         if (w == 0) rec(ctx->bev[1]);
+        if (gridded) {
+          e = launch_grid_tables_batch<T>(ctx->b_gargs.as<GridArgs<T>>(), r.it0, r.it1 - r.it0, st);
+          if (e == cudaSuccess)
+            e = launch_spread_batch<T>(ctx->b_gargs.as<GridArgs<T>>(), ctx->b_gmap.as<int2>() + r.g0,
+                                       (int)(r.g1 - r.g0), series, max_hw, st);
+          if (e != cudaSuccess) return e;
+          launches += 2;
+        }
         for (size_t bkt = 0; bkt < r.fb.size() && bkt < 7; ++bkt) {
           const FftBucket& fb = r.fb[bkt];
           e = launch_fft_batch<T>(ctx->b_fargs.as<FftArgs<T>>(), ctx->b_ftask.as<int4>() + fb.f0,
@@ -1666,7 +1907,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->green_r, &ctx->dp_eps, &ctx->dr_eps, &ctx->dp_h, &ctx->dr_h, &ctx->d_shapes, &ctx->d_bx, &ctx->d_by, &ctx->d_q,
                       &ctx->d_y, &ctx->d_grid, &ctx->d_table, &ctx->d_tw, &ctx->d_cnodes,
                       &ctx->d_coff, &ctx->d_cos, &ctx->d_lag, &ctx->d_flag, &ctx->d_pos,
-                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
+                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
                       &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_cand_r, &ctx->lu_cand_d, &ctx->lu_bar, &ctx->lu_err, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
                       &ctx->c_work2, &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
@@ -1679,7 +1920,8 @@ void cfft_destroy(cfft_ctx* ctx) {
     DevBuf* bb[] = {&ctx->b_cargs, &ctx->b_cdata, &ctx->b_iargs, &ctx->b_fargs, &ctx->b_bargs,
                     &ctx->b_cmap, &ctx->b_imap, &ctx->b_ftask, &ctx->b_btask, &ctx->b_count,
                     &ctx->b_cnodes, &ctx->b_coff, &ctx->b_cos, &ctx->b_contour, &ctx->b_y,
-                    &ctx->b_grid, &ctx->b_flag};
+                    &ctx->b_grid, &ctx->b_flag, &ctx->b_sargs, &ctx->b_smap, &ctx->b_gargs, &ctx->b_gmap,
+                    &ctx->b_coarse, &ctx->b_gtab};
     for (DevBuf* b : bb) b->release();
     for (auto& e : ctx->bev)
       if (e) cudaEventDestroy(e);

@@ -233,6 +233,54 @@ struct FftArgs {
   const cpx<T>* twiddle;                      // [sub_len] e^{-2 pi i t / sub_len}
   const cpx<T>* prec;                         // [n] input precorrection (null: none)
   cpx<T>* grid;                               // [series][2K+1]
+  // gridded transform (null: the series of FFTs): y holds the coarse samples, fft_len their
+  // FFT length, and output k is multiplied by out_factor[k + K]
+  const cpx<T>* out_factor;
+};
+
+// ---- spectral tables and gridding (k_grid.cu)
+
+// harmonics on the contour from the element's spectral tables D, E ([series][2][nc], sampled
+// at beta0 + i / inv_d): y = bw (P D - R beta^2 E)
+constexpr int kSpecOver = 8;   // samples per Nyquist step of the tables
+template <class T>
+struct SpecInterpArgs {
+  int n, nc, series;
+  double beta0, inv_d;
+  const cpx<T>* tab;
+  const double2* beta_c;
+  const double2* bw;
+  const double2* green_p;
+  const double2* green_r;
+  cpx<T>* y;               // out [series][n]
+};
+
+// shape of a gridded transform: coarse FFT length m, Gaussian exp(-a z^2) of half width hw
+// cells, at most kmax nodes per cell, cells with nodes and with active nodes, coarse samples
+struct GridShape {
+  int m, hw, kmax, n_cells, act_cells, nc;
+  double a, y_scale;
+};
+// Fills g and returns true when the gridded transform serves this contour and grid: height *
+// rho_max <= 3.5, a coarse grid (m >= 2 (2K + 1), a power of two >= min_m) no finer than the contour's
+// own transform (m <= fft_len) and a Gaussian within the staging buffer.  Otherwise the
+// series of FFTs runs.
+bool grid_plan(bool fp64, int n, int64_t fft_len, int n_active, int grid_half, double ds, double height,
+               double rho_max, int min_m, GridShape* g);
+
+template <class T>
+struct GridArgs {
+  int n, series, grid_half, sigma;
+  int m, hw, kmax, n_cells, act_cells, nc;
+  int64_t fft_len;           // P: node j lies at (j + 1/2) m / P cells
+  double a, y_scale, inv_norm;   // inv_norm = sqrt(a / pi)
+  const double* bi_rel;      // [n]
+  const cpx<T>* prec;        // [n] or null
+  const cpx<T>* y;           // [series][n]
+  T* wre;                    // [2 hw][kmax][n_cells]
+  T* wim;                    // [2 hw][kmax][act_cells]
+  cpx<T>* out_factor;        // [2K + 1]
+  cpx<T>* coarse;            // out [series][nc]
 };
 
 template <class T>
@@ -272,6 +320,28 @@ struct FillArgs {
 };
 
 // host launchers (one translation unit per stage)
+void spectral_table_shape(bool fp64, double elem_radius, double beta_max, int* nc, double* beta0, double* d);
+void launch_spectral_nodes(int nc, double beta0, double d, double2* beta, double2* bw, double2* gp, double2* gr,
+                           cudaStream_t s);
+template <class T>
+cudaError_t launch_spectral_interp(const SpecInterpArgs<T>& a, cudaStream_t s);
+// contour nodes per block of the batched interpolation
+template <class T>
+int spectral_interp_nodes();
+template <class T>
+cudaError_t launch_spectral_interp_batch(const SpecInterpArgs<T>* items, const int2* map, int n_blocks, int series,
+                                         cudaStream_t s);
+template <class T>
+cudaError_t launch_grid_tables(const GridArgs<T>& a, cudaStream_t s);
+template <class T>
+cudaError_t launch_grid_tables_batch(const GridArgs<T>* items, int item0, int n_items, cudaStream_t s);
+template <class T>
+cudaError_t launch_spread(const GridArgs<T>& a, cudaStream_t s);
+// coarse samples per block of the batched spreading
+int spread_samples();
+template <class T>
+cudaError_t launch_spread_batch(const GridArgs<T>* items, const int2* map, int n_blocks, int series, int max_hw,
+                                cudaStream_t s);
 void launch_contour(const ContourArgs& a, const ContourData& d, cudaStream_t s);
 template <class T>
 void launch_twiddle(cpx<T>* tw, int len, cudaStream_t s);

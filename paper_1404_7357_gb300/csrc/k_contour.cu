@@ -162,7 +162,7 @@ __global__ void nonfinite_kernel(const cpx<T>* buf, int64_t count, int* flag) {
 }  // namespace
 
 void launch_contour(const ContourArgs& a, const ContourData& d, cudaStream_t s) {
-  contour_kernel<<<(a.n + 255) / 256, 256, 0, s>>>(a, d);
+  contour_kernel<<<(a.n + 63) / 64, 64, 0, s>>>(a, d);
 }
 
 void launch_contour_batch(const ContourArgs* items, const ContourData* data, const int2* map,

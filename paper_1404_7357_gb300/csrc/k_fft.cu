@@ -19,6 +19,8 @@
 // One CTA owns one (series, k2): it loops over the Taylor terms, runs each
 // length-L FFT in shared memory (radix-4 Stockham passes staged through
 // registers), and accumulates (H s_k)^n/n! times the needed outputs.  The
+// With the gridded transform (k_grid.cu) the same task runs once, on the coarse samples
+// (a.y, length M for P) and multiplies every output by its factor (a.out_factor).  The
 // result is written demodulated by exp(+i beta_max s / 2) so that the
 // back-projection interpolates a function whose spectrum is centred on zero:
 //   grid[series][k + K] = g_q(s_k) exp(i pi k / sigma),   k = -K..K.
@@ -549,7 +551,10 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
   // fac[o]: the running factor of output o's coefficient, (H s)^n / n! for the Taylor
   // series, exp(a) (a/2)^m / m! for the Chebyshev series (a = H s / 2)
   const T dsh = (T)a.ds_height;
-  for (int o = tid; o < n_out; o += NT) {
+  // gridded transform: one term, each needed output used once, written as it is formed
+  const cpx<T>* of = a.out_factor;
+  cpx<T>* out = a.grid + (size_t)series * (2 * K + 1);
+  for (int o = tid; o < n_out && !of; o += NT) {
     acc[o] = mk((T)0, (T)0);
     fac[o] = cheb ? exp((T)0.5 * dsh * (T)(k2 + D * (t_lo + o))) : (T)1;
   }
@@ -629,7 +634,8 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
         const int tt = t <= t_hi ? t : t - L;
         if (tt >= t_lo && tt <= t_hi) {
           const int o = tt - t_lo;
-          acc[o] = acc[o] + coef(o) * v;
+          if (of) out[k2 + D * tt + K] = v * of[k2 + D * tt + K];
+          else acc[o] = acc[o] + coef(o) * v;
         }
       };
       if (t_hi < L / 16 && t_lo > -(L / 16)) last_pass_pruned<T, LOG2L, NT>(buf, thi, tlo, t_lo, t_hi, use);
@@ -643,12 +649,13 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
     for (int o = tid; o < n_out; o += NT) {
       int t = t_lo + o;
       int idx = t & (L - 1);  // t mod L (two's complement)
-      acc[o] = acc[o] + coef(o) * buf[bidx(idx)];
+      if (of) out[k2 + D * t + K] = buf[bidx(idx)] * of[k2 + D * t + K];
+      else acc[o] = acc[o] + coef(o) * buf[bidx(idx)];
     }
     __syncthreads();
   }
+  if (of) return;
   // ---- half-sample phase exp(-i pi k / P) and demodulation exp(+i pi k / sigma)
-  cpx<T>* out = a.grid + (size_t)series * (2 * K + 1);
   const int64_t two_p = 2 * P;
   for (int o = tid; o < n_out; o += NT) {
     int k = k2 + D * (t_lo + o);
@@ -714,7 +721,7 @@ template <class T, int LOG2L>
 cudaError_t launch_l(const FftArgs<T>& a, cudaStream_t s) {
   constexpr int NT = FftShape<LOG2L>::NT;
   const int D = a.n_sub;
-  const int n_out_max = (2 * a.grid_half + 1) / D + 2;
+  const int n_out_max = a.out_factor ? 0 : (2 * a.grid_half + 1) / D + 2;
   const int hi = (a.n + 127) / 128;
   // the stored active inputs pay when at least two terms after the first read them
   const int arrays = a.expansion == 1 ? 2 : 1;
