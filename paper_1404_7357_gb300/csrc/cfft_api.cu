@@ -141,7 +141,7 @@ struct cfft_ctx {
   int lu_diag[5] = {0, 0, 0, 0, 0};
   cfft_solve_info solve_info{};
   // the 2-D Cartesian C-FFT table and its work buffers
-  DevBuf c_tab, c_work, c_work2, c_im, c_gx, c_gy, c_flag;
+  DevBuf c_tab, c_work, c_im, c_gx, c_gy, c_flag;
   bool has_ctab = false;
   cfft_cartesian_info c_info{};
   // tensor-core spectra: float copies of the element and its GEMM B operand
@@ -1910,7 +1910,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
                       &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_cand_r, &ctx->lu_cand_d, &ctx->lu_bar, &ctx->lu_err, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
-                      &ctx->c_work2, &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
+                      &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
                       &ctx->tc_bmat_mirror, &ctx->tc_shapes};
     for (DevBuf* b : bufs) b->release();
     for (auto& e : ctx->ev)
@@ -2651,8 +2651,7 @@ cfft_status cartesian_impl(cfft_ctx* ctx, int n, double rho_max, int order) {
   CFFT_CUDA(cudaStreamSynchronize(st), "upload");   // the staging vectors die at scope end
   const size_t big = (size_t)pairs * p * p * es;
   CFFT_CUDA(ctx->c_tab.ensure(big), "alloc Cartesian table");
-  CFFT_CUDA(ctx->c_work.ensure(big), "alloc Cartesian work");
-  CFFT_CUDA(ctx->c_work2.ensure(big), "alloc Cartesian work");
+  CFFT_CUDA(ctx->c_work.ensure(big / 2), "alloc Cartesian work");
   CFFT_CUDA(ctx->c_im.ensure((size_t)pairs * n * n * es), "alloc Cartesian spectrum");
   CFFT_CUDA(ctx->c_gx.ensure((size_t)n * n * sizeof(T)), "alloc Cartesian spectrum");
   CFFT_CUDA(ctx->c_gy.ensure((size_t)n * n * sizeof(T)), "alloc Cartesian spectrum");
@@ -2681,8 +2680,7 @@ cfft_status cartesian_impl(cfft_ctx* ctx, int n, double rho_max, int order) {
     if (!e) CFFT_CUDA(cudaEventCreate(&e), "event");
   CFFT_CUDA(cudaEventRecord(ctx->ev[0], st), "event");
   cudaError_t e = cartesian_tabulate<T>(a, order, ctx->c_tab.as<cpx<T>>(), ctx->c_work.as<cpx<T>>(),
-                                        ctx->c_work2.as<cpx<T>>(), ctx->c_im.as<cpx<T>>(), ctx->c_gx.as<T>(),
-                                        ctx->c_gy.as<T>(), st);
+                                        ctx->c_im.as<cpx<T>>(), ctx->c_gx.as<T>(), ctx->c_gy.as<T>(), st);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "Cartesian C-FFT");
   CFFT_CUDA(cudaEventRecord(ctx->ev[1], st), "event");
   CFFT_CUDA(cudaMemsetAsync(ctx->c_flag.p, 0, sizeof(int), st), "flag");

@@ -488,11 +488,11 @@ struct CartArgs {
   const T* by;
   const cpx<T>* q;   // [n_basis][q_stride], bases sorted by shape class
 };
-// the refined table [pairs][2N][2N] (dx-major) up to Taylor order `order`; work, work2:
-// [pairs][2N][2N]; im: [pairs][N][N]; gx, gy: [N][N]
+// the refined table [pairs][2N][2N] (dx-major) up to Taylor order `order`; work: [pairs][N][2N]
+// (row transforms of one power); im: [pairs][N][N]; gx, gy: [N][N]
 template <class T>
-cudaError_t cartesian_tabulate(const CartArgs<T>& a, int order, cpx<T>* table, cpx<T>* work, cpx<T>* work2,
-                               cpx<T>* im, T* gx, T* gy, cudaStream_t s);
+cudaError_t cartesian_tabulate(const CartArgs<T>& a, int order, cpx<T>* table, cpx<T>* work, cpx<T>* im, T* gx,
+                               T* gy, cudaStream_t s);
 template <class T, class TO>
 cudaError_t cartesian_fill(const cpx<T>* table, int p, int m, double x0, double step, double rho_max, int n_el,
                            const double* pos, void* z, int64_t ld, int* err, cudaStream_t s);
