@@ -317,6 +317,7 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
       }
     }
     __syncthreads();
+#pragma unroll 2
     for (int t = 0; t < taps; ++t) {
       const int c = i - t;
       if (c < 0 || c >= a.n_cells) continue;
@@ -324,9 +325,15 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
       const T* wr = a.wre + ((int64_t)t * a.kmax + k0) * a.n_cells + c;
       const T* wi = a.wim + ((int64_t)t * a.kmax + k0) * a.act_cells + c;
       const float4* yp = ys + (c - c_lo);
-      for (int k = 0; k < kc; ++k) {
-        const T w = wr[(int64_t)k * a.n_cells];
-        const T q = act ? wi[(int64_t)k * a.act_cells] : (T)0;
+      // a cell's weights first (independent loads in flight), then its nodes
+      T w[kKc], q[kKc];
+#pragma unroll
+      for (int k = 0; k < kKc; ++k) {
+        w[k] = k < kc ? wr[(int64_t)k * a.n_cells] : (T)0;
+        q[k] = act && k < kc ? wi[(int64_t)k * a.act_cells] : (T)0;
+      }
+#pragma unroll
+      for (int k = 0; k < kKc; ++k) {
 #pragma unroll
         for (int v = 0; v < kSpreadVec; ++v) {
           cpx<T> y[PER];
@@ -341,11 +348,11 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
 #pragma unroll
           for (int u = 0; u < PER; ++u) {
             cpx<T>& z = acc[v * PER + u];
-            z.re = fma(w, y[u].re, z.re);
-            z.im = fma(w, y[u].im, z.im);
+            z.re = fma(w[k], y[u].re, z.re);
+            z.im = fma(w[k], y[u].im, z.im);
             if (act) {
-              z.re = fma(-q, y[u].im, z.re);
-              z.im = fma(q, y[u].re, z.im);
+              z.re = fma(-q[k], y[u].im, z.re);
+              z.im = fma(q[k], y[u].re, z.im);
             }
           }
         }
@@ -379,8 +386,9 @@ __global__ void __launch_bounds__(kSpreadThreads) spread_batch_kernel(const Grid
 size_t spread_smem(int hw) { return (size_t)kSpreadVec * kKc * ((kSpreadThreads + 2 * hw - 1) | 1) * 16; }
 
 int series_chunk(int series, int tiles) {
-  // about four blocks per SM, at least four series per block (its weights are formed once)
-  const int want = std::max(1, 4 * current_sm_count() / std::max(1, tiles));
+  // about sixteen blocks per SM (the table loads' latency needs that many warps: 72 us with
+  // four on the full-size patch), at least four series per block (its weights are formed once)
+  const int want = std::max(1, 16 * current_sm_count() / std::max(1, tiles));
   return std::max(std::min(series, 4), (series + want - 1) / want);
 }
 
