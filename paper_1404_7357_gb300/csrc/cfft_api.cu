@@ -115,12 +115,12 @@ struct cfft_ctx {
   DevBuf beta_c, weight, bw, bi_rel, green_p, green_r, dp_eps, dr_eps, dp_h, dr_h;
   int channels = 1;  // 1: table; 3: table, d/d eps_r, d/d h
   DevBuf d_shapes, d_bx, d_by, d_q, d_y, d_grid, d_table, d_tw, d_cnodes, d_coff, d_cos, d_lag, d_prec,
-      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_gres, d_gtab, d_coarse, d_snodes, d_spec;
+      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_gres, d_gtab, d_coarse, d_snodes, d_spec, d_sum;
   int tw_len = 0, tw_prec = -1;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   // batched sweep: plan arrays, scratch, stream, captured graph, tuned shape
   DevBuf b_cargs, b_cdata, b_iargs, b_fargs, b_bargs, b_cmap, b_imap, b_ftask, b_btask, b_count,
-      b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag, b_sargs, b_smap, b_gargs, b_gmap, b_coarse, b_gtab;
+      b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag, b_sargs, b_smap, b_gargs, b_gmap, b_coarse, b_gtab, b_sum, b_margs, b_omap, b_fmap, b_nmap;
   cudaStream_t bstream = nullptr;
   cudaEvent_t bev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t bgraph = nullptr;
@@ -318,6 +318,29 @@ void fill_grid_args(GridArgs<T>* ga, const GridShape& g, int n, int series, int 
   ga->wim = ga->wre + (size_t)2 * g.hw * g.kmax * g.n_cells;
 }
 
+// the sample sums of the back-projection `ba`, their buffers at `buf`: folded samples, far
+// sums, row weights
+template <class T>
+void set_sum_args(SumArgs<T>* sa, const SumPlan& p, const BackprojArgs<T>& ba, T* buf) {
+  sa->series_per_q = ba.series_per_q;
+  sa->n_harm = ba.n_harm;
+  sa->q_max = ba.q_max;
+  sa->n_rho = ba.n_rho;
+  sa->grid_half = ba.grid_half;
+  sa->sigma = ba.sigma;
+  sa->n_cells = p.cells;
+  sa->cell_rows = p.cell_rows;
+  sa->k_used = p.k_used;
+  sa->k_pad = p.k_pad;
+  sa->d_rho = ba.d_rho;
+  sa->d_s = ba.d_s;
+  sa->grid = ba.grid;
+  sa->table = ba.table;
+  sa->fold = buf;
+  sa->far = reinterpret_cast<cpx<T>*>(buf + p.fold);     // p.fold is a multiple of 64
+  sa->wrow = sa->far + p.far;
+}
+
 // the transform task of a gridded transform: one term over the coarse samples, length m
 template <class T>
 void set_gridded_fft(FftArgs<T>* fa, const GridArgs<T>& ga) {
@@ -383,9 +406,19 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   const int n_terms = taylor + (sc.series == 1 ? 2 : 1);
   const int64_t P = (int64_t)sigma * n;
   const double ds = 2.0 * kPi / ((double)P * step);
-  const int K = (int)std::ceil(rho_max / ds) + bp_taps / 2 + 2;
+  int K = (int)std::ceil(rho_max / ds) + bp_taps / 2 + 2;
   if (2 * (int64_t)K + 1 > P)
     return fail(ctx, CFFT_ERR_ARG, "rho_max exceeds the unaliased range 2 pi / step of the contour");
+  // an explicit order, series or sub-FFT length asks for the direct pipeline: the spectra at
+  // every node, the series of FFTs, the quadrature in alpha for every row
+  const bool direct = ctx->taylor_req >= 0 || ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0 || ctx->opt[CFFT_OPT_FFT_SUB_LEN] > 0;
+  // sums over the grid samples (k_backproject_sum.cu) beside the matrix forms; they read a few
+  // samples more
+  bool sums = !direct && !(ctx->opt[CFFT_OPT_BP_GATHER] > 0) && (fp64 || !(ctx->opt[CFFT_OPT_BP_SIMT] > 0));
+  if (sums) {
+    const int need = (int)std::ceil(rho_max / ds) + sum_grid_extra(fp64, bp_taps, bp_es ? 1 : 0);
+    if (2 * (int64_t)need + 1 <= P) K = std::max(K, need);
+  }
   // sub-FFT length: power of two dividing P, within shared memory
   const int l_max = fp64 ? 8192 : 16384;
   int L = 1;
@@ -408,9 +441,6 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   if (ctx->height <= 0) n_active = 0;
   if (n_active < 0) n_active = 0;
 
-  // an explicit order, series or sub-FFT length asks for the direct pipeline: the spectra at
-  // every node and the series of FFTs
-  const bool direct = ctx->taylor_req >= 0 || ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0 || l_req > 0;
   GridShape gs{};
   const bool gridded = !direct && grid_plan(fp64, n, P, n_active, K, ds, ctx->height, rho_max, 256, &gs);
   if (gridded) {
@@ -657,6 +687,14 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   const int rchunk = pform ? backproject_pm_rows() : (wform ? backproject_w_rows() : 32);
   const int n_chunks = (n_rho + rchunk - 1) / rchunk;
   const double d_rho = rho_max / (n_rho - 1);
+  // rows formed by sums over the grid samples; the matrix forms then run on the chunks of the
+  // rows below (all harmonics' first rows lie in the first n_low chunks)
+  SumPlan sp{};
+  sums = sums && (tform || wform) &&
+         sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q, &sp);
+  const int n_low = sums ? std::min(n_chunks, (sum_first_row(d_rho / ds, ctx->q_max, fp64) + rchunk - 1) / rchunk)
+                         : n_chunks;
+  int low_nodes = 0;
   std::vector<int> cn(n_chunks);
   std::vector<int64_t> coff(n_chunks);
   int64_t tot = 0;
@@ -672,7 +710,8 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
     cn[c] = alpha_nodes(beta_abs_max, rho_top, ctx->q_max, margin, alpha_cbrt_coef(fp64));
     const int rows_c = r_top + 1 - c * rchunk;
     bp_nodes += (double)cn[c] * rows_c * series;
-    if (pform || wform) {
+    if (c < n_low) low_nodes = std::max(low_nodes, cn[c]);
+    if ((pform || wform) && c < n_low) {
       // matrix columns: both signs of k (matrix form) or k >= -(taps/2) with the grid folded
       // about k = 0 (paired-harmonic form, which also visits only the nodes alpha <= pi/2)
       const int kmax_c = std::min(K - 1, (int)std::ceil(rho_top / ds) + bp_taps);
@@ -705,8 +744,8 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   CFFT_CUDA(cudaMemcpyAsync(ctx->d_coff.p, coff.data(), n_chunks * sizeof(int64_t), cudaMemcpyHostToDevice, st), "upload");
   CFFT_CUDA(cudaMemcpyAsync(ctx->d_lag.p, lag.data(), bp_taps * sizeof(double), cudaMemcpyHostToDevice, st), "upload");
   if (ch == 0) {
-    CFFT_CUDA(launch_chunk_cosines(ctx->d_cnodes.as<int>(), ctx->d_coff.as<int64_t>(), n_chunks,
-                                   max_nodes, ctx->d_cos.as<double>(), st), "cosine kernel");
+    CFFT_CUDA(launch_chunk_cosines(ctx->d_cnodes.as<int>(), ctx->d_coff.as<int64_t>(), n_low,
+                                   low_nodes, ctx->d_cos.as<double>(), st), "cosine kernel");
     ++launches;
   }
   int group = 8;
@@ -736,6 +775,18 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   ba.grid = ctx->d_grid.as<cpx<T>>();
   ba.table = dst.as<cpx<T>>() + ch * table_elems;
   ba.kern = bp_es ? 1 : 0;
+  if (sums) {
+    SumArgs<T> sa{};
+    CFFT_CUDA(ctx->d_sum.ensure(sp.fold * sizeof(T) + (sp.far + sp.wrow) * sizeof(cpx<T>)), "alloc back-projection");
+    set_sum_args<T>(&sa, sp, ba, ctx->d_sum.as<T>());
+    CFFT_CUDA(launch_backproject_sum<T>(sa, bp_taps, ba.kern, sp.splits, sp.tiles, st), "back-projection sums");
+    launches += sp.splits > 1 ? 5 : 4;
+    ba.low_h = d_rho / ds;
+    // real weights: half a complex multiply-add each, over the near window of every row and
+    // the cells' points
+    bp_macs += 0.5 * series * ((double)n_rho * (2.0 * sp.cell_rows * ba.low_h + 40.0) +
+                               0.5 * sp.cells * (fp64 ? 20.0 : 10.0) * sp.k_used);
+  }
   bp_form_used = tform ? 3 : (pform ? 2 : (wform ? 1 : 0));
   if (pform || wform) {
     ba.chunk_nodes = ctx->d_cnodes.as<int>();
@@ -744,15 +795,15 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
     if constexpr (sizeof(T) == 4) {
       if (tform) {
         ba.err = ctx->d_flag.as<int>() + 2;
-        CFFT_CUDA(launch_backproject_tc(ba, n_chunks, max_nodes, st), "backprojection kernel (tensor cores)");
+        CFFT_CUDA(launch_backproject_tc(ba, n_low, low_nodes, st), "backprojection kernel (tensor cores)");
         bp_tc = true;
       } else if (pform) {
         CFFT_CUDA(launch_backproject_pm(ba, n_chunks, max_nodes, st), "backprojection kernel");
       } else {
-        CFFT_CUDA(launch_backproject_w<T>(ba, n_chunks, max_nodes, st), "backprojection kernel");
+        CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, st), "backprojection kernel");
       }
     } else {
-      CFFT_CUDA(launch_backproject_w<T>(ba, n_chunks, max_nodes, st), "backprojection kernel");
+      CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, st), "backprojection kernel");
     }
   } else {
     CFFT_CUDA(launch_backproject_impl<T>(ba, ctx->d_cnodes.as<int>(), ctx->d_coff.as<int64_t>(),
@@ -1111,6 +1162,7 @@ struct BatchItemPlan {
   int na_need;   // angular samples the item's own spectra need (a power of two)
   int64_t P;
   double step, ds, beta_abs;
+  SumPlan sum;   // rows formed by sums over the grid samples (sum.cells = 0: none)
   GridShape g;   // gridded transform (when every item of the batch takes it)
 };
 
@@ -1176,6 +1228,23 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   if (l_common < 1024) return fail(ctx, CFFT_ERR_ARG, "batch: sigma * n must be divisible by 1024");
   if (n_alpha % 4 != 0) return fail(ctx, CFFT_ERR_ARG, "n_alpha must be a multiple of 4");
 
+  // sums over the grid samples, as in the single tabulation
+  bool any_sum = false;
+  {
+    bool allowed = !(ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0) && (tform_b || fp64);
+    for (int i = 0; i < n_items; ++i) allowed = allowed && items[i].taylor_order < 0;
+    for (int i = 0; i < n_items; ++i) {
+      BatchItemPlan& p = ip[i];
+      p.sum = SumPlan{};
+      if (!allowed) continue;
+      const int need = (int)std::ceil(rho_max / p.ds) + sum_grid_extra(fp64, bp_taps, bp_kern);
+      if (2 * (int64_t)need + 1 <= p.P) p.K = std::max(p.K, need);
+      any_sum = sum_plan(fp64, n_rho, d_rho, p.ds, sigma, p.K, bp_taps, bp_kern, q_max, pairs, &p.sum) || any_sum;
+    }
+  }
+  auto sum_scratch = [&](const BatchItemPlan& p) {   // elements of T, a multiple of 4
+    return (p.sum.fold + 2 * (p.sum.far + p.sum.wrow) + 3) / 4 * 4;
+  };
   // the gridded transform and the spectral tables (k_grid.cu), each when every item would
   // take it in a tabulation of its own; the tables are shared by all items
   bool gridded = !(ctx->opt[CFFT_OPT_CONTOUR_SERIES] > 0);
@@ -1234,24 +1303,27 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   // ---- waves: consecutive items whose harmonics + transform grids fit the wave scratch
   struct Wave { int i0, i1; };
   std::vector<Wave> waves;
-  size_t max_nodes_wave = 0, max_y = 0, max_grid = 0, max_coarse = 0, max_gtab = 0;
+  size_t max_nodes_wave = 0, max_y = 0, max_grid = 0, max_coarse = 0, max_gtab = 0, max_sum = 0;
   {
     int i0 = 0;
-    size_t nodes = 0, yb = 0, gb = 0, cb = 0, tb = 0;
+    size_t nodes = 0, yb = 0, gb = 0, cb = 0, tb = 0, sb = 0;
     for (int i = 0; i < n_items; ++i) {
       size_t yi = (size_t)series * ip[i].n * sizeof(cpx<T>);
       size_t gi = (size_t)series * (2 * ip[i].K + 1) * sizeof(cpx<T>);
       const size_t ci = gridded ? (size_t)series * ip[i].g.nc * sizeof(cpx<T>) : 0;
       const size_t ti = gridded ? grid_scratch(ip[i]) * sizeof(T) : 0;
-      if (i > i0 && yb + gb + cb + tb + yi + gi + ci + ti > kWaveScratch) {
+      const size_t si = sum_scratch(ip[i]) * sizeof(T);
+      if (i > i0 && yb + gb + cb + tb + sb + yi + gi + ci + ti + si > kWaveScratch) {
         waves.push_back({i0, i});
         i0 = i;
-        nodes = yb = gb = cb = tb = 0;
+        nodes = yb = gb = cb = tb = sb = 0;
       }
       cb += ci;
       tb += ti;
       max_coarse = std::max(max_coarse, cb);
       max_gtab = std::max(max_gtab, tb);
+      sb += si;
+      max_sum = std::max(max_sum, sb);
       nodes += ip[i].n;
       yb += yi;
       gb += gi;
@@ -1268,6 +1340,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     CFFT_CUDA(ctx->b_coarse.ensure(max_coarse), "alloc batch gridding");
     CFFT_CUDA(ctx->b_gtab.ensure(max_gtab), "alloc batch gridding");
   }
+  if (any_sum) CFFT_CUDA(ctx->b_sum.ensure(max_sum), "alloc batch back-projection");
   if (spec_tab) CFFT_CUDA(ctx->d_spec.ensure((size_t)series * 2 * nc_spec * sizeof(cpx<T>)), "alloc spectra");
 
   // contour buffers carved from b_contour: beta_c, weight, bw, green_p, green_r (double2), bi_rel (double)
@@ -1334,7 +1407,11 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     std::vector<BackprojArgs<T>> hba(n_items);
     std::vector<SpecInterpArgs<T>> hsa(n_items);
     std::vector<GridArgs<T>> hga(n_items);
+    std::vector<SumArgs<T>> hma(n_items);
     std::vector<int2> cmap, imap, smap, gmap;   // contour, integrand, interpolation, spreading blocks
+    std::vector<int2> omap, fmap, nmap;          // folding, far and near blocks of the sample sums
+    const bool sum_b = any_sum && (fp64 || tform_b);   // beside the tensor-core or the FP64 form
+    int max_splits = 1;
     std::vector<int4> ftask, btask;
     std::vector<int> cnodes((size_t)n_items * n_chunks);
     std::vector<int64_t> coff((size_t)n_items * n_chunks);
@@ -1345,6 +1422,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       size_t c0, c1, i0, im, i1, f0, f1, b0, b1;
       std::vector<FftBucket> fb;
       size_t s0, s1, g0, g1;   // interpolation and spreading blocks
+      size_t o0, o1, h0, h1, n0, n1;   // folding, far and near blocks
       int it0, it1;            // items
     };
     std::vector<WaveRanges> wr;
@@ -1406,8 +1484,8 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     }
     for (const Wave& w : waves) {
       WaveRanges r{cmap.size(), 0, imap.size(), 0, 0, ftask.size(), 0, btask.size(), 0, {}, smap.size(), 0,
-                   gmap.size(), 0, w.i0, w.i1};
-      size_t coarse_off = 0, gtab_off = 0;
+                   gmap.size(), 0, omap.size(), 0, fmap.size(), 0, nmap.size(), 0, w.i0, w.i1};
+      size_t coarse_off = 0, gtab_off = 0, sum_off = 0;
       // the 128-angle items' integrand blocks first
       for (int i = w.i0; i < w.i1; ++i)
         if (item_na[i] != n_alpha && !spec_tab)
@@ -1525,14 +1603,27 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         ba.cosv = ctx->b_cos.as<double>();
         ba.err = tform_b ? ctx->b_flag.as<int>() + 1 : nullptr;
         ba.kern = bp_es ? 1 : 0;
+        hma[i] = SumArgs<T>{};
+        const bool sum_i = sum_b && p.sum.cells > 0;
+        if (sum_i) {
+          set_sum_args<T>(&hma[i], p.sum, ba, ctx->b_sum.as<T>() + sum_off);
+          sum_off += sum_scratch(p);
+          ba.low_h = d_rho / p.ds;
+          max_splits = std::max(max_splits, p.sum.splits);
+          for (int k = 0; k < p.sum.k_pad; k += sum_fold_samples()) omap.push_back(make_int2(i, k));
+          for (int t = p.sum.tiles - 1; t >= 0; --t) fmap.push_back(make_int2(i, t * sum_tile_rows()));
+          for (int row = 0; row < n_rho; row += sum_tile_rows()) nmap.push_back(make_int2(i, row));
+        }
         for (int c = n_chunks - 1; c >= 0; --c) {  // larger rho (more nodes) first
           int rows = std::min((c + 1) * rchunk, n_rho) - c * rchunk;
+          auto low = [&](int q) { return !sum_i || c * rchunk < sum_first_row(ba.low_h, q, fp64); };
           if (pform_b) {
             const int n_sc = (pairs + backproject_pm_series_chunk() - 1) / backproject_pm_series_chunk();
             for (int pq = 0; pq <= q_max; ++pq)
-              for (int sc = 0; sc < n_sc; ++sc) btask.push_back(make_int4(i, pq, c, sc));
+              for (int sc = 0; sc < n_sc && low(pq); ++sc) btask.push_back(make_int4(i, pq, c, sc));
           } else {
-            for (int q = 0; q < nh; ++q) btask.push_back(make_int4(i, q, c, 0));
+            for (int q = 0; q < nh; ++q)
+              if (low(std::abs(q - q_max))) btask.push_back(make_int4(i, q, c, 0));
           }
           work_bp += (double)cnodes[(size_t)i * n_chunks + c] * rows * series;
         }
@@ -1545,6 +1636,9 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       r.b1 = btask.size();
       r.s1 = smap.size();
       r.g1 = gmap.size();
+      r.o1 = omap.size();
+      r.h1 = fmap.size();
+      r.n1 = nmap.size();
       // FFT tasks of the wave grouped by sub-FFT length (one persistent launch per length),
       // the larger transforms first inside each group
       std::stable_sort(ftask.begin() + r.f0, ftask.end(),
@@ -1597,6 +1691,12 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       CFFT_CUDA(up(ctx->b_sargs, hsa.data(), hsa.size() * sizeof(SpecInterpArgs<T>)), "upload plan");
       CFFT_CUDA(up(ctx->b_smap, smap.data(), smap.size() * sizeof(int2)), "upload plan");
     }
+    if (sum_b) {
+      CFFT_CUDA(up(ctx->b_margs, hma.data(), hma.size() * sizeof(SumArgs<T>)), "upload plan");
+      CFFT_CUDA(up(ctx->b_omap, omap.data(), omap.size() * sizeof(int2)), "upload plan");
+      CFFT_CUDA(up(ctx->b_fmap, fmap.data(), fmap.size() * sizeof(int2)), "upload plan");
+      CFFT_CUDA(up(ctx->b_nmap, nmap.data(), nmap.size() * sizeof(int2)), "upload plan");
+    }
     if (gridded) {
       CFFT_CUDA(up(ctx->b_gargs, hga.data(), hga.size() * sizeof(GridArgs<T>)), "upload plan");
       CFFT_CUDA(up(ctx->b_gmap, gmap.data(), gmap.size() * sizeof(int2)), "upload plan");
@@ -1625,7 +1725,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                         (long long)n_chunks, (long long)max_nodes, (long long)max_seg, (long long)max_nout,
                         (long long)max_active, (long long)max_n_item, (long long)cos_total,
                         (long long)zt_arrays, (long long)gridded, (long long)spec_tab, (long long)max_hw,
-                        (long long)(spec_tab ? nc_spec : 0)})
+                        (long long)sum_b, (long long)max_splits, (long long)(spec_tab ? nc_spec : 0)})
       add(v);
     for (const void* ptr : {ctx->d_tw.p, ctx->b_cnodes.p, ctx->b_coff.p, ctx->b_cos.p, ctx->b_count.p,
                             ctx->b_cargs.p, ctx->b_cdata.p, ctx->b_iargs.p, ctx->b_fargs.p, ctx->b_bargs.p,
@@ -1633,10 +1733,13 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                             ctx->b_y.p, ctx->b_grid.p, ctx->b_contour.p, ctx->d_bx.p, ctx->d_by.p, ctx->d_q.p,
                             ctx->d_shapes.p, ctx->tc_bx.p, ctx->tc_by.p, ctx->tc_bmat_mirror.p,
                             ctx->d_spec.p, ctx->d_snodes.p, ctx->b_sargs.p, ctx->b_smap.p, ctx->b_gargs.p,
-                            ctx->b_gmap.p, ctx->b_coarse.p, ctx->b_gtab.p})
+                            ctx->b_gmap.p, ctx->b_coarse.p, ctx->b_gtab.p, ctx->b_sum.p, ctx->b_margs.p,
+                            ctx->b_omap.p, ctx->b_fmap.p, ctx->b_nmap.p})
       add((long long)(uintptr_t)ptr);
     for (const WaveRanges& r : wr) {
-      for (size_t v : {r.c0, r.c1, r.i0, r.i1, r.f0, r.f1, r.b0, r.b1, r.s0, r.s1, r.g0, r.g1}) add((long long)v);
+      for (size_t v : {r.c0, r.c1, r.i0, r.i1, r.f0, r.f1, r.b0, r.b1, r.s0, r.s1, r.g0, r.g1, r.o0, r.o1, r.h0, r.h1, r.n0,
+                       r.n1})
+        add((long long)v);
       for (const FftBucket& fb : r.fb) {
         add(fb.log2L);
         add((long long)fb.f0);
@@ -1739,6 +1842,15 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
           ++launches;
         }
         if (w == 0) rec(ctx->bev[2]);
+        if (r.n1 > r.n0) {
+          e = launch_backproject_sum_batch<T>(ctx->b_margs.as<SumArgs<T>>(), r.it0, r.it1 - r.it0, n_rho,
+                                              ctx->b_omap.as<int2>() + r.o0, (int)(r.o1 - r.o0),
+                                              ctx->b_fmap.as<int2>() + r.h0, (int)(r.h1 - r.h0),
+                                              ctx->b_nmap.as<int2>() + r.n0, (int)(r.n1 - r.n0), max_splits, q_max,
+                                              pairs, bp_taps, bp_kern, st);
+          if (e != cudaSuccess) return e;
+          launches += 5;
+        }
         if constexpr (sizeof(T) == 4) {
           if (tform_b)
             e = launch_backproject_tc_batch(ctx->b_bargs.as<BackprojArgs<float>>(),
@@ -1907,7 +2019,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->green_r, &ctx->dp_eps, &ctx->dr_eps, &ctx->dp_h, &ctx->dr_h, &ctx->d_shapes, &ctx->d_bx, &ctx->d_by, &ctx->d_q,
                       &ctx->d_y, &ctx->d_grid, &ctx->d_table, &ctx->d_tw, &ctx->d_cnodes,
                       &ctx->d_coff, &ctx->d_cos, &ctx->d_lag, &ctx->d_flag, &ctx->d_pos,
-                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
+                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
                       &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_cand_r, &ctx->lu_cand_d, &ctx->lu_bar, &ctx->lu_err, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
                       &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
@@ -1921,7 +2033,8 @@ void cfft_destroy(cfft_ctx* ctx) {
                     &ctx->b_cmap, &ctx->b_imap, &ctx->b_ftask, &ctx->b_btask, &ctx->b_count,
                     &ctx->b_cnodes, &ctx->b_coff, &ctx->b_cos, &ctx->b_contour, &ctx->b_y,
                     &ctx->b_grid, &ctx->b_flag, &ctx->b_sargs, &ctx->b_smap, &ctx->b_gargs, &ctx->b_gmap,
-                    &ctx->b_coarse, &ctx->b_gtab};
+                    &ctx->b_coarse, &ctx->b_gtab, &ctx->b_sum, &ctx->b_margs, &ctx->b_omap, &ctx->b_fmap,
+                    &ctx->b_nmap};
     for (DevBuf* b : bb) b->release();
     for (auto& e : ctx->bev)
       if (e) cudaEventDestroy(e);

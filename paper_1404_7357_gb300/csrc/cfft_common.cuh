@@ -4,6 +4,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 #include <vector>
@@ -297,7 +298,50 @@ struct BackprojArgs {
   const double* cosv;      // node cosines
   int* err;                // tensor-core form: bit 5 set when a wait ran past its bound
   int kern;                // interpolation kernel: 0 Lagrange, 1 ES (precorrected grid)
+  // > 0: only the rows below sum_first_row(low_h, |q|) are formed (the sample sums form the
+  // others); the rho step in grid samples
+  double low_h;
 };
+
+// first row that the sums over grid samples serve for harmonics +-p (k_backproject_sum.cu); h:
+// the rho step in grid samples
+__host__ __device__ inline int sum_first_row(double h, int p, bool fp64) {
+  const double u = (fp64 ? 1.6 : 0.8) * (double)p * (double)p;
+  const double r = ceil((u > 48.0 ? u : 48.0) / h);
+  return r < 2.0e9 ? (int)r : 2000000000;
+}
+
+// back-projection by sums over the grid samples
+template <class T>
+struct SumArgs {
+  int series_per_q, n_harm, q_max, n_rho, grid_half, sigma;
+  int n_cells, cell_rows;  // n_cells = 0: not in use
+  int k_used, k_pad;       // samples k >= 0 the rows read, and the folded arrays' length
+  double d_rho, d_s;
+  const cpx<T>* grid;      // [series][2K+1]
+  cpx<T>* table;           // [series][n_rho]
+  cpx<T>* wrow;            // [end sample][n_rho]
+  T* fold;                 // [|q|][chunk][G+, i G-][k_pad][64]
+  cpx<T>* far;             // [split][|q|][chunk][cell][point][32]
+};
+struct SumPlan {
+  int cells, cell_rows, k_used, k_pad, splits, tiles;
+  size_t fold, far, wrow;  // elements of the three buffers (real, complex, complex)
+};
+// false (and an empty plan) where the sums do not serve: another zero padding than the end
+// weights were made for, a grid that ends before the end samples, no row far enough out
+bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int grid_half, int taps, int kern, int q_max,
+              int series_per_q, SumPlan* p);
+int sum_grid_extra(bool fp64, int taps, int kern);
+int sum_tile_rows();
+int sum_fold_samples();
+template <class T>
+cudaError_t launch_backproject_sum(const SumArgs<T>& a, int taps, int kern, int splits, int tiles, cudaStream_t s);
+template <class T>
+cudaError_t launch_backproject_sum_batch(const SumArgs<T>* items, int first, int n_items, int n_rho, const int2* fold_map,
+                                         int n_fold, const int2* far_map, int n_far, const int2* near_map, int n_near,
+                                         int max_splits, int q_max, int series_per_q, int taps, int kern,
+                                         cudaStream_t s);
 
 // back-projection with the W x G+- product on the tensor cores (FP32-mixed)
 size_t backproject_tc_smem(int max_nodes);

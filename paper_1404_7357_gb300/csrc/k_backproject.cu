@@ -266,8 +266,10 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
   const int S = a.series_per_q;
   const int S2 = wbp_series_pad<T>(S);
   const int r0 = tile * a.rchunk;                 // a.rchunk == kWR
-  const int r1 = min(r0 + a.rchunk, a.n_rho);
   const int q = qi - a.q_max;
+  const int r_end = a.low_h > 0.0 ? min(a.n_rho, sum_first_row(a.low_h, abs(q), sizeof(T) == 8)) : a.n_rho;
+  if (r0 >= r_end) return;                        // the sample sums form this tile
+  const int r1 = min(r0 + a.rchunk, r_end);
   const int np = a.chunk_nodes[tile];
   const int tid = threadIdx.x;
   // shared layout: W [WK][WR + 2] | G [WK][S2] | node cos | cos(q alpha) | row node ranges

@@ -81,7 +81,9 @@ __device__ __forceinline__ void bp_tc_task(const BackprojArgs<float>& a, int til
   constexpr TcLayout LY = tc_layout();
   const int S = a.series_per_q;
   const int r0 = tile * kTR;
-  const int r1 = min(r0 + kTR, a.n_rho);
+  const int r_end = a.low_h > 0.0 ? min(a.n_rho, sum_first_row(a.low_h, p, false)) : a.n_rho;
+  if (r0 >= r_end) return;                   // the sample sums form this tile
+  const int r1 = min(r0 + kTR, r_end);
   const int np = a.chunk_nodes[tile];
   const int nhalf = (np + 1) / 2;            // nodes with alpha <= pi / 2
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
