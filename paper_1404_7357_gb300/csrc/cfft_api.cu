@@ -332,6 +332,7 @@ void set_sum_args(SumArgs<T>* sa, const SumPlan& p, const BackprojArgs<T>& ba, T
   sa->cell_rows = p.cell_rows;
   sa->k_used = p.k_used;
   sa->k_pad = p.k_pad;
+  sa->split = p.split;
   sa->d_rho = ba.d_rho;
   sa->d_s = ba.d_s;
   sa->grid = ba.grid;
@@ -691,7 +692,8 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   // rows below (all harmonics' first rows lie in the first n_low chunks)
   SumPlan sp{};
   sums = sums && (tform || wform) &&
-         sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q, &sp);
+         sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q,
+                  ctx->sm_count, &sp);
   const int n_low = sums ? std::min(n_chunks, (sum_first_row(d_rho / ds, ctx->q_max, fp64) + rchunk - 1) / rchunk)
                          : n_chunks;
   int low_nodes = 0;
@@ -1239,7 +1241,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       if (!allowed) continue;
       const int need = (int)std::ceil(rho_max / p.ds) + sum_grid_extra(fp64, bp_taps, bp_kern);
       if (2 * (int64_t)need + 1 <= p.P) p.K = std::max(p.K, need);
-      any_sum = sum_plan(fp64, n_rho, d_rho, p.ds, sigma, p.K, bp_taps, bp_kern, q_max, pairs, &p.sum) || any_sum;
+      any_sum = sum_plan(fp64, n_rho, d_rho, p.ds, sigma, p.K, bp_taps, bp_kern, q_max, pairs, ctx->sm_count, &p.sum) || any_sum;
     }
   }
   auto sum_scratch = [&](const BatchItemPlan& p) {   // elements of T, a multiple of 4

@@ -306,8 +306,10 @@ struct BackprojArgs {
 // first row that the sums over grid samples serve for harmonics +-p (k_backproject_sum.cu); h:
 // the rho step in grid samples
 __host__ __device__ inline int sum_first_row(double h, int p, bool fp64) {
-  const double u = (fp64 ? 1.6 : 0.8) * (double)p * (double)p;
-  const double r = ceil((u > 48.0 ? u : 48.0) / h);
+  // end weights against Bessel functions there (single tones, times 2 pi): float32 8e-8,
+  // float64 1e-13, falling like u^-3 and faster beyond
+  const double u = (fp64 ? 1.0 : 0.5) * (double)p * (double)p;
+  const double r = ceil((u > 40.0 ? u : 40.0) / h);
   return r < 2.0e9 ? (int)r : 2000000000;
 }
 
@@ -317,21 +319,22 @@ struct SumArgs {
   int series_per_q, n_harm, q_max, n_rho, grid_half, sigma;
   int n_cells, cell_rows;  // n_cells = 0: not in use
   int k_used, k_pad;       // samples k >= 0 the rows read, and the folded arrays' length
+  int split;               // samples of a far block's share of a sum
   double d_rho, d_s;
   const cpx<T>* grid;      // [series][2K+1]
   cpx<T>* table;           // [series][n_rho]
   cpx<T>* wrow;            // [end sample][n_rho]
-  T* fold;                 // [|q|][chunk][G+, i G-][k_pad][64]
-  cpx<T>* far;             // [split][|q|][chunk][cell][point][32]
+  T* fold;                 // [|q|][chunk of 16 or 4 series][G+, i G-][k_pad][64 or 16 columns]
+  cpx<T>* far;             // [split][|q|][chunk][cell][point][32 or 8]
 };
 struct SumPlan {
-  int cells, cell_rows, k_used, k_pad, splits, tiles;
+  int cells, cell_rows, k_used, k_pad, split, splits, tiles;
   size_t fold, far, wrow;  // elements of the three buffers (real, complex, complex)
 };
 // false (and an empty plan) where the sums do not serve: another zero padding than the end
 // weights were made for, a grid that ends before the end samples, no row far enough out
 bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int grid_half, int taps, int kern, int q_max,
-              int series_per_q, SumPlan* p);
+              int series_per_q, int sms, SumPlan* p);
 int sum_grid_extra(bool fp64, int taps, int kern);
 int sum_tile_rows();
 int sum_fold_samples();

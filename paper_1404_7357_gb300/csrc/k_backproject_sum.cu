@@ -30,10 +30,12 @@
 //   far    the sums at the cells' points: tiles of 64 points, weights formed 32 samples at a time
 //          in shared memory and multiplied by the folded samples in registers (4 x 4 per
 //          thread); a sum is split over kSplit samples a block, then added in order
-//   near   64 rows: the samples from kc up, the end samples' imaginary weights, and the
-//          interpolation of the far sums as one more short product
-// Bound by the FP32 (FP64) pipe: a weight (T_q from the binary power of e^{i alpha}, one
-// reciprocal square root) costs about as much as its 64 products.
+//   near   64 rows: the samples from kc up (real and, at the end samples, imaginary weights
+//          formed together), and the interpolation of the far sums as one more short product
+// A block column holds 16 series per sign, or 4 where there are no more than 4 (one or two
+// MBFs: a column of 16 would mostly multiply zeros).  Bound by the FP32 (FP64) pipe: a weight
+// (T_q from the binary power of e^{i alpha}, one reciprocal square root) costs about as much as
+// its 64 products.
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -48,11 +50,11 @@ namespace {
 
 constexpr int kSR = 64;        // rows (points) of a block's tile
 constexpr int kSK = 32;        // samples per step
-constexpr int kSS = 16;        // series per sign
-constexpr int kSC = 4 * kSS;   // columns: 32 series x (re, im)
 constexpr int kSThreads = 256;
 constexpr int kSPitch = kSR + 4;
-constexpr int kSplit = 512;    // samples of a far block's share of a sum
+
+// series per sign of a block column (16 or 4), and its columns: both signs, (re, im)
+inline int sum_chunk(int series_per_q) { return series_per_q <= 4 ? 4 : 16; }
 
 template <class T>
 constexpr int kPts = sizeof(T) == 4 ? 10 : 20;   // Chebyshev points per cell
@@ -118,23 +120,28 @@ __device__ __forceinline__ T cheb_out(T z, int p) {
   return (T)0.5 * (r + (T)1 / r);
 }
 
-template <class T>
-__device__ __forceinline__ void fma4x4(T (&acc)[4][4], const T* x, const T* y) {
-  T xv[4], yv[4];
-  if constexpr (sizeof(T) == 4) {
-    const float4 p = *reinterpret_cast<const float4*>(x), q = *reinterpret_cast<const float4*>(y);
-    xv[0] = p.x; xv[1] = p.y; xv[2] = p.z; xv[3] = p.w;
-    yv[0] = q.x; yv[1] = q.y; yv[2] = q.z; yv[3] = q.w;
+// acc[4 rows][J columns] += x[4] y[J] (J = 4 or 1), 16-byte shared loads
+template <class T, int J>
+__device__ __forceinline__ void ld_vec(const T* p, T* v) {
+  if constexpr (J == 1) {
+    v[0] = p[0];
+  } else if constexpr (sizeof(T) == 4) {
+    const float4 q = *reinterpret_cast<const float4*>(p);
+    v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
   } else {
-    const double2 p0 = reinterpret_cast<const double2*>(x)[0], p1 = reinterpret_cast<const double2*>(x)[1];
-    const double2 q0 = reinterpret_cast<const double2*>(y)[0], q1 = reinterpret_cast<const double2*>(y)[1];
-    xv[0] = p0.x; xv[1] = p0.y; xv[2] = p1.x; xv[3] = p1.y;
-    yv[0] = q0.x; yv[1] = q0.y; yv[2] = q1.x; yv[3] = q1.y;
+    const double2 q0 = reinterpret_cast<const double2*>(p)[0], q1 = reinterpret_cast<const double2*>(p)[1];
+    v[0] = q0.x; v[1] = q0.y; v[2] = q1.x; v[3] = q1.y;
   }
+}
+template <class T, int J>
+__device__ __forceinline__ void fma4(T (&acc)[4][J], const T* x, const T* y) {
+  T xv[4], yv[J];
+  ld_vec<T, 4>(x, xv);
+  ld_vec<T, J>(y, yv);
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = fma(xv[i], yv[j], acc[i][j]);
+    for (int j = 0; j < J; ++j) acc[i][j] = fma(xv[i], yv[j], acc[i][j]);
 }
 
 // ---- end weights of the rows: [end sample][row]
@@ -154,10 +161,11 @@ __device__ __forceinline__ void sum_row_weights(const SumArgs<T>& a, int r) {
 }
 
 // ---- folded samples of kSK consecutive k of |q| = p, chunk sc
-template <class T, int TAPS, int KERN>
+template <class T, int TAPS, int KERN, int kSS>
 __device__ __forceinline__ void sum_fold_tile(const SumArgs<T>& a, int k0, int p, int sc) {
   constexpr int HALF = TAPS / 2 - 1;
   constexpr int NW = KERN == 1 ? TAPS : 1;
+  constexpr int kSC = 4 * kSS;
   __shared__ T G[2][kSK][kSC + 1];
   const int tid = threadIdx.x;
   T cw[NW];
@@ -206,7 +214,7 @@ __device__ __forceinline__ void sum_fold_tile(const SumArgs<T>& a, int k0, int p
 }
 
 // a step's samples into shared memory: 16-byte asynchronous copies
-template <class T>
+template <class T, int kSC>
 __device__ __forceinline__ void sum_fetch(const T* src, T* dst, int n_k) {
   const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
   const char* s = reinterpret_cast<const char*>(src);
@@ -215,10 +223,10 @@ __device__ __forceinline__ void sum_fetch(const T* src, T* dst, int n_k) {
   asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-template <class T>
+template <class T, int kSS>
 struct SumSmem {
-  T W[kSK][kSPitch];
-  T G[2][kSK][kSC];
+  T W[2][kSK][kSPitch];
+  T G[2][kSK][4 * kSS];
 };
 
 // samples the far sums of the points of the tile starting at row0 reach
@@ -228,11 +236,13 @@ __device__ __forceinline__ int sum_reach(const SumArgs<T>& a, int row0) {
   return sum_cell(a, min(row0 + kSR - 1, n_pts - 1) / kPts<T>).kc;
 }
 
-template <class T>
-__device__ __forceinline__ void sum_far_tile(const SumArgs<T>& a, int row0, int p, int sc, int split, SumSmem<T>& sm) {
+template <class T, int kSS>
+__device__ __forceinline__ void sum_far_tile(const SumArgs<T>& a, int row0, int p, int sc, int split,
+                                             SumSmem<T, kSS>& sm) {
+  constexpr int kSC = 4 * kSS, J = kSC / 16;
   const int n_pts = a.n_cells * kPts<T>;
   const int tid = threadIdx.x;
-  const int k_beg = split * kSplit, k_end = min(sum_reach(a, row0), k_beg + kSplit);
+  const int k_beg = split * a.split, k_end = min(sum_reach(a, row0), k_beg + a.split);
   // cells of rows below |q| = p's first row are not summed
   const int last = min(row0 + kSR - 1, n_pts - 1) / kPts<T>;
   if (k_beg >= k_end || (last + 1) * a.cell_rows <= sum_first_row(a.d_rho / a.d_s, p, sizeof(T) == 8)) return;
@@ -242,14 +252,14 @@ __device__ __forceinline__ void sum_far_tile(const SumArgs<T>& a, int row0, int 
   const T off = sum_point(c, pt % kPts<T>);
   const T inv_u = (T)1 / (c.o + off);
   const int ty = tid >> 4, tx = tid & 15;
-  T acc[4][4];
+  T acc[4][J];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+    for (int j = 0; j < J; ++j) acc[i][j] = (T)0;
   const int S = a.series_per_q, n_sc = (S + kSS - 1) / kSS;
   const T* fold = a.fold + ((size_t)p * n_sc + sc) * 2 * a.k_pad * kSC;
-  sum_fetch(fold + (size_t)k_beg * kSC, &sm.G[0][0][0], kSK);
+  sum_fetch<T, kSC>(fold + (size_t)k_beg * kSC, &sm.G[0][0][0], kSK);
   for (int k0 = k_beg, buf = 0; k0 < k_end; k0 += kSK, buf ^= 1) {
 #pragma unroll
     for (int m = 0; m < kSK / 4; ++m) {
@@ -262,32 +272,32 @@ __device__ __forceinline__ void sum_far_tile(const SumArgs<T>& a, int row0, int 
         w = cheb_in<T>(kf * inv_u, de * ir * inv_u, p) * ir;
         if (k == 0) w *= (T)0.5;
       }
-      sm.W[kl][wrow] = w;
+      sm.W[0][kl][wrow] = w;
     }
     const bool more = k0 + kSK < k_end;
-    if (more) sum_fetch(fold + (size_t)(k0 + kSK) * kSC, &sm.G[buf ^ 1][0][0], kSK);
+    if (more) sum_fetch<T, kSC>(fold + (size_t)(k0 + kSK) * kSC, &sm.G[buf ^ 1][0][0], kSK);
     if (more) asm volatile("cp.async.wait_group 1;" ::: "memory");
     else asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll 8
-    for (int k = 0; k < kSK; ++k) fma4x4(acc, &sm.W[k][4 * ty], &sm.G[buf][k][4 * tx]);
+    for (int k = 0; k < kSK; ++k) fma4<T, J>(acc, &sm.W[0][k][4 * ty], &sm.G[buf][k][J * tx]);
     __syncthreads();
   }
-  cpx<T>* out = a.far + ((((size_t)split * (a.q_max + 1) + p) * n_sc + sc) * n_pts) * (2 * kSS);
+  T* out = reinterpret_cast<T*>(a.far) + ((((size_t)split * (a.q_max + 1) + p) * n_sc + sc) * n_pts) * kSC;
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int row = row0 + 4 * ty + i;
     if (row >= n_pts) continue;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) out[(size_t)row * (2 * kSS) + 2 * tx + h] = mk(acc[i][2 * h], acc[i][2 * h + 1]);
+    for (int j = 0; j < J; ++j) out[(size_t)row * kSC + J * tx + j] = acc[i][j];
   }
 }
 
 // the far sums of kSR points: the splits added to the first
-template <class T>
+template <class T, int kSS>
 __device__ __forceinline__ void sum_splits(const SumArgs<T>& a, int row0, int p, int sc) {
   const int n_pts = a.n_cells * kPts<T>, n_sc = (a.series_per_q + kSS - 1) / kSS;
-  const int n = (sum_reach(a, row0) + kSplit - 1) / kSplit;
+  const int n = (sum_reach(a, row0) + a.split - 1) / a.split;
   const int last = min(row0 + kSR - 1, n_pts - 1) / kPts<T>;
   if (n < 2 || (last + 1) * a.cell_rows <= sum_first_row(a.d_rho / a.d_s, p, sizeof(T) == 8)) return;
   const size_t stride = (size_t)(a.q_max + 1) * n_sc * n_pts * (2 * kSS);
@@ -301,8 +311,9 @@ __device__ __forceinline__ void sum_splits(const SumArgs<T>& a, int row0, int p,
 }
 
 // kSR rows from row0 on: near sums, end samples, far interpolation, stores
-template <class T>
-__device__ __forceinline__ void sum_near_tile(const SumArgs<T>& a, int row0, int p, int sc, SumSmem<T>& sm) {
+template <class T, int kSS>
+__device__ __forceinline__ void sum_near_tile(const SumArgs<T>& a, int row0, int p, int sc, SumSmem<T, kSS>& sm) {
+  constexpr int kSC = 4 * kSS, J = kSC / 16;
   constexpr int IN = SumShape<T>::kIn, OUT = SumShape<T>::kOut, NE = SumShape<T>::kEnd;
   const int r_min = sum_first_row(a.d_rho / a.d_s, p, sizeof(T) == 8);
   if (row0 + kSR <= r_min || row0 >= a.n_rho) return;
@@ -321,52 +332,54 @@ __device__ __forceinline__ void sum_near_tile(const SumArgs<T>& a, int row0, int
   const T kuf = (T)ku;
   const T inv_u = (T)1 / (kuf + f);
   const int ty = tid >> 4, tx = tid & 15;
-  T acc[4][4];
+  T acc[4][J];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = (T)0;
+    for (int j = 0; j < J; ++j) acc[i][j] = (T)0;
   const int S = a.series_per_q, n_sc = (S + kSS - 1) / kSS;
   const T* fold_p = a.fold + ((size_t)p * n_sc + sc) * 2 * a.k_pad * kSC;
   const T* fold_m = fold_p + (size_t)a.k_pad * kSC;
-  // weight of sample k for this thread's row: part 0 real, 1 imaginary
-  auto weight = [&](int k, int part) -> T {
+  // weight of sample k for this thread's row (imaginary at the end samples only)
+  auto weight = [&](int k) -> cpx<T> {
     const int j = k - (ku + 1 - IN);
-    if (!live || k < c.kc || j >= NE || (part == 1 && j < 0)) return (T)0;
+    if (!live || k < c.kc || j >= NE) return mk((T)0, (T)0);
     const T kf = (T)k, d = (kuf - kf) + f, e = (kuf + kf) + f;   // u - k, u + k
-    T w;
     if (j < 0) {
       const T de = d * e, ir = rsqrt(de);
-      w = cheb_in<T>(kf * inv_u, de * ir * inv_u, p) * ir;
-    } else {
-      const T root = sqrt(fabs(d) * e) * inv_u;
-      w = d >= (T)0 ? cheb_in<T>(kf * inv_u, root, p) : cheb_out<T>(kf * inv_u + root, p);
-      const cpx<T> wj = a.wrow[(size_t)j * a.n_rho + r];
-      w *= rsqrt(e) * (part ? wj.im : wj.re);
+      const T w = cheb_in<T>(kf * inv_u, de * ir * inv_u, p) * ir;
+      return mk(k == 0 ? (T)0.5 * w : w, (T)0);
     }
-    return k == 0 ? (T)0.5 * w : w;
+    const T root = sqrt(fabs(d) * e) * inv_u;
+    const T w = (d >= (T)0 ? cheb_in<T>(kf * inv_u, root, p) : cheb_out<T>(kf * inv_u + root, p)) * rsqrt(e);
+    return w * a.wrow[(size_t)j * a.n_rho + r];
   };
-  auto step = [&](const T* fold, int k0, int part) {
-    sum_fetch(fold + (size_t)k0 * kSC, &sm.G[0][0][0], kSK);
+  // steps below the tile's first end sample take the real weights alone
+  const int b_beg = (int)floor((double)max(row0, r_min) * h) + 1 - IN;
+  for (int k0 = k_beg; k0 < k_end; k0 += kSK) {
+    const bool end = k0 + kSK > b_beg;
+    sum_fetch<T, kSC>(fold_p + (size_t)k0 * kSC, &sm.G[0][0][0], kSK);
+    if (end) sum_fetch<T, kSC>(fold_m + (size_t)k0 * kSC, &sm.G[1][0][0], kSK);
 #pragma unroll
-    for (int m = 0; m < kSK / 4; ++m) sm.W[kw + 4 * m][wrow] = weight(k0 + kw + 4 * m, part);
+    for (int m = 0; m < kSK / 4; ++m) {
+      const cpx<T> w = weight(k0 + kw + 4 * m);
+      sm.W[0][kw + 4 * m][wrow] = w.re;
+      if (end) sm.W[1][kw + 4 * m][wrow] = w.im;
+    }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
+    for (int part = 0; part < (end ? 2 : 1); ++part)
 #pragma unroll 8
-    for (int k = 0; k < kSK; ++k) fma4x4(acc, &sm.W[k][4 * ty], &sm.G[0][k][4 * tx]);
+      for (int k = 0; k < kSK; ++k) fma4<T, J>(acc, &sm.W[part][k][4 * ty], &sm.G[part][k][J * tx]);
     __syncthreads();
-  };
-  for (int k0 = k_beg; k0 < k_end; k0 += kSK) step(fold_p, k0, 0);
-  // end samples of the tile's rows, from the first live row's on
-  const int b_beg = max(0, (int)floor((double)max(row0, r_min) * h) + 1 - IN) / 4 * 4;
-  for (int k0 = b_beg; k0 < k_end; k0 += kSK) step(fold_m, k0, 1);
+  }
   // far sums of the tile's cells, interpolated (barycentric weights of the Chebyshev points)
   constexpr int P = kPts<T>;
-  const cpx<T>* far = a.far + (((size_t)p * n_sc + sc) * a.n_cells * P) * (2 * kSS);
+  const T* far = reinterpret_cast<const T*>(a.far) + (((size_t)p * n_sc + sc) * a.n_cells * P) * kSC;
   const int cell1 = min(row0 + kSR - 1, a.n_rho - 1) / a.cell_rows;
   for (int cell = row0 / a.cell_rows; cell <= cell1; ++cell) {
     if (sum_cell(a, cell).kc == 0 || (cell + 1) * a.cell_rows <= r_min) continue;
-    sum_fetch(reinterpret_cast<const T*>(far + (size_t)cell * P * (2 * kSS)), &sm.G[0][0][0], P);
+    sum_fetch<T, kSC>(far + (size_t)cell * P * kSC, &sm.G[0][0][0], P);
     if (kw == 0) {
       const bool mine = live && r / a.cell_rows == cell;
       const T x = (kuf - c.o) + f;
@@ -379,39 +392,35 @@ __device__ __forceinline__ void sum_near_tile(const SumArgs<T>& a, int row0, int
         sincospi_((T)(2 * i + 1) / (T)(2 * P), &s1, &c1);
         if (dx == (T)0) at = i;
         const T b = ((i & 1) ? -s1 : s1) / (dx == (T)0 ? (T)1 : dx);
-        sm.W[i][wrow] = b;
+        sm.W[0][i][wrow] = b;
         sum += b;
       }
       const T inv = (T)1 / sum;
 #pragma unroll
       for (int i = 0; i < P; ++i)
-        sm.W[i][wrow] = !mine ? (T)0 : (at >= 0 ? (at == i ? (T)1 : (T)0) : sm.W[i][wrow] * inv);
+        sm.W[0][i][wrow] = !mine ? (T)0 : (at >= 0 ? (at == i ? (T)1 : (T)0) : sm.W[0][i][wrow] * inv);
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
 #pragma unroll 5
-    for (int k = 0; k < P; ++k) fma4x4(acc, &sm.W[k][4 * ty], &sm.G[0][k][4 * tx]);
+    for (int k = 0; k < P; ++k) fma4<T, J>(acc, &sm.W[0][k][4 * ty], &sm.G[0][k][J * tx]);
     __syncthreads();
   }
   // stores through shared memory: 64 consecutive rows of a series
   const T norm = (T)(1.0 / (2.0 * 3.14159265358979323846 * 3.14159265358979323846));
-  cpx<T>* tile = reinterpret_cast<cpx<T>*>(&sm.G[0][0][0]);   // [16 series][kSR]
-  static_assert(sizeof(sm.G) >= kSS * kSR * sizeof(cpx<T>), "output tile");
-  for (int half = 0; half < (p > 0 ? 2 : 1); ++half) {
-    if (tx / 8 == half) {
+  T* tile = &sm.G[0][0][0];                       // [column][kSR]
+  static_assert(sizeof(sm.G) >= (size_t)kSC * kSR * sizeof(T), "output tile");
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int g = 0; g < 2; ++g)
-          tile[(2 * (tx & 7) + g) * kSR + 4 * ty + i] = mk(norm * acc[i][2 * g], norm * acc[i][2 * g + 1]);
-    }
-    __syncthreads();
-    const int qi = half == 0 ? a.q_max + p : a.q_max - p;
-    for (int e = tid; e < kSS * kSR; e += kSThreads) {
-      const int g = sc * kSS + e / kSR, row = row0 + e % kSR;
-      if (g < S && row < a.n_rho && row >= r_min) a.table[((size_t)g * a.n_harm + qi) * a.n_rho + row] = tile[e];
-    }
-    __syncthreads();
+    for (int j = 0; j < J; ++j) tile[(J * tx + j) * kSR + 4 * ty + i] = norm * acc[i][j];
+  __syncthreads();
+  for (int e = tid; e < 2 * kSS * kSR; e += kSThreads) {
+    const int c2 = e / kSR, rr = e % kSR, row = row0 + rr;
+    const int g = sc * kSS + (c2 & (kSS - 1));
+    if (g >= S || row >= a.n_rho || row < r_min || (c2 >= kSS && p == 0)) continue;
+    const int qi = c2 < kSS ? a.q_max + p : a.q_max - p;
+    a.table[((size_t)g * a.n_harm + qi) * a.n_rho + row] = mk(tile[(2 * c2) * kSR + rr], tile[(2 * c2 + 1) * kSR + rr]);
   }
 }
 
@@ -419,25 +428,25 @@ template <class T>
 __global__ void __launch_bounds__(128) sum_rows_kernel(SumArgs<T> a) {
   sum_row_weights<T>(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
-template <class T, int TAPS, int KERN>
+template <class T, int TAPS, int KERN, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_fold_kernel(SumArgs<T> a) {
-  sum_fold_tile<T, TAPS, KERN>(a, blockIdx.x * kSK, blockIdx.y, blockIdx.z);
+  sum_fold_tile<T, TAPS, KERN, kSS>(a, blockIdx.x * kSK, blockIdx.y, blockIdx.z);
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_far_kernel(SumArgs<T> a, int n_tiles, int n_p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int t = blockIdx.x;   // the largest rho (most splits) first
-  sum_far_tile<T>(a, (n_tiles - 1 - t / n_p) * kSR, t % n_p, blockIdx.y, blockIdx.z,
-                  *reinterpret_cast<SumSmem<T>*>(smem_raw));
+  sum_far_tile<T, kSS>(a, (n_tiles - 1 - t / n_p) * kSR, t % n_p, blockIdx.y, blockIdx.z,
+                  *reinterpret_cast<SumSmem<T, kSS>*>(smem_raw));
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(256) sum_splits_kernel(SumArgs<T> a) {
-  sum_splits<T>(a, blockIdx.x * kSR, blockIdx.y, blockIdx.z);
+  sum_splits<T, kSS>(a, blockIdx.x * kSR, blockIdx.y, blockIdx.z);
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_near_kernel(SumArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  sum_near_tile<T>(a, blockIdx.x * kSR, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T>*>(smem_raw));
+  sum_near_tile<T, kSS>(a, blockIdx.x * kSR, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T, kSS>*>(smem_raw));
 }
 
 // batched forms: maps of (item, first sample | point | row)
@@ -446,31 +455,31 @@ __global__ void __launch_bounds__(128) sum_rows_batch_kernel(const SumArgs<T>* i
   const SumArgs<T> a = items[first + blockIdx.y];
   if (a.n_cells > 0) sum_row_weights<T>(a, blockIdx.x * blockDim.x + threadIdx.x);
 }
-template <class T, int TAPS, int KERN>
+template <class T, int TAPS, int KERN, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_fold_batch_kernel(const SumArgs<T>* items, const int2* map) {
   const int2 bm = map[blockIdx.x];
   const SumArgs<T> a = items[bm.x];
-  sum_fold_tile<T, TAPS, KERN>(a, bm.y, blockIdx.y, blockIdx.z);
+  sum_fold_tile<T, TAPS, KERN, kSS>(a, bm.y, blockIdx.y, blockIdx.z);
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_far_batch_kernel(const SumArgs<T>* items, const int2* map, int n_p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 bm = map[blockIdx.x / n_p];
   const SumArgs<T> a = items[bm.x];
-  sum_far_tile<T>(a, bm.y, blockIdx.x % n_p, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T>*>(smem_raw));
+  sum_far_tile<T, kSS>(a, bm.y, blockIdx.x % n_p, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T, kSS>*>(smem_raw));
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(256) sum_splits_batch_kernel(const SumArgs<T>* items, const int2* map) {
   const int2 bm = map[blockIdx.x];
   const SumArgs<T> a = items[bm.x];
-  sum_splits<T>(a, bm.y, blockIdx.y, blockIdx.z);
+  sum_splits<T, kSS>(a, bm.y, blockIdx.y, blockIdx.z);
 }
-template <class T>
+template <class T, int kSS>
 __global__ void __launch_bounds__(kSThreads) sum_near_batch_kernel(const SumArgs<T>* items, const int2* map) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 bm = map[blockIdx.x];
   const SumArgs<T> a = items[bm.x];
-  sum_near_tile<T>(a, bm.y, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T>*>(smem_raw));
+  sum_near_tile<T, kSS>(a, bm.y, blockIdx.y, blockIdx.z, *reinterpret_cast<SumSmem<T, kSS>*>(smem_raw));
 }
 
 template <class T, class F>
@@ -483,15 +492,56 @@ cudaError_t by_kernel(int kern, int taps, F f) {
   return f(std::integral_constant<int, 16>{}, std::integral_constant<int, 0>{});
 }
 
-template <class T>
+template <class T, int kSS>
 cudaError_t sum_smem_opt_in() {
-  const int bytes = (int)sizeof(SumSmem<T>);
-  for (const void* k : {(const void*)sum_far_kernel<T>, (const void*)sum_near_kernel<T>,
-                        (const void*)sum_far_batch_kernel<T>, (const void*)sum_near_batch_kernel<T>}) {
+  const int bytes = (int)sizeof(SumSmem<T, kSS>);
+  for (const void* k : {(const void*)sum_far_kernel<T, kSS>, (const void*)sum_near_kernel<T, kSS>,
+                        (const void*)sum_far_batch_kernel<T, kSS>, (const void*)sum_near_batch_kernel<T, kSS>}) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+template <class T, int kSS>
+cudaError_t launch_sums(const SumArgs<T>& a, int taps, int kern, int splits, int tiles, cudaStream_t s) {
+  cudaError_t e = sum_smem_opt_in<T, kSS>();
+  if (e != cudaSuccess) return e;
+  const size_t smem = sizeof(SumSmem<T, kSS>);
+  const int n_p = a.q_max + 1, n_sc = (a.series_per_q + kSS - 1) / kSS;
+  sum_rows_kernel<T><<<(a.n_rho + 31) / 32, 32, 0, s>>>(a);
+  e = by_kernel<T>(kern, taps, [&](auto tp, auto kn) {
+    sum_fold_kernel<T, decltype(tp)::value, decltype(kn)::value, kSS>
+        <<<dim3(a.k_pad / kSK, n_p, n_sc), kSThreads, 0, s>>>(a);
+    return cudaGetLastError();
+  });
+  if (e != cudaSuccess) return e;
+  sum_far_kernel<T, kSS><<<dim3(tiles * n_p, n_sc, splits), kSThreads, smem, s>>>(a, tiles, n_p);
+  if (splits > 1) sum_splits_kernel<T, kSS><<<dim3(tiles, n_p, n_sc), 256, 0, s>>>(a);
+  sum_near_kernel<T, kSS><<<dim3((a.n_rho + kSR - 1) / kSR, n_p, n_sc), kSThreads, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
+template <class T, int kSS>
+cudaError_t launch_sums_batch(const SumArgs<T>* items, int first, int n_items, int n_rho, const int2* fold_map,
+                              int n_fold, const int2* far_map, int n_far, const int2* near_map, int n_near,
+                              int max_splits, int q_max, int series_per_q, int taps, int kern, cudaStream_t s) {
+  cudaError_t e = sum_smem_opt_in<T, kSS>();
+  if (e != cudaSuccess) return e;
+  const size_t smem = sizeof(SumSmem<T, kSS>);
+  const int n_p = q_max + 1, n_sc = (series_per_q + kSS - 1) / kSS;
+  for (int i = 0; i < n_items; i += 32768)
+    sum_rows_batch_kernel<T><<<dim3((n_rho + 127) / 128, std::min(32768, n_items - i)), 128, 0, s>>>(items, first + i);
+  e = by_kernel<T>(kern, taps, [&](auto tp, auto kn) {
+    sum_fold_batch_kernel<T, decltype(tp)::value, decltype(kn)::value, kSS>
+        <<<dim3(n_fold, n_p, n_sc), kSThreads, 0, s>>>(items, fold_map);
+    return cudaGetLastError();
+  });
+  if (e != cudaSuccess) return e;
+  sum_far_batch_kernel<T, kSS><<<dim3(n_far * n_p, n_sc, max_splits), kSThreads, smem, s>>>(items, far_map, n_p);
+  if (max_splits > 1) sum_splits_batch_kernel<T, kSS><<<dim3(n_far, n_p, n_sc), 256, 0, s>>>(items, far_map);
+  sum_near_batch_kernel<T, kSS><<<dim3(n_near, n_p, n_sc), kSThreads, smem, s>>>(items, near_map);
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -502,7 +552,7 @@ int sum_grid_extra(bool fp64, int taps, int kern) {
 }
 
 bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int grid_half, int taps, int kern, int q_max,
-              int series_per_q, SumPlan* p) {
+              int series_per_q, int sms, SumPlan* p) {
   *p = SumPlan{};
   const int out = fp64 ? EndShape<double>::kOut : EndShape<float>::kOut;
   if (sigma != (fp64 ? EndShape<double>::kSigma : EndShape<float>::kSigma)) return false;
@@ -516,11 +566,18 @@ bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int gri
   p->k_used = (int)std::floor(top) + out + 1;
   p->k_pad = (p->k_used + 4 + kSK) / kSK * kSK + kSK;   // steps may start at any multiple of 4
   const int pts = fp64 ? kPts<double> : kPts<float>;
-  p->splits = std::max(1, (p->k_used + kSplit - 1) / kSplit);
+  const int ss = sum_chunk(series_per_q);
   p->tiles = (p->cells * pts + kSR - 1) / kSR;
-  const size_t blocks = (size_t)(q_max + 1) * ((series_per_q + kSS - 1) / kSS);
-  p->fold = blocks * 2 * p->k_pad * kSC;
-  p->far = (size_t)p->splits * blocks * p->cells * pts * 2 * kSS;
+  const size_t blocks = (size_t)(q_max + 1) * ((series_per_q + ss - 1) / ss);
+  // a far sum is split over blocks of 64 to 512 samples: about eight blocks per SM (half the
+  // (tile, split) pairs lie beyond their tile's reach), at most 16 splits
+  p->split = 512;
+  while (p->split > 64 && (int64_t)p->tiles * blocks * (p->k_used / p->split + 1) < 16 * sms &&
+         p->k_used / (p->split / 2) < 16)
+    p->split /= 2;
+  p->splits = std::max(1, (p->k_used + p->split - 1) / p->split);
+  p->fold = blocks * 2 * p->k_pad * 4 * ss;
+  p->far = (size_t)p->splits * blocks * p->cells * pts * 2 * ss;
   p->wrow = (size_t)(fp64 ? SumShape<double>::kEnd : SumShape<float>::kEnd) * n_rho;
   return true;
 }
@@ -530,20 +587,8 @@ int sum_fold_samples() { return kSK; }
 
 template <class T>
 cudaError_t launch_backproject_sum(const SumArgs<T>& a, int taps, int kern, int splits, int tiles, cudaStream_t s) {
-  cudaError_t e = sum_smem_opt_in<T>();
-  if (e != cudaSuccess) return e;
-  const int n_p = a.q_max + 1, n_sc = (a.series_per_q + kSS - 1) / kSS;
-  sum_rows_kernel<T><<<(a.n_rho + 127) / 128, 128, 0, s>>>(a);
-  e = by_kernel<T>(kern, taps, [&](auto tp, auto kn) {
-    sum_fold_kernel<T, decltype(tp)::value, decltype(kn)::value>
-        <<<dim3(a.k_pad / kSK, n_p, n_sc), kSThreads, 0, s>>>(a);
-    return cudaGetLastError();
-  });
-  if (e != cudaSuccess) return e;
-  sum_far_kernel<T><<<dim3(tiles * n_p, n_sc, splits), kSThreads, sizeof(SumSmem<T>), s>>>(a, tiles, n_p);
-  if (splits > 1) sum_splits_kernel<T><<<dim3(tiles, n_p, n_sc), 256, 0, s>>>(a);
-  sum_near_kernel<T><<<dim3((a.n_rho + kSR - 1) / kSR, n_p, n_sc), kSThreads, sizeof(SumSmem<T>), s>>>(a);
-  return cudaGetLastError();
+  return sum_chunk(a.series_per_q) == 4 ? launch_sums<T, 4>(a, taps, kern, splits, tiles, s)
+                                        : launch_sums<T, 16>(a, taps, kern, splits, tiles, s);
 }
 
 template <class T>
@@ -551,21 +596,9 @@ cudaError_t launch_backproject_sum_batch(const SumArgs<T>* items, int first, int
                                          int n_fold, const int2* far_map, int n_far, const int2* near_map, int n_near,
                                          int max_splits, int q_max, int series_per_q, int taps, int kern,
                                          cudaStream_t s) {
-  cudaError_t e = sum_smem_opt_in<T>();
-  if (e != cudaSuccess) return e;
-  const int n_p = q_max + 1, n_sc = (series_per_q + kSS - 1) / kSS;
-  for (int i = 0; i < n_items; i += 32768)
-    sum_rows_batch_kernel<T><<<dim3((n_rho + 127) / 128, std::min(32768, n_items - i)), 128, 0, s>>>(items, first + i);
-  e = by_kernel<T>(kern, taps, [&](auto tp, auto kn) {
-    sum_fold_batch_kernel<T, decltype(tp)::value, decltype(kn)::value>
-        <<<dim3(n_fold, n_p, n_sc), kSThreads, 0, s>>>(items, fold_map);
-    return cudaGetLastError();
-  });
-  if (e != cudaSuccess) return e;
-  sum_far_batch_kernel<T><<<dim3(n_far * n_p, n_sc, max_splits), kSThreads, sizeof(SumSmem<T>), s>>>(items, far_map, n_p);
-  if (max_splits > 1) sum_splits_batch_kernel<T><<<dim3(n_far, n_p, n_sc), 256, 0, s>>>(items, far_map);
-  sum_near_batch_kernel<T><<<dim3(n_near, n_p, n_sc), kSThreads, sizeof(SumSmem<T>), s>>>(items, near_map);
-  return cudaGetLastError();
+  auto run = sum_chunk(series_per_q) == 4 ? launch_sums_batch<T, 4> : launch_sums_batch<T, 16>;
+  return run(items, first, n_items, n_rho, fold_map, n_fold, far_map, n_far, near_map, n_near, max_splits, q_max,
+             series_per_q, taps, kern, s);
 }
 
 template cudaError_t launch_backproject_sum<float>(const SumArgs<float>&, int, int, int, int, cudaStream_t);
