@@ -155,8 +155,8 @@ typedef enum {
  *   SOLVE_GRID_PANEL  a value > 0 runs every LU panel of cfft_solve_reduced
  *                as a cooperative launch over the grid (pivot keys
  *                published and polled in global memory per column) instead
- *                of on one
- *                thread-block cluster for panels of at most 2048 rows */
+ *                of on one thread-block cluster where its shared memory
+ *                holds the panel's rows */
 typedef enum {
   CFFT_OPT_N_ALPHA = 0,
   CFFT_OPT_SIGMA = 1,
@@ -629,30 +629,29 @@ cfft_status cfft_port_currents(cfft_ctx* ctx, int n_elements, int port, const vo
  * when complex128 != 0, else complex64.  n is at most the order whose panel
  * rows fit the panel CTAs' shared memory (48,640 in complex64 and 24,320 in
  * complex128 on 152 SMs) and at most 65535; beyond, CFFT_ERR_ARG.
- * mode 0: LU with partial pivoting (|re| + |im| of the column, compared on
- *         the leading 32 bits of its double, ties to the lowest row) in the
- *         matrix's own precision.
+ * mode 0: LU with partial pivoting (|re| + |im| of the column, compared as
+ *         floats in complex64 and on the leading 32 bits of the double in
+ *         complex128, ties to the lowest row) in the matrix's own precision.
  * mode 1 (complex128 only): the LU of a complex64 copy, then iterative
  *         refinement in float64 against z: x += LU^-1 (v - z x) until the
  *         correction falls below float64 resolution or the residual stops
  *         falling (at most 30 steps).
- * The factorization runs in panels of 64 columns: one launch per panel (pivot
- * search and elimination, one barrier per column: the hardware barrier of one
- * thread-block cluster of 16 or 8 CTAs, candidates and pivot rows read from
- * the peers' shared memory, for panels of at most 2048 rows that fit that
- * cluster's shared memory; otherwise a cooperative launch over the grid whose
- * CTAs publish their candidates' pivot keys, tagged with the column, in
- * global memory and poll them with a bound), the panel's row moves applied to
- * the whole matrix, a
- * triangular solve for
- * the panel's rows and a complex matrix product for the trailing matrix.  In
+ * The factorization runs in panels of 64 columns (pivot search and
+ * elimination, one exchange per column): one launch per panel of at most 2048
+ * rows, two halves of 32 columns for a longer one.  A launch whose rows fit
+ * the shared memory of one thread-block cluster of 16 or 8 CTAs runs there,
+ * the CTAs sending their candidate rows into each other's shared memory; any
+ * other is a cooperative launch over the grid whose CTAs publish their
+ * candidates' pivot keys, tagged with the column, in global memory.  Every
+ * wait has a bound.  Then the panel's row moves applied to
+ * the whole matrix, a triangular solve for the panel's rows and a complex matrix product for the trailing matrix.  In
  * complex64 that product runs on the tensor cores (three TF32 products, FP32
  * accumulation) unless the option SOLVE_SIMT is > 0, which keeps it on the
  * FP32 pipe.
  * cfft_get_solve_info reports the times and the relative residual
  * |v - z x| / |v| computed in float64 from z.  Errors: CFFT_ERR_ARG,
  * CFFT_ERR_OOM, CFFT_ERR_NUMERIC (a zero pivot: z singular), CFFT_ERR_TIMEOUT
- * (a grid-barrier or tensor-core wait gave up).  Synchronizes. */
+ * (a panel's or the tensor cores' wait gave up).  Synchronizes. */
 cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, int64_t ld, const void* v,
                                void* i_out, int complex128, int mode);
 
@@ -660,7 +659,8 @@ cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, int64_t ld, 
  * (ms, CUDA events on the context stream; the solve includes refinement),
  * relative residual, order n, mode, refinement steps (mode 1), panel width,
  * update_tc = 1 when the trailing updates ran on the tensor cores, the number
- * of panels that ran on one thread-block cluster and its CTA count (0: none). */
+ * of panels that ran whole (in one launch) on one thread-block cluster and its
+ * CTA count (0: none). */
 typedef struct {
   double ms_factor, ms_solve, residual;
   int n, mode, refinements, panel_width, update_tc, cluster_panels, panel_cluster;

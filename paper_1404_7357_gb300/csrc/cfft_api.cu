@@ -2574,7 +2574,7 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   const int nb = lu_panel_width();
   const int panels = (n + nb - 1) / nb;
   CFFT_CUDA(ctx->lu_moves.ensure((size_t)panels * 2 * nb * sizeof(int2)), "alloc LU");
-  CFFT_CUDA(ctx->lu_nmoves.ensure((size_t)panels * sizeof(int)), "alloc LU");
+  CFFT_CUDA(ctx->lu_nmoves.ensure((size_t)panels * 2 * sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_v.ensure((size_t)ctx->sm_count * 2 * sizeof(double)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_r.ensure((size_t)ctx->sm_count * 2 * sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_d.ensure((size_t)ctx->sm_count * 2 * nb * 16), "alloc LU");

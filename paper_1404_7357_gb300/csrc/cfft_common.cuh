@@ -546,8 +546,9 @@ cudaError_t cartesian_fill(const cpx<T>* table, int p, int m, double x0, double 
 
 // dense LU of the reduced system (k_solve.cu): device work arrays of one factorization
 struct LuWork {
-  int2* moves;         // [panels][2 * panel width] row moves (source, destination)
-  int* n_moves;        // [panels]
+  int2* moves;         // [panels][2][panel width] row moves (source, destination): a whole panel's
+                       // list, or one list per half
+  int* n_moves;        // [panels][2]
   double* cand_val;    // [2][SMs] 64-bit words: the panel CTAs' pivot keys with column tags
   int* cand_row;       // (unused)
   void* cand_data;     // [2][SMs][panel width] complex, the element type: the candidates' entries

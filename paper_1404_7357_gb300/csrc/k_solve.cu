@@ -6,22 +6,23 @@
 //
 // LU (right-looking, row-major, panels of kNb columns):
 //   panel    one launch over the panel's rows: per column, every CTA proposes its
-//            largest |re| + |im| among the rows not yet chosen (compared on the
-//            leading 32 bits of the double, ties: lowest row), a barrier, every
-//            CTA takes the same pivot, reads the pivot row and
-//            eliminates the column from its own rows.  Pivoting is logical: rows
-//            stay where they are and the chosen rows are recorded; one barrier per
-//            column.  A panel of at most 2048 rows (that fits the shared memory
-//            of one thread-block cluster, 16 CTAs, else 8) runs on the cluster:
-//            the CTAs exchange candidates and the pivot row through distributed
-//            shared memory with the cluster's hardware barrier.  Longer panels
+//            largest |re| + |im| among the rows not yet chosen (complex64 compared
+//            as floats, complex128 on the leading 32 bits; ties: lowest row), a
+//            barrier, every CTA takes the same pivot, gets the pivot row and
+//            eliminates the column from its own rows, the next column's entries
+//            first, so that the exchange of its candidates overlaps the rest.
+//            Pivoting is logical: rows stay where they are and the chosen rows are
+//            recorded; one barrier per column.  A panel of more than 2048 rows runs
+//            as two halves of 32 columns.  What fits the shared memory of one
+//            thread-block cluster (16 CTAs, else 8) runs there: the CTAs send
+//            their candidate rows into each other's shared memory.  Longer panels
 //            run cooperatively over the grid: each CTA publishes its candidate's
 //            key with a column tag in global memory, and polling the keys (with
 //            a bound) is the grid barrier.
 //   moves    the panel's pivot rows go to rows k..k+kb-1 and the rows they
 //            displace to the vacated places, as a list of (source, destination)
 //            row moves applied to every column of the matrix.
-//   trsm     U12 = L11^-1 A12 (unit lower L11), one thread per column.
+//   trsm     U12 = L11^-1 A12 (unit lower L11), four columns per warp at once.
 //   gemm     A22 -= L21 U12, K = the panel: in complex64 on the tensor cores (the
 //            complex product as a real GEMM, three TF32 products), otherwise
 //            64 x 64 tiles of complex entries on the FP32 / FP64 pipe.
@@ -66,6 +67,9 @@ __device__ __forceinline__ cpx<T> crecip(cpx<T> z) {
   return cdiv(mk((T)1, (T)0), z);
 }
 
+// a panel row's pitch in shared memory: odd, so that a column's entries lie in different banks
+__host__ __device__ constexpr int cl_pitch(int kb) { return kb | 1; }
+
 template <class T>
 struct PanelArgs {
   cpx<T>* a;
@@ -78,13 +82,18 @@ struct PanelArgs {
   int* err;           // bit 1: a barrier wait ran out; bit 2: zero pivot
 };
 
-// pivot key of row `row` with |re| + |im| = metric: the leading 32 bits of the metric (a
-// non-negative double, so its bits order like its value: exponent and 20 mantissa bits),
-// then the lower row (rows below 65535); the low 16 bits stay free for a column tag.  The
-// largest key is the pivot, so the choice does not depend on how the rows are split
-// between CTAs; 0 stands for no candidate.
-__device__ __forceinline__ unsigned long long pivot_key(double metric, int row) {
-  return (((unsigned long long)__double_as_longlong(metric) >> 32) << 32) |
+// pivot key of row `row` with entry v: the leading 32 bits of |re| + |im| (non-negative, so its
+// bits order like its value; a float whole, a double's exponent and 20 mantissa bits), then the
+// lower row (rows below 65535); the low 16 bits stay free for a column tag.  The largest key is
+// the pivot, so the choice does not depend on how the rows are split between CTAs; 0 stands for
+// no candidate.  (complex64 in its own type: three conversions and an addition on the FP64 pipe
+// per entry were most of a column's 1,100 cycles in the cluster form.)
+__device__ __forceinline__ unsigned long long pivot_key(cpx<float> v, int row) {
+  return ((unsigned long long)__float_as_uint(fabsf(v.re) + fabsf(v.im)) << 32) |
+         ((unsigned long long)(0xFFFFu - (unsigned)row) << 16);
+}
+__device__ __forceinline__ unsigned long long pivot_key(cpx<double> v, int row) {
+  return (((unsigned long long)__double_as_longlong(fabs(v.re) + fabs(v.im)) >> 32) << 32) |
          ((unsigned long long)(0xFFFFu - (unsigned)row) << 16);
 }
 __device__ __forceinline__ int key_row(unsigned long long key) { return 0xFFFF - (int)((key >> 16) & 0xFFFFu); }
@@ -92,18 +101,11 @@ __device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsig
   return a > b ? a : b;
 }
 
-// the largest key of this CTA's rows not chosen yet in column j (every thread gets it)
-template <class T, int kWarps>
-__device__ __forceinline__ unsigned long long cta_best_key(const cpx<T>* rows, const unsigned char* chosen,
-                                                           int nr, int kb, int j, int lo,
-                                                           unsigned long long* wk) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  unsigned long long best = 0;
-  for (int i = tid; i < nr; i += blockDim.x) {
-    if (chosen[i]) continue;
-    const cpx<T> v = rows[i * kb + j];
-    best = umax64(best, pivot_key(fabs((double)v.re) + fabs((double)v.im), lo + i));
-  }
+// the largest of the CTA's keys (every thread gets it); `wk` is not written again before the
+// caller's next barrier
+template <int kWarps>
+__device__ __forceinline__ unsigned long long cta_max_key(unsigned long long best, unsigned long long* wk) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) best = umax64(best, __shfl_xor_sync(0xffffffffu, best, off));
   if (lane == 0) wk[warp] = best;
@@ -111,110 +113,194 @@ __device__ __forceinline__ unsigned long long cta_best_key(const cpx<T>* rows, c
   unsigned long long b = wk[0];
 #pragma unroll
   for (int w = 1; w < kWarps; ++w) b = umax64(b, wk[w]);
-  __syncthreads();   // wk is rewritten at the next column
   return b;
 }
 
-// the panel's row moves from its pivots (one thread): rows k+j <- pivot j; the rows of
-// [k, k+kb) that were not chosen go to the places the chosen rows outside that range
-// leave free, both in increasing order
+// A panel column, both forms.  Column j's elimination is split so that the exchange of column
+// j + 1's candidates overlaps most of it:
+//   panel_column   the multipliers of column j and the new entries of column j + 1 (one thread
+//                  per row), and the CTA's best key of column j + 1;
+//   panel_row      the remaining entries of that best row (warp 0), which is then published;
+//   panel_rest     the remaining entries of the other rows (the other warps), while warp 0
+//                  exchanges keys and reads the pivot row.
+// Every entry takes the same operations in the same order as an elimination column by column.
+
+// column j with pivot row `pr` (entries j.. in prow): returns this thread's best key of j + 1
+template <class T>
+__device__ __forceinline__ unsigned long long panel_column(cpx<T>* rows, unsigned char* chosen, int nr, int kb, int j,
+                                                           int lo, int pr, const cpx<T>* prow) {
+  const cpx<T> inv = crecip(prow[0]);
+  unsigned long long best = 0;
+  for (int i = threadIdx.x; i < nr; i += blockDim.x) {
+    if (lo + i == pr) chosen[i] = 1;
+    if (chosen[i]) continue;
+    cpx<T>* row = rows + (size_t)i * cl_pitch(kb) + j;
+    const cpx<T> l = row[0] * inv;
+    row[0] = l;
+    if (j + 1 < kb) {
+      cpx<T> v = row[1];
+      cmac(v, mk(-l.re, -l.im), prow[1]);
+      row[1] = v;
+      best = umax64(best, pivot_key(v, lo + i));
+    }
+  }
+  return best;
+}
+
+// entries j + 2.. of local row i, one warp
+template <class T>
+__device__ __forceinline__ void panel_row(cpx<T>* rows, int i, int kb, int j, const cpx<T>* prow) {
+  cpx<T>* row = rows + (size_t)i * cl_pitch(kb) + j;
+  const cpx<T> l = row[0];
+  const cpx<T> ml = mk(-l.re, -l.im);
+  for (int t = 2 + (int)(threadIdx.x & 31); t < kb - j; t += 32) cmac(row[t], ml, prow[t]);
+}
+
+// entries j + 2.. of every row not chosen but `skip`, warps 1 .. kWarps - 1
+template <class T, int kWarps>
+__device__ __forceinline__ void panel_rest(cpx<T>* rows, const unsigned char* chosen, int nr, int kb, int j, int skip,
+                                           const cpx<T>* prow) {
+  constexpr int kBatch = sizeof(T) == 4 ? 4 : 2;   // rows in flight per warp
+  const int lane = threadIdx.x & 31, pitch = cl_pitch(kb);
+  for (int t = 2 + lane; t - lane < kb - j; t += 32) {
+    const bool in = t < kb - j;
+    const cpx<T> pt = in ? prow[t] : mk((T)0, (T)0);
+    for (int i0 = (int)(threadIdx.x >> 5) - 1; i0 < nr; i0 += kBatch * (kWarps - 1)) {
+      cpx<T> l[kBatch], v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const cpx<T>* row = rows + (size_t)min(i0 + u * (kWarps - 1), nr - 1) * pitch + j;
+        l[u] = row[0];
+        v[u] = in ? row[t] : mk((T)0, (T)0);
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) cmac(v[u], mk(-l[u].re, -l[u].im), pt);
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        const int i = i0 + u * (kWarps - 1);
+        if (in && i < nr && i != skip && !chosen[i]) rows[(size_t)i * pitch + j + t] = v[u];
+      }
+    }
+  }
+}
+
+// the panel's row moves from its pivots (every thread of the CTA, at least kNb): pivot j to row
+// k + j, and the rows of the block that no column chose, in ascending order, to the rows that
+// pivots from below the block left, in ascending order.  Every source is read before any
+// destination is written, so the order of the list does not matter.
 template <class T>
 __device__ void panel_record_moves(const PanelArgs<T>& p, const int* s_piv) {
-  const int kb = p.kb;
-  int nm = 0, nd = 0, nv = 0;
-  int displaced[kNb], vacated[kNb];
-  for (int j = 0; j < kb; ++j) {
-    if (s_piv[j] != p.k + j) p.moves[nm++] = make_int2(s_piv[j], p.k + j);
-    if (s_piv[j] >= p.k + kb) vacated[nv++] = s_piv[j];
+  __shared__ int displaced[kNb], vacated[kNb], taken[kNb], nm, nd;
+  const int kb = p.kb, t = threadIdx.x;
+  if (t < kNb) taken[t] = 0;
+  if (t == 0) nm = nd = 0;
+  __syncthreads();
+  const int pr = t < kb ? s_piv[t] : -1;
+  if (pr >= p.k && pr < p.k + kb) taken[pr - p.k] = 1;
+  __syncthreads();
+  if (t < kb) {
+    if (pr != p.k + t) p.moves[atomicAdd(&nm, 1)] = make_int2(pr, p.k + t);
+    int d = 0, v = 0;
+    for (int u = 0; u < kb; ++u) {
+      d += u < t && !taken[u];
+      v += s_piv[u] >= p.k + kb && s_piv[u] < pr;
+    }
+    if (!taken[t]) {
+      displaced[d] = p.k + t;
+      atomicAdd(&nd, 1);
+    }
+    if (pr >= p.k + kb) vacated[v] = pr;   // as many as there are displaced rows
   }
-  for (int r = p.k; r < p.k + kb; ++r) {
-    bool taken = false;
-    for (int j = 0; j < kb; ++j) taken = taken || s_piv[j] == r;
-    if (!taken) displaced[nd++] = r;
-  }
-  // nd == nv: both count the pivots from outside [k, k+kb)
-  for (int t = 0; t < nd && t < nv; ++t) {
-    int m = t;
-    for (int u = t + 1; u < nv; ++u)
-      if (vacated[u] < vacated[m]) m = u;
-    const int tmp = vacated[t];
-    vacated[t] = vacated[m];
-    vacated[m] = tmp;
-    p.moves[nm++] = make_int2(displaced[t], vacated[t]);
-  }
-  *p.n_moves = nm;
+  __syncthreads();
+  if (t < nd) p.moves[nm + t] = make_int2(displaced[t], vacated[t]);
+  if (t == 0) *p.n_moves = nm + nd;
 }
 
 // One panel of kb columns on rows k..n-1, cooperative over the grid.  Each CTA holds its
-// slice of rows in shared memory for the whole panel.  Per column it stages its best
-// candidate's remaining entries in global memory, then publishes its pivot key tagged with
-// the column (one 64-bit store after a fence); warp 0 of every CTA polls the G keys of the
-// column until all carry the tag (the poll is the grid barrier, and it delivers the
-// candidates), every CTA takes the largest key as the pivot and reads that row's entries.
-// Keys and entries are double-buffered by column parity: a CTA publishes column j + 2 only
-// after it has seen every key of column j + 1, which each CTA publishes after its reads of
-// column j.  Every poll is bounded; a CTA whose poll runs out leaves the panel, and the
-// others then run out on its missing keys.
+// slice of rows in shared memory for the whole panel.  Per column warp 0 completes its CTA's
+// best candidate row, stages its remaining entries in global memory, publishes its pivot key
+// tagged with the column (one 64-bit store after a fence) and polls the G keys of the column
+// until all carry the tag (the poll is the grid barrier, and it delivers the candidates), takes
+// the largest as the pivot and reads that row's entries; the other warps meanwhile finish the
+// previous column's elimination.  Keys and entries are double-buffered by column parity: a CTA
+// publishes column j + 2 only after it has seen every key of column j + 1, which each CTA
+// publishes after its reads of column j.  Every poll is bounded; a CTA whose poll runs out
+// leaves the panel, and the others then run out on its missing keys.  Bound by two trips
+// through L2 per column (key, row).
 template <class T>
 __global__ void __launch_bounds__(kPanelThreads) lu_panel_kernel(PanelArgs<T> p) {
   constexpr int kWarps = kPanelThreads / 32;
+  constexpr int kSlots = 8;   // keys per lane: at most 256 CTAs
   const int G = gridDim.x, g = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int R = p.n - p.k, kb = p.kb;
+  const int R = p.n - p.k, kb = p.kb, pitch = cl_pitch(kb);
   const int per = (R + G - 1) / G;
   const int lo = p.k + min(g * per, R), hi = p.k + min((g + 1) * per, R), nr = hi - lo;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<T>* rows = reinterpret_cast<cpx<T>*>(smem_raw);                       // [per][kb]
-  unsigned char* chosen = smem_raw + (size_t)per * kb * sizeof(cpx<T>);     // [per]
-  __shared__ cpx<T> prow[kNb];
+  cpx<T>* rows = reinterpret_cast<cpx<T>*>(smem_raw);                       // [per][pitch]
+  unsigned char* chosen = smem_raw + (size_t)per * pitch * sizeof(cpx<T>);  // [per]
+  __shared__ cpx<T> prow[2][kNb];                                           // by column parity
   __shared__ unsigned long long wk[kWarps];
   __shared__ unsigned long long s_win;
   __shared__ int s_piv[kNb];
   __shared__ int s_fail;
   for (int e = tid; e < nr * kb; e += blockDim.x)
-    rows[e] = p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb];
+    rows[(size_t)(e / kb) * pitch + e % kb] = p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb];
   for (int i = tid; i < per; i += blockDim.x) chosen[i] = 0;
   if (tid == 0) s_fail = 0;
   __syncthreads();
+  unsigned long long mine = 0;
+  for (int i = tid; i < nr; i += blockDim.x) {
+    const cpx<T> v = rows[(size_t)i * pitch];
+    mine = umax64(mine, pivot_key(v, lo + i));
+  }
+  mine = cta_max_key<kWarps>(mine, wk);
   bool ok = true;
   for (int j = 0; j < kb; ++j) {
     const int buf = (p.k + j) & 1;
     const unsigned long long tag = (unsigned long long)((p.k + j) & 0xFFFF);
-    const unsigned long long mine = cta_best_key<T, kWarps>(rows, chosen, nr, kb, j, lo, wk);
-    if (mine != 0) {
-      const int bl = key_row(mine) - lo;
-      for (int t = tid; t < kb - j; t += blockDim.x)
-        p.cand_data[((size_t)buf * G + g) * kNb + t] = rows[bl * kb + j + t];
-    }
-    __syncthreads();
-    if (tid == 0) {
-      __threadfence();   // the entries before the key
-      *reinterpret_cast<volatile unsigned long long*>(p.slot + buf * G + g) = mine | tag;
-    }
+    const int bl = mine != 0 ? key_row(mine) - lo : -1;
+    const cpx<T>* prev = prow[(j & 1) ^ 1];     // pivot row of column j - 1
     if (warp == 0) {
+      if (bl >= 0) {
+        if (j > 0) panel_row(rows, bl, kb, j - 1, prev);
+        __syncwarp();
+        for (int t = lane; t < kb - j; t += 32)
+          p.cand_data[((size_t)buf * G + g) * kNb + t] = rows[(size_t)bl * pitch + j + t];
+      }
+      __threadfence();   // the entries before the key
+      __syncwarp();
+      if (lane == 0) *reinterpret_cast<volatile unsigned long long*>(p.slot + buf * G + g) = mine | tag;
+      const volatile unsigned long long* sp = reinterpret_cast<const volatile unsigned long long*>(p.slot + buf * G);
       unsigned long long kmax = 0;
-      bool fine = true;
-      for (int t = lane; t < G && fine; t += 32) {
-        const volatile unsigned long long* sp = reinterpret_cast<const volatile unsigned long long*>(p.slot + buf * G + t);
-        unsigned polls = 0;
-        unsigned long long x = *sp;
-        while ((x & 0xFFFFull) != tag) {
-          if (++polls > kBarrierPolls) {
-            fine = false;
-            break;
-          }
-          if (polls > 256) __nanosleep(32);
-          x = *sp;
+      bool fine = false;
+      for (unsigned polls = 0; polls <= kBarrierPolls && !fine; ++polls) {
+        unsigned long long x[kSlots];
+#pragma unroll
+        for (int u = 0; u < kSlots; ++u) x[u] = lane + 32 * u < G ? sp[lane + 32 * u] : tag;
+        fine = true;
+        kmax = 0;
+#pragma unroll
+        for (int u = 0; u < kSlots; ++u) {
+          fine = fine && (x[u] & 0xFFFFull) == tag;
+          kmax = umax64(kmax, x[u] & ~0xFFFFull);
         }
-        kmax = umax64(kmax, x & ~0xFFFFull);
+        if (polls > 256) __nanosleep(32);
       }
       const bool all_fine = __all_sync(0xffffffffu, fine);
 #pragma unroll
       for (int off = 16; off > 0; off >>= 1) kmax = umax64(kmax, __shfl_xor_sync(0xffffffffu, kmax, off));
       __threadfence();   // the winner's entries after its key
+      const int w_row = kmax != 0 ? key_row(kmax) : -1;
+      if (all_fine && w_row >= p.k && w_row < p.n) {
+        const int w = (w_row - p.k) / per;   // the CTA whose candidate it is
+        for (int t = lane; t < kb - j; t += 32) prow[j & 1][t] = ldcg(p.cand_data + ((size_t)buf * G + w) * kNb + t);
+      }
       if (lane == 0) {
         s_win = kmax;
         if (!all_fine) s_fail = 1;
       }
+    } else if (j > 0) {
+      panel_rest<T, kWarps>(rows, chosen, nr, kb, j - 1, bl, prev);
     }
     __syncthreads();
     if (s_fail) {
@@ -229,29 +315,10 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel_kernel(PanelArgs<T> p)
       break;
     }
     if ((win >> 32) == 0 && tid == 0 && g == 0) atomicOr(p.err, 4);   // a zero pivot
-    const int w = (pr - p.k) / per;   // the CTA whose candidate it is
-    for (int t = tid; t < kb - j; t += blockDim.x) prow[t] = ldcg(p.cand_data + ((size_t)buf * G + w) * kNb + t);
-    if (tid == 0) {
-      if (pr >= lo && pr < hi) chosen[pr - lo] = 1;
-      s_piv[j] = pr;
-    }
-    __syncthreads();
-    const cpx<T> inv = crecip(prow[0]);
-    // eliminate column j from this CTA's other rows: the multipliers first (one thread per
-    // row), then the updates (one warp per row, lanes over columns; rows independent)
-    for (int i = tid; i < nr; i += blockDim.x)
-      if (!chosen[i]) rows[i * kb + j] = rows[i * kb + j] * inv;
-    __syncthreads();
-#pragma unroll 4
-    for (int i = warp; i < nr; i += kWarps) {
-      if (chosen[i]) continue;
-      cpx<T>* row = rows + i * kb + j;
-      const cpx<T> l = row[0];
-      const cpx<T> ml = mk(-l.re, -l.im);
-      for (int t = 1 + lane; t < kb - j; t += 32) cmac(row[t], ml, prow[t]);
-    }
-    __syncthreads();
+    if (tid == 0) s_piv[j] = pr;
+    mine = cta_max_key<kWarps>(panel_column(rows, chosen, nr, kb, j, lo, pr, prow[j & 1]), wk);
   }
+  __syncthreads();
   if (!ok) {
     // the panel stopped (a zero pivot or a wait that ran out): no row moves for it
     if (tid == 0 && s_fail) atomicOr(p.err, 2);
@@ -259,8 +326,8 @@ __global__ void __launch_bounds__(kPanelThreads) lu_panel_kernel(PanelArgs<T> p)
     return;
   }
   for (int e = tid; e < nr * kb; e += blockDim.x)
-    p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb] = rows[e];
-  if (g == 0 && tid == 0) panel_record_moves(p, s_piv);
+    p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb] = rows[(size_t)(e / kb) * pitch + e % kb];
+  if (g == 0) panel_record_moves(p, s_piv);
 }
 
 // ---- the panel inside one thread-block cluster (distributed shared memory)
@@ -274,110 +341,229 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// the address of `p` (this CTA's shared memory) in the shared memory of cluster CTA `rank`
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
+// the shared-memory address `a` of this CTA in the shared memory of cluster CTA `rank`
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, int rank) {
   uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(tc::smem_u32(p)), "r"(rank));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   return r;
 }
-__device__ __forceinline__ unsigned long long ld_cluster_u64(uint32_t a) {
-  unsigned long long v;
-  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(a) : "memory");
-  return v;
+// `bytes` (a multiple of 16) of this CTA's shared memory to a peer's (a cluster address), counted
+// by the peer's mbarrier
+__device__ __forceinline__ void bulk_to_peer(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(src), "r"(bytes), "r"(mbar)
+               : "memory");
 }
-__device__ __forceinline__ cpx<float> ld_cluster_cpx(const cpx<float>*, uint32_t a) {
-  float x, y;
-  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(x), "=f"(y) : "r"(a) : "memory");
-  return mk(x, y);
+// the largest of the lanes' keys: the two halves in turn
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+  return (unsigned long long)hi << 32 | lo;
 }
-__device__ __forceinline__ cpx<double> ld_cluster_cpx(const cpx<double>*, uint32_t a) {
-  double x, y;
-  asm volatile("ld.shared::cluster.v2.f64 {%0, %1}, [%2];" : "=d"(x), "=d"(y) : "r"(a) : "memory");
-  return mk(x, y);
+
+constexpr int kClWarps = 16;             // warps of a cluster panel's CTA that hold rows
+constexpr int kClSenders = 4;            // warps that send its candidates
+constexpr int kClThreads = 32 * (kClWarps + kClSenders);
+constexpr int kClSlots = 3;              // columns of candidates held
+constexpr unsigned kClPolls = 1u << 20;  // bound of a wait for a column's candidates
+// bytes of one candidate: its key, the reciprocal of its first entry (at 16), its entries (at 32)
+template <class T>
+__host__ __device__ constexpr uint32_t cand_bytes(int kb) {
+  return 32u + (uint32_t)((kb * sizeof(cpx<T>) + 15) & ~(size_t)15);
+}
+template <class T>
+__host__ __device__ constexpr int cl_batch() {   // rows a warp has in flight
+  return sizeof(T) == 4 ? 4 : 2;
+}
+// shared bytes of a CTA of `per` rows in a cluster of G: received candidates, own candidates,
+// rows (and what a batch reads past the last)
+template <class T>
+__host__ __device__ constexpr size_t cl_smem(int G, int per, int kb) {
+  return (size_t)kClSlots * (G + 1) * cand_bytes<T>(kb) + (size_t)(per + cl_batch<T>()) * cl_pitch(kb) * sizeof(cpx<T>);
 }
 
 // One panel of kb columns on rows k..n-1, the grid being one cluster of G CTAs.  Each CTA
-// holds its slice of rows in shared memory for the whole panel.  Per column it posts its
-// best pivot key in its own shared memory, the cluster barrier, then every CTA reads the
-// G keys and takes the largest (the same pivot as the grid form), and reads the pivot row
-// from the owner's shared memory.  The candidate slots are double-buffered by column: a CTA writes
-// the slot of column j + 2 only after the barrier of column j + 1, which every CTA passes
-// after its reads of column j.  A chosen row is never written again in the panel, so the
-// pivot row is read while its owner eliminates its other rows.  A last cluster barrier
-// keeps every CTA's shared memory in place until no peer reads it.
+// holds its slice of rows in shared memory for the whole panel, each of its row warps a share of
+// them.  Per column the sending warps bring the CTA's best candidate row up to date and send its
+// key, its entries and the reciprocal of the first to all G CTAs (one bulk copy each, counted by
+// the receivers' mbarriers); meanwhile the row warps finish the previous column on their other
+// rows.  All wait for the G candidates in their own shared memory and take the largest key (the
+// same pivot as the grid form); the row warps divide the column of their rows, form their next
+// column and that column's best key.  One trip between SMs and one block barrier per column; no
+// row warp reads another's rows.  Three columns of candidates are held: a CTA sends column j + 3
+// after it has column j + 2 of every peer, which a peer sends after the block barrier behind its
+// last use of column j.  Every wait is bounded; a last cluster barrier keeps every CTA's shared
+// memory in place until all have stopped sending.
+//
+// A serial chain per column: the CTA's best key, its row, the copies, the pivot, the column.
+// Sending by 16-byte remote stores took 220 cycles per peer, by bulk copies of one warp 65;
+// a cluster barrier, then reads of the keys and of the pivot row from the peers, 3,400.
 template <class T>
-__global__ void __launch_bounds__(kPanelThreads) lu_panel_cluster_kernel(PanelArgs<T> p) {
-  constexpr int kWarps = kPanelThreads / 32;
+__global__ void __launch_bounds__(kClThreads) lu_panel_cluster_kernel(PanelArgs<T> p) {
+  constexpr int kBatch = cl_batch<T>();
   const int G = gridDim.x, g = (int)cluster_rank(), tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int R = p.n - p.k, kb = p.kb;
   const int per = (R + G - 1) / G;
   const int lo = p.k + min(g * per, R), hi = p.k + min((g + 1) * per, R), nr = hi - lo;
+  const int pitch = cl_pitch(kb);
+  const uint32_t slot = cand_bytes<T>(kb);
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  cpx<T>* rows = reinterpret_cast<cpx<T>*>(smem_raw);                       // [per][kb]
-  unsigned char* chosen = smem_raw + (size_t)per * kb * sizeof(cpx<T>);     // [per]
-  __shared__ cpx<T> prow[kNb];
-  __shared__ unsigned long long wk[kWarps];
+  unsigned char* recv = smem_raw;                            // [kClSlots][G][slot]
+  unsigned char* own = recv + kClSlots * G * slot;           // [kClSlots][slot]
+  cpx<T>* rows = reinterpret_cast<cpx<T>*>(own + kClSlots * slot);   // [per + kBatch][pitch]
+  __shared__ uint64_t mbar[kClSlots];
+  __shared__ unsigned long long wk[2][kClWarps];   // the row warps' best keys, by column parity
   __shared__ int s_piv[kNb];
-  __shared__ unsigned long long s_ck[2];   // this CTA's key of the column, by column parity
-  __shared__ unsigned long long s_win;
-  for (int e = tid; e < nr * kb; e += blockDim.x)
-    rows[e] = p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb];
-  for (int i = tid; i < per; i += blockDim.x) chosen[i] = 0;
+  __shared__ int s_fail[2];   // error bits, by column parity: every warp leaves at the same column
+  for (int e = tid; e < nr * kb; e += kClThreads)
+    rows[(size_t)(e / kb) * pitch + e % kb] = p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb];
+  if (tid == 0) {
+    s_fail[0] = s_fail[1] = 0;
+    for (int i = 0; i < kClSlots; ++i) tc::mbar_init(&mbar[i], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  cluster_sync_all();
+  // this warp's rows r0 .. r0 + nw - 1 of the CTA's (at most 64: a bit each while not chosen)
+  const int q = (per + kClWarps - 1) / kClWarps;
+  const int r0 = min(warp * q, nr), nw = warp < kClWarps ? min(q, nr - r0) : 0;
+  unsigned long long alive = nw == 64 ? ~0ull : (1ull << nw) - 1;
+  {
+    unsigned long long best = 0;
+    for (int i = lane; i < nw; i += 32) {
+      const cpx<T> v = rows[(size_t)(r0 + i) * pitch];
+      best = umax64(best, pivot_key(v, lo + r0 + i));
+    }
+    best = warp_max_key(best);
+    if (lane == 0 && warp < kClWarps) wk[0][warp] = best;
+  }
   __syncthreads();
-  bool ok = true;
+  uint32_t prev_at = 0;   // where recv holds the pivot row of column j - 1, from that column on
+  int fail = 0, b = 0;
+  uint32_t phase = 0;
   for (int j = 0; j < kb; ++j) {
-    const int buf = j & 1;
-    const unsigned long long mine = cta_best_key<T, kWarps>(rows, chosen, nr, kb, j, lo, wk);
-    if (tid == 0) s_ck[buf] = mine;
-    cluster_sync_all();
-    // the pivot: the largest key over the cluster (the same choice in every CTA)
-    if (warp == 0) {
-      unsigned long long kmax = lane < G ? ld_cluster_u64(cluster_addr(&s_ck[buf], lane)) : 0ull;
+    const int cnt = kb - j;
+    const int nv = (int)((cnt * sizeof(cpx<T>) + 15) / 16);   // 16-byte pieces of a candidate's entries
+    if (tid == 0)
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(tc::smem_u32(&mbar[b])),
+                   "r"((uint32_t)G * (32u + 16u * (uint32_t)nv))
+                   : "memory");
+    const unsigned long long mine = warp_max_key(lane < kClWarps ? wk[j & 1][lane] : 0ull);
+    const int bl = mine != 0 ? key_row(mine) - lo : -1;
+    const cpx<T>* prev = reinterpret_cast<const cpx<T>*>(recv + prev_at);
+    if (warp >= kClWarps) {
+      const cpx<T>* row = rows + max(bl, 0) * pitch + j;
+      unsigned char* out = own + b * slot;
+      if (warp == kClWarps) {
+        // the candidate row's entries j.., with column j - 1's elimination (not written back:
+        // its warp takes them from what arrives)
+        const bool upd = j > 0 && bl >= 0;
+        const cpx<T> l = upd ? row[-1] : mk((T)0, (T)0);
+        const cpx<T> ml = mk(-l.re, -l.im);
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) kmax = umax64(kmax, __shfl_xor_sync(0xffffffffu, kmax, off));
-      if (lane == 0) s_win = kmax;
+        for (int u = 0; u < 2; ++u) {
+          const int e = lane + 32 * u;
+          if (e < cnt) {
+            cpx<T> v = row[e];
+            if (upd && e >= 1) cmac(v, ml, prev[e + 1]);
+            reinterpret_cast<cpx<T>*>(out + 32)[e] = v;
+          }
+        }
+      } else if (warp == kClWarps + 1 && lane == 0) {
+        *reinterpret_cast<unsigned long long*>(out) = mine;
+        *reinterpret_cast<cpx<T>*>(out + 16) = crecip(row[0]);
+      }
+      tc::fence_proxy_async();
+      asm volatile("bar.sync 1, %0;" ::"n"(32 * kClSenders) : "memory");
+      const int c = (warp - kClWarps) + kClSenders * lane;
+      if (c < G)
+        bulk_to_peer(cluster_addr(tc::smem_u32(recv + (b * G + g) * slot), c), tc::smem_u32(out),
+                     32u + 16u * (uint32_t)nv, cluster_addr(tc::smem_u32(&mbar[b]), c));
     }
-    __syncthreads();
-    const unsigned long long win = s_win;
+    if (j > 0) {
+      // entries j + 1.. of column j - 1's elimination on the warp's other rows: lanes over
+      // columns, kBatch rows in flight (the rows a batch reads past the warp's are not stored)
+      unsigned long long todo = alive;
+      if (bl >= r0 && bl < r0 + nw) todo &= ~(1ull << (bl - r0));
+      for (int c = 1 + lane; c - lane < cnt; c += 32) {
+        const bool in = c < cnt;
+        const int cc = in ? c : 0;
+        const cpx<T> pc = prev[cc + 1];
+        cpx<T>* row = rows + r0 * pitch + j;
+        for (int i0 = 0; i0 < nw; i0 += kBatch, row += kBatch * pitch) {
+          cpx<T> l[kBatch], v[kBatch];
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u) {
+            l[u] = row[u * pitch - 1];
+            v[u] = row[u * pitch + cc];
+          }
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u) cmac(v[u], mk(-l[u].re, -l[u].im), pc);
+          const unsigned bits = in ? (unsigned)(todo >> i0) : 0u;
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u)
+            if ((bits >> u) & 1) row[u * pitch + cc] = v[u];
+        }
+      }
+    }
+    __syncwarp();
+    // the candidates of column j, and the pivot
+    const bool got = tc::mbar_wait(&mbar[b], phase, kClPolls);
+    const unsigned char* at = recv + b * G * slot;
+    const unsigned long long key = got && lane < G ? *reinterpret_cast<const unsigned long long*>(at + lane * slot) : 0ull;
+    const unsigned long long win = warp_max_key(key);
     const int pr = win != 0 ? key_row(win) : -1;
-    if (!(pr >= p.k && pr < p.n)) {   // no row left (cannot happen with n - k >= kb): every CTA stops here
-      if (tid == 0 && g == 0) atomicOr(p.err, 4);
-      ok = false;
-      break;
+    const bool ok = pr >= p.k && pr < p.n;   // no row left cannot happen with n - k >= kb
+    unsigned long long best = 0;
+    if (ok) {
+      const int who = __ffs((int)__ballot_sync(0xffffffffu, key == win)) - 1;   // the CTA whose candidate it is
+      const unsigned char* cand = at + who * slot;
+      const cpx<T> inv = *reinterpret_cast<const cpx<T>*>(cand + 16);
+      prev_at = (b * G + who) * slot + 32;
+      const int mine_pr = pr - lo - r0;
+      if (mine_pr >= 0 && mine_pr < nw) alive &= ~(1ull << mine_pr);
+      if (bl >= r0 && bl < r0 + nw) {   // the entries of the CTA's candidate, back into its row
+        const cpx<T>* mc = reinterpret_cast<const cpx<T>*>(at + g * slot + 32);
+        for (int e = 1 + lane; e < cnt; e += 32) rows[bl * pitch + j + e] = mc[e];
+        __syncwarp();
+      }
+      const cpx<T> p1 = j + 1 < kb ? reinterpret_cast<const cpx<T>*>(cand + 32)[1] : mk((T)0, (T)0);
+      for (int i = lane; i < nw; i += 32) {
+        if (!((alive >> i) & 1)) continue;
+        cpx<T>* row = rows + (r0 + i) * pitch + j;
+        const cpx<T> l = row[0] * inv;
+        row[0] = l;
+        if (j + 1 < kb) {
+          cpx<T> v = row[1];
+          cmac(v, mk(-l.re, -l.im), p1);
+          row[1] = v;
+          best = umax64(best, pivot_key(v, lo + r0 + i));
+        }
+      }
+      best = warp_max_key(best);
     }
-    if ((win >> 32) == 0 && tid == 0 && g == 0) atomicOr(p.err, 4);   // a zero pivot
-    {
-      // the pivot row's entries j.. from its owner (its local row pr - lo_w, lo_w = k + w per)
-      const int w = (pr - p.k) / per;
-      const int lrow = pr - (p.k + w * per);
-      const cpx<T>* src = rows + (size_t)lrow * kb + j;
-      for (int t = tid; t < kb - j; t += blockDim.x) prow[t] = ld_cluster_cpx(src, cluster_addr(src + t, w));
+    if (lane == 0) {
+      if (warp < kClWarps) wk[(j + 1) & 1][warp] = best;
+      if (!ok) s_fail[j & 1] = got ? 4 : 2;
     }
     if (tid == 0) {
-      if (pr >= lo && pr < hi) chosen[pr - lo] = 1;
       s_piv[j] = pr;
+      if (ok && (win >> 32) == 0 && g == 0) atomicOr(p.err, 4);   // a zero pivot
     }
     __syncthreads();
-    const cpx<T> inv = crecip(prow[0]);
-    for (int i = tid; i < nr; i += blockDim.x)
-      if (!chosen[i]) rows[i * kb + j] = rows[i * kb + j] * inv;
-    __syncthreads();
-#pragma unroll 4
-    for (int i = warp; i < nr; i += kWarps) {
-      if (chosen[i]) continue;
-      cpx<T>* row = rows + i * kb + j;
-      const cpx<T> l = row[0];
-      const cpx<T> ml = mk(-l.re, -l.im);
-      for (int t = 1 + lane; t < kb - j; t += 32) cmac(row[t], ml, prow[t]);
+    fail = s_fail[j & 1];
+    if (fail != 0) break;
+    if (++b == kClSlots) {
+      b = 0;
+      phase ^= 1;
     }
-    __syncthreads();
   }
-  if (ok) {
-    for (int e = tid; e < nr * kb; e += blockDim.x)
-      p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb] = rows[e];
-    if (g == 0 && tid == 0) panel_record_moves(p, s_piv);
-  } else if (tid == 0 && g == 0) {
-    *p.n_moves = 0;   // the panel stopped: no row moves for it
+  if (fail == 0) {
+    for (int e = tid; e < nr * kb; e += kClThreads)
+      p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb] = rows[(size_t)(e / kb) * pitch + e % kb];
+    if (g == 0) panel_record_moves(p, s_piv);
+  } else if (tid == 0) {
+    atomicOr(p.err, fail);
+    if (g == 0) *p.n_moves = 0;   // the panel stopped: no row moves for it
   }
   cluster_sync_all();
 }
@@ -405,63 +591,84 @@ __global__ void __launch_bounds__(256) lu_moves_kernel(cpx<T>* a, int64_t ld, in
     if (col < n_cols && mv[m].x >= 0) a[(int64_t)mv[m].y * ld + col] = buf[m][cl];
 }
 
-// Column-oriented substitution with one warp: the right-hand side's entries of rows
-// lane and lane + 32 stay in the lane's registers; at step j the solved entry x_j is
+// Column-oriented substitution with one warp, NC right-hand sides in flight: their entries of
+// rows lane and lane + 32 stay in the lane's registers; at step j the solved entries x_j are
 // shuffled to every lane, and the rows below (lower) or above (upper) subtract their
 // coefficient times x_j.  M: the kb x kb diagonal block in shared memory (row stride ms).
-template <class T, bool UPPER>
-__device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb, cpx<T>& x0, cpx<T>& x1) {
+template <class T, bool UPPER, int NC>
+__device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb, cpx<T> (&x0)[NC], cpx<T> (&x1)[NC]) {
   const int lane = threadIdx.x & 31;
   for (int s = 0; s < kb; ++s) {
     const int j = UPPER ? kb - 1 - s : s;
-    if (UPPER) {   // x_j /= U_jj by the lane that holds row j
-      if (j < 32 && lane == j) x0 = cdiv(x0, M[j * ms + j]);
-      if (j >= 32 && lane == j - 32) x1 = cdiv(x1, M[j * ms + j]);
-    }
-    const T r0 = __shfl_sync(0xffffffffu, j < 32 ? x0.re : x1.re, j & 31);
-    const T i0 = __shfl_sync(0xffffffffu, j < 32 ? x0.im : x1.im, j & 31);
-    const cpx<T> xj = mk(-r0, -i0);
     const bool t0 = UPPER ? lane < j : (lane > j && lane < kb);
     const bool t1 = UPPER ? lane + 32 < j : (lane + 32 > j && lane + 32 < kb);
-    if (t0) cmac(x0, M[lane * ms + j], xj);
-    if (t1) cmac(x1, M[(lane + 32) * ms + j], xj);
+    const cpx<T> m0 = t0 ? M[lane * ms + j] : mk((T)0, (T)0), m1 = t1 ? M[(lane + 32) * ms + j] : mk((T)0, (T)0);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      if (UPPER) {   // x_j /= U_jj by the lane that holds row j
+        if (j < 32 && lane == j) x0[c] = cdiv(x0[c], M[j * ms + j]);
+        if (j >= 32 && lane == j - 32) x1[c] = cdiv(x1[c], M[j * ms + j]);
+      }
+      const T r0 = __shfl_sync(0xffffffffu, j < 32 ? x0[c].re : x1[c].re, j & 31);
+      const T i0 = __shfl_sync(0xffffffffu, j < 32 ? x0[c].im : x1[c].im, j & 31);
+      const cpx<T> xj = mk(-r0, -i0);
+      if (t0) cmac(x0[c], m0, xj);
+      if (t1) cmac(x1[c], m1, xj);
+    }
   }
 }
 
-// U12 = L11^-1 A12 on rows k..k+kb-1: L11 and a tile of 32 columns in shared memory,
-// one warp per column (lanes over rows), the tile stored back coalesced
+// U12 = L11^-1 A12 on rows k..k+kb-1 and columns k+kb..nc-1: L11 and a tile of 32 columns in
+// shared memory, four columns per warp at once (lanes over rows; a serial chain of kb steps,
+// so the columns of a warp share it), the tile stored back coalesced
 template <class T>
-__global__ void __launch_bounds__(256) lu_trsm_kernel(cpx<T>* a, int64_t ld, int n, int k, int kb) {
-  constexpr int TC = 32, LS = kNb + 1;
+__global__ void __launch_bounds__(256) lu_trsm_kernel(cpx<T>* a, int64_t ld, int nc, int k, int kb) {
+  constexpr int TC = 32, LS = kNb + 1, NC = TC / 8;
   extern __shared__ __align__(16) unsigned char sm[];
-  cpx<T>* L = reinterpret_cast<cpx<T>*>(sm);          // [kb][LS]
+  cpx<T>* L = reinterpret_cast<cpx<T>*>(sm);          // [kNb][LS]
   cpx<T>* X = L + kNb * LS;                            // [kNb][TC]
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int c0 = k + kb + blockIdx.x * TC;
-  for (int e = tid; e < kb * kb; e += blockDim.x) L[(e / kb) * LS + e % kb] = a[(int64_t)(k + e / kb) * ld + k + e % kb];
-  for (int e = tid; e < kb * TC; e += blockDim.x) {
-    const int r = e / TC, c = e % TC;
-    X[r * TC + c] = c0 + c < n ? a[(int64_t)(k + r) * ld + c0 + c] : mk((T)0, (T)0);
+  // (every load of a thread in flight at once)
+  cpx<T> vl[kNb * kNb / 256], vx[kNb * TC / 256];
+#pragma unroll
+  for (int u = 0; u < kNb * kNb / 256; ++u) {
+    const int r = (tid + 256 * u) / kNb, c = tid % kNb;
+    vl[u] = r < kb && c < kb ? a[(int64_t)(k + r) * ld + k + c] : mk((T)0, (T)0);
+  }
+#pragma unroll
+  for (int u = 0; u < kNb * TC / 256; ++u) {
+    const int r = (tid + 256 * u) / TC, c = tid % TC;
+    vx[u] = r < kb && c0 + c < nc ? a[(int64_t)(k + r) * ld + c0 + c] : mk((T)0, (T)0);
+  }
+#pragma unroll
+  for (int u = 0; u < kNb * kNb / 256; ++u) L[((tid + 256 * u) / kNb) * LS + tid % kNb] = vl[u];
+#pragma unroll
+  for (int u = 0; u < kNb * TC / 256; ++u) X[((tid + 256 * u) / TC) * TC + tid % TC] = vx[u];
+  __syncthreads();
+  cpx<T> x0[NC], x1[NC];
+#pragma unroll
+  for (int u = 0; u < NC; ++u) {
+    x0[u] = lane < kb ? X[lane * TC + warp * NC + u] : mk((T)0, (T)0);
+    x1[u] = lane + 32 < kb ? X[(lane + 32) * TC + warp * NC + u] : mk((T)0, (T)0);
+  }
+  warp_substitute<T, false, NC>(L, LS, kb, x0, x1);
+#pragma unroll
+  for (int u = 0; u < NC; ++u) {
+    if (lane < kb) X[lane * TC + warp * NC + u] = x0[u];
+    if (lane + 32 < kb) X[(lane + 32) * TC + warp * NC + u] = x1[u];
   }
   __syncthreads();
-  for (int c = warp; c < TC; c += blockDim.x / 32) {
-    cpx<T> x0 = lane < kb ? X[lane * TC + c] : mk((T)0, (T)0);
-    cpx<T> x1 = lane + 32 < kb ? X[(lane + 32) * TC + c] : mk((T)0, (T)0);
-    warp_substitute<T, false>(L, LS, kb, x0, x1);
-    if (lane < kb) X[lane * TC + c] = x0;
-    if (lane + 32 < kb) X[(lane + 32) * TC + c] = x1;
-  }
-  __syncthreads();
   for (int e = tid; e < kb * TC; e += blockDim.x) {
     const int r = e / TC, c = e % TC;
-    if (c0 + c < n) a[(int64_t)(k + r) * ld + c0 + c] = X[r * TC + c];
+    if (c0 + c < nc) a[(int64_t)(k + r) * ld + c0 + c] = X[r * TC + c];
   }
 }
 
-// A22 -= L21 U12: a 64 x 64 tile of complex entries per block, 256 threads with 4 x 4 each,
+// A22 -= L21 U12 (columns below nc): a 64 x 64 tile of complex entries per block, 256 threads with 4 x 4 each,
 // the whole K (the panel width) staged in shared memory (A transposed, padded)
 template <class T>
-__global__ void __launch_bounds__(256) lu_gemm_kernel(cpx<T>* a, int64_t ld, int n, int k, int kb) {
+__global__ void __launch_bounds__(256) lu_gemm_kernel(cpx<T>* a, int64_t ld, int n, int nc, int k, int kb) {
   constexpr int BM = 64, BN = 64, PA = BM + 1;
   extern __shared__ unsigned char sm[];
   cpx<T>* As = reinterpret_cast<cpx<T>*>(sm);   // [kb][PA]
@@ -474,7 +681,7 @@ __global__ void __launch_bounds__(256) lu_gemm_kernel(cpx<T>* a, int64_t ld, int
   }
   for (int e = tid; e < kb * BN; e += 256) {
     const int kk = e / BN, col = e % BN;
-    Bs[kk * BN + col] = c0 + col < n ? a[(int64_t)(k + kk) * ld + c0 + col] : mk((T)0, (T)0);
+    Bs[kk * BN + col] = c0 + col < nc ? a[(int64_t)(k + kk) * ld + c0 + col] : mk((T)0, (T)0);
   }
   __syncthreads();
   const int ty = tid >> 4, tx = tid & 15;
@@ -501,7 +708,7 @@ __global__ void __launch_bounds__(256) lu_gemm_kernel(cpx<T>* a, int64_t ld, int
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       const int cc = c0 + tx * 4 + j;
-      if (cc < n) {
+      if (cc < nc) {
         cpx<T>& z = a[(int64_t)r * ld + cc];
         z = z - acc[i][j];
       }
@@ -697,13 +904,15 @@ __global__ void __launch_bounds__(256, 2) lu_gemm_tc_kernel(cpx<float>* a, int64
   if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
-// every panel's row moves on the right-hand side, in panel order (one block)
+// every panel's row moves on the right-hand side, in panel order (one block); two lists per
+// panel, the second that of the panel's second half where it ran in two
 template <class T>
 __global__ void lu_vector_moves_kernel(cpx<T>* x, int n, int n_panels, const int2* moves, const int* n_moves) {
   __shared__ cpx<T> buf[2 * kNb];
-  for (int pnl = 0; pnl < n_panels; ++pnl) {
-    const int nm = max(0, min(n_moves[pnl], 2 * kNb));
-    const int2* mv = moves + (size_t)pnl * 2 * kNb;
+  for (int h = 0; h < 2 * n_panels; ++h) {
+    const int nm = max(0, min(n_moves[h], (h & 1) ? kNb : 2 * kNb));
+    if (nm == 0) continue;
+    const int2* mv = moves + (size_t)h * kNb;
     auto valid = [&](int2 v) { return v.x >= 0 && v.x < n && v.y >= 0 && v.y < n; };
     for (int m = threadIdx.x; m < nm; m += blockDim.x)
       if (valid(mv[m])) buf[m] = x[mv[m].x];
@@ -724,11 +933,11 @@ __device__ void block_solve(const cpx<T>* a, int64_t ld, int k, int kb, const cp
   __syncthreads();
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
-    cpx<T> x0 = lane < kb ? src[k + lane] : mk((T)0, (T)0);
-    cpx<T> x1 = lane + 32 < kb ? src[k + lane + 32] : mk((T)0, (T)0);
-    warp_substitute<T, UPPER>(D, LS, kb, x0, x1);
-    if (lane < kb) xb[lane] = x0;
-    if (lane + 32 < kb) xb[lane + 32] = x1;
+    cpx<T> x0[1] = {lane < kb ? src[k + lane] : mk((T)0, (T)0)};
+    cpx<T> x1[1] = {lane + 32 < kb ? src[k + lane + 32] : mk((T)0, (T)0)};
+    warp_substitute<T, UPPER, 1>(D, LS, kb, x0, x1);
+    if (lane < kb) xb[lane] = x0[0];
+    if (lane + 32 < kb) xb[lane + 32] = x1[0];
   }
   __syncthreads();
 }
@@ -922,18 +1131,22 @@ int lu_panel_grid(int rows, int sms) {
 }
 
 // the most rows of a panel of kb columns that one cluster of cs CTAs holds in shared
-// memory (the opt-in limit per CTA less room for the kernel's static words)
+// memory (the opt-in limit per CTA less room for the kernel's static words), at most 64 per warp
 template <class T>
 int cluster_panel_rows(int cs, int kb, int smem_optin) {
-  const int64_t avail = std::max<int64_t>(0, (int64_t)smem_optin - 4096);
-  return (int)std::min<int64_t>((int64_t)cs * (avail / ((int64_t)kb * (int64_t)sizeof(cpx<T>) + 1)), 1 << 30);
+  const int64_t avail = std::max<int64_t>(0, (int64_t)smem_optin - 4096 - (int64_t)cl_smem<T>(cs, 0, kb));
+  const int64_t per = std::min<int64_t>(avail / ((int64_t)cl_pitch(kb) * (int64_t)sizeof(cpx<T>)), 64 * kClWarps);
+  return (int)(cs * per);
 }
 
-// panels of at most this many rows run on the cluster: there its cheaper barrier wins
-// (GB300, 16 CTAs: 12.2 ms against 15.0 for the whole 2,000^2 complex64 factorization);
-// on longer panels the elimination work of its 16 CTAs outweighs it (8,000^2 with every
-// panel that fits on the cluster: 90.3 ms against 83.6 on the grid)
-constexpr int kClusterPanelRows = 2048;
+// panels of more than this many rows run as two halves of kNb / 2 columns (the second after
+// the first's update of its columns): half the elimination per column, and twice the rows fit
+// the cluster (12,880 in complex64, 6,032 in complex128 with 16 CTAs; beyond, the grid form).
+// Below, a half's own launches and narrow update (about 15 us) cost more than that gives.
+// GB300, 8,000^2 complex64, every panel: 42.2 ms (2,048 rows and more on the grid, whole; the
+// cluster's CTAs reading each other's candidates behind its barrier, one row per warp at a
+// time) -> 19 ms
+constexpr int kWholePanelRows = 2048;
 
 // cluster size of the cluster panels on this device: 16 CTAs where the device schedules
 // such a cluster with the shared memory it needs, else 8, else 0 (grid panels only)
@@ -950,7 +1163,7 @@ int choose_panel_cluster(int smem_optin, cudaStream_t s) {
   for (int c : {16, 8}) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
-    cfg.blockDim = dim3(kPanelThreads);
+    cfg.blockDim = dim3(kClThreads);
     cfg.dynamicSmemBytes = (size_t)dyn;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
@@ -974,7 +1187,7 @@ int lu_max_order(int sms) {
 
 template <class T>
 cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_t s) {
-  const int sms = current_sm_count();
+  const int sms = std::min(current_sm_count(), 256);   // lu_panel_kernel polls up to 256 CTAs' keys
   const int n_panels = (n + kNb - 1) / kNb;
   if (lu_panel_grid<T>(n, sms) > sms) return cudaErrorInvalidValue;
   if (n > 65535) return cudaErrorInvalidValue;   // rows and column tags are 16-bit fields of the pivot keys
@@ -984,7 +1197,7 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
   e = cudaMemsetAsync(w.err, 0, sizeof(int), s);
   if (e != cudaSuccess) return e;
   // no row moves until a panel records its own (a panel that stops early records none)
-  e = cudaMemsetAsync(w.n_moves, 0, (size_t)n_panels * sizeof(int), s);
+  e = cudaMemsetAsync(w.n_moves, 0, (size_t)2 * n_panels * sizeof(int), s);
   if (e != cudaSuccess) return e;
   const size_t trsm_smem = (size_t)kNb * (kNb + 1 + 32) * sizeof(cpx<T>);
   const size_t gemm_smem = (size_t)kNb * (65 + 64) * sizeof(cpx<T>);
@@ -992,7 +1205,7 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
   size_t panel_smem0 = 0;
   for (int pnl = 0; pnl < n_panels; ++pnl) {
     const int R = n - pnl * kNb, G = lu_panel_grid<T>(R, sms), per = (R + G - 1) / G;
-    panel_smem0 = std::max(panel_smem0, (size_t)per * kNb * sizeof(cpx<T>) + (size_t)per + 16);
+    panel_smem0 = std::max(panel_smem0, (size_t)per * cl_pitch(kNb) * sizeof(cpx<T>) + (size_t)per + 16);
   }
   if ((e = cudaFuncSetAttribute(lu_panel_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)panel_smem0)) != cudaSuccess)
@@ -1022,17 +1235,17 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
   const int cs = w.panel_cluster ? choose_panel_cluster<T>(smem_optin, s) : 0;
   w.diag[3] = 0;
   w.diag[4] = cs;
-  for (int pnl = 0; pnl < n_panels; ++pnl) {
-    const int k = pnl * kNb, kb = std::min(kNb, n - k), R = n - k;
+  // columns k .. k + kb - 1 as panel list h (its row moves on all columns included)
+  auto panel = [&](int k, int kb, int h, bool whole) -> cudaError_t {
+    const int R = n - k;
     PanelArgs<T> pa{a, ld, n, k, kb, reinterpret_cast<unsigned long long*>(w.cand_val),
-                    reinterpret_cast<cpx<T>*>(w.cand_data), w.moves + (size_t)pnl * 2 * kNb, w.n_moves + pnl,
-                    w.err};
-    if (cs > 0 && R <= std::min(kClusterPanelRows, cluster_panel_rows<T>(cs, kb, smem_optin))) {
-      const int per = (R + cs - 1) / cs;
+                    reinterpret_cast<cpx<T>*>(w.cand_data), w.moves + (size_t)h * kNb, w.n_moves + h, w.err};
+    cudaError_t e;
+    if (cs > 0 && R <= cluster_panel_rows<T>(cs, kb, smem_optin)) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(cs);
-      cfg.blockDim = dim3(kPanelThreads);
-      cfg.dynamicSmemBytes = (size_t)per * kb * sizeof(cpx<T>) + (size_t)per + 16;
+      cfg.blockDim = dim3(kClThreads);
+      cfg.dynamicSmemBytes = cl_smem<T>(cs, (R + cs - 1) / cs, kb);
       cfg.stream = s;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeClusterDimension;
@@ -1042,11 +1255,11 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
       cfg.attrs = at;
       cfg.numAttrs = 1;
       if ((e = cudaLaunchKernelEx(&cfg, lu_panel_cluster_kernel<T>, pa)) != cudaSuccess) return e;
-      ++w.diag[3];
+      if (whole) ++w.diag[3];
     } else {
       const int G = std::min(lu_panel_grid<T>(R, sms), per_sm * sms);   // all CTAs resident
       const int per = (R + G - 1) / G;
-      const size_t psmem = (size_t)per * kb * sizeof(cpx<T>) + (size_t)per + 16;
+      const size_t psmem = (size_t)per * cl_pitch(kb) * sizeof(cpx<T>) + (size_t)per + 16;
       void* args[] = {&pa};
       w.diag[0] = G;
       w.diag[1] = per_sm;
@@ -1055,7 +1268,19 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
                                            psmem, s)) != cudaSuccess)
         return e;
     }
-    lu_moves_kernel<T><<<(n + 15) / 16, 256, 0, s>>>(a, ld, n, w.moves + (size_t)pnl * 2 * kNb, w.n_moves + pnl);
+    lu_moves_kernel<T><<<(n + 15) / 16, 256, 0, s>>>(a, ld, n, pa.moves, pa.n_moves);
+    return cudaGetLastError();
+  };
+  for (int pnl = 0; pnl < n_panels; ++pnl) {
+    const int k = pnl * kNb, kb = std::min(kNb, n - k), hb = kNb / 2;
+    if (n - k <= kWholePanelRows) {
+      if ((e = panel(k, kb, 2 * pnl, true)) != cudaSuccess) return e;
+    } else {   // kb = kNb
+      if ((e = panel(k, hb, 2 * pnl, false)) != cudaSuccess) return e;
+      lu_trsm_kernel<T><<<1, 256, trsm_smem, s>>>(a, ld, k + kb, k, hb);
+      lu_gemm_kernel<T><<<dim3(1, (n - k - hb + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, k + kb, k, hb);
+      if ((e = panel(k + hb, hb, 2 * pnl + 1, false)) != cudaSuccess) return e;
+    }
     const int rest = n - k - kb;
     if (rest > 0) {
       lu_trsm_kernel<T><<<(rest + 31) / 32, 256, trsm_smem, s>>>(a, ld, n, k, kb);
@@ -1064,9 +1289,9 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
           lu_gemm_tc_kernel<<<dim3((rest + kUN / 2 - 1) / (kUN / 2), (rest + kUM - 1) / kUM), 256, kUSmem, s>>>(
               a, ld, n, k, kb, w.err);
         else
-          lu_gemm_kernel<T><<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, k, kb);
+          lu_gemm_kernel<T><<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, n, k, kb);
       } else {
-        lu_gemm_kernel<T><<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, k, kb);
+        lu_gemm_kernel<T><<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, n, k, kb);
       }
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
