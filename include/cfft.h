@@ -643,9 +643,10 @@ cfft_status cfft_port_currents(cfft_ctx* ctx, int n_elements, int port, const vo
  * the CTAs sending their candidate rows into each other's shared memory; any
  * other is a cooperative launch over the grid whose CTAs publish their
  * candidates' pivot keys, tagged with the column, in global memory.  Every
- * wait has a bound.  Then the panel's row moves applied to
- * the whole matrix, a triangular solve for the panel's rows and a complex matrix product for the trailing matrix.  In
- * complex64 that product runs on the tensor cores (three TF32 products, FP32
+ * wait has a bound.  Then the panel's row moves applied to the whole matrix,
+ * a triangular solve for the panel's rows and a complex matrix product for
+ * the trailing matrix.  The substitutions run in blocks of 64 rows, one
+ * cooperative launch each.  In complex64 the product runs on the tensor cores (three TF32 products, FP32
  * accumulation) unless the option SOLVE_SIMT is > 0, which keeps it on the
  * FP32 pipe.
  * cfft_get_solve_info reports the times and the relative residual

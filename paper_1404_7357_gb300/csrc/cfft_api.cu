@@ -136,7 +136,7 @@ struct cfft_ctx {
   std::vector<std::complex<double>> q_user;
   DevBuf d_quser;
   // dense LU of the reduced system: the factored copy, work arrays, vectors, timing
-  DevBuf lu_a, lu_moves, lu_nmoves, lu_cand_v, lu_cand_r, lu_cand_d, lu_bar, lu_err, lu_x, lu_y, lu_x64, lu_r, lu_sums;
+  DevBuf lu_a, lu_moves, lu_nmoves, lu_cand_v, lu_perm, lu_cand_d, lu_words, lu_err, lu_x, lu_y, lu_x64, lu_r, lu_sums;
   cudaEvent_t lu_ev[3] = {nullptr, nullptr, nullptr};
   int lu_diag[5] = {0, 0, 0, 0, 0};
   cfft_solve_info solve_info{};
@@ -2022,7 +2022,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->d_y, &ctx->d_grid, &ctx->d_table, &ctx->d_tw, &ctx->d_cnodes,
                       &ctx->d_coff, &ctx->d_cos, &ctx->d_lag, &ctx->d_flag, &ctx->d_pos,
                       &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
-                      &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_cand_r, &ctx->lu_cand_d, &ctx->lu_bar, &ctx->lu_err, &ctx->lu_x,
+                      &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_perm, &ctx->lu_cand_d, &ctx->lu_words, &ctx->lu_err, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
                       &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
                       &ctx->tc_bmat_mirror, &ctx->tc_shapes};
@@ -2576,21 +2576,33 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   CFFT_CUDA(ctx->lu_moves.ensure((size_t)panels * 2 * nb * sizeof(int2)), "alloc LU");
   CFFT_CUDA(ctx->lu_nmoves.ensure((size_t)panels * 2 * sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_v.ensure((size_t)ctx->sm_count * 2 * sizeof(double)), "alloc LU");
-  CFFT_CUDA(ctx->lu_cand_r.ensure((size_t)ctx->sm_count * 2 * sizeof(int)), "alloc LU");
+  CFFT_CUDA(ctx->lu_perm.ensure((size_t)n * sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_d.ensure((size_t)ctx->sm_count * 2 * nb * 16), "alloc LU");
-  CFFT_CUDA(ctx->lu_bar.ensure((size_t)panels * sizeof(unsigned)), "alloc LU");
+  CFFT_CUDA(ctx->lu_words.ensure((size_t)n * 2 * 4 * sizeof(unsigned long long)), "alloc LU");
   CFFT_CUDA(ctx->lu_err.ensure(sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_sums.ensure(4 * sizeof(double)), "alloc LU");
   w->moves = ctx->lu_moves.as<int2>();
   w->n_moves = ctx->lu_nmoves.as<int>();
   w->cand_val = ctx->lu_cand_v.as<double>();
-  w->cand_row = ctx->lu_cand_r.as<int>();
+  w->perm = ctx->lu_perm.as<int>();
   w->cand_data = ctx->lu_cand_d.p;
   w->diag = ctx->lu_diag;
-  w->bar = ctx->lu_bar.as<unsigned>();
+  w->words = ctx->lu_words.as<unsigned long long>();
   w->err = ctx->lu_err.as<int>();
   w->tc_update = ctx->opt[CFFT_OPT_SOLVE_SIMT] > 0 ? 0 : 1;
   w->panel_cluster = ctx->opt[CFFT_OPT_SOLVE_GRID_PANEL] > 0 ? 0 : 1;
+  return CFFT_OK;
+}
+
+// the error bits of the LU kernels so far, read behind them
+cfft_status lu_flags(cfft_ctx* ctx, const LuWork& w) {
+  int flag = 0;
+  CFFT_CUDA(cudaMemcpyAsync(&flag, w.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "LU flag");
+  CFFT_CUDA(cudaStreamSynchronize(ctx->stream), "LU");
+  if (flag & 2) return fail(ctx, CFFT_ERR_TIMEOUT, "LU panel: a wait for the pivot candidates ran past its bound");
+  if (flag & 4) return fail(ctx, CFFT_ERR_NUMERIC, "LU: the reduced matrix is singular (zero pivot)");
+  if (flag & 8) return fail(ctx, CFFT_ERR_TIMEOUT, "LU update: a tensor-core wait ran past its bound");
+  if (flag & 16) return fail(ctx, CFFT_ERR_TIMEOUT, "LU substitution: a wait for a solved block ran past its bound");
   return CFFT_OK;
 }
 
@@ -2604,13 +2616,7 @@ cfft_status lu_factor_checked(cfft_ctx* ctx, int n, const LuWork& w) {
                 ", shared bytes " + std::to_string(w.diag[2]) + ")";
     return st;
   }
-  int flag = 0;
-  CFFT_CUDA(cudaMemcpyAsync(&flag, w.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "LU flag");
-  CFFT_CUDA(cudaStreamSynchronize(ctx->stream), "LU factorization");
-  if (flag & 2) return fail(ctx, CFFT_ERR_TIMEOUT, "LU panel: a poll of the pivot keys ran past its bound");
-  if (flag & 4) return fail(ctx, CFFT_ERR_NUMERIC, "LU: the reduced matrix is singular (zero pivot)");
-  if (flag & 8) return fail(ctx, CFFT_ERR_TIMEOUT, "LU update: a tensor-core wait ran past its bound");
-  return CFFT_OK;
+  return lu_flags(ctx, w);
 }
 
 cfft_status read_sums(cfft_ctx* ctx, double* h, int count) {
@@ -2712,7 +2718,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[2], st), "event");
     CFFT_CUDA(residual_f64(z, ld, n, i_out, v, nullptr, ctx->lu_sums.as<double>(), st), "residual");
   }
-  if ((s = read_sums(ctx, h, 2)) != CFFT_OK) return s;
+  if ((s = read_sums(ctx, h, 2)) != CFFT_OK || (s = lu_flags(ctx, w)) != CFFT_OK) return s;
   float ms = 0.f;
   cfft_solve_info& in = ctx->solve_info;
   in = cfft_solve_info{};

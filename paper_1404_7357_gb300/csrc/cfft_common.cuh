@@ -550,11 +550,11 @@ struct LuWork {
                        // list, or one list per half
   int* n_moves;        // [panels][2]
   double* cand_val;    // [2][SMs] 64-bit words: the panel CTAs' pivot keys with column tags
-  int* cand_row;       // (unused)
+  int* perm;           // [n] the factors' row order
   void* cand_data;     // [2][SMs][panel width] complex, the element type: the candidates' entries
-  unsigned* bar;       // (unused)
+  unsigned long long* words;  // [2][n] solved entries with tags: 2 (complex64) or 4 words each
   int* err;            // bit 1: a key poll ran out; bit 2: zero pivot; bit 3: a tensor-core
-                       // wait of the trailing update ran out
+                       // wait of the trailing update ran out; bit 4: a wait of a substitution
   int* diag;           // host: [5] panel grid, resident CTAs per SM, shared bytes of the last grid
                        // panel; panels run on one cluster, CTAs per cluster (0: none)
   int tc_update;       // complex64: the trailing update on the tensor cores

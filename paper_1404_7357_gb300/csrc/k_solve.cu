@@ -26,15 +26,14 @@
 //   gemm     A22 -= L21 U12, K = the panel: in complex64 on the tensor cores (the
 //            complex product as a real GEMM, three TF32 products), otherwise
 //            64 x 64 tiles of complex entries on the FP32 / FP64 pipe.
-// The solve applies every panel's moves to the right-hand side, then blocked
-// forward (unit L) and backward (U) substitution: per panel one launch whose
-// CTAs each solve the small diagonal block (one warp) and update their rows.
+// The solve takes the right-hand side in the factors' row order, then forward (unit L)
+// and backward (U) substitution, one cooperative launch each: block rows of 64 dealt to
+// the CTAs, solved entries passed on through tagged words in global memory.
 //
-// Every poll of the grid panel is bounded: a poll that runs out sets an error bit,
-// and every CTA leaves the panel (the host then returns CFFT_ERR_TIMEOUT).  The
-// cluster barrier is the hardware's own: every CTA of the cluster is resident by
-// construction, and every CTA takes every barrier (the pivot, and so any early
-// stop, is the same decision in all of them).
+// Every wait is bounded: one that runs out sets an error bit, and the CTAs leave the
+// kernel (the host then returns CFFT_ERR_TIMEOUT).  The cluster barriers before and
+// behind a cluster panel are the hardware's own: every CTA of the cluster is resident
+// by construction and takes both.
 #include <algorithm>
 
 #include "cfft_common.cuh"
@@ -593,10 +592,12 @@ __global__ void __launch_bounds__(256) lu_moves_kernel(cpx<T>* a, int64_t ld, in
 
 // Column-oriented substitution with one warp, NC right-hand sides in flight: their entries of
 // rows lane and lane + 32 stay in the lane's registers; at step j the solved entries x_j are
-// shuffled to every lane, and the rows below (lower) or above (upper) subtract their
-// coefficient times x_j.  M: the kb x kb diagonal block in shared memory (row stride ms).
+// shuffled to every lane, and the rows below (lower, unit diagonal) or above (upper, rd the
+// diagonal's reciprocals) subtract their coefficient times x_j.  M: the kb x kb diagonal block
+// in shared memory (row stride ms).
 template <class T, bool UPPER, int NC>
-__device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb, cpx<T> (&x0)[NC], cpx<T> (&x1)[NC]) {
+__device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb, const cpx<T>* rd, cpx<T> (&x0)[NC],
+                                                cpx<T> (&x1)[NC]) {
   const int lane = threadIdx.x & 31;
   for (int s = 0; s < kb; ++s) {
     const int j = UPPER ? kb - 1 - s : s;
@@ -605,15 +606,23 @@ __device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb,
     const cpx<T> m0 = t0 ? M[lane * ms + j] : mk((T)0, (T)0), m1 = t1 ? M[(lane + 32) * ms + j] : mk((T)0, (T)0);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (UPPER) {   // x_j /= U_jj by the lane that holds row j
-        if (j < 32 && lane == j) x0[c] = cdiv(x0[c], M[j * ms + j]);
-        if (j >= 32 && lane == j - 32) x1[c] = cdiv(x1[c], M[j * ms + j]);
+      cpx<T> xj = mk(__shfl_sync(0xffffffffu, j < 32 ? x0[c].re : x1[c].re, j & 31),
+                     __shfl_sync(0xffffffffu, j < 32 ? x0[c].im : x1[c].im, j & 31));
+      if (UPPER) {
+        const cpx<T> y = xj;
+        xj = y * rd[j];
+        if constexpr (sizeof(T) == 8) {   // the quotient's last bits, as a division would have them
+          cpx<T> r = y;
+          const cpx<T> d = M[j * ms + j];
+          cmac(r, mk(-xj.re, -xj.im), d);
+          cmac(xj, r, rd[j]);
+        }
+        if (lane == j) x0[c] = xj;
+        if (lane + 32 == j) x1[c] = xj;
       }
-      const T r0 = __shfl_sync(0xffffffffu, j < 32 ? x0[c].re : x1[c].re, j & 31);
-      const T i0 = __shfl_sync(0xffffffffu, j < 32 ? x0[c].im : x1[c].im, j & 31);
-      const cpx<T> xj = mk(-r0, -i0);
-      if (t0) cmac(x0[c], m0, xj);
-      if (t1) cmac(x1[c], m1, xj);
+      xj = mk(-xj.re, -xj.im);
+      if ((UPPER || j < 31) && t0) cmac(x0[c], m0, xj);
+      if ((!UPPER || j > 32) && t1) cmac(x1[c], m1, xj);
     }
   }
 }
@@ -652,7 +661,7 @@ __global__ void __launch_bounds__(256) lu_trsm_kernel(cpx<T>* a, int64_t ld, int
     x0[u] = lane < kb ? X[lane * TC + warp * NC + u] : mk((T)0, (T)0);
     x1[u] = lane + 32 < kb ? X[(lane + 32) * TC + warp * NC + u] : mk((T)0, (T)0);
   }
-  warp_substitute<T, false, NC>(L, LS, kb, x0, x1);
+  warp_substitute<T, false, NC>(L, LS, kb, nullptr, x0, x1);
 #pragma unroll
   for (int u = 0; u < NC; ++u) {
     if (lane < kb) X[lane * TC + warp * NC + u] = x0[u];
@@ -904,88 +913,266 @@ __global__ void __launch_bounds__(256, 2) lu_gemm_tc_kernel(cpx<float>* a, int64
   if (warp == 0) tc::tmem_dealloc(tmem, 256);
 }
 
-// every panel's row moves on the right-hand side, in panel order (one block); two lists per
-// panel, the second that of the panel's second half where it ran in two
-template <class T>
-__global__ void lu_vector_moves_kernel(cpx<T>* x, int n, int n_panels, const int2* moves, const int* n_moves) {
-  __shared__ cpx<T> buf[2 * kNb];
-  for (int h = 0; h < 2 * n_panels; ++h) {
-    const int nm = max(0, min(n_moves[h], (h & 1) ? kNb : 2 * kNb));
-    if (nm == 0) continue;
-    const int2* mv = moves + (size_t)h * kNb;
-    auto valid = [&](int2 v) { return v.x >= 0 && v.x < n && v.y >= 0 && v.y < n; };
-    for (int m = threadIdx.x; m < nm; m += blockDim.x)
-      if (valid(mv[m])) buf[m] = x[mv[m].x];
+// the row order of the factors: row i holds the matrix's row perm[i], every panel's row moves
+// applied in panel order (two lists per panel, the second that of the panel's second half where
+// it ran in two).  One block, the order in shared memory (n <= 65535), kPermLists lists at a
+// time: on a vector in global memory the lists took 1 us each (8,000: 0.25 ms per right-hand
+// side); once per factorization
+constexpr int kPermLists = 32;
+__global__ void __launch_bounds__(256) lu_order_kernel(int n, int n_lists, const int2* moves, const int* n_moves,
+                                                       int* perm) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  unsigned short* p = reinterpret_cast<unsigned short*>(sm);
+  __shared__ int2 mv[kPermLists * kNb];
+  __shared__ int nm[kPermLists];
+  for (int i = threadIdx.x; i < n; i += 256) p[i] = (unsigned short)i;
+  for (int h0 = 0; h0 < n_lists; h0 += kPermLists) {
+    const int cnt = min(kPermLists, n_lists - h0);
     __syncthreads();
-    for (int m = threadIdx.x; m < nm; m += blockDim.x)
-      if (valid(mv[m])) x[mv[m].y] = buf[m];
+    if ((int)threadIdx.x < cnt)
+      nm[threadIdx.x] = max(0, min(n_moves[h0 + threadIdx.x], ((h0 + threadIdx.x) & 1) ? kNb : 2 * kNb));
+    for (int e = threadIdx.x; e < cnt * kNb; e += 256) mv[e] = moves[(size_t)h0 * kNb + e];
     __syncthreads();
+    for (int h = 0; h < cnt; ++h) {
+      if (nm[h] == 0) continue;   // the same in every thread
+      const int m = threadIdx.x;  // at most 2 kNb moves; a whole panel's list runs on into its second place
+      int2 v = make_int2(-1, -1);
+      unsigned short r = 0;
+      if (m < nm[h]) {
+        v = mv[h * kNb + m];
+        if (v.x >= 0 && v.x < n && v.y >= 0 && v.y < n) r = p[v.x];
+        else v.x = -1;
+      }
+      __syncthreads();
+      if (v.x >= 0) p[v.y] = r;
+      __syncthreads();
+    }
   }
+  __syncthreads();
+  for (int i = threadIdx.x; i < n; i += 256) perm[i] = p[i];
+}
+static_assert(kPermLists % 2 == 0, "a panel's two lists are staged together");
+
+// A solved entry on its way to the other CTAs: 32 bits of value under a tag per 64-bit word, so
+// that a reader that finds the tag has the value (no flag, no fence)
+constexpr unsigned kSolvedTag = 1;
+__device__ __forceinline__ unsigned long long tag_word(unsigned v) {
+  return (unsigned long long)kSolvedTag << 32 | v;
+}
+template <class T>
+struct Solved;
+template <>
+struct Solved<float> {
+  static constexpr int kWords = 2;
+  static __device__ __forceinline__ void put(volatile unsigned long long* w, cpx<float> v) {
+    w[0] = tag_word(__float_as_uint(v.re));
+    w[1] = tag_word(__float_as_uint(v.im));
+  }
+  static __device__ __forceinline__ cpx<float> value(const unsigned long long* w) {
+    return mk(__uint_as_float((unsigned)w[0]), __uint_as_float((unsigned)w[1]));
+  }
+};
+template <>
+struct Solved<double> {
+  static constexpr int kWords = 4;
+  static __device__ __forceinline__ void put(volatile unsigned long long* w, cpx<double> v) {
+    w[0] = tag_word((unsigned)__double2loint(v.re));
+    w[1] = tag_word((unsigned)__double2hiint(v.re));
+    w[2] = tag_word((unsigned)__double2loint(v.im));
+    w[3] = tag_word((unsigned)__double2hiint(v.im));
+  }
+  static __device__ __forceinline__ cpx<double> value(const unsigned long long* w) {
+    return mk(__hiloint2double((int)(unsigned)w[1], (int)(unsigned)w[0]),
+              __hiloint2double((int)(unsigned)w[3], (int)(unsigned)w[2]));
+  }
+};
+
+// acc[u] (row 8 warp + u, u < 8) summed over the warp's lanes: halving exchanges, after which
+// lane 4 u' holds a whole row; returns that row's sum and its index in the warp (all lanes)
+template <class T>
+__device__ __forceinline__ cpx<T> rows_sum(cpx<T> (&acc)[8], int& row) {
+  const int lane = threadIdx.x & 31;
+  row = 0;
+#pragma unroll
+  for (int half = 4, off = 16; half > 0; half >>= 1, off >>= 1) {
+    const bool up = (lane & off) != 0;
+    row += up ? half : 0;
+#pragma unroll
+    for (int u = 0; u < half; ++u) {
+      const cpx<T> keep = up ? acc[u + half] : acc[u], give = up ? acc[u] : acc[u + half];
+      acc[u].re = keep.re + __shfl_xor_sync(0xffffffffu, give.re, off);
+      acc[u].im = keep.im + __shfl_xor_sync(0xffffffffu, give.im, off);
+    }
+  }
+  cpx<T> v = acc[0];
+#pragma unroll
+  for (int off = 2; off > 0; off >>= 1) {
+    v.re += __shfl_xor_sync(0xffffffffu, v.re, off);
+    v.im += __shfl_xor_sync(0xffffffffu, v.im, off);
+  }
+  return v;
 }
 
-// the diagonal block of rows k..k+kb-1 into shared memory (coalesced), then one warp
-// solves it against src[k..k+kb) (unit lower: forward; upper: backward) into xb
+// One row of a kNb x kNb matrix (row stride kNb + 1, shared) times a vector: four threads per
+// row, the sum in all four
+template <class T>
+__device__ __forceinline__ cpx<T> row_times(const cpx<T>* M, const cpx<T>* v) {
+  const int r = threadIdx.x >> 2, part = threadIdx.x & 3;
+  cpx<T> s = mk((T)0, (T)0);
+#pragma unroll
+  for (int q = 0; q < kNb / 4; ++q) cmac(s, M[r * (kNb + 1) + part + 4 * q], v[part + 4 * q]);
+#pragma unroll
+  for (int off = 1; off < 4; off <<= 1) {
+    s.re += __shfl_xor_sync(0xffffffffu, s.re, off);
+    s.im += __shfl_xor_sync(0xffffffffu, s.im, off);
+  }
+  return s;
+}
+
+template <class T>
+constexpr size_t subst_smem() {   // the diagonal block, and its inverse (complex64)
+  return (size_t)(sizeof(T) == 4 ? 2 : 1) * kNb * (kNb + 1) * sizeof(cpx<T>);
+}
+
+// x with L x = b[order] (unit lower) or U x = b (UPPER), one cooperative launch: block rows of
+// kNb, dealt to the CTAs in the order in which they are solved, so the lowest unsolved one always
+// has a CTA at work on it.  A CTA subtracts the solved blocks as they appear (its next tile's
+// loads in flight meanwhile), solves its diagonal block and publishes the entries.  complex64
+// inverts the diagonal block while it waits and multiplies by the inverse, with one step of
+// refinement against the block itself, so that the error is that of a substitution; in complex128
+// the FP64 pipe makes the three products (13 us) and the inverse (50 us and more) dearer than a
+// substitution of 64 serial steps.  Bound by the chain of blocks: publish, poll, one tile, the
+// diagonal block.  One launch per block row with a serial substitution in every CTA took 15 us
+// (forward) and 25 us (backward) per block in complex64.
 template <class T, bool UPPER>
-__device__ void block_solve(const cpx<T>* a, int64_t ld, int k, int kb, const cpx<T>* src, cpx<T>* D,
-                            cpx<T>* xb) {
-  constexpr int LS = kNb + 1;
-  for (int e = threadIdx.x; e < kb * kb; e += blockDim.x) D[(e / kb) * LS + e % kb] = a[(int64_t)(k + e / kb) * ld + k + e % kb];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    cpx<T> x0[1] = {lane < kb ? src[k + lane] : mk((T)0, (T)0)};
-    cpx<T> x1[1] = {lane + 32 < kb ? src[k + lane + 32] : mk((T)0, (T)0)};
-    warp_substitute<T, UPPER, 1>(D, LS, kb, x0, x1);
-    if (lane < kb) xb[lane] = x0[0];
-    if (lane + 32 < kb) xb[lane + 32] = x1[0];
-  }
-  __syncthreads();
-}
-
-// forward step of panel k: y_b = L11^-1 x_b (written to y), x[r] -= L[r][k..] y_b for the
-// rows below (one warp per row)
-template <class T>
-__global__ void __launch_bounds__(256) lu_forward_kernel(const cpx<T>* a, int64_t ld, int n, int k, int kb,
-                                                         cpx<T>* x, cpx<T>* y) {
-  __shared__ cpx<T> yb[kNb];
+__global__ void __launch_bounds__(256) lu_substitute_kernel(const cpx<T>* a, int64_t ld, int n, const int* order,
+                                                            const cpx<T>* b, cpx<T>* x, unsigned long long* words,
+                                                            int* err) {
+  constexpr int LS = kNb + 1, W = Solved<T>::kWords;
   extern __shared__ __align__(16) unsigned char sm[];
-  block_solve<T, false>(a, ld, k, kb, x, reinterpret_cast<cpx<T>*>(sm), yb);
-  if (blockIdx.x == 0)
-    for (int t = threadIdx.x; t < kb; t += blockDim.x) y[k + t] = yb[t];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int r = k + kb + blockIdx.x * nw + warp; r < n; r += gridDim.x * nw) {
-    cpx<T> acc = mk((T)0, (T)0);
-    for (int j = lane; j < kb; j += 32) cmac(acc, a[(int64_t)r * ld + k + j], yb[j]);
+  cpx<T>* D = reinterpret_cast<cpx<T>*>(sm);   // the diagonal block
+  cpx<T>* V = D + kNb * LS;                     // its inverse (complex64)
+  __shared__ cpx<T> xs[2][kNb], rhs[kNb], sol[kNb], rd[kNb];
+  __shared__ int s_fail;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nb = (n + kNb - 1) / kNb;
+  const cpx<T> zero = mk((T)0, (T)0);
+  if (tid == 0) s_fail = 0;
+  for (int t = blockIdx.x; t < nb; t += gridDim.x) {
+    const int k = kNb * (UPPER ? nb - 1 - t : t), kb = min(kNb, n - k);
+    __syncthreads();
+    cpx<T> v[kNb * kNb / 256];
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      acc.re += __shfl_xor_sync(0xffffffffu, acc.re, off);
-      acc.im += __shfl_xor_sync(0xffffffffu, acc.im, off);
+    for (int u = 0; u < kNb * kNb / 256; ++u) {
+      const int r = (tid >> 6) + 4 * u, c = tid & 63;
+      v[u] = r < kb && c < kb ? a[(int64_t)(k + r) * ld + k + c] : mk(r == c ? (T)1 : (T)0, (T)0);
+      if (UPPER ? r > c : r < c) v[u] = zero;
+      if (!UPPER && r == c) v[u] = mk((T)1, (T)0);
     }
-    if (lane == 0) x[r] = x[r] - acc;
-  }
-}
-
-// backward step of panel k: x_b = U11^-1 y_b (written to x), y[r] -= U[r][k..] x_b for the
-// rows above
-template <class T>
-__global__ void __launch_bounds__(256) lu_backward_kernel(const cpx<T>* a, int64_t ld, int k, int kb,
-                                                          cpx<T>* y, cpx<T>* x) {
-  __shared__ cpx<T> xb[kNb];
-  extern __shared__ __align__(16) unsigned char sm[];
-  block_solve<T, true>(a, ld, k, kb, y, reinterpret_cast<cpx<T>*>(sm), xb);
-  if (blockIdx.x == 0)
-    for (int t = threadIdx.x; t < kb; t += blockDim.x) x[k + t] = xb[t];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int r = blockIdx.x * nw + warp; r < k; r += gridDim.x * nw) {
-    cpx<T> acc = mk((T)0, (T)0);
-    for (int j = lane; j < kb; j += 32) cmac(acc, a[(int64_t)r * ld + k + j], xb[j]);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      acc.re += __shfl_xor_sync(0xffffffffu, acc.re, off);
-      acc.im += __shfl_xor_sync(0xffffffffu, acc.im, off);
+    for (int u = 0; u < kNb * kNb / 256; ++u) D[((tid >> 6) + 4 * u) * LS + (tid & 63)] = v[u];
+    if (tid < kb) rhs[tid] = b[order ? order[k + tid] : k + tid];
+    if (tid >= kb && tid < kNb) rhs[tid] = zero;
+    __syncthreads();
+    if (UPPER) {
+      if (tid < kNb) rd[tid] = crecip(D[tid * LS + tid]);
+      __syncthreads();
     }
-    if (lane == 0) y[r] = y[r] - acc;
+    if constexpr (sizeof(T) == 4) {
+      cpx<T> x0[8], x1[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        x0[u] = mk(lane == 8 * warp + u ? (T)1 : (T)0, (T)0);
+        x1[u] = mk(lane + 32 == 8 * warp + u ? (T)1 : (T)0, (T)0);
+      }
+      warp_substitute<T, UPPER, 8>(D, LS, kNb, rd, x0, x1);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        V[lane * LS + 8 * warp + u] = x0[u];
+        V[(lane + 32) * LS + 8 * warp + u] = x1[u];
+      }
+    }
+    // the solved blocks: rows k + 8 warp + u, columns lane and lane + 32 of each
+    cpx<T> acc[8], m0[8], m1[8];
+    auto load = [&](int s) {
+      const int c = kNb * (UPPER ? nb - 1 - s : s) + lane;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int r = k + 8 * warp + u;
+        const cpx<T>* p = a + (int64_t)r * ld + c;
+        m0[u] = r < n && c < n ? ldcg(p) : zero;
+        m1[u] = r < n && c + 32 < n ? ldcg(p + 32) : zero;
+      }
+    };
+#pragma unroll
+    for (int u = 0; u < 8; ++u) acc[u] = zero;
+    if (t > 0) load(0);
+    for (int s = 0; s < t; ++s) {
+      if (warp == 0) {
+        const int c = kNb * (UPPER ? nb - 1 - s : s) + lane;
+        const volatile unsigned long long* p = words + (size_t)c * W;
+        unsigned long long w[2][W];
+        bool have = false;
+        for (unsigned polls = 0; polls <= kBarrierPolls && !have; ++polls) {
+          if (polls > 0 && t - s > 2) __nanosleep(200);   // the next blocks first
+          have = true;
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int q = 0; q < W; ++q) {
+              w[h][q] = c + 32 * h < n ? p[32 * h * W + q] : tag_word(0);
+              have = have && (unsigned)(w[h][q] >> 32) == kSolvedTag;
+            }
+        }
+        if (!have) s_fail = 1;
+        xs[s & 1][lane] = Solved<T>::value(w[0]);
+        xs[s & 1][lane + 32] = Solved<T>::value(w[1]);
+      }
+      __syncthreads();
+      if (s_fail) break;
+      const cpx<T> y0 = xs[s & 1][lane], y1 = xs[s & 1][lane + 32];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        cmac(acc[u], m0[u], y0);
+        cmac(acc[u], m1[u], y1);
+      }
+      if (s + 1 < t) load(s + 1);
+    }
+    int row;
+    const cpx<T> sum = rows_sum(acc, row);
+    if ((lane & 3) == 0) rhs[8 * warp + row] = rhs[8 * warp + row] - sum;
+    __syncthreads();
+    if (s_fail) break;
+    if constexpr (sizeof(T) == 8) {
+      if (warp == 0) {
+        cpx<T> x0[1] = {rhs[lane]}, x1[1] = {rhs[lane + 32]};
+        warp_substitute<T, UPPER, 1>(D, LS, kb, rd, x0, x1);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int r = lane + 32 * h;
+          const cpx<T> z = h ? x1[0] : x0[0];
+          if (r < kb) {
+            Solved<T>::put(words + (size_t)(k + r) * W, z);
+            x[k + r] = z;
+          }
+        }
+      }
+      continue;
+    }
+    const int r = tid >> 2;
+    const cpx<T> y = row_times(V, rhs);
+    if ((tid & 3) == 0) sol[r] = y;
+    __syncthreads();
+    const cpx<T> dy = row_times(D, sol);
+    if ((tid & 3) == 0) xs[0][r] = rhs[r] - dy;
+    __syncthreads();
+    const cpx<T> z = y + row_times(V, xs[0]);
+    if ((tid & 3) == 0 && r < kb) {
+      Solved<T>::put(words + (size_t)(k + r) * W, z);
+      x[k + r] = z;
+    }
   }
+  if (tid == 0 && s_fail) atomicOr(err, 16);
 }
 
 // r = b - Z x in float64 from the float64 matrix (one warp per row), and |r|^2, |b|^2 sums
@@ -1296,31 +1483,38 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  const size_t osmem = (size_t)n * sizeof(unsigned short);
+  if ((e = cudaFuncSetAttribute(lu_order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)osmem)) !=
+      cudaSuccess)
+    return e;
+  lu_order_kernel<<<1, 256, osmem, s>>>(n, 2 * n_panels, w.moves, w.n_moves, w.perm);
+  return cudaGetLastError();
 }
 
 template <class T>
 cudaError_t lu_solve(const cpx<T>* a, int64_t ld, int n, const LuWork& w, cpx<T>* x, cpx<T>* y, cudaStream_t s) {
-  const int sms = current_sm_count();
-  const int n_panels = (n + kNb - 1) / kNb;
-  const size_t dsm = (size_t)kNb * (kNb + 1) * sizeof(cpx<T>);
+  constexpr size_t smem = subst_smem<T>();
+  const size_t bytes = (size_t)n * Solved<T>::kWords * sizeof(unsigned long long);
+  unsigned long long* words[2] = {w.words, w.words + (size_t)n * Solved<T>::kWords};
+  int G = std::min((n + kNb - 1) / kNb, current_sm_count());
+  const int* order = w.perm;
+  const int* none = nullptr;
+  const cpx<T>* xc = x;
+  const cpx<T>* yc = y;
+  int* err = w.err;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(lu_forward_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)) !=
-      cudaSuccess)
+  if ((e = cudaMemsetAsync(w.words, 0, 2 * bytes, s)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(lu_substitute_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem)) != cudaSuccess ||
+      (e = cudaFuncSetAttribute(lu_substitute_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)smem)) != cudaSuccess)
     return e;
-  if ((e = cudaFuncSetAttribute(lu_backward_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)) !=
-      cudaSuccess)
+  void* fwd[] = {&a, &ld, &n, &order, &xc, &y, &words[0], &err};
+  if ((e = cudaLaunchCooperativeKernel((const void*)lu_substitute_kernel<T, false>, dim3(G), dim3(256), fwd, smem,
+                                       s)) != cudaSuccess)
     return e;
-  lu_vector_moves_kernel<T><<<1, 128, 0, s>>>(x, n, n_panels, w.moves, w.n_moves);
-  for (int pnl = 0; pnl < n_panels; ++pnl) {
-    const int k = pnl * kNb, kb = std::min(kNb, n - k);
-    lu_forward_kernel<T><<<grid_for(n - k - kb, 8, 2 * sms), 256, dsm, s>>>(a, ld, n, k, kb, x, y);
-  }
-  for (int pnl = n_panels - 1; pnl >= 0; --pnl) {
-    const int k = pnl * kNb, kb = std::min(kNb, n - k);
-    lu_backward_kernel<T><<<grid_for(k, 8, 2 * sms), 256, dsm, s>>>(a, ld, k, kb, y, x);
-  }
-  return cudaGetLastError();
+  void* bwd[] = {&a, &ld, &n, &none, &yc, &x, &words[1], &err};
+  return cudaLaunchCooperativeKernel((const void*)lu_substitute_kernel<T, true>, dim3(G), dim3(256), bwd, smem, s);
 }
 
 cudaError_t residual_f64(const void* z, int64_t ld, int n, const void* x, const void* b, void* r, double* sums,
