@@ -2594,6 +2594,9 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   return CFFT_OK;
 }
 
+// row stride of the context's copy of an n x n matrix: whole 128-byte lines
+int64_t lu_stride(int n) { return ((int64_t)n + 15) & ~(int64_t)15; }
+
 // the error bits of the LU kernels so far, read behind them
 cfft_status lu_flags(cfft_ctx* ctx, const LuWork& w) {
   int flag = 0;
@@ -2609,7 +2612,7 @@ cfft_status lu_flags(cfft_ctx* ctx, const LuWork& w) {
 // factor the context's copy of Z (element type T, dense n x n) and report the panel status
 template <class T>
 cfft_status lu_factor_checked(cfft_ctx* ctx, int n, const LuWork& w) {
-  cudaError_t e = lu_factor<T>(ctx->lu_a.as<cpx<T>>(), n, n, w, ctx->stream);
+  cudaError_t e = lu_factor<T>(ctx->lu_a.as<cpx<T>>(), lu_stride(n), n, w, ctx->stream);
   if (e != cudaSuccess) {
     cfft_status st = cuda_fail(ctx, e, "LU factorization");
     ctx->err += " (panel grid " + std::to_string(w.diag[0]) + ", resident per SM " + std::to_string(w.diag[1]) +
@@ -2664,28 +2667,28 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
     return fail(ctx, CFFT_ERR_ARG, "solve: order " + std::to_string(n) + " exceeds " + std::to_string(n_lim) +
                 " (the panel's rows must fit the shared memory of the panel CTAs; pivot keys hold 16-bit rows)");
   const size_t es = fp64_lu ? 16 : 8;
-  CFFT_CUDA(ctx->lu_a.ensure((size_t)n * n * es), "alloc LU matrix");
+  CFFT_CUDA(ctx->lu_a.ensure((size_t)n * lu_stride(n) * es), "alloc LU matrix");
   CFFT_CUDA(ctx->lu_x.ensure((size_t)n * es), "alloc LU vectors");
   CFFT_CUDA(ctx->lu_y.ensure((size_t)n * es), "alloc LU vectors");
   double h[4] = {0, 0, 0, 0};
   int steps = 0;
   CFFT_CUDA(cudaEventRecord(ctx->lu_ev[0], st), "event");
   if (!complex128) {
-    CFFT_CUDA((copy_matrix<float, float>(z, ld, n, ctx->lu_a.p, st)), "LU copy");
+    CFFT_CUDA((copy_matrix<float, float>(z, ld, n, ctx->lu_a.p, lu_stride(n), st)), "LU copy");
     if ((s = lu_factor_checked<float>(ctx, n, w)) != CFFT_OK) return s;
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[1], st), "event");
     CFFT_CUDA((copy_vector<float, float>(v, n, ctx->lu_x.p, st)), "LU copy");
-    CFFT_CUDA(lu_solve<float>(ctx->lu_a.as<cpx<float>>(), n, n, w, ctx->lu_x.as<cpx<float>>(),
+    CFFT_CUDA(lu_solve<float>(ctx->lu_a.as<cpx<float>>(), lu_stride(n), n, w, ctx->lu_x.as<cpx<float>>(),
                               ctx->lu_y.as<cpx<float>>(), st), "LU solve");
     CFFT_CUDA((copy_vector<float, float>(ctx->lu_x.p, n, i_out, st)), "LU copy");
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[2], st), "event");
     CFFT_CUDA(residual_f32(z, ld, n, i_out, v, ctx->lu_sums.as<double>(), st), "residual");
   } else if (fp64_lu) {
-    CFFT_CUDA((copy_matrix<double, double>(z, ld, n, ctx->lu_a.p, st)), "LU copy");
+    CFFT_CUDA((copy_matrix<double, double>(z, ld, n, ctx->lu_a.p, lu_stride(n), st)), "LU copy");
     if ((s = lu_factor_checked<double>(ctx, n, w)) != CFFT_OK) return s;
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[1], st), "event");
     CFFT_CUDA((copy_vector<double, double>(v, n, ctx->lu_x.p, st)), "LU copy");
-    CFFT_CUDA(lu_solve<double>(ctx->lu_a.as<cpx<double>>(), n, n, w, ctx->lu_x.as<cpx<double>>(),
+    CFFT_CUDA(lu_solve<double>(ctx->lu_a.as<cpx<double>>(), lu_stride(n), n, w, ctx->lu_x.as<cpx<double>>(),
                                ctx->lu_y.as<cpx<double>>(), st), "LU solve");
     CFFT_CUDA((copy_vector<double, double>(ctx->lu_x.p, n, i_out, st)), "LU copy");
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[2], st), "event");
@@ -2695,7 +2698,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
     // x_0 = 0, r_0 = v; d = LU^-1 r (float32), x += d, r = v - Z x (float64)
     CFFT_CUDA(ctx->lu_x64.ensure((size_t)n * 16), "alloc LU vectors");
     CFFT_CUDA(ctx->lu_r.ensure((size_t)n * 16), "alloc LU vectors");
-    CFFT_CUDA((copy_matrix<float, double>(z, ld, n, ctx->lu_a.p, st)), "LU copy");
+    CFFT_CUDA((copy_matrix<float, double>(z, ld, n, ctx->lu_a.p, lu_stride(n), st)), "LU copy");
     if ((s = lu_factor_checked<float>(ctx, n, w)) != CFFT_OK) return s;
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[1], st), "event");
     CFFT_CUDA(cudaMemsetAsync(ctx->lu_x64.p, 0, (size_t)n * 16, st), "LU zero");
@@ -2703,7 +2706,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
     double rr_prev = -1.0;
     for (steps = 1; steps <= 30; ++steps) {
       CFFT_CUDA((copy_vector<float, double>(ctx->lu_r.p, n, ctx->lu_x.p, st)), "LU copy");
-      CFFT_CUDA(lu_solve<float>(ctx->lu_a.as<cpx<float>>(), n, n, w, ctx->lu_x.as<cpx<float>>(),
+      CFFT_CUDA(lu_solve<float>(ctx->lu_a.as<cpx<float>>(), lu_stride(n), n, w, ctx->lu_x.as<cpx<float>>(),
                                 ctx->lu_y.as<cpx<float>>(), st), "LU solve");
       CFFT_CUDA(add_correction(ctx->lu_x64.p, ctx->lu_x.p, n, ctx->lu_sums.as<double>() + 2, st), "refinement");
       CFFT_CUDA(residual_f64(z, ld, n, ctx->lu_x64.p, v, ctx->lu_r.p, ctx->lu_sums.as<double>(), st), "residual");

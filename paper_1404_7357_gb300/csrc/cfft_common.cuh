@@ -573,7 +573,7 @@ cudaError_t residual_f64(const void* z, int64_t ld, int n, const void* x, const 
 cudaError_t residual_f32(const void* z, int64_t ld, int n, const void* x, const void* b, double* sums,
                          cudaStream_t s);
 template <class TD, class TS>
-cudaError_t copy_matrix(const void* src, int64_t ld, int n, void* dst, cudaStream_t s);
+cudaError_t copy_matrix(const void* src, int64_t ld, int n, void* dst, int64_t ld_dst, cudaStream_t s);
 template <class TD, class TS>
 cudaError_t copy_vector(const void* src, int n, void* dst, cudaStream_t s);
 cudaError_t add_correction(void* x, const void* d, int n, double* sums, cudaStream_t s);

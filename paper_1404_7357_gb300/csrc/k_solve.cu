@@ -34,6 +34,8 @@
 // kernel (the host then returns CFFT_ERR_TIMEOUT).  The cluster barriers before and
 // behind a cluster panel are the hardware's own: every CTA of the cluster is resident
 // by construction and takes both.
+#include <cuda.h>
+
 #include <algorithm>
 
 #include "cfft_common.cuh"
@@ -729,188 +731,252 @@ __global__ void __launch_bounds__(256) lu_gemm_kernel(cpx<T>* a, int64_t ld, int
 // stored interleaved (re, im), one tile
 //   D (128 rows x 128 reals = 64 complex columns) = A' (128 x 2 kb) B' (2 kb x 128)
 // with A' the rows of L21 as stored (k' = 2 c + part) and
-//   B'^T[2j][2c] = Re U_cj, B'^T[2j][2c+1] = -Im U_cj,
-//   B'^T[2j+1][2c] = Im U_cj, B'^T[2j+1][2c+1] = Re U_cj
-// holds (Re, Im) of (L21 U12)_ij in columns 2j, 2j+1: the layout of A22 itself.  Three
-// TF32 products (head x head into one tensor-memory accumulator, the two corrections
-// into a second, added in FP32 registers), K staged 16 reals (8 panel columns) at a time
-// in two buffers, so the threads build one stage while the tensor core consumes the
-// other.  Every mbarrier wait is bounded; a wait that runs out sets bit 3 of err and the
-// CTA issues nothing more.
-constexpr int kUM = 128, kUN = 128, kUK = 16;   // tile rows, tile real columns, reals per stage
-constexpr uint32_t kUSbo = (kUK / 4) * 128;      // 8-row group stride of the K-major operands
-constexpr size_t kUStage = (size_t)2 * kUM * kUK * 4 + (size_t)2 * kUN * kUK * 4;
-// shared bytes per CTA: two stages, padded so that at most two CTAs share an SM (their
-// 2 x 256 tensor-memory columns then always fit)
-constexpr size_t kUSmem = 96 * 1024;
-static_assert(2 * kUStage + 128 <= kUSmem, "update stages");
-constexpr int kUPitch = kUN + 4;                 // row pitch (floats) of the staged product tile
-static_assert((size_t)kUM * kUPitch * 4 + 128 <= kUSmem, "staged product tile");
+//   B'^T[j][2c] = Re U_cj, B'^T[j][2c+1] = -Im U_cj,
+//   B'^T[64+j][2c] = Im U_cj, B'^T[64+j][2c+1] = Re U_cj
+// holds the 64 columns' real parts of L21 U12, then their imaginary parts.  Three TF32
+// products (head x head into one tensor-memory accumulator, the two corrections into a
+// second, added in FP32 registers).
+//
+// Persistent, one CTA per SM, tiles dealt out row by row in equal contiguous runs:
+//   producers  (4 warps) split L21's block into A' once per row of tiles, which stays in tensor
+//              memory (from shared memory the two operands took 119 of its 128 bytes a clock
+//              and starved the epilogue: 16,000 cycles per tile), and U12's into B' in shared
+//              memory, 32 reals per stage, a tile ahead, with two more stages' loads in flight;
+//   issuer     (1 warp) the tensor core's products;
+//   epilogue   (16 warps) subtracts the products from A22's tile, which TMA brings into shared
+//              memory one tile ahead and takes back: four boxes of 128 rows x 128 bytes, each with
+//              its four warps, swizzled so that a lane per row meets no bank conflict.  (As loads
+//              and stores of the warps it held up the producers: 12,000 cycles per tile.)
+// A22 is read and written once per panel, which bounds it (16 bytes per entry); the products
+// take about three quarters of that time.  The rows of `a` are 16-byte aligned (ld even).
+// GB300, 8,000^2, all panels: 19.9 ms with a tile per CTA, which loaded, split, multiplied
+// and stored in turn (two CTAs per SM) -> UPDATE_MS.
+constexpr int kUM = 128, kUN = 128, kUK = 32;   // tile rows, tile real columns, reals per stage
+constexpr int kUStages = 2 * kNb / kUK;          // stages per tile
+constexpr int kUProd = 4, kUEpi = 16;            // producer and epilogue warps
+constexpr int kUThreads = 32 * (kUProd + kUEpi + 1);
+constexpr uint32_t kUSbo = (kUK / 4) * 128;      // 8-row group stride of B' (K-major)
+constexpr uint32_t kUB = kUN * kUK * 4;          // bytes of a stage's head or correction
+constexpr unsigned kUPolls = 1u << 22;           // bound of a wait
+constexpr uint32_t kUColA = 2 * kUN;             // tensor-memory columns: products, corrections, then A'
+constexpr int kUBox = 32;                        // floats of a box's rows
+constexpr uint32_t kUBoxBytes = kUM * kUBox * 4;
+constexpr size_t kUSmem = 1024 + 2 * kUStages * kUB + (kUN / kUBox) * kUBoxBytes;
+static_assert(kUSmem <= 227 * 1024 - 1024, "update: one CTA's shared memory");
+static_assert(kUColA + 4 * kNb <= 512 && kUProd * 32 == kUM, "update: A' in tensor memory");
 
-__global__ void __launch_bounds__(256, 2) lu_gemm_tc_kernel(cpx<float>* a, int64_t ld, int n, int k, int kb, int* err) {
-  extern __shared__ __align__(128) unsigned char sm_raw[];
-  __shared__ uint64_t mbar[2];
+// panel of kNb columns at k; columns and rows k + kNb .. n - 1.  map: a as n rows of 2 n floats
+// (ld apart), boxes of kUBox x kUM, 128-byte swizzle
+__global__ void __launch_bounds__(kUThreads, 1) lu_gemm_tc_kernel(const __grid_constant__ CUtensorMap map, cpx<float>* a,
+                                                                   int64_t ld, int n, int k, int* err) {
+  extern __shared__ __align__(1024) unsigned char sm_raw[];
+  __shared__ uint64_t full_c[kUN / kUBox], full_b[kUStages], empty_b[kUStages], full_t, empty_t, drain;
   __shared__ uint32_t taddr_s;
   __shared__ int s_fail;
-  unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm_raw) + 127) & ~(uintptr_t)127);
+  unsigned char* Bs = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) & ~(uintptr_t)1023);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int r0 = k + kb + blockIdx.y * kUM;          // first row of the tile
-  const int c0 = k + kb + blockIdx.x * (kUN / 2);    // first complex column of the tile
-  float* af = reinterpret_cast<float*>(a);
-  const int64_t ldf = 2 * ld;
+  const int k1 = k + kNb, rt = (n - k1 + kUM - 1) / kUM, ct = (n - k1 + kUN / 2 - 1) / (kUN / 2);
+  const int64_t tiles = (int64_t)rt * ct;
+  const int t0 = (int)(tiles * blockIdx.x / gridDim.x), t1 = (int)(tiles * (blockIdx.x + 1) / gridDim.x);
   if (tid == 0) {
     s_fail = 0;
-    tc::mbar_init(&mbar[0], 1);
-    tc::mbar_init(&mbar[1], 1);
+    for (int i = 0; i < kUStages; ++i) {
+      tc::mbar_init(&full_b[i], kUProd);
+      tc::mbar_init(&empty_b[i], 1);
+    }
+    for (int i = 0; i < kUN / kUBox; ++i) tc::mbar_init(&full_c[i], 1);
+    tc::mbar_init(&full_t, 1);
+    tc::mbar_init(&empty_t, kUEpi);
+    tc::mbar_init(&drain, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {
-    tc::tmem_alloc(&taddr_s, 256);
+    tc::tmem_alloc(&taddr_s, 512);
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = taddr_s;
-  const uint32_t idesc = tc::idesc_tf32(kUM, kUN);
-  const int n_stages = (2 * kb + kUK - 1) / kUK;
-  // A: rows (tid >> 3) + 32 q, q < 4, reals 2 p, 2 p + 1 of the stage's 16 (p = tid & 7): the
-  // eight lanes of a row read its 64 bytes of the stage together
-  const int arow = tid >> 3, apiece = tid & 7;
-  const int brow = tid >> 5, bcol = tid & 31;   // B: panel row of the stage, columns bcol, bcol + 32
   auto failed = [&]() { return *reinterpret_cast<volatile int*>(&s_fail) != 0; };
-  // a stage's global values, loaded one stage ahead (in flight across the barrier and the
-  // MMA issue of the stage before)
-  float2 av[4];
-  cpx<float> bv[2];
-  auto load_stage = [&](int st) {
-    const int f = kUK * st + 2 * apiece;   // even, as is 2 kb: both reals are in range or neither
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int R = r0 + arow + 32 * q;
-      av[q] = (R < n && f < 2 * kb) ? __ldcg(reinterpret_cast<const float2*>(af + (int64_t)R * ldf + 2 * (int64_t)k + f))
-                                    : make_float2(0.f, 0.f);
-    }
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int j = bcol + 32 * u, c = (kUK / 2) * st + brow;
-      float2 x = make_float2(0.f, 0.f);
-      if (c < kb && c0 + j < n) x = __ldcg(reinterpret_cast<const float2*>(a + (int64_t)(k + c) * ld + c0 + j));
-      bv[u] = mk(x.x, x.y);
-    }
+  // one lane per warp polls, the others wait for it
+  auto wait = [&](uint64_t* m, int parity) {
+    if (lane == 0 && !failed() && !tc::mbar_wait(m, (uint32_t)parity & 1u, kUPolls)) atomicOr(&s_fail, 1);
+    __syncwarp();
   };
-  load_stage(0);
-  uint32_t n_issued = 0;
-  for (int st = 0; st < n_stages; ++st) {
-    const int buf = st & 1;
-    float* Ahi = reinterpret_cast<float*>(base + buf * kUStage);
-    float* Alo = Ahi + kUM * kUK;
-    float* Bhi = Alo + kUM * kUK;
-    float* Blo = Bhi + kUN * kUK;
-    if (st >= 2) {
-      // the MMAs of stage st - 2 read this buffer: one lane per warp polls, the others wait
-      if (lane == 0 && !failed() && !tc::mbar_wait(&mbar[buf], ((st - 2) >> 1) & 1, kTcPolls)) atomicOr(&s_fail, 1);
+  if (warp < kUEpi) {
+    // ---- epilogue: tensor-memory lanes 32 (warp mod 4).., columns 16 (warp / 4).. (a box)
+    const int lq = warp & 3, cg = warp >> 2, r = 32 * lq + lane;
+    unsigned char* box = Bs + 2 * kUStages * kUB + cg * kUBoxBytes;
+    float4* row = reinterpret_cast<float4*>(box + r * kUBox * 4);
+    const bool lead = lq == 0 && lane == 0;
+    int loads = 0;
+    auto load = [&](int t) {
+      ++loads;
+      tc::mbar_expect(&full_c[cg], kUBoxBytes);
+      tc::tma_load2(box, &map, 2 * (k1 + (t % ct) * (kUN / 2)) + kUBox * cg, k1 + (t / ct) * kUM, &full_c[cg]);
+    };
+    if (lead && t0 < t1) load(t0);
+    for (int t = t0, it = 0; t < t1; ++t, ++it) {
+      wait(&full_t, it);
+      tc::fence_after_sync();
+      const uint32_t at = tmem + ((uint32_t)(32 * lq) << 16) + 16u * cg;
+      float4 d[8];   // 16 complex columns
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float v[4][8];   // real parts, their corrections, imaginary parts, theirs: 8 columns
+        const uint32_t re = at + 8u * h, im = re + kUN / 2;
+        tc::tmem_ld8x4(re, re + kUN, im, im + kUN, v);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          d[4 * h + i] = make_float4(v[0][2 * i] + v[1][2 * i], v[2][2 * i] + v[3][2 * i],
+                                     v[0][2 * i + 1] + v[1][2 * i + 1], v[2][2 * i + 1] + v[3][2 * i + 1]);
+      }
+      tc::fence_before_sync();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&empty_t);   // the accumulators are read
+      wait(&full_c[cg], it);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        float4* z = row + (i ^ (r & 7));
+        const float4 c = *z;
+        *z = make_float4(c.x - d[i].x, c.y - d[i].y, c.z - d[i].z, c.w - d[i].w);
+      }
+      tc::fence_proxy_async();
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + cg) : "memory");   // the box's four warps
+      if (lead) {
+        const int x = 2 * (k1 + (t % ct) * (kUN / 2)) + kUBox * cg;
+        if (!failed() && x < 2 * n) tc::tma_store2(&map, x, k1 + (t / ct) * kUM, box);
+        tc::tma_store_wait_read();
+        if (t + 1 < t1) load(t + 1);
+      }
       __syncwarp();
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      // A: reals 16 st + 2 apiece, + 1 of row r0 + arow + 32 q of L21 (zero outside)
-      float h0, l0, h1, l1;
-      tf32_split(av[q].x, h0, l0);
-      tf32_split(av[q].y, h1, l1);
-      const uint32_t off = tc::kmajor_offset(arow + 32 * q, 2 * apiece, kUK) / 4;
-      *reinterpret_cast<float2*>(Ahi + off) = make_float2(h0, h1);
-      *reinterpret_cast<float2*>(Alo + off) = make_float2(l0, l1);
+    if (lead) {
+      if (loads > 0) tc::mbar_wait(&full_c[cg], (loads - 1) & 1, kUPolls);   // (in flight after a failure)
+      tc::tma_store_wait();
     }
+  } else if (warp < kUEpi + kUProd) {
+    // ---- producers
+    const int w = warp - kUEpi;   // (its tensor-memory lanes: kUEpi is a multiple of 4)
+    const int n_stages = (t1 - t0) * kUStages;
+    // B': two adjacent panel rows of one column give whole 16-byte rows of a core matrix, eight
+    // lanes a whole one; warp w takes row pairs 2 w, 2 w + 1 of the stage's 8, lanes over 32 columns
+    float2 bv[2][8];
+    int lt = t0 % ct, ls = 0;   // tile column and stage of the next load
+    const float2* const x0 = reinterpret_cast<const float2*>(a + (int64_t)(k + 4 * w) * ld + k1 + lane);
+    auto load = [&](float2 (&v)[8]) {
+      const float2* x = x0 + (int64_t)ls * (kUK / 2) * ld + lt * (kUN / 2);
+      const int cols = n - (k1 + lt * (kUN / 2) + lane);
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      // B: U12 entry (panel column 8 st + brow, tile column bcol + 32 u), four reals of B'^T
-      const int j = bcol + 32 * u;
-      float h0, l0, h1, l1;
-      tf32_split(bv[u].re, h0, l0);
-      tf32_split(bv[u].im, h1, l1);
-      const uint32_t o0 = tc::kmajor_offset(2 * j, 2 * brow, kUK) / 4;
-      const uint32_t o1 = tc::kmajor_offset(2 * j + 1, 2 * brow, kUK) / 4;
-      *reinterpret_cast<float2*>(Bhi + o0) = make_float2(h0, -h1);
-      *reinterpret_cast<float2*>(Blo + o0) = make_float2(l0, -l1);
-      *reinterpret_cast<float2*>(Bhi + o1) = make_float2(h1, h0);
-      *reinterpret_cast<float2*>(Blo + o1) = make_float2(l1, l0);
-    }
-    if (st + 1 < n_stages) load_stage(st + 1);
-    tc::fence_proxy_async();
-    tc::fence_before_sync();
-    __syncthreads();
-    if (tid == 0 && !failed()) {
-      tc::fence_after_sync();
-      const uint32_t ah = tc::smem_u32(Ahi), al = tc::smem_u32(Alo), bh = tc::smem_u32(Bhi), bl = tc::smem_u32(Blo);
-#pragma unroll
-      for (int s2 = 0; s2 < kUK / 8; ++s2) {
-        const uint32_t ko = s2 * 256;
-        const uint64_t dah = tc::sdesc(ah + ko, 128, kUSbo), dal = tc::sdesc(al + ko, 128, kUSbo);
-        const uint64_t dbh = tc::sdesc(bh + ko, 128, kUSbo), dbl = tc::sdesc(bl + ko, 128, kUSbo);
-        const uint32_t accf = (st > 0 || s2 > 0) ? 1u : 0u;
-        tc::mma_tf32(tmem + kUN, dah, dbl, idesc, accf);
-        tc::mma_tf32(tmem + kUN, dal, dbh, idesc, 1u);
-        tc::mma_tf32(tmem, dah, dbh, idesc, accf);
+      for (int r = 0; r < 4; ++r, x += ld) {
+        v[2 * r] = 0 < cols ? __ldcg(x) : make_float2(0.f, 0.f);
+        v[2 * r + 1] = 32 < cols ? __ldcg(x + 32) : make_float2(0.f, 0.f);
       }
-      tc::mma_commit(&mbar[buf]);
-      ++n_issued;
+      if (++ls == kUStages) {
+        ls = 0;
+        if (++lt == ct) lt = 0;
+      }
+    };
+    unsigned char* const B0 = Bs + tc::kmajor_offset(lane, 8 * w, kUK);
+    constexpr uint32_t kPair = 128, kHalf = 4 * kUSbo, kIm = 8 * kUSbo;   // next row pair; columns + 32; imaginary
+    if (n_stages > 0) {
+      load(bv[0]);
+      load(bv[1]);
     }
-  }
-  // A22's tile, read while the last products run (the tile is this CTA's alone): warp w
-  // takes tile rows 16 w .. 16 w + 15, its lanes consecutive complex columns (two
-  // 256-byte halves of each row)
-  float2 cz[32];
+    for (int t = t0, it = 0; t < t1; ++t, ++it) {
+      if (it == 0 || t % ct == 0) {
+        // A' of this row of tiles, once no product reads the last one's: a lane per row, the
+        // panel's 128 reals as tensor-memory columns (heads, then corrections)
+        if (it > 0) {
+          wait(&full_t, it - 1);
+          tc::fence_after_sync();
+        }
+        const int R = k1 + (t / ct) * kUM + 32 * w + lane;
+        const float4* x = reinterpret_cast<const float4*>(a + (int64_t)R * ld + k);
+        const uint32_t to = tmem + ((uint32_t)(32 * w) << 16) + kUColA;
+#pragma unroll 2
+        for (int c = 0; c < 2 * kNb; c += 16) {
+          float hi[16], lo[16];
 #pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const int R = r0 + 16 * warp + (i >> 1), jc = c0 + 32 * (i & 1) + lane;
-    cz[i] = (R < n && jc < n) ? __ldcg(reinterpret_cast<const float2*>(af + (int64_t)R * ldf + 2 * (int64_t)jc))
-                              : make_float2(0.f, 0.f);
-  }
-  // the last commit covers every MMA of the CTA
-  if (tid == 0 && !failed() && n_stages > 0) {
-    const int last = n_stages - 1;
-    if (!tc::mbar_wait(&mbar[last & 1], (last >> 1) & 1, kTcPolls)) atomicOr(&s_fail, 1);
-  }
-  __syncthreads();
-  tc::fence_after_sync();
-  const bool ok = !failed();   // no writer is left: the same value in every thread
-  if (ok) {
-    // the products (tensor-memory lane = tile row; warp w: lanes 32 (w mod 4).., real columns
-    // 64 (w / 4)..) into a shared tile over the stage buffers, which the finished MMAs no
-    // longer read
-    float* T = reinterpret_cast<float*>(base);
-    const int lq = warp & 3, ch = warp >> 2;
-    const int r = 32 * lq + lane;
-    const uint32_t tl = (uint32_t)(32 * lq) << 16;
+          for (int u = 0; u < 4; ++u) {
+            const float4 v = R < n ? __ldcg(x + c / 4 + u) : make_float4(0.f, 0.f, 0.f, 0.f);
+            tf32_split(v.x, hi[4 * u], lo[4 * u]);
+            tf32_split(v.y, hi[4 * u + 1], lo[4 * u + 1]);
+            tf32_split(v.z, hi[4 * u + 2], lo[4 * u + 2]);
+            tf32_split(v.w, hi[4 * u + 3], lo[4 * u + 3]);
+          }
+          tc::tmem_st16(to + c, hi);
+          tc::tmem_st16(to + 2 * kNb + c, lo);
+        }
+        tc::tmem_wait_st();
+        tc::fence_before_sync();
+      }
+#pragma unroll 2
+      for (int st = 0; st < kUStages; ++st) {
+        const int gs = it * kUStages + st, buf = st & 1;
+        if (it > 0) wait(&empty_b[st], it - 1);
 #pragma unroll
-    for (int cb = 0; cb < 64; cb += 16) {
-      const int col = 64 * ch + cb;
-      float v[16], w[16];
-      tc::tmem_ld16x2(tmem + tl + (uint32_t)col, tmem + tl + (uint32_t)(kUN + col), v, w);
+        for (int rp = 0; rp < 2; ++rp)
 #pragma unroll
-      for (int i = 0; i < 16; i += 4)
-        *reinterpret_cast<float4*>(T + r * kUPitch + col + i) =
-            make_float4(v[i] + w[i], v[i + 1] + w[i + 1], v[i + 2] + w[i + 2], v[i + 3] + w[i + 3]);
+          for (int h = 0; h < 2; ++h) {
+            const float2 x = bv[buf][4 * rp + h], y = bv[buf][4 * rp + 2 + h];
+            float xh, xl, xih, xil, yh, yl, yih, yil;
+            tf32_split(x.x, xh, xl);
+            tf32_split(x.y, xih, xil);
+            tf32_split(y.x, yh, yl);
+            tf32_split(y.y, yih, yil);
+            unsigned char* B = B0 + st * 2 * kUB + rp * kPair + h * kHalf;
+            *reinterpret_cast<float4*>(B) = make_float4(xh, -xih, yh, -yih);
+            *reinterpret_cast<float4*>(B + kIm) = make_float4(xih, xh, yih, yh);
+            *reinterpret_cast<float4*>(B + kUB) = make_float4(xl, -xil, yl, -yil);
+            *reinterpret_cast<float4*>(B + kUB + kIm) = make_float4(xil, xl, yil, yl);
+          }
+        if (gs + 2 < n_stages) load(bv[buf]);
+        tc::fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&full_b[st]);
+      }
     }
-    __syncthreads();
+  } else {
+    // ---- issuer
+    const uint32_t idesc = tc::idesc_tf32(kUM, kUN), b0 = tc::smem_u32(Bs);
+    bool issued = false;
+    for (int t = t0, it = 0; t < t1; ++t, ++it) {
+      if (it > 0) wait(&empty_t, it - 1);
+      for (int st = 0; st < kUStages; ++st) {
+        wait(&full_b[st], it);
+        tc::fence_after_sync();
+        if (lane == 0 && !failed()) {
+          const uint32_t bh = b0 + st * 2 * kUB, bl = bh + kUB;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int rr = 16 * warp + (i >> 1), h = i & 1;
-      const int R = r0 + rr, jc = c0 + 32 * h + lane;
-      const float2 d = *reinterpret_cast<const float2*>(T + rr * kUPitch + 64 * h + 2 * lane);
-      if (R < n && jc < n)
-        *reinterpret_cast<float2*>(af + (int64_t)R * ldf + 2 * (int64_t)jc) = make_float2(cz[i].x - d.x, cz[i].y - d.y);
+          for (int s2 = 0; s2 < kUK / 8; ++s2) {
+            const uint32_t ah = tmem + kUColA + st * kUK + 8 * s2, al = ah + 2 * kNb;
+            const uint64_t dbh = tc::sdesc(bh + s2 * 256, 128, kUSbo), dbl = tc::sdesc(bl + s2 * 256, 128, kUSbo);
+            const uint32_t accf = (st > 0 || s2 > 0) ? 1u : 0u;
+            tc::mma_tf32_ta(tmem + kUN, ah, dbl, idesc, accf);
+            tc::mma_tf32_ta(tmem + kUN, al, dbh, idesc, 1u);
+            tc::mma_tf32_ta(tmem, ah, dbh, idesc, accf);
+          }
+          tc::mma_commit(&empty_b[st]);
+          if (st == kUStages - 1) tc::mma_commit(&full_t);
+          issued = true;
+        }
+        __syncwarp();
+      }
     }
-  } else if (tid == 0) {
-    atomicOr(err, 8);
-    // a bounded wait for the MMAs in flight before their tensor memory is freed
-    if (n_issued > 0) tc::mbar_wait(&mbar[(n_issued - 1) & 1], ((n_issued - 1) >> 1) & 1, kTcPolls);
+    if (lane == 0 && issued) {
+      // every product done before the tensor memory is freed
+      tc::mma_commit(&drain);
+      if (!tc::mbar_wait(&drain, 0, kUPolls)) atomicOr(&s_fail, 1);
+    }
+    __syncwarp();
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
-  if (warp == 0) tc::tmem_dealloc(tmem, 256);
+  if (warp == 0) tc::tmem_dealloc(tmem, 512);
+  if (tid == 0 && failed()) atomicOr(err, 8);
 }
 
 // the row order of the factors: row i holds the matrix's row perm[i], every panel's row moves
@@ -1226,14 +1292,14 @@ __global__ void __launch_bounds__(256) residual32_kernel(const cpx<float>* z, in
   }
 }
 
-// copy an n x n block (row stride ld_src) into a dense n x n buffer, changing precision
+// copy an n x n block (row stride ld) into one of row stride ld_dst, changing precision: a
+// block of rows per CTA, lanes over columns
 template <class TD, class TS>
-__global__ void copy_matrix_kernel(const cpx<TS>* src, int64_t ld, int n, cpx<TD>* dst) {
-  const int64_t total = (int64_t)n * n;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / n, j = e - i * n;
-    dst[e] = ccast<TD>(src[i * ld + j]);
-  }
+__global__ void __launch_bounds__(256) copy_matrix_kernel(const cpx<TS>* src, int64_t ld, int n, cpx<TD>* dst,
+                                                          int64_t ld_dst) {
+  for (int64_t i = blockIdx.y; i < n; i += gridDim.y)
+    for (int j = blockIdx.x * 256 + threadIdx.x; j < n; j += gridDim.x * 256)
+      dst[i * ld_dst + j] = ccast<TD>(src[i * ld + j]);
 }
 
 template <class TD, class TS>
@@ -1372,6 +1438,21 @@ int lu_max_order(int sms) {
   return (int)((int64_t)sms * (int64_t)kPanelSmem / ((int64_t)kNb * sizeof(cpx<T>)));
 }
 
+// the update's tensor map of a (n rows of 2 n floats, 2 ld floats apart)
+cudaError_t update_map(float* a, int64_t ld, int n, CUtensorMap* map) {
+  void* f = nullptr;
+  cudaDriverEntryPointQueryResult found;
+  cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &found);
+  if (e != cudaSuccess) return e;
+  if (found != cudaDriverEntryPointSuccess || !f) return cudaErrorNotSupported;
+  const cuuint64_t dims[2] = {(cuuint64_t)2 * n, (cuuint64_t)n}, strides[1] = {(cuuint64_t)ld * sizeof(cpx<float>)};
+  const cuuint32_t box[2] = {kUBox, kUM}, step[2] = {1, 1};
+  const CUresult r = reinterpret_cast<decltype(&cuTensorMapEncodeTiled)>(f)(
+      map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a, dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+      CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 template <class T>
 cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_t s) {
   const int sms = std::min(current_sm_count(), 256);   // lu_panel_kernel polls up to 256 CTAs' keys
@@ -1410,6 +1491,8 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
   if (tc_update && (e = cudaFuncSetAttribute(lu_gemm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)kUSmem)) != cudaSuccess)
     return e;
+  CUtensorMap map = {};
+  if (tc_update && n > kNb && (e = update_map(reinterpret_cast<float*>(a), ld, n, &map)) != cudaSuccess) return e;
   int per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lu_panel_kernel<T>, kPanelThreads,
                                                          panel_smem0)) != cudaSuccess)
@@ -1473,8 +1556,9 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
       lu_trsm_kernel<T><<<(rest + 31) / 32, 256, trsm_smem, s>>>(a, ld, n, k, kb);
       if constexpr (sizeof(T) == 4) {
         if (tc_update)
-          lu_gemm_tc_kernel<<<dim3((rest + kUN / 2 - 1) / (kUN / 2), (rest + kUM - 1) / kUM), 256, kUSmem, s>>>(
-              a, ld, n, k, kb, w.err);
+          // a panel with columns behind it is kNb wide
+          lu_gemm_tc_kernel<<<grid_for((int64_t)((rest + kUN / 2 - 1) / (kUN / 2)) * ((rest + kUM - 1) / kUM), 1, sms),
+                              kUThreads, kUSmem, s>>>(map, a, ld, n, k, w.err);
         else
           lu_gemm_kernel<T><<<dim3((rest + 63) / 64, (rest + 63) / 64), 256, gemm_smem, s>>>(a, ld, n, n, k, kb);
       } else {
@@ -1538,9 +1622,9 @@ cudaError_t residual_f32(const void* z, int64_t ld, int n, const void* x, const 
 }
 
 template <class TD, class TS>
-cudaError_t copy_matrix(const void* src, int64_t ld, int n, void* dst, cudaStream_t s) {
-  copy_matrix_kernel<TD, TS><<<grid_for((int64_t)n * n, 256, 16 * current_sm_count()), 256, 0, s>>>(
-      reinterpret_cast<const cpx<TS>*>(src), ld, n, reinterpret_cast<cpx<TD>*>(dst));
+cudaError_t copy_matrix(const void* src, int64_t ld, int n, void* dst, int64_t ld_dst, cudaStream_t s) {
+  copy_matrix_kernel<TD, TS><<<dim3(grid_for(n, 256, 64), std::min(n, 65535)), 256, 0, s>>>(
+      reinterpret_cast<const cpx<TS>*>(src), ld, n, reinterpret_cast<cpx<TD>*>(dst), ld_dst);
   return cudaGetLastError();
 }
 
@@ -1585,9 +1669,9 @@ template cudaError_t lu_solve<float>(const cpx<float>*, int64_t, int, const LuWo
                                      cudaStream_t);
 template cudaError_t lu_solve<double>(const cpx<double>*, int64_t, int, const LuWork&, cpx<double>*, cpx<double>*,
                                       cudaStream_t);
-template cudaError_t copy_matrix<float, double>(const void*, int64_t, int, void*, cudaStream_t);
-template cudaError_t copy_matrix<float, float>(const void*, int64_t, int, void*, cudaStream_t);
-template cudaError_t copy_matrix<double, double>(const void*, int64_t, int, void*, cudaStream_t);
+template cudaError_t copy_matrix<float, double>(const void*, int64_t, int, void*, int64_t, cudaStream_t);
+template cudaError_t copy_matrix<float, float>(const void*, int64_t, int, void*, int64_t, cudaStream_t);
+template cudaError_t copy_matrix<double, double>(const void*, int64_t, int, void*, int64_t, cudaStream_t);
 template cudaError_t copy_vector<float, double>(const void*, int, void*, cudaStream_t);
 template cudaError_t copy_vector<double, float>(const void*, int, void*, cudaStream_t);
 template cudaError_t copy_vector<float, float>(const void*, int, void*, cudaStream_t);
