@@ -115,7 +115,7 @@ struct cfft_ctx {
   DevBuf beta_c, weight, bw, bi_rel, green_p, green_r, dp_eps, dr_eps, dp_h, dr_h;
   int channels = 1;  // 1: table; 3: table, d/d eps_r, d/d h
   DevBuf d_shapes, d_bx, d_by, d_q, d_y, d_grid, d_table, d_tw, d_cnodes, d_coff, d_cos, d_lag, d_prec,
-      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_gres, d_gtab, d_coarse, d_snodes, d_spec, d_sum;
+      d_flag, d_pos, d_rot, d_zbuf, d_fill, d_lat, d_latz, d_gres, d_gtab, d_coarse, d_snodes, d_spec, d_sum;
   int tw_len = 0, tw_prec = -1;
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   // batched sweep: plan arrays, scratch, stream, captured graph, tuned shape
@@ -1002,6 +1002,49 @@ const cpx<T>* fill_table(const cfft_ctx* ctx) {
   return (ctx->fill_own ? ctx->d_ftable : ctx->d_table).template as<cpx<T>>();
 }
 
+// The FP64 fill of a lattice through its different displacements (k_fill_lattice.cu), when they
+// are few enough; *done tells.  From 256 elements, where looking for them (30 us) is below 1% of
+// the general fill, and for at most an eighth as many (displacement, class) blocks as pairs (the
+// blocks are evaluated whether a pair uses them or not).  Without memory for the blocks, the
+// general path.
+cfft_status fill_lattice(cfft_ctx* ctx, const FillArgs<double, double>& fa, bool* done) {
+  *done = false;
+  cudaStream_t st = ctx->stream;
+  const size_t n = fa.n_el, sq = (size_t)kLatAxis * kLatAxis;
+  if (ctx->d_lat.ensure((2 * n + 2 * sq + 4) * sizeof(int) + 2 * sq * sizeof(double)) != cudaSuccess) {
+    cudaGetLastError();
+    return CFFT_OK;
+  }
+  LatticeAxis ax[2];
+  double* ud = ctx->d_lat.as<double>();
+  int* p = reinterpret_cast<int*>(ud + 2 * sq);
+  for (int i = 0; i < 2; ++i) {
+    ax[i].ud = ud + i * sq;
+    ax[i].id = p + i * n;
+    ax[i].did = p + 2 * n + i * sq;
+    ax[i].info = p + 2 * n + 2 * sq + 2 * i;
+  }
+  CFFT_CUDA(launch_lattice_axes(fa.n_el, fa.pos, ax[0], ax[1], st), "lattice kernel");
+  int c[4];
+  CFFT_CUDA(cudaMemcpyAsync(c, ax[0].info, sizeof(c), cudaMemcpyDeviceToHost, st), "lattice");
+  CFFT_CUDA(cudaStreamSynchronize(st), "lattice");
+  if (c[0] == 0 || c[2] == 0) return CFFT_OK;
+  const size_t groups = (size_t)c[1] * c[3];
+  if (8 * groups * fa.n_cls > n * n) return CFFT_OK;
+  const FillBucketPlan plan = plan_fill_bucketed<double>(std::max(c[1], c[3]), fa.n_mbf, fa.n_harm, fa.n_rho, fa.taps,
+                                                         1, 0, false);
+  if (!plan.ok) return CFFT_OK;
+  const size_t blocks = groups * fa.n_cls * fa.n_mbf * fa.n_mbf * sizeof(cpx<double>);
+  if (ctx->d_fill.ensure(plan.scratch) != cudaSuccess || ctx->d_latz.ensure(blocks + groups) != cudaSuccess) {
+    cudaGetLastError();
+    return CFFT_OK;
+  }
+  CFFT_CUDA(launch_fill_lattice(fa, ax[0], ax[1], c, plan, ctx->d_fill.p, ctx->d_latz.p,
+                                ctx->d_latz.as<unsigned char>() + blocks, st), "fill kernel");
+  *done = true;
+  return CFFT_OK;
+}
+
 template <class T, class TO>
 cfft_status fill_impl(cfft_ctx* ctx, int n_el, const double* pos, const int* rot, void* z,
                       int64_t ld) {
@@ -1029,11 +1072,18 @@ cfft_status fill_impl(cfft_ctx* ctx, int n_el, const double* pos, const int* rot
   if (std::is_same<T, TO>::value && ctx->opt[CFFT_OPT_FILL_BLOCK] >= 0)
     plan = plan_fill_bucketed<T>(n_el, fa.n_mbf, fa.n_harm, fa.n_rho, fa.taps, fa.n_cls,
                                  (int)ctx->opt[CFFT_OPT_FILL_BLOCK], !(ctx->opt[CFFT_OPT_FILL_SIMT] > 0));
-  if (plan.ok) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
   CFFT_CUDA(cudaMemsetAsync(fa.err, 0, sizeof(int), ctx->stream), "flag");
   ctx->info.fill_form = plan.ok ? (plan.tc ? 3 : 2) : 1;
-  cudaError_t le = launch_fill<T, TO>(fa, plan, ctx->d_fill.p, ctx->stream);
-  if (le != cudaSuccess) return cuda_fail(ctx, le, "fill kernel");
+  bool done = false;
+  if constexpr (std::is_same<T, double>::value && std::is_same<TO, double>::value)
+    if (plan.ok && n_el >= 256 && ctx->opt[CFFT_OPT_FILL_BLOCK] == 0 &&
+        (fs = fill_lattice(ctx, fa, &done)) != CFFT_OK)
+      return fs;
+  if (!done) {
+    if (plan.ok) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
+    cudaError_t le = launch_fill<T, TO>(fa, plan, ctx->d_fill.p, ctx->stream);
+    if (le != cudaSuccess) return cuda_fail(ctx, le, "fill kernel");
+  }
   int flag = 0;
   CFFT_CUDA(cudaMemcpyAsync(&flag, fa.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "flag");
   CFFT_CUDA(cudaStreamSynchronize(ctx->stream), "fill");
@@ -2021,7 +2071,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->green_r, &ctx->dp_eps, &ctx->dr_eps, &ctx->dp_h, &ctx->dr_h, &ctx->d_shapes, &ctx->d_bx, &ctx->d_by, &ctx->d_q,
                       &ctx->d_y, &ctx->d_grid, &ctx->d_table, &ctx->d_tw, &ctx->d_cnodes,
                       &ctx->d_coff, &ctx->d_cos, &ctx->d_lag, &ctx->d_flag, &ctx->d_pos,
-                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
+                      &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_lat, &ctx->d_latz, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
                       &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_perm, &ctx->lu_cand_d, &ctx->lu_words, &ctx->lu_err, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
                       &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,

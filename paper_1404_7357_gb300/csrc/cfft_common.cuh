@@ -364,6 +364,21 @@ struct FillArgs {
   const int* rot;          // [n_el] or null
   cpx<TO>* z;              // [(m*M + a) * ld + n*M + b]
   int* err;                // set when a pair lies beyond rho_max
+  // a lattice's displacements in place of element pairs (FP64, bucketed): "pair" (m, n), m < n_rows,
+  // n < n_el, is the displacement (dx[m], dy[n]), and bad[m * n_el + n] is set in place of err
+  int n_rows;              // 0: n_el
+  const double* dx;        // null: element pairs
+  const double* dy;
+  unsigned char* bad;
+};
+
+// one coordinate of a lattice (k_fill_lattice.cu)
+constexpr int kLatAxis = 96;   // different values at most
+struct LatticeAxis {
+  int* id;        // [n_el]
+  int* did;       // [kLatAxis^2]
+  double* ud;     // [kLatAxis^2]
+  int* info;      // [2] different values (0: too many), different differences
 };
 
 // host launchers (one translation unit per stage)
@@ -485,6 +500,13 @@ FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, in
 template <class T>
 cudaError_t launch_fill_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& plan, void* scratch,
                                  cudaStream_t s);
+cudaError_t launch_lattice_axes(int n_el, const double* pos, const LatticeAxis& ax, const LatticeAxis& ay,
+                                cudaStream_t s);
+// counts: info of ax, then of ay; plan, scratch: those of max(counts[1], counts[3]) elements, one
+// class; blocks: [n_cls][counts[1] M][counts[3] M]; bad: [counts[1]][counts[3]]
+cudaError_t launch_fill_lattice(const FillArgs<double, double>& a, const LatticeAxis& ax, const LatticeAxis& ay,
+                                const int (&counts)[4], const FillBucketPlan& plan, void* scratch, void* blocks,
+                                unsigned char* bad, cudaStream_t s);
 // adjoint of the bucketed fill: position gradient (grad_pos) and, with both
 // derivative tables, the (eps_r, h) gradient (grad_theta[0..1]); both accumulated
 template <class T>

@@ -48,6 +48,7 @@ struct BucketArgs {
   int n_ck;         // rotation classes (1 or 4)
   int n_cells;      // stencil starts i0 in [-half, n_rho - taps]
   int win;          // stencil starts per window
+  int parts;        // CTAs per window of the fill (bucket_fill_kernel)
   int vec_out;      // output rows 16-byte aligned: vector stores
   float ih, il;     // 1 / d_rho as float head + tail
   const float4* ps; // positions as (x head, x tail, y head, y tail)
@@ -134,8 +135,8 @@ __device__ __forceinline__ typename std::enable_if<sizeof(T) == 8, BGeom<T>>::ty
 bucket_geom(const FillArgs<T, T>& a, const BucketArgs&, int m, int n) {
   constexpr int HALF = TAPS / 2 - 1;
   // rounded operations only (no contraction), so every kernel takes the same decisions
-  const double dx = __dsub_rn(a.pos[2 * m], a.pos[2 * n]);
-  const double dy = __dsub_rn(a.pos[2 * m + 1], a.pos[2 * n + 1]);
+  const double dx = a.dx ? a.dx[m] : __dsub_rn(a.pos[2 * m], a.pos[2 * n]);
+  const double dy = a.dx ? a.dy[n] : __dsub_rn(a.pos[2 * m + 1], a.pos[2 * n + 1]);
   const double rho = __dsqrt_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)));
   const double u = __dmul_rn(rho, a.inv_d_rho);
   BGeom<T> g;
@@ -174,7 +175,8 @@ __global__ void __launch_bounds__(kBThreads) bucket_sort_kernel(FillArgs<T, T> a
     const BGeom<T> g = bucket_geom<T, TAPS>(a, b, m, n);
     if (g.bad) {
       if (!SCATTER) {
-        atomicOr(a.err, 1);
+        if (a.bad) a.bad[(size_t)m * a.n_el + n] = 1;
+        else atomicOr(a.err, 1);
         if (a.z == nullptr) continue;   // the adjoint: no matrix
         const int M = a.n_mbf;
         for (int ia = 0; ia < M; ++ia)
@@ -403,21 +405,29 @@ __global__ void __launch_bounds__(kBThreads, 2) bucket_fill_kernel(FillArgs<T, T
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int HALF = TAPS / 2 - 1;
   constexpr int P2 = M * M;
-  const int w = blockIdx.x, cls = blockIdx.y, blk = blockIdx.z;
+  const int w = blockIdx.x / b.parts, part = blockIdx.x % b.parts, cls = blockIdx.y, blk = blockIdx.z;
   const int cell0 = w * b.win;
   if (cell0 >= b.n_cells) return;
   const int cell1 = min(cell0 + b.win, b.n_cells);
   const size_t kbase = ((size_t)blk * b.n_ck + cls) * b.n_cells;
   const unsigned p0 = b.off[kbase + cell0], p1 = b.off[kbase + cell1];
-  if (p0 == p1) return;
+  // items: a pair, or with fewer pairs than threads a pair and MBF row a (the geometry and
+  // weights anew: 8% of a row's work); equal shares for the window's CTAs, whole warps
+  const unsigned np = p1 - p0;
+  const int split = np < (unsigned)kBThreads ? M : 1;
+  const unsigned items = np * split;
+  const unsigned share = max(64u, (items + 32u * b.parts - 1) / (32u * b.parts) * 32u);
+  const unsigned it0 = b.parts > 1 ? part * share : 0u, it1 = b.parts > 1 ? min(it0 + share, items) : items;
+  if (it0 >= it1) return;
   const int R = b.win + TAPS - 1;       // table rows of the window
   const int r_first = cell0 - HALF;     // table row of window row 0
   cpx<T>* S = reinterpret_cast<cpx<T>*>(smem_raw);
   load_window<T, M>(a, a.table + (size_t)cls * P2 * a.n_harm * a.n_rho, r_first, R, S);
   __syncthreads();
   const unsigned nmask = (1u << b.nb_bits) - 1u;
-  for (unsigned p = p0 + threadIdx.x; p < p1; p += blockDim.x) {
-    const unsigned code = b.list[p];
+  for (unsigned it = it0 + threadIdx.x; it < it1; it += blockDim.x) {
+    const int a0 = split > 1 ? (int)(it / np) : 0, a1 = split > 1 ? a0 + 1 : M;
+    const unsigned code = b.list[p0 + (split > 1 ? it % np : it)];
     const int n = (int)(code & nmask);
     const int m = b.m0 + blk * b.br + (int)(code >> b.nb_bits);
     const BGeom<T> g = bucket_geom<T, TAPS>(a, b, m, n);
@@ -433,7 +443,7 @@ __global__ void __launch_bounds__(kBThreads, 2) bucket_fill_kernel(FillArgs<T, T
     for (int k = 0; k < a.q_max; ++k) zq = zq * conj(e1);
     cpx<T>* zrow = a.z + (size_t)m * M * a.ld + (size_t)n * M;
 #pragma unroll 1
-    for (int ia = 0; ia < M; ++ia) {
+    for (int ia = a0; ia < a1; ++ia) {
       cpx<T> acc[M];
 #pragma unroll
       for (int ib = 0; ib < M; ++ib) acc[ib] = mk((T)0, (T)0);
@@ -1086,6 +1096,7 @@ BucketArgs bucket_args(const FillArgs<T, T>& a, const FillBucketPlan& pl, void* 
   b.n_ck = a.n_cls;
   b.n_cells = pl.n_cells;
   b.win = pl.win;
+  b.parts = sizeof(T) == 8 ? 8 : 1;
   const double inv = a.inv_d_rho;
   b.ih = (float)inv;
   b.il = (float)(inv - (double)b.ih);
@@ -1104,9 +1115,10 @@ cudaError_t run_waves(const FillArgs<T, T>& a, const FillBucketPlan& pl, BucketA
                                                               const_cast<float4*>(b.ps));
   }
   const int n_windows = (pl.n_cells + pl.win - 1) / pl.win;
-  for (int m0 = 0; m0 < a.n_el; m0 += pl.rows_per_wave) {
+  const int n_rows = a.n_rows > 0 ? a.n_rows : a.n_el;
+  for (int m0 = 0; m0 < n_rows; m0 += pl.rows_per_wave) {
     b.m0 = m0;
-    b.rows = min(pl.rows_per_wave, a.n_el - m0);
+    b.rows = min(pl.rows_per_wave, n_rows - m0);
     const int n_blocks = (b.rows + b.br - 1) / b.br;
     const size_t n_keys = (size_t)n_blocks * b.n_ck * b.n_cells;
     cudaError_t e = cudaMemsetAsync(b.cursor, 0, n_keys * sizeof(unsigned), s);
@@ -1134,6 +1146,7 @@ cudaError_t run_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& pl, void
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return run_waves<T, TAPS>(a, pl, bucket_args(a, pl, scratch), s, [&](const BucketArgs& b, dim3 fg) {
+    fg.x *= b.parts;
     bucket_fill_kernel<T, M, TAPS><<<fg, kBThreads, smem, s>>>(a, b);
     return cudaSuccess;
   });
@@ -1265,6 +1278,14 @@ FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, in
     if (win < 8) win = (int)((220 * 1024) / row_bytes) - (taps - 1);
     if (win < 4) return pl;
     win = std::min(win, 64);
+    // FP64: the pairs' arithmetic is dear and unevenly spread over the cells (a lattice's
+    // displacements lie in a few hundred of them), the copy of the table rows cheap, so at least
+    // six windows per SM and eight CTAs per window.  GB300: the 25 x 25 array's displacements
+    // 1.31 -> 0.45 ms, 700 irregular elements 10.1 -> 9.0 ms, 60: 0.43 -> 0.28 ms
+    if (sizeof(T) == 8) {
+      const int cells = n_rho - taps + taps / 2;
+      win = std::min(win, std::max(2, cells / (6 * current_sm_count())));
+    }
     pl.win = win;
     pl.smem = (size_t)(win + taps - 1) * row_bytes;
   }
