@@ -91,7 +91,9 @@ typedef enum {
  *                the same quadrature; the matrix form needs at most 64 series
  *                per harmonic and 8, 12 or 16 taps)
  *   FILL_BLOCK   test elements per row block of the bucketed fill and of
- *                its adjoint (default 1024); a value < 0 selects the per-row
+ *                its adjoint (default 0: automatic, and the fill of few
+ *                element pairs or of a lattice may take another form); a
+ *                value < 0 selects the per-row
  *                kernels, which also serve the cases the bucketed forms do
  *                not cover (M other than 1, 2, 4; fill taps other than 8, 12,
  *                16; an output or gradient precision different from the
@@ -469,8 +471,9 @@ cfft_status cfft_fill_backward_residual(cfft_ctx* ctx, int n_elements, const dou
  * multiply-adds of the interpolation-matrix products (rows x grid columns x
  * series, every harmonic) and work_bp_stencils the node stencils added into
  * the matrices (rows x angular nodes x matrices).  fill_form: the form of the
- * last cfft_fill_reduced_matrix: 1 per-row, 2 bucketed on the FP32 pipe, 3 on
- * the tensor cores (0: no fill yet).  fill_err_est: the estimated
+ * last cfft_fill_reduced_matrix: 1 per-row, 2 bucketed on the FP32 or FP64
+ * pipe, 3 on the tensor cores, 4 direct (few pairs: up to 6144 in FP32, 2048
+ * in FP64; 0: no fill yet).  fill_err_est: the estimated
  * interpolation error of the fill on the tabulated grid, relative to the
  * table maximum (-1: not estimated); fill_refine: the factor r of the grid
  * the fill interpolates (0: no fill since the last tabulation); fill_n_rho:

@@ -64,6 +64,20 @@ class FillProblem:
             if pin:
                 self.ctx.set_option(cfft.OPT_CONTOUR_SERIES, own)
 
+    def fill(self, pos, z):
+        # For the same reason the float32 matrix keeps the sorted fill's order of sums where few
+        # elements would take the direct one: a row block of the whole array, which is the sorted
+        # fill's own choice there, selects it.  A row block set by the caller stays as it is.
+        own = self.ctx._options.get(cfft.OPT_FILL_BLOCK, 0.0)
+        pin = self.precision == cfft.CFFT_FP32_MIXED and own == 0 and pos.shape[0] <= 1024
+        if pin:
+            self.ctx.set_option(cfft.OPT_FILL_BLOCK, pos.shape[0])
+        try:
+            self.ctx.fill_reduced_matrix(pos, self.rot, z)
+        finally:
+            if pin:
+                self.ctx.set_option(cfft.OPT_FILL_BLOCK, own)
+
     @property
     def dtype(self):
         return torch.complex128 if self.precision == cfft.CFFT_FP64 else torch.complex64
@@ -77,7 +91,7 @@ class ReducedMatrix(torch.autograd.Function):
         a = pos.shape[0]
         m = problem.element.n_mbf
         z = torch.empty((a * m, a * m), dtype=problem.dtype, device=pos.device)
-        problem.ctx.fill_reduced_matrix(pos.detach().contiguous(), problem.rot, z)
+        problem.fill(pos.detach().contiguous(), z)
         fctx.save_for_backward(pos.detach(), eps_h.detach())
         fctx.problem = problem
         return z

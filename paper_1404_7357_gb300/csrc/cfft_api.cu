@@ -1072,15 +1072,17 @@ cfft_status fill_impl(cfft_ctx* ctx, int n_el, const double* pos, const int* rot
   if (std::is_same<T, TO>::value && ctx->opt[CFFT_OPT_FILL_BLOCK] >= 0)
     plan = plan_fill_bucketed<T>(n_el, fa.n_mbf, fa.n_harm, fa.n_rho, fa.taps, fa.n_cls,
                                  (int)ctx->opt[CFFT_OPT_FILL_BLOCK], !(ctx->opt[CFFT_OPT_FILL_SIMT] > 0));
+  plan.direct = plan.ok && ctx->opt[CFFT_OPT_FILL_BLOCK] == 0 && 
+                (int64_t)n_el * n_el <= direct_pairs(sizeof(T) == 8);
   CFFT_CUDA(cudaMemsetAsync(fa.err, 0, sizeof(int), ctx->stream), "flag");
-  ctx->info.fill_form = plan.ok ? (plan.tc ? 3 : 2) : 1;
+  ctx->info.fill_form = plan.direct ? 4 : plan.ok ? (plan.tc ? 3 : 2) : 1;
   bool done = false;
   if constexpr (std::is_same<T, double>::value && std::is_same<TO, double>::value)
     if (plan.ok && n_el >= 256 && ctx->opt[CFFT_OPT_FILL_BLOCK] == 0 &&
         (fs = fill_lattice(ctx, fa, &done)) != CFFT_OK)
       return fs;
   if (!done) {
-    if (plan.ok) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
+    if (plan.ok && !plan.direct) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
     cudaError_t le = launch_fill<T, TO>(fa, plan, ctx->d_fill.p, ctx->stream);
     if (le != cudaSuccess) return cuda_fail(ctx, le, "fill kernel");
   }

@@ -493,7 +493,10 @@ struct FillBucketPlan {
   bool tc;                 // the tensor-core form (FP32, M = 4, 8 taps)
   int win, n_cells, nb_bits, block_rows, rows_per_wave;
   size_t n_keys_max, smem, scratch;
+  bool direct;             // few pairs: no sort, a block per pair (fill only)
 };
+// pairs up to which fill_direct_kernel is the faster fill
+constexpr int64_t direct_pairs(bool fp64) { return fp64 ? 2048 : 6144; }
 template <class T>
 FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, int taps, int n_cls,
                                   int block_rows, bool tc);

@@ -156,12 +156,15 @@ __device__ __forceinline__ int bucket_class(const int* rot, int n_ck, int m, int
   return (n_ck == 1 || rot == nullptr) ? 0 : 2 * (rot[m] != 0) + (rot[n] != 0);
 }
 
-__global__ void split_positions_kernel(const double* pos, int n_el, float4* ps) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_el) return;
+__device__ __forceinline__ float4 split_position(const double* pos, int i) {
   const double x = pos[2 * i], y = pos[2 * i + 1];
   const float xh = (float)x, yh = (float)y;
-  ps[i] = make_float4(xh, (float)(x - (double)xh), yh, (float)(y - (double)yh));
+  return make_float4(xh, (float)(x - (double)xh), yh, (float)(y - (double)yh));
+}
+
+__global__ void split_positions_kernel(const double* pos, int n_el, float4* ps) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n_el) ps[i] = split_position(pos, i);
 }
 
 // pass 1 (count) and pass 2 (scatter) of the counting sort of this wave's pairs
@@ -473,6 +476,94 @@ __global__ void __launch_bounds__(kBThreads, 2) bucket_fill_kernel(FillArgs<T, T
       }
       store_row<T, M>(zrow + (size_t)ia * a.ld, acc, b.vec_out != 0);
     }
+  }
+}
+
+// e^{i q phi} from e^{i phi} by squarings (|q| < 2^31)
+template <class T>
+__device__ __forceinline__ cpx<T> phase_power(cpx<T> e, int q) {
+  cpx<T> p = mk((T)1, (T)0);
+  for (int k = q < 0 ? -q : q; k > 0; k >>= 1) {
+    if (k & 1) p = p * e;
+    e = e * e;
+  }
+  return q < 0 ? conj(p) : p;
+}
+
+// The fill of few pairs: a block per pair, straight from the table.  One warp forms the
+// stencil and its weights; lanes take harmonics (their taps are adjacent in the table), the
+// warps MBF pairs, and a warp sum ends each.  The sort, its scans and the buckets' table slices
+// are 9 launches and a serial chain of 60 us and more for any number of pairs; here a pair costs
+// its 17 KB of table rows (M = 4, 17 harmonics, 8 taps), and in FP64 its weights on the FP64 pipe.
+// GB300, M = 4, sorted -> direct per call, elements: FP32 24: 78 -> 39 us, 64: 102 -> 66,
+// 100: 106 -> 113; FP64 8: 170 -> 53 us, 48: 296 -> 271, 64: 375 -> 409: the lines between
+// (direct_pairs).
+template <class T, int M, int TAPS>
+__global__ void __launch_bounds__(128) fill_direct_kernel(FillArgs<T, T> a, BucketArgs b) {
+  constexpr int P2 = M * M, W = 4, AB = P2 < W ? 1 : P2 / W;   // MBF pairs per warp
+  __shared__ T wt_s[TAPS];
+  __shared__ cpx<T> e_s;
+  __shared__ int i0_s, bad_s;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int m = blockIdx.x / a.n_el, n = blockIdx.x - m * a.n_el;
+  cpx<T>* zb = a.z + (size_t)m * M * a.ld + (size_t)n * M;
+  if (warp == 0) {
+    BGeom<T> g;
+    if constexpr (sizeof(T) == 4) g = bucket_geom_ps<TAPS>(a, b, split_position(a.pos, m), split_position(a.pos, n));
+    else g = bucket_geom<T, TAPS>(a, b, m, n);
+    T wt[TAPS];
+    stencil_weights<T, TAPS, false>(g.x, wt, nullptr);
+    if (lane == 0) {
+#pragma unroll
+      for (int t = 0; t < TAPS; ++t) wt_s[t] = wt[t];
+      e_s = mk(g.ex, g.ey);
+      i0_s = g.i0;
+      bad_s = g.bad;
+      if (g.bad) atomicOr(a.err, 1);
+    }
+  }
+  __syncthreads();
+  if (bad_s) {
+    for (int e = threadIdx.x; e < P2; e += blockDim.x) zb[(size_t)(e / M) * a.ld + e % M] = mk((T)0, (T)0);
+    return;
+  }
+  if (warp * AB >= P2) return;
+  const int i0 = i0_s;
+  const cpx<T>* tab = a.table + ((size_t)bucket_class(a.rot, b.n_ck, m, n) * P2 + warp * AB) * a.n_harm * a.n_rho;
+  cpx<T> acc[AB];
+#pragma unroll
+  for (int u = 0; u < AB; ++u) acc[u] = mk((T)0, (T)0);
+  for (int qi = lane; qi < a.n_harm; qi += 32) {
+    const bool odd = (qi - a.q_max) & 1;
+    const cpx<T> ph = phase_power(e_s, qi - a.q_max);
+#pragma unroll
+    for (int u = 0; u < AB; ++u) {
+      const cpx<T>* row = tab + ((size_t)u * a.n_harm + qi) * a.n_rho;
+      cpx<T> x[TAPS];
+#pragma unroll
+      for (int t = 0; t < TAPS; ++t) {   // rows below 0 by parity; a stencil never passes the end
+        const int r = i0 + t;
+        x[t] = row[r < 0 ? -r : r];
+        if (r < 0 && odd) x[t] = mk(-x[t].re, -x[t].im);
+      }
+      cpx<T> v = mk((T)0, (T)0);
+#pragma unroll
+      for (int t = 0; t < TAPS; ++t) {
+        v.re = fma(wt_s[t], x[t].re, v.re);
+        v.im = fma(wt_s[t], x[t].im, v.im);
+      }
+      cmac(acc[u], ph, v);
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < AB; ++u) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      acc[u].re += __shfl_xor_sync(0xffffffffu, acc[u].re, off);
+      acc[u].im += __shfl_xor_sync(0xffffffffu, acc[u].im, off);
+    }
+    const int ab = warp * AB + u;
+    if (lane == u) zb[(size_t)(ab / M) * a.ld + ab % M] = acc[u];
   }
 }
 
@@ -1141,6 +1232,10 @@ cudaError_t run_waves(const FillArgs<T, T>& a, const FillBucketPlan& pl, BucketA
 
 template <class T, int M, int TAPS>
 cudaError_t run_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& pl, void* scratch, cudaStream_t s) {
+  if (pl.direct) {
+    fill_direct_kernel<T, M, TAPS><<<a.n_el * a.n_el, 128, 0, s>>>(a, bucket_args(a, pl, scratch));
+    return cudaGetLastError();
+  }
   const size_t smem = pl.smem;
   cudaError_t e = cudaFuncSetAttribute(bucket_fill_kernel<T, M, TAPS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1318,7 +1413,7 @@ cudaError_t launch_fill_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& 
                                  cudaStream_t s) {
   if (!pl.ok) return cudaErrorInvalidValue;
   if constexpr (sizeof(T) == 4) {
-    if (pl.tc) return run_fill_tc(a, pl, scratch, s);
+    if (pl.tc && !pl.direct) return run_fill_tc(a, pl, scratch, s);
   }
   switch (a.n_mbf) {
     case 1: return run_taps<T, 1>(a, pl, scratch, s);
