@@ -694,8 +694,12 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   sums = sums && (tform || wform) &&
          sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q,
                   ctx->sm_count, &sp);
-  const int n_low = sums ? std::min(n_chunks, (sum_first_row(d_rho / ds, ctx->q_max, fp64) + rchunk - 1) / rchunk)
-                         : n_chunks;
+  const int low_rows = sums ? std::min(n_rho, sum_first_row(d_rho / ds, ctx->q_max, fp64)) : n_rho;
+  const int rchunk = pform ? backproject_pm_rows()
+                     : !wform ? 32
+                     : sums ? backproject_w_low_rows(low_rows, 2 * ctx->q_max + 1) : backproject_w_rows();
+  const int n_chunks = (n_rho + rchunk - 1) / rchunk;
+  const int n_low = std::min(n_chunks, (low_rows + rchunk - 1) / rchunk);
   int low_nodes = 0;
   std::vector<int> cn(n_chunks);
   std::vector<int64_t> coff(n_chunks);
@@ -755,7 +759,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   while (group > 1 && backproject_smem<T>(group, max_seg, max_nodes) > smem_cap) --group;
   if (!wform && backproject_smem<T>(group, max_seg, max_nodes) > smem_cap)
     return fail(ctx, CFFT_ERR_ARG, "rho_max too large for one shared-memory segment");
-  if (wform && backproject_w_smem<T>(max_nodes, series_per_q) > smem_cap)
+  if (wform && backproject_w_smem<T>(rchunk, max_nodes, series_per_q) > smem_cap)
     return fail(ctx, CFFT_ERR_ARG, "rho_max too large for the angular node table");
   if (pform && (tform ? backproject_tc_smem(max_nodes) : backproject_pm_smem(max_nodes)) > smem_cap)
     return fail(ctx, CFFT_ERR_ARG, "rho_max too large for the angular node table");
@@ -1509,7 +1513,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     CFFT_CUDA(ctx->b_cos.ensure(cos_total * sizeof(double)), "alloc plan");
     CFFT_CUDA(ctx->d_tw.ensure((size_t)L * sizeof(cpx<T>)), "alloc twiddles");
     if (pform_b ? (tform_b ? backproject_tc_smem(max_nodes) : backproject_pm_smem(max_nodes)) > 225 * 1024
-                : (backproject_w_smem<T>(max_nodes, pairs) > 225 * 1024 || pairs > 64))
+                : (backproject_w_smem<T>(backproject_w_rows(), max_nodes, pairs) > 225 * 1024 || pairs > 64))
       return fail(ctx, CFFT_ERR_ARG, "batch: rho_max too large for the angular node table");
     const int group = std::min(8, pairs);
     double work_bp = 0, work_fft = 0;

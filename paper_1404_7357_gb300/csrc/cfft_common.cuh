@@ -452,7 +452,7 @@ cudaError_t launch_backproject_batch(const BackprojArgs<T>* items, const int4* t
 cudaError_t launch_chunk_cosines(const int* n_nodes, const int64_t* offset, int n_chunks,
                                  int max_nodes, double* cosv, cudaStream_t s);
 template <class T>
-size_t backproject_w_smem(int max_nodes, int series);
+size_t backproject_w_smem(int rows, int max_nodes, int series);
 // paired-harmonic matrix form (FP32-mixed, taps 8/12/16): tiles of backproject_pm_rows()
 // rows, tasks (tile, |q|, chunk of backproject_pm_series_chunk() series per sign)
 size_t backproject_pm_smem(int max_nodes);
@@ -464,6 +464,7 @@ cudaError_t launch_backproject_pm_batch(const BackprojArgs<float>* items, const 
                                         cudaStream_t s);
 int backproject_w_rows();
 template <class T>
+int backproject_w_low_rows(int n_rows, int n_harm);   // low rows beside the sums
 cudaError_t launch_backproject_w(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s);
 template <class T>
 cudaError_t launch_backproject_w_batch(const BackprojArgs<T>* items, const int4* tasks, int n_tasks,

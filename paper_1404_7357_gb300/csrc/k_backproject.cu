@@ -231,7 +231,7 @@ __device__ __forceinline__ void backproject_task(const BackprojArgs<T>& a, int g
 // all MBF pairs of that q (a register-tiled complex product; 2 rows x up to
 // 8 series per thread).  The weights of a node are computed once per q instead
 // of once per series, and the grid values are read once per tile.
-constexpr int kWR = 64;       // rows per tile
+// rows per tile (WR): 64, or 16 where 64 leave SMs without a tile (backproject_w_rows)
 constexpr int kWK = 64;       // grid points per tile
 constexpr int kWThreads = 256;
 constexpr int kWSeriesMax = 64;
@@ -240,9 +240,9 @@ template <class T>
 __host__ __device__ constexpr int wbp_series_pad(int series) { return (series + 1) & ~1; }
 
 template <class T>
-__host__ __device__ constexpr size_t wbp_smem_bytes(int n_nodes_max, int series) {
-  return (size_t)kWK * (kWR + 2) * sizeof(cpx<T>) + (size_t)kWK * wbp_series_pad<T>(series) * sizeof(cpx<T>) +
-         (size_t)n_nodes_max * (sizeof(NodeCos<T>) + sizeof(T)) + (size_t)(2 * kWR) * sizeof(int) + 64;
+__host__ __device__ constexpr size_t wbp_smem_bytes(int rows, int n_nodes_max, int series) {
+  return (size_t)kWK * (rows + 2) * sizeof(cpx<T>) + (size_t)kWK * wbp_series_pad<T>(series) * sizeof(cpx<T>) +
+         (size_t)n_nodes_max * (sizeof(NodeCos<T>) + sizeof(T)) + (size_t)(2 * rows) * sizeof(int) + 64;
 }
 
 // two adjacent complex values from shared memory (16-byte aligned)
@@ -258,14 +258,14 @@ __device__ __forceinline__ void ld_pair(const cpx<T>* p, cpx<T>& x0, cpx<T>& x1)
   }
 }
 
-template <class T, int TAPS>
+template <class T, int TAPS, int WR>
 __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int tile, int qi,
                                                    unsigned char* smem_raw) {
   constexpr int HALF = TAPS / 2 - 1;
-  constexpr int kSub = kWThreads / kWR;            // threads per row in the scatter
+  constexpr int kSub = kWThreads / WR;            // threads per row in the scatter
   const int S = a.series_per_q;
   const int S2 = wbp_series_pad<T>(S);
-  const int r0 = tile * a.rchunk;                 // a.rchunk == kWR
+  const int r0 = tile * a.rchunk;                 // a.rchunk == WR
   const int q = qi - a.q_max;
   const int r_end = a.low_h > 0.0 ? min(a.n_rho, sum_first_row(a.low_h, abs(q), sizeof(T) == 8)) : a.n_rho;
   if (r0 >= r_end) return;                        // the sample sums form this tile
@@ -274,11 +274,11 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
   const int tid = threadIdx.x;
   // shared layout: W [WK][WR + 2] | G [WK][S2] | node cos | cos(q alpha) | row node ranges
   cpx<T>* W = reinterpret_cast<cpx<T>*>(smem_raw);
-  cpx<T>* G = W + kWK * (kWR + 2);
+  cpx<T>* G = W + kWK * (WR + 2);
   NodeCos<T>* scos = reinterpret_cast<NodeCos<T>*>(G + kWK * S2);
   T* scq = reinterpret_cast<T*>(scos + np);
   int* l_lo = reinterpret_cast<int*>(scq + np);
-  int* l_hi = l_lo + kWR;
+  int* l_hi = l_lo + WR;
   const int four_np = 4 * np;
   for (int t = tid; t < np; t += blockDim.x) {
     const double c = a.cosv[a.chunk_off[tile] + t];
@@ -307,17 +307,18 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
   // GEMM thread layout: a warp holds 8 row pairs x 4 series pairs, so each of its
   // shared-memory loads covers one 128-byte line (W) or a broadcast (G)
   const int lane = tid & 31, warp = tid >> 5;
-  const int rp = (warp & 3) * 8 + (lane & 7);     // rows 2 rp, 2 rp + 1
-  const int sp = (warp >> 2) * 4 + (lane >> 3);   // series 2 sp, 2 sp + 1 (+ 16 per pass)
-  constexpr int NPASS = kWSeriesMax / 16;
+  constexpr int RW = WR / 16, SP = 8 * (8 / RW);  // warps over rows; series per pass
+  const int rp = (warp % RW) * 8 + (lane & 7);    // rows 2 rp, 2 rp + 1
+  const int sp = (warp / RW) * 4 + (lane >> 3);   // series 2 sp, 2 sp + 1 (+ SP per pass)
+  constexpr int NPASS = kWSeriesMax / SP;
   cpx<T> acc[NPASS][4];                           // [pass][row0 s0, row0 s1, row1 s0, row1 s1]
 #pragma unroll
   for (int j = 0; j < NPASS; ++j)
 #pragma unroll
     for (int k = 0; k < 4; ++k) acc[j][k] = mk((T)0, (T)0);
-  const int npass = (S2 + 15) / 16;
+  const int npass = (S2 + SP - 1) / SP;
   // scatter layout: kSub threads per row, nodes interleaved among them
-  const int srow = tid % kWR, ssub = tid / kWR;
+  const int srow = tid % WR, ssub = tid / WR;
   const double arow = (double)(r0 + srow) * a.d_rho / a.d_s;
   const double rho_top = (r1 - 1) * a.d_rho;
   const int kmax = min(a.grid_half - 1, (int)ceil(rho_top / a.d_s) + TAPS);
@@ -326,7 +327,7 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
   for (int kt = 0; kt < n_tiles; ++kt) {
     const int k0 = k_first + kt * kWK;
     // ---- zero W, load the grid tile of every series of this q, find node ranges
-    for (int t = tid; t < kWK * (kWR + 2); t += blockDim.x) W[t] = mk((T)0, (T)0);
+    for (int t = tid; t < kWK * (WR + 2); t += blockDim.x) W[t] = mk((T)0, (T)0);
     for (int t = tid; t < kWK * S2; t += blockDim.x) {
       const int g = t / kWK, kk = t - g * kWK;
       const int k = k0 + kk;
@@ -334,7 +335,7 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
                            ? a.grid[((size_t)g * a.n_harm + qi) * (2 * a.grid_half + 1) + k + a.grid_half]
                            : mk((T)0, (T)0);
     }
-    if (tid < kWR) {
+    if (tid < WR) {
       const int r = r0 + tid;
       int lo = 0, hi = -1;
       if (r < r1) {
@@ -417,7 +418,7 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
         for (int m = 0; m < TAPS; ++m) {
           const int kk = kb + m;
           if (kk >= 0 && kk < kWK) {
-            T* dst = reinterpret_cast<T*>(&W[kk * (kWR + 2) + srow]);
+            T* dst = reinterpret_cast<T*>(&W[kk * (WR + 2) + srow]);
             atomicAdd(dst, wc.re * w[m]);
             atomicAdd(dst + 1, wc.im * w[m]);
           }
@@ -429,13 +430,13 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
 #pragma unroll 4
     for (int kk = 0; kk < kWK; ++kk) {
       cpx<T> w0, w1;
-      ld_pair(W + kk * (kWR + 2) + 2 * rp, w0, w1);
+      ld_pair(W + kk * (WR + 2) + 2 * rp, w0, w1);
       const cpx<T>* gk = G + kk * S2 + 2 * sp;
 #pragma unroll
       for (int j = 0; j < NPASS; ++j) {
-        if (j < npass && 2 * sp + 16 * j < S2) {
+        if (j < npass && 2 * sp + SP * j < S2) {
           cpx<T> g0, g1;
-          ld_pair(gk + 16 * j, g0, g1);
+          ld_pair(gk + SP * j, g0, g1);
           cmac(acc[j][0], w0, g0);
           cmac(acc[j][1], w0, g1);
           cmac(acc[j][2], w1, g0);
@@ -451,7 +452,7 @@ __device__ __forceinline__ void backproject_w_task(const BackprojArgs<T>& a, int
   for (int j = 0; j < NPASS; ++j) {
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int g = 2 * sp + 16 * j + (k & 1);
+      const int g = 2 * sp + SP * j + (k & 1);
       const int r = (k < 2) ? ra : rb;
       if (j < npass && g < S && r < r1)
         a.table[((size_t)g * a.n_harm + qi) * a.n_rho + r] = mk(acc[j][k].re * norm, acc[j][k].im * norm);
@@ -722,10 +723,10 @@ backproject_pm_batch_kernel(const BackprojArgs<float>* items, const int4* tasks,
   }
 }
 
-template <class T, int TAPS>
+template <class T, int TAPS, int WR>
 __global__ void __launch_bounds__(kWThreads) backproject_w_kernel(BackprojArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  backproject_w_task<T, TAPS>(a, blockIdx.x, blockIdx.y, smem_raw);
+  backproject_w_task<T, TAPS, WR>(a, blockIdx.x, blockIdx.y, smem_raw);
 }
 
 // persistent form over (item, row tile, harmonic) tasks
@@ -742,7 +743,7 @@ backproject_w_batch_kernel(const BackprojArgs<T>* items, const int4* tasks, int 
     if (t >= n_tasks) break;
     const int4 tk = tasks[t];
     const BackprojArgs<T> a = items[tk.x];
-    backproject_w_task<T, TAPS>(a, tk.z, tk.y, smem_raw);
+    backproject_w_task<T, TAPS, 64>(a, tk.z, tk.y, smem_raw);
     __syncthreads();
   }
 }
@@ -851,23 +852,35 @@ template cudaError_t launch_backproject_batch<double>(const BackprojArgs<double>
                                                       int*, int, int, int, int, int, cudaStream_t);
 
 template <class T>
-size_t backproject_w_smem(int max_nodes, int series) { return wbp_smem_bytes<T>(max_nodes, series); }
-int backproject_w_rows() { return kWR; }
+size_t backproject_w_smem(int rows, int max_nodes, int series) { return wbp_smem_bytes<T>(rows, max_nodes, series); }
+// rows per tile of the matrix form: 64; for the low rows below the sums 16 where 64-row tiles of
+// every harmonic are fewer than two per SM.  GB300, FP64: strip, 18 tiles of 64 rows 316 us, of
+// 16 rows 131 us; patch, 264 tiles of 64 rows 1,312 us, of 16 rows 780 us
+int backproject_w_rows() { return 64; }
+int backproject_w_low_rows(int n_rows, int n_harm) {
+  return (int64_t)((n_rows + 63) / 64) * n_harm < 2 * (int64_t)current_sm_count() ? 16 : 64;
+}
 
-template <class T, int TAPS>
-cudaError_t launch_w_taps(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s) {
-  const size_t smem = wbp_smem_bytes<T>(max_nodes, a.series_per_q);
-  cudaError_t e = cudaFuncSetAttribute(backproject_w_kernel<T, TAPS>,
+template <class T, int TAPS, int WR>
+cudaError_t launch_w_rows(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s) {
+  const size_t smem = wbp_smem_bytes<T>(WR, max_nodes, a.series_per_q);
+  cudaError_t e = cudaFuncSetAttribute(backproject_w_kernel<T, TAPS, WR>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(n_tiles, a.n_harm);
-  backproject_w_kernel<T, TAPS><<<grid, kWThreads, smem, s>>>(a);
+  backproject_w_kernel<T, TAPS, WR><<<grid, kWThreads, smem, s>>>(a);
   return cudaGetLastError();
+}
+
+template <class T, int TAPS>
+cudaError_t launch_w_taps(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s) {
+  return a.rchunk == 16 ? launch_w_rows<T, TAPS, 16>(a, n_tiles, max_nodes, s)
+                        : launch_w_rows<T, TAPS, 64>(a, n_tiles, max_nodes, s);
 }
 
 template <class T>
 cudaError_t launch_backproject_w(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s) {
-  if (a.series_per_q > kWSeriesMax || a.rchunk != kWR) return cudaErrorInvalidValue;
+  if (a.series_per_q > kWSeriesMax || (a.rchunk != 64 && a.rchunk != 16)) return cudaErrorInvalidValue;
   switch (a.taps) {
     case 8: return launch_w_taps<T, 8>(a, n_tiles, max_nodes, s);
     case 12: return launch_w_taps<T, 12>(a, n_tiles, max_nodes, s);
@@ -879,7 +892,7 @@ cudaError_t launch_backproject_w(const BackprojArgs<T>& a, int n_tiles, int max_
 template <class T, int TAPS>
 cudaError_t launch_w_batch_taps(const BackprojArgs<T>* items, const int4* tasks, int n_tasks,
                                 int* counter, int max_nodes, int series, int n_ctas, cudaStream_t s) {
-  const size_t smem = wbp_smem_bytes<T>(max_nodes, series);
+  const size_t smem = wbp_smem_bytes<T>(64, max_nodes, series);
   cudaError_t e = cudaFuncSetAttribute(backproject_w_batch_kernel<T, TAPS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -905,8 +918,8 @@ cudaError_t launch_backproject_w_batch(const BackprojArgs<T>* items, const int4*
   }
 }
 
-template size_t backproject_w_smem<float>(int, int);
-template size_t backproject_w_smem<double>(int, int);
+template size_t backproject_w_smem<float>(int, int, int);
+template size_t backproject_w_smem<double>(int, int, int);
 template cudaError_t launch_backproject_w<float>(const BackprojArgs<float>&, int, int, cudaStream_t);
 template cudaError_t launch_backproject_w<double>(const BackprojArgs<double>&, int, int, cudaStream_t);
 template cudaError_t launch_backproject_w_batch<float>(const BackprojArgs<float>*, const int4*, int, int*,
