@@ -580,6 +580,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
     launch_spectral_nodes(nc_spec, spec_beta0, spec_d, sn, sn + 2 * nc_spec, sn + 4 * nc_spec, sn + 6 * nc_spec, st);
     ++launches;
     CFFT_CUDA(cudaGetLastError(), "spectral nodes kernel");
+    ia.tables = 1;
     ia.beta_c = sn;
     ia.bw = sn + 2 * nc_spec;
     ia.green_p = sn + 4 * nc_spec;
@@ -685,8 +686,6 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   const bool pform = !fp64 && taps_ok && !gather;
   const bool tform = pform && !(ctx->opt[CFFT_OPT_BP_SIMT] > 0);   // its products on the tensor cores
   const bool wform = !pform && series_per_q <= 64 && taps_ok && !gather;
-  const int rchunk = pform ? backproject_pm_rows() : (wform ? backproject_w_rows() : 32);
-  const int n_chunks = (n_rho + rchunk - 1) / rchunk;
   const double d_rho = rho_max / (n_rho - 1);
   // rows formed by sums over the grid samples; the matrix forms then run on the chunks of the
   // rows below (all harmonics' first rows lie in the first n_low chunks)
@@ -1835,6 +1834,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         ia.bx = ctx->d_bx.as<T>();
         ia.by = ctx->d_by.as<T>();
         ia.q = ctx->d_q.as<cpx<T>>();
+        ia.tables = 1;
         ia.beta_c = sn;
         ia.bw = sn + 2 * nc_spec;
         ia.green_p = sn + 4 * nc_spec;

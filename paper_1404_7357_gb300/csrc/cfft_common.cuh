@@ -199,6 +199,7 @@ struct IntegrandArgs {
   int n, n_alpha, q_max, n_cls;  // n_cls computed classes (1 or 3)
   int n_mbf;                      // real MBF count (q holds a padded column count)
   int n_shape, n_basis;
+  int tables;                     // 1: the nodes are spectral_nodes' (real; D, then E on the same nodes)
   const ShapeClass* shapes;       // device, n_shape
   const T* bx;                    // device, basis centres x (sorted by class)
   const T* by;
@@ -463,8 +464,8 @@ cudaError_t launch_backproject_pm_batch(const BackprojArgs<float>* items, const 
                                         int* counter, int taps, int kern, int max_nodes, int n_ctas,
                                         cudaStream_t s);
 int backproject_w_rows();
-template <class T>
 int backproject_w_low_rows(int n_rows, int n_harm);   // low rows beside the sums
+template <class T>
 cudaError_t launch_backproject_w(const BackprojArgs<T>& a, int n_tiles, int max_nodes, cudaStream_t s);
 template <class T>
 cudaError_t launch_backproject_w_batch(const BackprojArgs<T>* items, const int4* tasks, int n_tasks,
