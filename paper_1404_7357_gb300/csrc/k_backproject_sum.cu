@@ -575,9 +575,13 @@ bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int gri
   while (p->split > 64 && (int64_t)p->tiles * blocks * (p->k_used / p->split + 1) < 16 * sms &&
          p->k_used / (p->split / 2) < 16)
     p->split /= 2;
+  // ... and as large as it takes to keep the splits' sums, a sixth of the table each, to 256 MB
+  const size_t per_split = blocks * p->cells * pts * 2 * ss;
+  while (p->split < p->k_used && (size_t)((p->k_used + p->split - 1) / p->split) * per_split * (fp64 ? 16 : 8) > ((size_t)256 << 20))
+    p->split *= 2;
   p->splits = std::max(1, (p->k_used + p->split - 1) / p->split);
   p->fold = blocks * 2 * p->k_pad * 4 * ss;
-  p->far = (size_t)p->splits * blocks * p->cells * pts * 2 * ss;
+  p->far = p->splits * per_split;
   p->wrow = (size_t)(fp64 ? SumShape<double>::kEnd : SumShape<float>::kEnd) * n_rho;
   return true;
 }

@@ -264,7 +264,10 @@ __global__ void grid_table_batch_kernel(const GridArgs<T>* items, int item0) {
 // The block's nodes are staged in shared memory as [vector][k][cell] (k the node's place in
 // its cell, absent ones zero), 16 bytes per vector (two series in float32, one in float64):
 // consecutive threads read consecutive cells of the nodes and of the weight tables, and a
-// weight serves kSb series.  Cells with many nodes go through in chunks of kKc nodes.
+// weight serves kSb series.  Cells with many nodes go through in chunks of kKc nodes.  With SUB
+// tap groups a block has 1 / SUB as many samples and SUB threads for each, every SUB-th tap: for
+// few series, whose blocks are fewer than the SMs and serial (strip, FP64: 15 blocks 112 us ->
+// 33 us).
 constexpr int kSpreadThreads = 128;
 constexpr int kSpreadVec = 4;        // 16-byte vectors per node
 constexpr int kKc = 4;               // nodes of a cell staged at a time
@@ -276,20 +279,21 @@ struct SpreadShape {
   static constexpr int kSb = kSpreadVec * kPer;
 };
 
-template <class T>
+template <class T, int SUB>
 __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0, unsigned char* smem_raw,
                                             int* s_first) {
   constexpr int PER = SpreadShape<T>::kPer, SB = SpreadShape<T>::kSb;
   const int tid = threadIdx.x;
   const int taps = 2 * a.hw;
   const int c_lo = i0 - taps + 1;                       // first cell that reaches this tile
-  const int ncell = kSpreadThreads + taps - 1;          // cells of the tile
+  constexpr int kSamples = kSpreadThreads / SUB;
+  const int ncell = kSamples + taps - 1;                // cells of the tile
   const int pitch = ncell | 1;
   float4* ys = reinterpret_cast<float4*>(smem_raw);     // [vector][kKc][pitch]
   for (int c = tid; c <= ncell; c += kSpreadThreads)
     s_first[c] = min(first_node(a.fft_len, a.m, c_lo + c), a.n);
   __syncthreads();
-  const int i = i0 + tid;
+  const int i = i0 + tid % kSamples, sub = tid / kSamples;
   cpx<T> acc[SB];
 #pragma unroll
   for (int u = 0; u < SB; ++u) acc[u] = mk((T)0, (T)0);
@@ -318,7 +322,7 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
     }
     __syncthreads();
 #pragma unroll 2
-    for (int t = 0; t < taps; ++t) {
+    for (int t = sub; t < taps; t += SUB) {
       const int c = i - t;
       if (c < 0 || c >= a.n_cells) continue;
       const bool act = c < a.act_cells;
@@ -360,6 +364,18 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
     }
     __syncthreads();
   }
+  if constexpr (SUB > 1) {
+    // the tap groups' sums, in order (the staging buffer holds kSpreadThreads SB entries)
+    cpx<T>* part = reinterpret_cast<cpx<T>*>(smem_raw);
+#pragma unroll
+    for (int u = 0; u < SB; ++u) part[u * kSpreadThreads + tid] = acc[u];
+    __syncthreads();
+    if (sub > 0) return;
+#pragma unroll
+    for (int u = 0; u < SB; ++u)
+#pragma unroll
+      for (int g = 1; g < SUB; ++g) acc[u] = acc[u] + part[u * kSpreadThreads + g * kSamples + tid];
+  }
   if (i < a.nc) {
 #pragma unroll
     for (int u = 0; u < SB; ++u)
@@ -367,11 +383,11 @@ __device__ __forceinline__ void spread_tile(const GridArgs<T>& a, int i0, int s0
   }
 }
 
-template <class T>
+template <class T, int SUB>
 __global__ void __launch_bounds__(kSpreadThreads) spread_kernel(GridArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int s_first[kSpreadThreads + 2 * kMaxHw + 1];
-  spread_tile<T>(a, blockIdx.x * kSpreadThreads, blockIdx.y * SpreadShape<T>::kSb, smem_raw, s_first);
+  spread_tile<T, SUB>(a, blockIdx.x * (kSpreadThreads / SUB), blockIdx.y * SpreadShape<T>::kSb, smem_raw, s_first);
 }
 
 template <class T>
@@ -380,10 +396,10 @@ __global__ void __launch_bounds__(kSpreadThreads) spread_batch_kernel(const Grid
   __shared__ int s_first[kSpreadThreads + 2 * kMaxHw + 1];
   const int2 bm = map[blockIdx.x];
   const GridArgs<T> a = items[bm.x];
-  spread_tile<T>(a, bm.y, blockIdx.y * SpreadShape<T>::kSb, smem_raw, s_first);
+  spread_tile<T, 1>(a, bm.y, blockIdx.y * SpreadShape<T>::kSb, smem_raw, s_first);
 }
 
-size_t spread_smem(int hw) { return (size_t)kSpreadVec * kKc * ((kSpreadThreads + 2 * hw - 1) | 1) * 16; }
+size_t spread_smem(int hw, int samples) { return (size_t)kSpreadVec * kKc * ((samples + 2 * hw - 1) | 1) * 16; }
 
 int series_chunk(int series, int tiles) {
   // about sixteen blocks per SM (the table loads' latency needs that many warps: 72 us with
@@ -475,9 +491,15 @@ cudaError_t launch_grid_tables_batch(const GridArgs<T>* items, int item0, int n_
 
 template <class T>
 cudaError_t launch_spread(const GridArgs<T>& a, cudaStream_t s) {
-  spread_kernel<T><<<dim3((a.nc + kSpreadThreads - 1) / kSpreadThreads,
-                          (a.series + SpreadShape<T>::kSb - 1) / SpreadShape<T>::kSb),
-                     kSpreadThreads, spread_smem(a.hw), s>>>(a);
+  constexpr int kSub = 4;
+  const int chunks = (a.series + SpreadShape<T>::kSb - 1) / SpreadShape<T>::kSb;
+  const int tiles = (a.nc + kSpreadThreads - 1) / kSpreadThreads;
+  if ((int64_t)tiles * chunks < current_sm_count()) {
+    constexpr int n = kSpreadThreads / kSub;
+    spread_kernel<T, kSub><<<dim3((a.nc + n - 1) / n, chunks), kSpreadThreads, spread_smem(a.hw, n), s>>>(a);
+  } else {
+    spread_kernel<T, 1><<<dim3(tiles, chunks), kSpreadThreads, spread_smem(a.hw, kSpreadThreads), s>>>(a);
+  }
   return cudaGetLastError();
 }
 
@@ -487,7 +509,7 @@ template <class T>
 cudaError_t launch_spread_batch(const GridArgs<T>* items, const int2* map, int n_blocks, int series, int max_hw,
                                 cudaStream_t s) {
   spread_batch_kernel<T><<<dim3(n_blocks, (series + SpreadShape<T>::kSb - 1) / SpreadShape<T>::kSb), kSpreadThreads,
-                           spread_smem(max_hw), s>>>(items, map);
+                           spread_smem(max_hw, kSpreadThreads), s>>>(items, map);
   return cudaGetLastError();
 }
 
