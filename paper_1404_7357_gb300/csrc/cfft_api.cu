@@ -5,6 +5,7 @@
 #include <complex>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <new>
 #include <string>
@@ -122,6 +123,8 @@ struct cfft_ctx {
   DevBuf b_cargs, b_cdata, b_iargs, b_fargs, b_bargs, b_cmap, b_imap, b_ftask, b_btask, b_count,
       b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag, b_sargs, b_smap, b_gargs, b_gmap, b_coarse, b_gtab, b_sum, b_margs, b_omap, b_fmap, b_nmap;
   cudaStream_t bstream = nullptr;
+  cudaStream_t side = nullptr;     // forked from and joined to `stream` inside a call
+  cudaEvent_t side_ev[2] = {nullptr, nullptr};
   cudaEvent_t bev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t bgraph = nullptr;
   std::string bsig;           // signature of the captured graph
@@ -780,17 +783,30 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   ba.grid = ctx->d_grid.as<cpx<T>>();
   ba.table = dst.as<cpx<T>>() + ch * table_elems;
   ba.kern = bp_es ? 1 : 0;
+  std::function<cudaError_t()> launch_sums;
+  cudaStream_t bst = st;
   if (sums) {
     SumArgs<T> sa{};
     CFFT_CUDA(ctx->d_sum.ensure(sp.fold * sizeof(T) + (sp.far + sp.wrow) * sizeof(cpx<T>)), "alloc back-projection");
     set_sum_args<T>(&sa, sp, ba, ctx->d_sum.as<T>());
-    CFFT_CUDA(launch_backproject_sum<T>(sa, bp_taps, ba.kern, sp.splits, sp.tiles, st), "back-projection sums");
+    launch_sums = [=]() { return launch_backproject_sum<T>(sa, bp_taps, ba.kern, sp.splits, sp.tiles, st); };
     launches += sp.splits > 1 ? 5 : 4;
     ba.low_h = d_rho / ds;
     // real weights: half a complex multiply-add each, over the near window of every row and
     // the cells' points
     bp_macs += 0.5 * series * ((double)n_rho * (2.0 * sp.cell_rows * ba.low_h + 40.0) +
                                0.5 * sp.cells * (fp64 ? 20.0 : 10.0) * sp.k_used);
+  }
+  if (sums) {
+    // the low rows' few tiles and the sums side by side (they share the grid and write different
+    // rows): the tiles, 12 to 34 in float32, run for 75 to 100 us on as many SMs
+    if (!ctx->side) {
+      CFFT_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking), "stream");
+      for (auto& e : ctx->side_ev) CFFT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event");
+    }
+    CFFT_CUDA(cudaEventRecord(ctx->side_ev[0], st), "event");
+    CFFT_CUDA(cudaStreamWaitEvent(ctx->side, ctx->side_ev[0], 0), "stream");
+    bst = ctx->side;
   }
   bp_form_used = tform ? 3 : (pform ? 2 : (wform ? 1 : 0));
   if (pform || wform) {
@@ -800,20 +816,25 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
     if constexpr (sizeof(T) == 4) {
       if (tform) {
         ba.err = ctx->d_flag.as<int>() + 2;
-        CFFT_CUDA(launch_backproject_tc(ba, n_low, low_nodes, st), "backprojection kernel (tensor cores)");
+        CFFT_CUDA(launch_backproject_tc(ba, n_low, low_nodes, bst), "backprojection kernel (tensor cores)");
         bp_tc = true;
       } else if (pform) {
         CFFT_CUDA(launch_backproject_pm(ba, n_chunks, max_nodes, st), "backprojection kernel");
       } else {
-        CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, st), "backprojection kernel");
+        CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, bst), "backprojection kernel");
       }
     } else {
-      CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, st), "backprojection kernel");
+      CFFT_CUDA(launch_backproject_w<T>(ba, n_low, low_nodes, bst), "backprojection kernel");
     }
   } else {
     CFFT_CUDA(launch_backproject_impl<T>(ba, ctx->d_cnodes.as<int>(), ctx->d_coff.as<int64_t>(),
                                          ctx->d_cos.as<double>(), ctx->d_lag.as<double>(), n_chunks,
                                          max_nodes, max_seg, st), "backprojection kernel");
+  }
+  if (sums) {
+    CFFT_CUDA(launch_sums(), "back-projection sums");
+    CFFT_CUDA(cudaEventRecord(ctx->side_ev[1], ctx->side), "event");
+    CFFT_CUDA(cudaStreamWaitEvent(st, ctx->side_ev[1], 0), "stream");
   }
   ++launches;
   if (cls_s == 4) {
@@ -2096,6 +2117,9 @@ void cfft_destroy(cfft_ctx* ctx) {
     for (DevBuf* b : bb) b->release();
     for (auto& e : ctx->bev)
       if (e) cudaEventDestroy(e);
+    for (auto& e : ctx->side_ev)
+      if (e) cudaEventDestroy(e);
+    if (ctx->side) cudaStreamDestroy(ctx->side);
     if (ctx->bgraph) cudaGraphExecDestroy(ctx->bgraph);
     if (ctx->bstream) cudaStreamDestroy(ctx->bstream);
   }
