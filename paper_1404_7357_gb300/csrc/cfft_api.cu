@@ -358,6 +358,25 @@ void set_gridded_fft(FftArgs<T>* fa, const GridArgs<T>& ga) {
   fa->out_factor = ga.out_factor;
 }
 
+// the context's second stream behind `st`, and `st` behind it again
+cudaError_t make_side(cfft_ctx* ctx) {
+  cudaError_t e = cudaSuccess;
+  if (!ctx->side) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
+  for (auto& ev : ctx->side_ev)
+    if (e == cudaSuccess && !ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+  return e;
+}
+cudaError_t fork_side(cfft_ctx* ctx, cudaStream_t st) {
+  cudaError_t e = make_side(ctx);
+  if (e == cudaSuccess) e = cudaEventRecord(ctx->side_ev[0], st);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->side_ev[0], 0);
+  return e;
+}
+cudaError_t join_side(cfft_ctx* ctx, cudaStream_t st) {
+  cudaError_t e = cudaEventRecord(ctx->side_ev[1], ctx->side);
+  return e == cudaSuccess ? cudaStreamWaitEvent(st, ctx->side_ev[1], 0) : e;
+}
+
 // One tabulation into `dst` on n_rho points rho_r = r rho_max / (n_rho - 1).  primary: the
 // table of cfft_tabulate_reactions (its diagnostics go to ctx->info); otherwise the table
 // that the fill interpolates when the tabulated grid misses the fill's target.
@@ -800,12 +819,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   if (sums) {
     // the low rows' few tiles and the sums side by side (they share the grid and write different
     // rows): the tiles, 12 to 34 in float32, run for 75 to 100 us on as many SMs
-    if (!ctx->side) {
-      CFFT_CUDA(cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking), "stream");
-      for (auto& e : ctx->side_ev) CFFT_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event");
-    }
-    CFFT_CUDA(cudaEventRecord(ctx->side_ev[0], st), "event");
-    CFFT_CUDA(cudaStreamWaitEvent(ctx->side, ctx->side_ev[0], 0), "stream");
+    CFFT_CUDA(fork_side(ctx, st), "stream");
     bst = ctx->side;
   }
   bp_form_used = tform ? 3 : (pform ? 2 : (wform ? 1 : 0));
@@ -833,8 +847,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   }
   if (sums) {
     CFFT_CUDA(launch_sums(), "back-projection sums");
-    CFFT_CUDA(cudaEventRecord(ctx->side_ev[1], ctx->side), "event");
-    CFFT_CUDA(cudaStreamWaitEvent(st, ctx->side_ev[1], 0), "stream");
+    CFFT_CUDA(join_side(ctx, st), "stream");
   }
   ++launches;
   if (cls_s == 4) {
@@ -1106,7 +1119,8 @@ cfft_status fill_impl(cfft_ctx* ctx, int n_el, const double* pos, const int* rot
         (fs = fill_lattice(ctx, fa, &done)) != CFFT_OK)
       return fs;
   if (!done) {
-    if (plan.ok && !plan.direct) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
+    // (the direct form reserves the sorted one's scratch too: memory runs out at the same calls)
+    if (plan.ok) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
     cudaError_t le = launch_fill<T, TO>(fa, plan, ctx->d_fill.p, ctx->stream);
     if (le != cudaSuccess) return cuda_fail(ctx, le, "fill kernel");
   }
@@ -1921,7 +1935,33 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
           ++launches;
         }
         if (w == 0) rec(ctx->bev[2]);
-        if (r.n1 > r.n0) {
+        // the low rows' tiles beside the sums (they share the grids and write different rows)
+        const bool split_rows = r.n1 > r.n0;
+        cudaStream_t lst = st;
+        if (split_rows) {
+          if ((e = fork_side(ctx, st)) != cudaSuccess) return e;
+          lst = ctx->side;
+        }
+        if constexpr (sizeof(T) == 4) {
+          if (tform_b)
+            e = launch_backproject_tc_batch(ctx->b_bargs.as<BackprojArgs<float>>(),
+                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0), counters,
+                                            bp_taps, bp_kern, max_nodes, ctx->sm_count, lst);
+          else if (pform_b)
+            e = launch_backproject_pm_batch(ctx->b_bargs.as<BackprojArgs<float>>(),
+                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0), counters,
+                                            bp_taps, bp_kern, max_nodes, ctx->sm_count, lst);
+          else
+            e = launch_backproject_w_batch<T>(ctx->b_bargs.as<BackprojArgs<T>>(),
+                                              ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0),
+                                              counters, bp_taps, max_nodes, pairs, ctx->sm_count, lst);
+        } else {
+          e = launch_backproject_w_batch<T>(ctx->b_bargs.as<BackprojArgs<T>>(),
+                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0),
+                                            counters, bp_taps, max_nodes, pairs, ctx->sm_count, lst);
+        }
+        if (e != cudaSuccess) return e;
+        if (split_rows) {
           e = launch_backproject_sum_batch<T>(ctx->b_margs.as<SumArgs<T>>(), r.it0, r.it1 - r.it0, n_rho,
                                               ctx->b_omap.as<int2>() + r.o0, (int)(r.o1 - r.o0),
                                               ctx->b_fmap.as<int2>() + r.h0, (int)(r.h1 - r.h0),
@@ -1929,24 +1969,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                                               pairs, bp_taps, bp_kern, st);
           if (e != cudaSuccess) return e;
           launches += 5;
-        }
-        if constexpr (sizeof(T) == 4) {
-          if (tform_b)
-            e = launch_backproject_tc_batch(ctx->b_bargs.as<BackprojArgs<float>>(),
-                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0), counters,
-                                            bp_taps, bp_kern, max_nodes, ctx->sm_count, st);
-          else if (pform_b)
-            e = launch_backproject_pm_batch(ctx->b_bargs.as<BackprojArgs<float>>(),
-                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0), counters,
-                                            bp_taps, bp_kern, max_nodes, ctx->sm_count, st);
-          else
-            e = launch_backproject_w_batch<T>(ctx->b_bargs.as<BackprojArgs<T>>(),
-                                              ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0),
-                                              counters, bp_taps, max_nodes, pairs, ctx->sm_count, st);
-        } else {
-          e = launch_backproject_w_batch<T>(ctx->b_bargs.as<BackprojArgs<T>>(),
-                                            ctx->b_btask.as<int4>() + r.b0, (int)(r.b1 - r.b0),
-                                            counters, bp_taps, max_nodes, pairs, ctx->sm_count, st);
+          e = join_side(ctx, st);
         }
         if (e != cudaSuccess) return e;
         ++launches;
@@ -1954,6 +1977,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
       }
       return cudaGetLastError();
     };
+    CFFT_CUDA(make_side(ctx), "stream");   // (not inside a capture)
     if (mode == 2) return CFFT_OK;
     if (mode == 3) {
       // tuning run: plain launches, time the requested stage of the first wave

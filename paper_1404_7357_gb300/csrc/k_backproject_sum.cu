@@ -556,6 +556,9 @@ bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int gri
   *p = SumPlan{};
   const int out = fp64 ? EndShape<double>::kOut : EndShape<float>::kOut;
   if (sigma != (fp64 ? EndShape<double>::kSigma : EndShape<float>::kSigma)) return false;
+  // Lagrange stencils narrower than the precision's target asks for (an option) keep the quadrature
+  // that interpolates with them
+  if (kern == 0 && taps < (fp64 ? 16 : 12)) return false;
   const double h = d_rho / d_s, top = (n_rho - 1) * h;
   if ((int)std::ceil(top) + sum_grid_extra(fp64, taps, kern) > grid_half) return false;
   if (sum_first_row(h, 0, fp64) >= n_rho) return false;
