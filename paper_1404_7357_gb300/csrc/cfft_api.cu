@@ -124,7 +124,7 @@ struct cfft_ctx {
       b_cnodes, b_coff, b_cos, b_contour, b_y, b_grid, b_flag, b_sargs, b_smap, b_gargs, b_gmap, b_coarse, b_gtab, b_sum, b_margs, b_omap, b_fmap, b_nmap;
   cudaStream_t bstream = nullptr;
   cudaStream_t side = nullptr;     // forked from and joined to `stream` inside a call
-  cudaEvent_t side_ev[2] = {nullptr, nullptr};
+  cudaEvent_t side_ev[3] = {nullptr, nullptr, nullptr};
   cudaEvent_t bev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   cudaGraphExec_t bgraph = nullptr;
   std::string bsig;           // signature of the captured graph
@@ -361,7 +361,12 @@ void set_gridded_fft(FftArgs<T>* fa, const GridArgs<T>& ga) {
 // the context's second stream behind `st`, and `st` behind it again
 cudaError_t make_side(cfft_ctx* ctx) {
   cudaError_t e = cudaSuccess;
-  if (!ctx->side) e = cudaStreamCreateWithFlags(&ctx->side, cudaStreamNonBlocking);
+  if (!ctx->side) {
+    // of the highest priority: what is forked is short of CTAs and has a call's time to run in
+    int least = 0, greatest = 0;
+    e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side, cudaStreamNonBlocking, greatest);
+  }
   for (auto& ev : ctx->side_ev)
     if (e == cudaSuccess && !ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   return e;
@@ -2693,6 +2698,9 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   w->diag = ctx->lu_diag;
   w->words = ctx->lu_words.as<unsigned long long>();
   w->err = ctx->lu_err.as<int>();
+  CFFT_CUDA(make_side(ctx), "stream");
+  w->side = ctx->side;
+  for (int i = 0; i < 3; ++i) w->ev[i] = ctx->side_ev[i];
   w->tc_update = ctx->opt[CFFT_OPT_SOLVE_SIMT] > 0 ? 0 : 1;
   w->panel_cluster = ctx->opt[CFFT_OPT_SOLVE_GRID_PANEL] > 0 ? 0 : 1;
   return CFFT_OK;

@@ -584,6 +584,8 @@ struct LuWork {
                        // wait of the trailing update ran out; bit 4: a wait of a substitution
   int* diag;           // host: [5] panel grid, resident CTAs per SM, shared bytes of the last grid
                        // panel; panels run on one cluster, CTAs per cluster (0: none)
+  cudaStream_t side;   // second stream and events of the look-ahead
+  cudaEvent_t ev[3];
   int tc_update;       // complex64: the trailing update on the tensor cores
   int panel_cluster;   // 1: panels whose rows fit one cluster's shared memory run there
 };
