@@ -656,8 +656,10 @@ def stage_flops(inf, wl):
         # into the A and B rows and 16 for its position and phase
         weights = 2.0 * taps * (taps + 1) if inf.get("bp_kernel", 0) == 1 else 4.0 * taps
         sten = (weights + 2.0 * taps + 16.0) * inf["work_bp_stencils"]
-        bp = {"algorithmic": prod + sten, "fp32": sten if form == 3 else prod + sten,
-              "tensor": inf.get("tc_flops_backproject", 0.0) if form == 3 else 0.0}
+        # form 3 executes its products on the tensor cores (a third of the executed flops each);
+        # what is left of them are the sample sums, on the FP32 pipe
+        tc = inf.get("tc_flops_backproject", 0.0) if form == 3 else 0.0
+        bp = {"algorithmic": prod + sten, "fp32": sten + (max(0.0, prod - tc / 3.0) if form == 3 else prod), "tensor": tc}
     else:
         bp = {"algorithmic": per_node, "fp32": per_node, "tensor": 0.0}
     bp["per_node_unit"] = per_node

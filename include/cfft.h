@@ -279,8 +279,12 @@ cfft_status cfft_contour_series_order(double x, cfft_precision precision, int se
  * computed by the C-FFT: MBF spectra along the contour (Eq. 11), the kernel
  * H = M_t . G . M_b^* (Eq. 10), azimuthal harmonics, the contour factor
  * (Eq. 22: in the weights of a gridded FFT, or as a series of zero-padded
- * FFTs, Eq. 23-24; see CONTOUR_SERIES) and a back-projection over the angle
- * to the uniform rho grid.  The back-projection's midpoint rule in the angle takes,
+ * FFTs, Eq. 23-24; see CONTOUR_SERIES) and a back-projection to the uniform
+ * rho grid.  Where the gridded FFT applies the spectra come from tables in
+ * beta, and the rows from rho of max(40, q^2 / 2) samples of the transform
+ * grid up (FP64: max(40, q^2)) are sums over those samples with end weights;
+ * the other rows, and every row elsewhere, are integrals over the angle by
+ * the midpoint rule, which takes,
  * for the rows of each chunk up to rho, ceil((z + q_max)/2 + c z^(1/3) +
  * margin/2) + 1 nodes with z = |beta_c|max rho, margin = ALPHA_MARGIN (24)
  * and c = 4 in FP64, 2 in FP32-mixed: the first aliased angular harmonic
@@ -329,7 +333,13 @@ cfft_status cfft_copy_table(const cfft_ctx* ctx, void* dst, int64_t bytes, int d
  * share table rows run together on one copy of those rows in shared memory;
  * the context owns that scratch (4 bytes per element pair of up to 2^27 pairs
  * at a time, 8 bytes per (row block, class, table row), 16 bytes per element)
- * and keeps it for the next fill.
+ * and keeps it for the next fill.  With FILL_BLOCK at its default, few pairs
+ * (up to 6144 in FP32, 2048 in FP64) are filled straight from the table
+ * without the sort; and an FP64 array of 256 elements or more whose centres
+ * take at most 96 different x and y is filled through its different
+ * displacements, when (displacements x classes) are at most an eighth of the
+ * pairs and memory for their blocks is there (kept too), bit for bit as the
+ * sorted form would.
  * Accuracy: the fill's interpolation keeps within a quarter of the table
  * precision's target (1e-10 of the table maximum per (class, pair) for FP64,
  * 1e-5 for FP32-mixed) at every distance up to rho_max.  The first fill or
@@ -467,7 +477,7 @@ cfft_status cfft_fill_backward_residual(cfft_ctx* ctx, int n_elements, const dou
  * spectra_tc: 1 when the MBF spectra ran on the tensor cores; bp_form: 0 the
  * gather form of the back-projection, 1 the matrix form, 2 the paired-
  * harmonic matrix form, 3 the paired-harmonic form with its products on the
- * tensor cores; for the matrix forms work_bp_macs counts the complex
+ * tensor cores (with the sample sums: the form of the rows beside them); for the matrix forms work_bp_macs counts the complex
  * multiply-adds of the interpolation-matrix products (rows x grid columns x
  * series, every harmonic) and work_bp_stencils the node stencils added into
  * the matrices (rows x angular nodes x matrices).  fill_form: the form of the
