@@ -1824,6 +1824,12 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                         (long long)zt_arrays, (long long)gridded, (long long)spec_tab, (long long)max_hw,
                         (long long)sum_b, (long long)max_splits, (long long)(spec_tab ? nc_spec : 0)})
       add(v);
+    // the integrand's launches (the spectral tables' whole, the per-node forms' sizes) take these
+    // of the element's arguments by value
+    static_assert(sizeof(shape_args.tc_rmax) == sizeof(int), "bits of tc_rmax");
+    int rmax_bits;
+    std::memcpy(&rmax_bits, &shape_args.tc_rmax, sizeof(rmax_bits));
+    for (long long v : {(long long)ctx->shapes.size(), (long long)shape_args.tc_ncol, (long long)rmax_bits}) add(v);
     for (const void* ptr : {ctx->d_tw.p, ctx->b_cnodes.p, ctx->b_coff.p, ctx->b_cos.p, ctx->b_count.p,
                             ctx->b_cargs.p, ctx->b_cdata.p, ctx->b_iargs.p, ctx->b_fargs.p, ctx->b_bargs.p,
                             ctx->b_cmap.p, ctx->b_imap.p, ctx->b_ftask.p, ctx->b_btask.p, ctx->b_flag.p,
