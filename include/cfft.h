@@ -133,7 +133,8 @@ typedef enum {
  *                Gaussian weights that carry the contour factor, one FFT
  *                follows, and no series is summed; and the spectra come from
  *                tables in beta where the contour has at least four times
- *                their nodes.  An explicit series (1 or 2), order or sub-FFT
+ *                their nodes and its height is at most 1.5 of their steps
+ *                pi / (17 element radius).  An explicit series (1 or 2), order or sub-FFT
  *                length keeps the spectra at every node and the series of FFTs
  *   BP_KERNEL    interpolation kernel of the back-projection.  1: Lagrange
  *                polynomials on the transform grid g(s_k).  2: the ES
@@ -280,8 +281,8 @@ cfft_status cfft_contour_series_order(double x, cfft_precision precision, int se
  * H = M_t . G . M_b^* (Eq. 10), azimuthal harmonics, the contour factor
  * (Eq. 22: in the weights of a gridded FFT, or as a series of zero-padded
  * FFTs, Eq. 23-24; see CONTOUR_SERIES) and a back-projection to the uniform
- * rho grid.  Where the gridded FFT applies the spectra come from tables in
- * beta, and the rows from rho of max(40, q^2 / 2) samples of the transform
+ * rho grid.  Without an explicit order, series or sub-FFT length the spectra
+ * may come from tables in beta (CONTOUR_SERIES), and the rows from rho of max(40, q^2 / 2) samples of the transform
  * grid up (FP64: max(40, q^2)) are sums over those samples with end weights;
  * the other rows, and every row elsewhere, are integrals over the angle by
  * the midpoint rule, which takes,

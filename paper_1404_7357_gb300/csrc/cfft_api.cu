@@ -478,12 +478,12 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
     while ((1 << log2L) < L) ++log2L;
     D = gs.m / L;
   }
-  // the spectra from tables in beta (k_grid.cu) where those have far fewer nodes than the
-  // contour; short contours evaluate them at every node
+  // the spectra from tables in beta (k_grid.cu) where those serve; other contours evaluate them
+  // at every node
   int nc_spec = 0;
   double spec_beta0 = 0, spec_d = 0;
   spectral_table_shape(fp64, ctx->elem_radius, ctx->beta_max, &nc_spec, &spec_beta0, &spec_d);
-  const bool spec_tab = !direct && 4 * (int64_t)nc_spec <= n;
+  const bool spec_tab = !direct && spectral_tables_serve(nc_spec, spec_d, n, ctx->height);
 
   // ---- buffers
   if (gridded) {
@@ -1356,7 +1356,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     int nc = 0;
     double b0 = 0, d = 0;
     spectral_table_shape(fp64, ctx->elem_radius, items[i].beta_max, &nc, &b0, &d);
-    spec_tab = spec_tab && 4 * (int64_t)nc <= p.n;
+    spec_tab = spec_tab && spectral_tables_serve(nc, d, p.n, items[i].height);
     beta_top = std::max(beta_top, items[i].beta_max);
   }
   spec_tab = spec_tab && !direct;

@@ -384,6 +384,7 @@ struct LatticeAxis {
 
 // host launchers (one translation unit per stage)
 void spectral_table_shape(bool fp64, double elem_radius, double beta_max, int* nc, double* beta0, double* d);
+bool spectral_tables_serve(int nc, double d, int n, double height);
 void launch_spectral_nodes(int nc, double beta0, double d, double2* beta, double2* bw, double2* gp, double2* gr,
                            cudaStream_t s);
 template <class T>

@@ -9,12 +9,14 @@
 //    have compact support.  They are sampled on a uniform real grid of step pi / (tau os)
 //    (os = kSpecOver times denser than their Nyquist step; a few samples beyond both ends:
 //    D and E continue through beta = 0 and beta_max) and interpolated at every contour
-//    node, complex ones included (a polynomial is as good there as beside it), with
-//    Lagrange stencils.  An entire function of type tau interpolated by w central taps has
-//    the error |prod (x - t)| / w! (pi / os)^w: below 1e-9 of the table for w = 8, os = 8
-//    (float32), 2e-15 for w = 16, os = 8 (float64), measured on the 200-rooftop patch.  The
-//    paper tabulates the MBFs' Fourier transforms before its FFTs in the same spirit
-//    (Table II, "FT tabulation").
+//    node, complex ones included, with Lagrange stencils.  An entire function of type tau
+//    interpolated by w central taps has the error |prod (x - t)| / w! (pi / os)^w: on the real
+//    axis below 1e-9 of the table for w = 8, os = 8 (float32), 2e-15 for w = 16, os = 8
+//    (float64), measured on the 200-rooftop patch.  Off the axis that product grows, and so do
+//    the weights, which carry the table's rounding (sum |weight| of 8 taps: 50 two steps off
+//    the axis, 12,000 six steps off), so contours rising more than kSpecRise steps keep the
+//    spectra at every node (spectral_tables_serve).  The paper tabulates the MBFs' Fourier
+//    transforms before its FFTs in the same spirit (Table II, "FT tabulation").
 // 2. Gridding.  The transform in beta, g_q(s_k) = sum_j Y_j exp(-i beta_c,j s_k), is wanted
 //    on |k| <= K only, a small part of the period 2 pi / step that the contour's nodes
 //    resolve.  The nodes are spread onto a coarser grid in beta (spacing 2 pi / (M ds),
@@ -420,6 +422,18 @@ void spectral_table_shape(bool fp64, double elem_radius, double beta_max, int* n
   *nc = (need + 7) / 8 * 8;
   *d = step;
   *beta0 = (0.5 - (w / 2 + 1)) * step;
+}
+
+// Where the tables serve a contour of n nodes: far fewer table nodes than contour nodes, and a
+// contour that stays within kSpecRise table steps of the real axis.  Functions of the full type
+// (all weight at the ends of the support, the worst case), float32 / float64 error over their
+// maximum, by the rise in steps: 0: 3e-7 / 1e-13, 1: 2e-6 / 1e-12, 1.5: 5e-6 / 5e-12,
+// 2: 2e-5 / 2e-11, 3: 1e-4 / 3e-10, 6: 1e-2 / 2e-7 (an element's spectrum: a tenth of that).  A
+// contour six of its own node spacings high, the workloads' choice, rises at most 1.5 steps
+// wherever the first condition holds.
+constexpr double kSpecRise = 1.5;
+bool spectral_tables_serve(int nc, double d, int n, double height) {
+  return 4 * (int64_t)nc <= n && height <= kSpecRise * d;
 }
 
 void launch_spectral_nodes(int nc, double beta0, double d, double2* beta, double2* bw, double2* gp, double2* gr,
