@@ -128,7 +128,9 @@ typedef enum {
  *                remainder bound (Taylor on a tie).  With the automatic
  *                series and order, sub-FFT length included, the same
  *                transform runs gridded where that applies (height * rho_max
- *                <= 3.5 and a grid of at most half the contour's own period):
+ *                <= 3.5, a grid of at most half the contour's own period, and
+ *                no height so many cells of a small rho_max's shortest grid
+ *                that the Gaussian's weights would cost digits):
  *                the nodes are spread onto a coarse grid in beta with complex
  *                Gaussian weights that carry the contour factor, one FFT
  *                follows, and no series is summed; and the spectra come from
@@ -282,10 +284,10 @@ cfft_status cfft_contour_series_order(double x, cfft_precision precision, int se
  * (Eq. 22: in the weights of a gridded FFT, or as a series of zero-padded
  * FFTs, Eq. 23-24; see CONTOUR_SERIES) and a back-projection to the uniform
  * rho grid.  Without an explicit order, series or sub-FFT length the spectra
- * may come from tables in beta (CONTOUR_SERIES), and the rows from rho of max(40, q^2 / 2) samples of the transform
- * grid up (FP64: max(40, q^2)) are sums over those samples with end weights;
- * the other rows, and every row elsewhere, are integrals over the angle by
- * the midpoint rule, which takes,
+ * may come from tables in beta (CONTOUR_SERIES), and the rows from rho of
+ * max(40, q^2 / 2) samples of the transform grid up (FP64: max(40, q^2)) are
+ * sums over those samples with end weights; the other rows, and every row
+ * elsewhere, are integrals over the angle by the midpoint rule, which takes,
  * for the rows of each chunk up to rho, ceil((z + q_max)/2 + c z^(1/3) +
  * margin/2) + 1 nodes with z = |beta_c|max rho, margin = ALPHA_MARGIN (24)
  * and c = 4 in FP64, 2 in FP32-mixed: the first aliased angular harmonic

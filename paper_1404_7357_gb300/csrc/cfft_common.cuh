@@ -265,8 +265,8 @@ struct GridShape {
 };
 // Fills g and returns true when the gridded transform serves this contour and grid: height *
 // rho_max <= 3.5, a coarse grid (m >= 2 (2K + 1), a power of two >= min_m) no finer than the contour's
-// own transform (m <= fft_len) and a Gaussian within the staging buffer.  Otherwise the
-// series of FFTs runs.
+// own transform (m <= fft_len), a contour that does not rise too many of its cells, and a Gaussian
+// within the staging buffer.  Otherwise the series of FFTs runs.
 bool grid_plan(bool fp64, int n, int64_t fft_len, int n_active, int grid_half, double ds, double height,
                double rho_max, int min_m, GridShape* g);
 

@@ -465,8 +465,7 @@ cudaError_t launch_spectral_interp_batch(const SpecInterpArgs<T>* items, const i
 // declaration)
 bool grid_plan(bool fp64, int n, int64_t fft_len, int n_active, int grid_half, double ds, double height,
                double rho_max, int min_m, GridShape* g) {
-  // height rho_max up to 3 is the documented range of float32; beyond about 3.5 the complex
-  // weights' growth exp(a y^2) would cost digits
+  // height rho_max up to 3 is the documented range of float32
   if (!(height * rho_max <= 3.5)) return false;
   int64_t m = min_m;
   while (m < 2 * (2 * (int64_t)grid_half + 1)) m *= 2;
@@ -475,6 +474,12 @@ bool grid_plan(bool fp64, int n, int64_t fft_len, int n_active, int grid_half, d
   const double db = 2.0 * pi / ((double)m * ds), thc = 2.0 * pi * (grid_half + 1) / (double)m;
   const double y = n_active > 0 ? height / db : 0.0, far = 2.0 * pi - thc;
   g->a = (far * far - thc * thc) / 4.0 / (e + y * far);
+  // The complex weights grow to exp(a y^2) and must cancel.  A grid as fine as the outputs ask
+  // for (m below 8 K) keeps a y^2 below 4 up to height rho_max = 3.5; the shortest grid, min_m,
+  // with few outputs does not.  Error of the transform over its maximum by a y^2, float32: up to
+  // 5 below 1e-6 (that of a y^2 = 1), 8: 4e-6, 10: 3e-5, 13: 5e-4, 21: 4; float64: up to 7 below
+  // 2e-14, 8: 5e-14, 14: 2e-11.
+  if (g->a * y * y > (fp64 ? 7.0 : 5.0)) return false;
   g->hw = (int)std::ceil(std::sqrt(e / g->a));
   if (g->hw > kMaxHw) return false;
   g->m = (int)m;
