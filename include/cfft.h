@@ -286,7 +286,8 @@ cfft_status cfft_contour_series_order(double x, cfft_precision precision, int se
  * rho grid.  Without an explicit order, series or sub-FFT length the spectra
  * may come from tables in beta (CONTOUR_SERIES), and the rows from rho of
  * max(40, q^2 / 2) samples of the transform grid up (FP64: max(40, q^2)) are
- * sums over those samples with end weights; the other rows, and every row
+ * sums over those samples with end weights (harmonics |q| > 16 only where the
+ * rows lie at most 2.4 samples apart, FP64: 10); the other rows, and every row
  * elsewhere, are integrals over the angle by the midpoint rule, which takes,
  * for the rows of each chunk up to rho, ceil((z + q_max)/2 + c z^(1/3) +
  * margin/2) + 1 nodes with z = |beta_c|max rho, margin = ALPHA_MARGIN (24)

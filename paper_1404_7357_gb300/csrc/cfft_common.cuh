@@ -304,10 +304,20 @@ struct BackprojArgs {
   double low_h;
 };
 
+// The far part of the sample sums is interpolated over cells of rows (k_backproject_sum.cu), where
+// the weights of harmonic q turn up to about sqrt(width) times from row q^2 on.  Up to |q| =
+// kSumNarrow any width keeps the interpolation's error (single tones, times 2 pi) at 1.6e-7 in
+// float32 and 5e-15 in float64; above, a cell is at most sum_cell_width samples wide (2e-7,
+// 3e-14), where that leaves it kSumCellRows rows (of fewer, the far part's points would be as many
+// as the rows).  Wider: |q| = 32 7e-6, 64 6e-4 in float32 (6e-13, 3e-10 in float64).
+constexpr int kSumNarrow = 16, kSumCellRows = 16;
+__host__ __device__ constexpr double sum_cell_width(bool fp64) { return fp64 ? 150.0 : 36.0; }
+
 // first row that the sums over grid samples serve for harmonics +-p (k_backproject_sum.cu); h:
 // the rho step in grid samples
 __host__ __device__ inline int sum_first_row(double h, int p, bool fp64) {
-  // end weights against Bessel functions there (single tones, times 2 pi): float32 8e-8,
+  if (p > kSumNarrow && (kSumCellRows - 1) * h > sum_cell_width(fp64)) return 2000000000;   // none
+  // end weights against Bessel functions there (single tones, times 2 pi): float32 1e-7,
   // float64 1e-13, falling like u^-3 and faster beyond
   const double u = (fp64 ? 1.0 : 0.5) * (double)p * (double)p;
   const double r = ceil((u > 40.0 ? u : 40.0) / h);

@@ -11,17 +11,18 @@
 //   A_k + i B_k = w_j(u - floor(u)) T_q(k / u) / sqrt(u + k)  for the kIn + kOut end samples
 // (k = 0 with half weight).  No interpolation stencils, no angular nodes, and a weight that is
 // real and closed in form but for the end samples.  The part of a sum that lies far from a
-// row's end is a smooth function of rho, so the rows are taken in cells of 64 or 32: with [ua, ub]
-// a cell's extent in samples, the samples below kc = ua - (ub - ua) (and below the cell's end
-// samples) are summed at kPts
-// Chebyshev points of the cell only and interpolated (the nearest singularity lies three half
-// widths from the cell's middle: the error falls by 5.8 per point).
+// row's end is a smooth function of rho, so the rows are taken in cells of 64, 32 or less: with
+// [ua, ub] a cell's extent in samples, the samples below kc = ua - (ub - ua) (and below the cell's
+// end samples) are summed at kPts Chebyshev points of the cell only and interpolated (the nearest
+// singularity lies three half widths from the cell's middle: the error falls by 5.8 per point).
 //
-// The weights' accuracy is that of the end weights (4e-9 in float32, 2e-14 in float64) while
-// T_q(k / u) / sqrt(u + k) varies slowly over the end samples, that is from u of about q^2 up
+// The weights' accuracy is that of the end weights while T_q(k / u) / sqrt(u + k) varies slowly
+// over the end samples, that is from u of about q^2 / 2 (float32) or q^2 (float64) up
 // (sum_first_row); the rows below keep the quadrature in alpha.  Errors against Bessel functions
-// (single tones over the band, times 2 pi): float32 form 1e-8 at q = 16 from u = 200, float64 form
-// 2e-14 at q = 16 from u = 400.
+// (single tones over the band, times 2 pi) at the first row: float32 form 1e-7 at |q| = 12 and 16,
+// 2e-8 at 64, float64 form 1e-13 at 8, 2e-14 at 64; at twice that row a tenth.  The far part's
+// interpolation adds at most 2e-7 (float32) and 3e-14 (float64): cells are narrowed for |q| beyond
+// kSumNarrow, and where rows lie too far apart for that those |q| keep the quadrature.
 //
 // Kernels (q and -q share their weights; 16 series per sign and block column):
 //   rows   end weights w_j of every row
@@ -565,6 +566,9 @@ bool sum_plan(bool fp64, int n_rho, double d_rho, double d_s, int sigma, int gri
   // 64 rows to a cell, 32 where those are more than 40 samples wide: the near window (two
   // widths and the end samples) grows with the width, the far points with the number of cells
   p->cell_rows = 63.0 * h > 40.0 ? 32 : 64;
+  // narrower for high harmonics, while sum_first_row has the sums serve them
+  if (q_max > kSumNarrow && (kSumCellRows - 1) * h <= sum_cell_width(fp64))
+    p->cell_rows = std::min(p->cell_rows, 1 + (int)(sum_cell_width(fp64) / h));
   p->cells = (n_rho + p->cell_rows - 1) / p->cell_rows;
   p->k_used = (int)std::floor(top) + out + 1;
   p->k_pad = (p->k_used + 4 + kSK) / kSK * kSK + kSK;   // steps may start at any multiple of 4
