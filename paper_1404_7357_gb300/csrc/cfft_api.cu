@@ -139,7 +139,7 @@ struct cfft_ctx {
   std::vector<std::complex<double>> q_user;
   DevBuf d_quser;
   // dense LU of the reduced system: the factored copy, work arrays, vectors, timing
-  DevBuf lu_a, lu_moves, lu_nmoves, lu_cand_v, lu_perm, lu_cand_d, lu_words, lu_err, lu_x, lu_y, lu_x64, lu_r, lu_sums;
+  DevBuf lu_a, lu_moves, lu_nmoves, lu_cand_v, lu_perm, lu_cand_d, lu_words, lu_x, lu_y, lu_x64, lu_r, lu_sums;
   cudaEvent_t lu_ev[3] = {nullptr, nullptr, nullptr};
   int lu_diag[5] = {0, 0, 0, 0, 0};
   cfft_solve_info solve_info{};
@@ -2134,7 +2134,7 @@ void cfft_destroy(cfft_ctx* ctx) {
                       &ctx->d_y, &ctx->d_grid, &ctx->d_table, &ctx->d_tw, &ctx->d_cnodes,
                       &ctx->d_coff, &ctx->d_cos, &ctx->d_lag, &ctx->d_flag, &ctx->d_pos,
                       &ctx->d_rot, &ctx->d_zbuf, &ctx->d_fill, &ctx->d_lat, &ctx->d_latz, &ctx->d_gres, &ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum, &ctx->d_ftable, &ctx->d_fest, &ctx->d_quser, &ctx->lu_a, &ctx->lu_moves,
-                      &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_perm, &ctx->lu_cand_d, &ctx->lu_words, &ctx->lu_err, &ctx->lu_x,
+                      &ctx->lu_nmoves, &ctx->lu_cand_v, &ctx->lu_perm, &ctx->lu_cand_d, &ctx->lu_words, &ctx->lu_x,
                       &ctx->lu_y, &ctx->lu_x64, &ctx->lu_r, &ctx->lu_sums, &ctx->c_tab, &ctx->c_work,
                       &ctx->c_im, &ctx->c_gx, &ctx->c_gy, &ctx->c_flag, &ctx->tc_bx, &ctx->tc_by, &ctx->tc_bmat,
                       &ctx->tc_bmat_mirror, &ctx->tc_shapes};
@@ -2694,8 +2694,7 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   CFFT_CUDA(ctx->lu_perm.ensure((size_t)n * sizeof(int)), "alloc LU");
   CFFT_CUDA(ctx->lu_cand_d.ensure((size_t)ctx->sm_count * 2 * nb * 16), "alloc LU");
   CFFT_CUDA(ctx->lu_words.ensure((size_t)n * 2 * 4 * sizeof(unsigned long long)), "alloc LU");
-  CFFT_CUDA(ctx->lu_err.ensure(sizeof(int)), "alloc LU");
-  CFFT_CUDA(ctx->lu_sums.ensure(4 * sizeof(double)), "alloc LU");
+  CFFT_CUDA(ctx->lu_sums.ensure(5 * sizeof(double)), "alloc LU");   // four sums, the error bits
   w->moves = ctx->lu_moves.as<int2>();
   w->n_moves = ctx->lu_nmoves.as<int>();
   w->cand_val = ctx->lu_cand_v.as<double>();
@@ -2703,7 +2702,7 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   w->cand_data = ctx->lu_cand_d.p;
   w->diag = ctx->lu_diag;
   w->words = ctx->lu_words.as<unsigned long long>();
-  w->err = ctx->lu_err.as<int>();
+  w->err = reinterpret_cast<int*>(ctx->lu_sums.as<double>() + 4);
   CFFT_CUDA(make_side(ctx), "stream");
   w->side = ctx->side;
   for (int i = 0; i < 3; ++i) w->ev[i] = ctx->side_ev[i];
@@ -2715,11 +2714,13 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
 // row stride of the context's copy of an n x n matrix: whole 128-byte lines
 int64_t lu_stride(int n) { return ((int64_t)n + 15) & ~(int64_t)15; }
 
-// the error bits of the LU kernels so far, read behind them
-cfft_status lu_flags(cfft_ctx* ctx, const LuWork& w) {
-  int flag = 0;
-  CFFT_CUDA(cudaMemcpyAsync(&flag, w.err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "LU flag");
+// the error bits of the LU kernels so far and the four sums of the residual and the correction, in
+// one read behind them
+cfft_status lu_read(cfft_ctx* ctx, double (&h)[5]) {
+  CFFT_CUDA(cudaMemcpyAsync(h, ctx->lu_sums.p, sizeof(h), cudaMemcpyDeviceToHost, ctx->stream), "LU flag");
   CFFT_CUDA(cudaStreamSynchronize(ctx->stream), "LU");
+  int flag = 0;
+  std::memcpy(&flag, h + 4, sizeof(flag));
   if (flag & 2) return fail(ctx, CFFT_ERR_TIMEOUT, "LU panel: a wait for the pivot candidates ran past its bound");
   if (flag & 4) return fail(ctx, CFFT_ERR_NUMERIC, "LU: the reduced matrix is singular (zero pivot)");
   if (flag & 8) return fail(ctx, CFFT_ERR_TIMEOUT, "LU update: a tensor-core wait ran past its bound");
@@ -2737,13 +2738,8 @@ cfft_status lu_factor_checked(cfft_ctx* ctx, int n, const LuWork& w) {
                 ", shared bytes " + std::to_string(w.diag[2]) + ")";
     return st;
   }
-  return lu_flags(ctx, w);
-}
-
-cfft_status read_sums(cfft_ctx* ctx, double* h, int count) {
-  CFFT_CUDA(cudaMemcpyAsync(h, ctx->lu_sums.p, count * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream), "sums");
-  CFFT_CUDA(cudaStreamSynchronize(ctx->stream), "sums");
-  return CFFT_OK;
+  double h[5];
+  return lu_read(ctx, h);
 }
 
 }  // namespace
@@ -2788,7 +2784,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
   CFFT_CUDA(ctx->lu_a.ensure((size_t)n * lu_stride(n) * es), "alloc LU matrix");
   CFFT_CUDA(ctx->lu_x.ensure((size_t)n * es), "alloc LU vectors");
   CFFT_CUDA(ctx->lu_y.ensure((size_t)n * es), "alloc LU vectors");
-  double h[4] = {0, 0, 0, 0};
+  double h[5] = {0, 0, 0, 0, 0};
   int steps = 0;
   CFFT_CUDA(cudaEventRecord(ctx->lu_ev[0], st), "event");
   if (!complex128) {
@@ -2828,7 +2824,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
                                 ctx->lu_y.as<cpx<float>>(), st), "LU solve");
       CFFT_CUDA(add_correction(ctx->lu_x64.p, ctx->lu_x.p, n, ctx->lu_sums.as<double>() + 2, st), "refinement");
       CFFT_CUDA(residual_f64(z, ld, n, ctx->lu_x64.p, v, ctx->lu_r.p, ctx->lu_sums.as<double>(), st), "residual");
-      if ((s = read_sums(ctx, h, 4)) != CFFT_OK) return s;
+      if ((s = lu_read(ctx, h)) != CFFT_OK) return s;
       const double rr = h[0], dd = h[2], xx = h[3];
       // stop when the correction is below float64 resolution or the residual stops falling
       if (!(dd > 1e-30 * xx) || (rr_prev >= 0.0 && rr > 0.25 * rr_prev)) break;
@@ -2839,7 +2835,7 @@ extern "C" cfft_status cfft_solve_reduced(cfft_ctx* ctx, int n, const void* z, i
     CFFT_CUDA(cudaEventRecord(ctx->lu_ev[2], st), "event");
     CFFT_CUDA(residual_f64(z, ld, n, i_out, v, nullptr, ctx->lu_sums.as<double>(), st), "residual");
   }
-  if ((s = read_sums(ctx, h, 2)) != CFFT_OK || (s = lu_flags(ctx, w)) != CFFT_OK) return s;
+  if ((s = lu_read(ctx, h)) != CFFT_OK) return s;
   float ms = 0.f;
   cfft_solve_info& in = ctx->solve_info;
   in = cfft_solve_info{};

@@ -623,7 +623,7 @@ __device__ __forceinline__ void warp_substitute(const cpx<T>* M, int ms, int kb,
       if (UPPER) {
         const cpx<T> y = xj;
         xj = y * rd[j];
-        if constexpr (sizeof(T) == 8) {   // the quotient's last bits, as a division would have them
+        if constexpr (sizeof(T) == 8 || NC == 1) {   // the quotient's last bits, as a division would have them
           cpx<T> r = y;
           const cpx<T> d = M[j * ms + j];
           cmac(r, mk(-xj.re, -xj.im), d);
@@ -1117,9 +1117,10 @@ constexpr size_t subst_smem() {   // the diagonal block, and its inverse (comple
 // inverts the diagonal block while it waits and multiplies by the inverse, with one step of
 // refinement against the block itself, so that the error is that of a substitution; in complex128
 // the FP64 pipe makes the three products (13 us) and the inverse (50 us and more) dearer than a
-// substitution of 64 serial steps.  Bound by the chain of blocks: publish, poll, one tile, the
-// diagonal block.  One launch per block row with a serial substitution in every CTA took 15 us
-// (forward) and 25 us (backward) per block in complex64.
+// substitution of 64 serial steps, and so is the first block's, which waits for nothing (two
+// substitutions of 24 unknowns: 39 us with the inverses, 12 us without).  Bound by the chain of blocks:
+// publish, poll, one tile, the diagonal block.  One launch per block row with a serial substitution
+// in every CTA took 15 us (forward) and 25 us (backward) per block in complex64.
 template <class T, bool UPPER>
 __global__ void __launch_bounds__(256) lu_substitute_kernel(const cpx<T>* a, int64_t ld, int n, const int* order,
                                                             const cpx<T>* b, cpx<T>* x, unsigned long long* words,
@@ -1154,7 +1155,8 @@ __global__ void __launch_bounds__(256) lu_substitute_kernel(const cpx<T>* a, int
       if (tid < kNb) rd[tid] = crecip(D[tid * LS + tid]);
       __syncthreads();
     }
-    if constexpr (sizeof(T) == 4) {
+    const bool invert = sizeof(T) == 4 && t > 0;
+    if (invert) {
       cpx<T> x0[8], x1[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -1219,7 +1221,7 @@ __global__ void __launch_bounds__(256) lu_substitute_kernel(const cpx<T>* a, int
     if ((lane & 3) == 0) rhs[8 * warp + row] = rhs[8 * warp + row] - sum;
     __syncthreads();
     if (s_fail) break;
-    if constexpr (sizeof(T) == 8) {
+    if (!invert) {
       if (warp == 0) {
         cpx<T> x0[1] = {rhs[lane]}, x1[1] = {rhs[lane + 32]};
         warp_substitute<T, UPPER, 1>(D, LS, kb, rd, x0, x1);
@@ -1639,18 +1641,22 @@ cudaError_t lu_solve(const cpx<T>* a, int64_t ld, int n, const LuWork& w, cpx<T>
   const cpx<T>* yc = y;
   int* err = w.err;
   cudaError_t e;
-  if ((e = cudaMemsetAsync(w.words, 0, 2 * bytes, s)) != cudaSuccess) return e;
+  // one block row: no CTA waits for another, and no word is read
+  const bool coop = G > 1;
+  if (coop && (e = cudaMemsetAsync(w.words, 0, 2 * bytes, s)) != cudaSuccess) return e;
   if ((e = cudaFuncSetAttribute(lu_substitute_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(lu_substitute_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem)) != cudaSuccess)
     return e;
+  auto launch = [&](const void* f, void** args) {
+    return coop ? cudaLaunchCooperativeKernel(f, dim3(G), dim3(256), args, smem, s)
+                : cudaLaunchKernel(f, dim3(G), dim3(256), args, smem, s);
+  };
   void* fwd[] = {&a, &ld, &n, &order, &xc, &y, &words[0], &err};
-  if ((e = cudaLaunchCooperativeKernel((const void*)lu_substitute_kernel<T, false>, dim3(G), dim3(256), fwd, smem,
-                                       s)) != cudaSuccess)
-    return e;
+  if ((e = launch((const void*)lu_substitute_kernel<T, false>, fwd)) != cudaSuccess) return e;
   void* bwd[] = {&a, &ld, &n, &none, &yc, &x, &words[1], &err};
-  return cudaLaunchCooperativeKernel((const void*)lu_substitute_kernel<T, true>, dim3(G), dim3(256), bwd, smem, s);
+  return launch((const void*)lu_substitute_kernel<T, true>, bwd);
 }
 
 cudaError_t residual_f64(const void* z, int64_t ld, int n, const void* x, const void* b, void* r, double* sums,
