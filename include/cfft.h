@@ -608,6 +608,13 @@ cfft_status cfft_selftest_bounded_wait(cfft_ctx* ctx, unsigned polls);
  * context stays usable: a later call allocates what it needs again. */
 void cfft_test_fail_allocation(int after);
 
+/* The same for the groups of launches that a call makes while its second stream
+ * is forked from the context's (the sample sums of a tabulation or a batch, the
+ * look-ahead of a factorization): after `after` of them the next one reports a
+ * launch failure and the call returns CFFT_ERR_CUDA, with nothing that it
+ * launched left to run beside a later call. */
+void cfft_test_fail_forked_launch(int after);
+
 /* Reduced excitation of an array of identical elements (Section II, Eq. 4):
  *   v_red[m M + a] = sum_i conj(Q_ia) v[m][i]
  * for every element m and MBF a, with Q the coefficient matrix given to

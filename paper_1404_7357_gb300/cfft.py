@@ -31,7 +31,8 @@ EXPORTS = ["cfft_create", "cfft_destroy", "cfft_last_error", "cfft_set_substrate
            "cfft_debug_buffer", "cfft_synchronize", "cfft_backproject_static",
            "cfft_get_derivative_table", "cfft_fill_backward", "cfft_tabulate_batch",
            "cfft_get_batch_info", "cfft_mbf_spectra", "cfft_selftest_bounded_wait", "cfft_load_table",
-           "cfft_fill_backward_residual", "cfft_test_fail_allocation", "cfft_measure_peak",
+           "cfft_fill_backward_residual", "cfft_test_fail_allocation", "cfft_test_fail_forked_launch",
+           "cfft_measure_peak",
            "cfft_reduced_excitation", "cfft_port_excitation", "cfft_port_currents", "cfft_solve_reduced",
            "cfft_get_solve_info", "cfft_tabulate_cartesian", "cfft_get_cartesian_table", "cfft_fill_cartesian",
            "cfft_set_green_extraction"]
@@ -117,6 +118,7 @@ def _load():
         "cfft_fill_backward": ([P, I, P, P, P, L, I, P, P], I),
         "cfft_fill_backward_residual": ([P, I, P, P, P, P, I, P, P], I),
         "cfft_test_fail_allocation": ([I], None),
+        "cfft_test_fail_forked_launch": ([I], None),
         "cfft_tabulate_batch": ([P, I, ctypes.POINTER(BatchItem), I, D, I, I, P, I], I),
         "cfft_get_batch_info": ([P, ctypes.POINTER(BatchInfo)], I),
         "cfft_mbf_spectra": ([P, I, P, P], I),
@@ -563,6 +565,12 @@ def test_fail_allocation(after):
     """cfft_test_fail_allocation: after `after` successful device allocations the next one
     fails as out of memory (host-side injection; after < 0 disarms)."""
     _lib.cfft_test_fail_allocation(int(after))
+
+
+def test_fail_forked_launch(after):
+    """cfft_test_fail_forked_launch: after `after` successful launch groups beside the forked second
+    stream the next one fails (host-side injection; after < 0 disarms)."""
+    _lib.cfft_test_fail_forked_launch(int(after))
 
 
 PEAK_FP32, PEAK_FP64, PEAK_TF32, PEAK_BF16 = range(4)

@@ -38,6 +38,12 @@ constexpr double kPi = 3.14159265358979323846;
 // failure injection on the host (cfft_test_fail_allocation): the number of library
 // allocations still to succeed before one fails as out of memory; -1 = disarmed
 long g_alloc_countdown = -1;
+// the same for the launches made while the second stream is forked (cfft_test_fail_forked_launch)
+long g_fork_countdown = -1;
+bool fail_forked_launch() {
+  if (g_fork_countdown < 0) return false;
+  return g_fork_countdown-- == 0;
+}
 
 struct DevBuf {
   void* p = nullptr;
@@ -371,16 +377,35 @@ cudaError_t make_side(cfft_ctx* ctx) {
     if (e == cudaSuccess && !ev) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
   return e;
 }
-cudaError_t fork_side(cfft_ctx* ctx, cudaStream_t st) {
-  cudaError_t e = make_side(ctx);
-  if (e == cudaSuccess) e = cudaEventRecord(ctx->side_ev[0], st);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx->side, ctx->side_ev[0], 0);
-  return e;
-}
-cudaError_t join_side(cfft_ctx* ctx, cudaStream_t st) {
-  cudaError_t e = cudaEventRecord(ctx->side_ev[1], ctx->side);
-  return e == cudaSuccess ? cudaStreamWaitEvent(st, ctx->side_ev[1], 0) : e;
-}
+// The second stream forked behind `st`.  It is joined again by join(), or, when a call returns
+// between the two, by the destructor: what such a call has launched there must not run on beside
+// the next call's work on the same buffers (nor leave a capture with an open fork).
+class SideFork {
+ public:
+  SideFork(cfft_ctx* ctx, cudaStream_t st) : ctx_(ctx), st_(st) {}
+  SideFork(const SideFork&) = delete;
+  SideFork& operator=(const SideFork&) = delete;
+  ~SideFork() {
+    if (open_) join();
+  }
+  cudaError_t fork() {
+    cudaError_t e = make_side(ctx_);
+    if (e == cudaSuccess) e = cudaEventRecord(ctx_->side_ev[0], st_);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(ctx_->side, ctx_->side_ev[0], 0);
+    open_ = e == cudaSuccess;
+    return e;
+  }
+  cudaError_t join() {
+    open_ = false;
+    const cudaError_t e = cudaEventRecord(ctx_->side_ev[1], ctx_->side);
+    return e == cudaSuccess ? cudaStreamWaitEvent(st_, ctx_->side_ev[1], 0) : e;
+  }
+
+ private:
+  cfft_ctx* ctx_;
+  cudaStream_t st_;
+  bool open_ = false;
+};
 
 // One tabulation into `dst` on n_rho points rho_r = r rho_max / (n_rho - 1).  primary: the
 // table of cfft_tabulate_reactions (its diagnostics go to ctx->info); otherwise the table
@@ -809,6 +834,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   ba.kern = bp_es ? 1 : 0;
   std::function<cudaError_t()> launch_sums;
   cudaStream_t bst = st;
+  SideFork fork(ctx, st);
   if (sums) {
     SumArgs<T> sa{};
     CFFT_CUDA(ctx->d_sum.ensure(sp.fold * sizeof(T) + (sp.far + sp.wrow) * sizeof(cpx<T>)), "alloc back-projection");
@@ -824,7 +850,7 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   if (sums) {
     // the low rows' few tiles and the sums side by side (they share the grid and write different
     // rows): the tiles, 12 to 34 in float32, run for 75 to 100 us on as many SMs
-    CFFT_CUDA(fork_side(ctx, st), "stream");
+    CFFT_CUDA(fork.fork(), "stream");
     bst = ctx->side;
   }
   bp_form_used = tform ? 3 : (pform ? 2 : (wform ? 1 : 0));
@@ -851,8 +877,8 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
                                          max_nodes, max_seg, st), "backprojection kernel");
   }
   if (sums) {
-    CFFT_CUDA(launch_sums(), "back-projection sums");
-    CFFT_CUDA(join_side(ctx, st), "stream");
+    CFFT_CUDA(fail_forked_launch() ? cudaErrorLaunchOutOfResources : launch_sums(), "back-projection sums");
+    CFFT_CUDA(fork.join(), "stream");
   }
   ++launches;
   if (cls_s == 4) {
@@ -1949,8 +1975,9 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         // the low rows' tiles beside the sums (they share the grids and write different rows)
         const bool split_rows = r.n1 > r.n0;
         cudaStream_t lst = st;
+        SideFork fork(ctx, st);
         if (split_rows) {
-          if ((e = fork_side(ctx, st)) != cudaSuccess) return e;
+          if ((e = fork.fork()) != cudaSuccess) return e;
           lst = ctx->side;
         }
         if constexpr (sizeof(T) == 4) {
@@ -1973,6 +2000,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         }
         if (e != cudaSuccess) return e;
         if (split_rows) {
+          if (fail_forked_launch()) return cudaErrorLaunchOutOfResources;
           e = launch_backproject_sum_batch<T>(ctx->b_margs.as<SumArgs<T>>(), r.it0, r.it1 - r.it0, n_rho,
                                               ctx->b_omap.as<int2>() + r.o0, (int)(r.o1 - r.o0),
                                               ctx->b_fmap.as<int2>() + r.h0, (int)(r.h1 - r.h0),
@@ -1980,7 +2008,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
                                               pairs, bp_taps, bp_kern, st);
           if (e != cudaSuccess) return e;
           launches += 5;
-          e = join_side(ctx, st);
+          e = fork.join();
         }
         if (e != cudaSuccess) return e;
         ++launches;
@@ -2455,6 +2483,8 @@ cfft_status cfft_tabulate_batch(cfft_ctx* ctx, int n_items, const cfft_batch_ite
   cfft_status s = precision == CFFT_FP64
                       ? batch_impl<double>(ctx, n_items, items, q_max, rho_max, n_rho, tables, flags)
                       : batch_impl<float>(ctx, n_items, items, q_max, rho_max, n_rho, tables, flags);
+  // a batch that stopped half way leaves nothing running beside the context stream
+  if (s != CFFT_OK) cudaStreamSynchronize(ctx->bstream);
   return s;
 }
 
@@ -2616,6 +2646,7 @@ cfft_status ensure_tc_element(cfft_ctx* ctx) {
 }  // namespace
 
 extern "C" void cfft_test_fail_allocation(int after) { g_alloc_countdown = after < 0 ? -1 : after; }
+extern "C" void cfft_test_fail_forked_launch(int after) { g_fork_countdown = after < 0 ? -1 : after; }
 
 extern "C" cfft_status cfft_selftest_bounded_wait(cfft_ctx* ctx, unsigned polls) {
   if (!ctx) return CFFT_ERR_ARG;
@@ -2706,6 +2737,7 @@ cfft_status lu_work(cfft_ctx* ctx, int n, LuWork* w) {
   CFFT_CUDA(make_side(ctx), "stream");
   w->side = ctx->side;
   for (int i = 0; i < 3; ++i) w->ev[i] = ctx->side_ev[i];
+  w->fail_forked = fail_forked_launch;
   w->tc_update = ctx->opt[CFFT_OPT_SOLVE_SIMT] > 0 ? 0 : 1;
   w->panel_cluster = ctx->opt[CFFT_OPT_SOLVE_GRID_PANEL] > 0 ? 0 : 1;
   return CFFT_OK;

@@ -597,6 +597,7 @@ struct LuWork {
                        // panel; panels run on one cluster, CTAs per cluster (0: none)
   cudaStream_t side;   // second stream and events of the look-ahead
   cudaEvent_t ev[3];
+  bool (*fail_forked)();   // failure injection: a launch behind the fork is to fail
   int tc_update;       // complex64: the trailing update on the tensor cores
   int panel_cluster;   // 1: panels whose rows fit one cluster's shared memory run there
 };

@@ -1583,6 +1583,15 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
     if constexpr (sizeof(T) == 4)
       lu_gemm_tc_kernel<<<grid_for((int64_t)rt * ct, 1, ctas), kUThreads, kUSmem, st>>>(map, a, ld, n, k, cf, ct, w.err);
   };
+  // the second stream joined again when the factorization stops between its fork and its join
+  struct Fork {
+    const LuWork& w;
+    cudaStream_t s;
+    bool open = false;
+    ~Fork() {
+      if (open && cudaEventRecord(w.ev[2], w.side) == cudaSuccess) cudaStreamWaitEvent(s, w.ev[2], 0);
+    }
+  } fork{w, s};
   bool done = false;   // block column pnl was factored ahead
   for (int pnl = 0; pnl < n_panels; ++pnl) {
     const int k = pnl * kNb, kb = std::min(kNb, n - k), k1 = k + kb, rest = n - k1;
@@ -1606,13 +1615,16 @@ cudaError_t lu_factor(cpx<T>* a, int64_t ld, int n, const LuWork& w, cudaStream_
         if ((e = cudaEventRecord(w.ev[0], s)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(w.side, w.ev[0], 0)) != cudaSuccess)
           return e;
+        fork.open = true;
         update(k, k1, 1, sms, w.side);
+        if (w.fail_forked()) return cudaErrorLaunchOutOfResources;
         if ((e = block(pnl + 1, true, w.side, w.ev[1])) != cudaSuccess ||
             (e = cudaEventRecord(w.ev[2], w.side)) != cudaSuccess ||
             (e = cudaStreamWaitEvent(s, w.ev[1], 0)) != cudaSuccess)
           return e;
         update(k, k1 + kNb, ct - 1, sms - cs, s);
         if ((e = cudaStreamWaitEvent(s, w.ev[2], 0)) != cudaSuccess) return e;
+        fork.open = false;
       } else if (tc_update) {
         update(k, k1, ct, sms, s);
       } else {
