@@ -364,7 +364,8 @@ def bench_fill(torch, cfft, args, dev):
     flops_per_pair = m * m * nh * (4 * taps + 8)
     sec = sum(ms) / steps / 1e3
     form = ctx.info()["fill_form"]
-    res["form"] = {1: "per-row", 2: "bucketed, FP32 pipe", 3: "tensor cores"}.get(form, "none")
+    res["form"] = {1: "per-row", 2: "bucketed, FP32 pipe", 3: "tensor cores", 4: "direct",
+                   5: "displacements"}.get(form, "none")
     res["algorithmic_tflops"] = flops_per_pair * float(a) ** 2 / sec / 1e12
     if form == 3:
         kpad = (2 * nh + 7) // 8 * 8

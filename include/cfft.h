@@ -487,9 +487,9 @@ cfft_status cfft_fill_backward_residual(cfft_ctx* ctx, int n_elements, const dou
  * the matrices (rows x angular nodes x matrices).  fill_form: the form of the
  * last cfft_fill_reduced_matrix: 1 per-row, 2 bucketed on the FP32 or FP64
  * pipe, 3 on the tensor cores, 4 direct (few pairs: up to 6144 in FP32, 2048
- * in FP64; 0: no fill yet).  fill_err_est: the estimated
- * interpolation error of the fill on the tabulated grid, relative to the
- * table maximum (-1: not estimated); fill_refine: the factor r of the grid
+ * in FP64), 5 by an FP64 lattice's different displacements (0: no fill yet).
+ * fill_err_est: the estimated interpolation error of the fill on the tabulated
+ * grid, relative to the table maximum (-1: not estimated); fill_refine: the factor r of the grid
  * the fill interpolates (0: no fill since the last tabulation); fill_n_rho:
  * that grid's points (n_rho when the fill uses the tabulated table, else
  * (n_rho - 1) r + 1 + fill_taps / 2, reaching beyond rho_max).

@@ -1149,7 +1149,9 @@ cfft_status fill_impl(cfft_ctx* ctx, int n_el, const double* pos, const int* rot
     if (plan.ok && n_el >= 256 && ctx->opt[CFFT_OPT_FILL_BLOCK] == 0 &&
         (fs = fill_lattice(ctx, fa, &done)) != CFFT_OK)
       return fs;
-  if (!done) {
+  if (done) {
+    ctx->info.fill_form = 5;
+  } else {
     // (the direct form reserves the sorted one's scratch too: memory runs out at the same calls)
     if (plan.ok) CFFT_CUDA(ctx->d_fill.ensure(plan.scratch), "alloc fill scratch");
     cudaError_t le = launch_fill<T, TO>(fa, plan, ctx->d_fill.p, ctx->stream);
