@@ -136,8 +136,10 @@ typedef enum {
  *                follows, and no series is summed; and the spectra come from
  *                tables in beta where the contour has at least four times
  *                their nodes and its height is at most 1.5 of their steps
- *                pi / (17 element radius).  An explicit series (1 or 2), order or sub-FFT
- *                length keeps the spectra at every node and the series of FFTs
+ *                pi / (17 element radius).  An explicit series (1 or 2), order
+ *                or sub-FFT length keeps the spectra at every node and the
+ *                series of FFTs, and so does a lack of memory for the others'
+ *                buffers
  *   BP_KERNEL    interpolation kernel of the back-projection.  1: Lagrange
  *                polynomials on the transform grid g(s_k).  2: the ES
  *                kernel exp(beta (sqrt(1 - (2x/w)^2) - 1)) of width w = taps

@@ -495,32 +495,32 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   if (n_active < 0) n_active = 0;
 
   GridShape gs{};
-  const bool gridded = !direct && grid_plan(fp64, n, P, n_active, K, ds, ctx->height, rho_max, 256, &gs);
-  if (gridded) {
-    L = std::min(gs.m, l_max);
-    while (L > 256 && (int64_t)series * (gs.m / L) < 2 * ctx->sm_count) L /= 2;
-    log2L = 0;
-    while ((1 << log2L) < L) ++log2L;
-    D = gs.m / L;
-  }
+  bool gridded = !direct && grid_plan(fp64, n, P, n_active, K, ds, ctx->height, rho_max, 256, &gs);
   // the spectra from tables in beta (k_grid.cu) where those serve; other contours evaluate them
   // at every node
   int nc_spec = 0;
   double spec_beta0 = 0, spec_d = 0;
   spectral_table_shape(fp64, ctx->elem_radius, ctx->beta_max, &nc_spec, &spec_beta0, &spec_d);
-  const bool spec_tab = !direct && spectral_tables_serve(nc_spec, spec_d, n, ctx->height);
+  bool spec_tab = !direct && spectral_tables_serve(nc_spec, spec_d, n, ctx->height);
+
+  // ---- the back-projection's form
+  // the matrix-form back-projection handles up to 64 series per harmonic with 8/12/16 taps;
+  // otherwise the direct gather form runs
+  // FP32-mixed: the paired-harmonic matrix form (one interpolation matrix per |q|)
+  const bool taps_ok = bp_es ? (bp_taps == 6 || bp_taps == 8) : (bp_taps == 8 || bp_taps == 12 || bp_taps == 16);
+  const bool gather = ctx->opt[CFFT_OPT_BP_GATHER] > 0;
+  const bool pform = !fp64 && taps_ok && !gather;
+  const bool tform = pform && !(ctx->opt[CFFT_OPT_BP_SIMT] > 0);   // its products on the tensor cores
+  const bool wform = !pform && series_per_q <= 64 && taps_ok && !gather;
+  const double d_rho = rho_max / (n_rho - 1);
+  // rows formed by sums over the grid samples; the matrix forms then run on the chunks of the
+  // rows below (all harmonics' first rows lie in the first n_low chunks)
+  SumPlan sp{};
+  sums = sums && (tform || wform) &&
+         sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q,
+                  ctx->sm_count, &sp);
 
   // ---- buffers
-  if (gridded) {
-    const size_t nw = (size_t)2 * gs.hw * gs.kmax;
-    CFFT_CUDA(ctx->d_gtab.ensure(nw * (gs.n_cells + gs.act_cells) * sizeof(T) + (size_t)(2 * K + 2) * sizeof(cpx<T>)),
-              "alloc gridding");
-    CFFT_CUDA(ctx->d_coarse.ensure((size_t)series * gs.nc * sizeof(cpx<T>)), "alloc gridding");
-  }
-  if (spec_tab) {
-    CFFT_CUDA(ctx->d_snodes.ensure((size_t)8 * nc_spec * sizeof(double2)), "alloc spectra");
-    CFFT_CUDA(ctx->d_spec.ensure((size_t)series * 2 * nc_spec * sizeof(cpx<T>)), "alloc spectra");
-  }
   CFFT_CUDA(ctx->beta_c.ensure(n * sizeof(double2)), "alloc contour");
   CFFT_CUDA(ctx->weight.ensure(n * sizeof(double2)), "alloc contour");
   CFFT_CUDA(ctx->bw.ensure(n * sizeof(double2)), "alloc contour");
@@ -542,6 +542,40 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   }
   CFFT_CUDA(ctx->d_flag.ensure(sizeof(int) * 4), "alloc flag");
   CFFT_CUDA(cudaMemsetAsync(ctx->d_flag.as<int>() + 2, 0, sizeof(int), st), "flag");
+  // the buffers of the gridded transform, the spectral tables and the sample sums come last:
+  // without memory for them the direct pipeline runs on the others
+  auto extras = [&]() -> cudaError_t {
+    cudaError_t e = cudaSuccess;
+    auto need = [&](DevBuf& b, size_t bytes) {
+      if (e == cudaSuccess) e = b.ensure(bytes);
+    };
+    if (gridded) {
+      const size_t nw = (size_t)2 * gs.hw * gs.kmax;
+      need(ctx->d_gtab, nw * (gs.n_cells + gs.act_cells) * sizeof(T) + (size_t)(2 * K + 2) * sizeof(cpx<T>));
+      need(ctx->d_coarse, (size_t)series * gs.nc * sizeof(cpx<T>));
+    }
+    if (spec_tab) {
+      need(ctx->d_snodes, (size_t)8 * nc_spec * sizeof(double2));
+      need(ctx->d_spec, (size_t)series * 2 * nc_spec * sizeof(cpx<T>));
+    }
+    if (sums) need(ctx->d_sum, sp.fold * sizeof(T) + (sp.far + sp.wrow) * sizeof(cpx<T>));
+    return e;
+  };
+  const cudaError_t extra = extras();
+  if (extra == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    for (DevBuf* b : {&ctx->d_gtab, &ctx->d_coarse, &ctx->d_snodes, &ctx->d_spec, &ctx->d_sum}) b->release();
+    gridded = spec_tab = sums = false;
+  } else {
+    CFFT_CUDA(extra, "alloc transform");
+  }
+  if (gridded) {
+    L = std::min(gs.m, l_max);
+    while (L > 256 && (int64_t)series * (gs.m / L) < 2 * ctx->sm_count) L /= 2;
+    log2L = 0;
+    while ((1 << log2L) < L) ++log2L;
+    D = gs.m / L;
+  }
   // MBF spectra on the tensor cores (FP32-mixed rooftop elements), unless disabled
   bool tc_spectra = false;
   if (!fp64 && !(ctx->opt[CFFT_OPT_SPECTRA_SIMT] > 0) && (n_alpha == 128 || n_alpha == 256)) {
@@ -730,21 +764,6 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   if (ch == 0) CFFT_CUDA(cudaEventRecord(ctx->ev[3], st), "event");
 
   // ---- a5: back-projection to the rho grid
-  // the matrix-form back-projection handles up to 64 series per harmonic with 8/12/16 taps;
-  // otherwise the direct gather form runs
-  // FP32-mixed: the paired-harmonic matrix form (one interpolation matrix per |q|)
-  const bool taps_ok = bp_es ? (bp_taps == 6 || bp_taps == 8) : (bp_taps == 8 || bp_taps == 12 || bp_taps == 16);
-  const bool gather = ctx->opt[CFFT_OPT_BP_GATHER] > 0;
-  const bool pform = !fp64 && taps_ok && !gather;
-  const bool tform = pform && !(ctx->opt[CFFT_OPT_BP_SIMT] > 0);   // its products on the tensor cores
-  const bool wform = !pform && series_per_q <= 64 && taps_ok && !gather;
-  const double d_rho = rho_max / (n_rho - 1);
-  // rows formed by sums over the grid samples; the matrix forms then run on the chunks of the
-  // rows below (all harmonics' first rows lie in the first n_low chunks)
-  SumPlan sp{};
-  sums = sums && (tform || wform) &&
-         sum_plan(fp64, n_rho, d_rho, ds, sigma, K, bp_taps, bp_es ? 1 : 0, ctx->q_max, series_per_q,
-                  ctx->sm_count, &sp);
   const int low_rows = sums ? std::min(n_rho, sum_first_row(d_rho / ds, ctx->q_max, fp64)) : n_rho;
   const int rchunk = pform ? backproject_pm_rows()
                      : !wform ? 32
@@ -837,7 +856,6 @@ cfft_status tabulate_impl(cfft_ctx* ctx, int n_rho, double rho_max, DevBuf& dst,
   SideFork fork(ctx, st);
   if (sums) {
     SumArgs<T> sa{};
-    CFFT_CUDA(ctx->d_sum.ensure(sp.fold * sizeof(T) + (sp.far + sp.wrow) * sizeof(cpx<T>)), "alloc back-projection");
     set_sum_args<T>(&sa, sp, ba, ctx->d_sum.as<T>());
     launch_sums = [=]() { return launch_backproject_sum<T>(sa, bp_taps, ba.kern, sp.splits, sp.tiles, st); };
     launches += sp.splits > 1 ? 5 : 4;
@@ -1395,16 +1413,6 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
     return ((size_t)2 * p.g.hw * p.g.kmax * (p.g.n_cells + p.g.act_cells) + 2 * (2 * (size_t)p.K + 2) + 3) / 4 * 4;
   };
 
-  // ---- signature (graph and tuning cache key)
-  std::string sig = std::to_string(n_items) + ":" + std::to_string(q_max) + ":" + std::to_string(n_rho) +
-                    ":" + std::to_string(rho_max) + ":" + std::to_string(sizeof(T)) + ":" +
-                    std::to_string(n_alpha) + ":" + std::to_string((size_t)tables) + ":" +
-                    std::to_string(ctx->n_basis) + ":" + std::to_string(M) + ":" + std::to_string(bp_taps) + ":" +
-                    std::to_string(bp_kern) + ":" + std::to_string(gridded) + std::to_string(spec_tab);
-  for (int i = 0; i < n_items; ++i)
-    sig += ":" + std::to_string(ip[i].n) + "/" + std::to_string(ip[i].taylor) + "/" + std::to_string(ip[i].series) +
-           "/" + std::to_string(ip[i].na_need);
-
   // ---- element data in T (shared by all items)
   {
     std::vector<T> hx(ctx->n_basis), hy(ctx->n_basis);
@@ -1461,12 +1469,37 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
   CFFT_CUDA(ctx->b_contour.ensure(max_nodes_wave * (4 * sizeof(double2) + sizeof(double) + sizeof(double2) + 64)), "alloc batch contour");
   CFFT_CUDA(ctx->b_y.ensure(max_y), "alloc batch harmonics");
   CFFT_CUDA(ctx->b_grid.ensure(max_grid), "alloc batch grid");
-  if (gridded) {
-    CFFT_CUDA(ctx->b_coarse.ensure(max_coarse), "alloc batch gridding");
-    CFFT_CUDA(ctx->b_gtab.ensure(max_gtab), "alloc batch gridding");
+  // without memory for the gridded transform, the tables and the sums: the direct pipeline, as in
+  // the single tabulation
+  {
+    cudaError_t e = cudaSuccess;
+    auto need = [&](DevBuf& b, size_t bytes) {
+      if (e == cudaSuccess) e = b.ensure(bytes);
+    };
+    if (gridded) {
+      need(ctx->b_coarse, max_coarse);
+      need(ctx->b_gtab, max_gtab);
+    }
+    if (any_sum) need(ctx->b_sum, max_sum);
+    if (spec_tab) need(ctx->d_spec, (size_t)series * 2 * nc_spec * sizeof(cpx<T>));
+    if (e == cudaErrorMemoryAllocation) {
+      cudaGetLastError();
+      for (DevBuf* b : {&ctx->b_coarse, &ctx->b_gtab, &ctx->b_sum, &ctx->d_spec}) b->release();
+      gridded = spec_tab = any_sum = false;
+    } else {
+      CFFT_CUDA(e, "alloc batch transform");
+    }
   }
-  if (any_sum) CFFT_CUDA(ctx->b_sum.ensure(max_sum), "alloc batch back-projection");
-  if (spec_tab) CFFT_CUDA(ctx->d_spec.ensure((size_t)series * 2 * nc_spec * sizeof(cpx<T>)), "alloc spectra");
+
+  // ---- signature (graph and tuning cache key)
+  std::string sig = std::to_string(n_items) + ":" + std::to_string(q_max) + ":" + std::to_string(n_rho) +
+                    ":" + std::to_string(rho_max) + ":" + std::to_string(sizeof(T)) + ":" +
+                    std::to_string(n_alpha) + ":" + std::to_string((size_t)tables) + ":" +
+                    std::to_string(ctx->n_basis) + ":" + std::to_string(M) + ":" + std::to_string(bp_taps) + ":" +
+                    std::to_string(bp_kern) + ":" + std::to_string(gridded) + std::to_string(spec_tab);
+  for (int i = 0; i < n_items; ++i)
+    sig += ":" + std::to_string(ip[i].n) + "/" + std::to_string(ip[i].taylor) + "/" + std::to_string(ip[i].series) +
+           "/" + std::to_string(ip[i].na_need);
 
   // contour buffers carved from b_contour: beta_c, weight, bw, green_p, green_r (double2), bi_rel (double)
   double2* c_beta = ctx->b_contour.as<double2>();
