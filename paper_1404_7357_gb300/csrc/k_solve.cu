@@ -564,9 +564,14 @@ __global__ void __launch_bounds__(kClThreads) lu_panel_cluster_kernel(PanelArgs<
     for (int e = tid; e < nr * kb; e += kClThreads)
       p.a[(int64_t)(lo + e / kb) * p.ld + p.k + e % kb] = rows[(size_t)(e / kb) * pitch + e % kb];
     if (g == 0) panel_record_moves(p, s_piv);
-  } else if (tid == 0) {
-    atomicOr(p.err, fail);
-    if (g == 0) *p.n_moves = 0;   // the panel stopped: no row moves for it
+  } else if (warp == 0) {
+    if (lane == 0) {
+      atomicOr(p.err, fail);
+      if (g == 0) *p.n_moves = 0;   // the panel stopped: no row moves for it
+    }
+    // once more, with the same bound, for candidates still on their way here: no CTA's shared
+    // memory goes while a copy into it or out of it may be in flight
+    tc::mbar_wait(&mbar[b], phase, kClPolls);
   }
   cluster_sync_all();
 }
