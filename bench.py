@@ -676,10 +676,10 @@ def stage_flops(inf, wl):
     }
 
 
-# DRAM bytes (read + write) per launch of each table kernel on the full patch-m4 workload,
-# from one ncu capture of the current kernel (None: changed since its last capture);
-# valid only for the default table sizes
-KERNEL_DRAM_BYTES = {"integrand": None, "fft": None, "backproject": None}
+# DRAM bytes (read + write) of each table stage's kernels on the full patch-m4 workload, from one
+# ncu capture (profiles/table_kernels_gridded.md); valid only for the default table sizes
+KERNEL_DRAM_BYTES = {"integrand": 0.5e6 + 9.9e6, "fft": 0.2e6 + 73.0e6 + 17.5e6,
+                     "backproject": 0.8e6 + 17.8e6 + 9.1e6 + 25.6e6 + 25.0e6}
 
 
 def pipe_peaks(peaks):
@@ -729,7 +729,7 @@ def roofline(infos, wl, peaks, clk):
     return {"kernel": dominant, "bound": "tensor" if d["bound"] == "tensor" else "alu",
             "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic.get(dominant),
-            "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
+            "traffic_unit": "bytes of the stage's kernels (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
             "peak_note": "%s; peak source: %s" % (kind, source),
             "peaks_tflops": {"fp32": p32, "tf32": ptc}, "stages": stages,
             "algorithmic_flops_per_launch": fl[dominant]["algorithmic"],

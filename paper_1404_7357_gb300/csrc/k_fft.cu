@@ -18,7 +18,7 @@
 // i.e. for every residue k2 one length-L FFT of a folded, pre-twiddled input.
 // One CTA owns one (series, k2): it loops over the Taylor terms, runs each
 // length-L FFT in shared memory (radix-4 Stockham passes staged through
-// registers), and accumulates (H s_k)^n/n! times the needed outputs.  The
+// registers), and accumulates (H s_k)^n/n! times the needed outputs.
 // With the gridded transform (k_grid.cu) the same task runs once, on the coarse samples
 // (a.y, length M for P) and multiplies every output by its factor (a.out_factor).  The
 // result is written demodulated by exp(+i beta_max s / 2) so that the

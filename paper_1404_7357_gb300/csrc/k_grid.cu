@@ -33,11 +33,12 @@
 //    the 8 (float32) or 14 (float64) terms of the contour factor's series, and it is as long
 //    as the wanted outputs need, not as the contour's nodes do.
 //
-// Measured (GB300, before -> after, same table error): the 16-pair patch table (n 16384,
-// 8192 rho points, float32) integrand 1247 -> 154 us (tables 77, interpolation 74; float32
-// stores bound the latter), transform 1170 -> 188 us (spreading 100: shared-memory
-// bandwidth, 16 bytes per node, tap and pair of series; FFT 74: one 512-thread CTA per SM);
-// float64 (n 4096) integrand 19.5 -> 1.8 ms, transform 24.4 -> 1.2 ms (FP64 pipe).
+// Measured (GB300, before -> now, same table error): the 16-pair patch table (n 16384, 8192 rho
+// points, float32) integrand 1247 -> 126 us (tables 77, interpolation 49; one serial chain on 72
+// blocks and float32 issue bound them), transform 1170 -> 157 us (spreading 65: shared-memory
+// bandwidth, 16 bytes per node, tap and pair of series; FFT 75: one 512-thread CTA per SM; spreading
+// weights 17); float64 (n 4096) integrand 19.5 -> 0.82 ms (tables 0.37, interpolation 0.46),
+// transform 24.4 -> 1.13 ms (FP64 pipe).
 #include <algorithm>
 #include <cmath>
 
