@@ -1187,7 +1187,7 @@ BucketArgs bucket_args(const FillArgs<T, T>& a, const FillBucketPlan& pl, void* 
   b.n_ck = a.n_cls;
   b.n_cells = pl.n_cells;
   b.win = pl.win;
-  b.parts = sizeof(T) == 8 ? 8 : 1;
+  b.parts = 1;
   const double inv = a.inv_d_rho;
   b.ih = (float)inv;
   b.il = (float)(inv - (double)b.ih);
@@ -1240,7 +1240,18 @@ cudaError_t run_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& pl, void
   cudaError_t e = cudaFuncSetAttribute(bucket_fill_kernel<T, M, TAPS>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return run_waves<T, TAPS>(a, pl, bucket_args(a, pl, scratch), s, [&](const BucketArgs& b, dim3 fg) {
+  return run_waves<T, TAPS>(a, pl, bucket_args(a, pl, scratch), s, [&](BucketArgs b, dim3 fg) {
+    // FP64: the pairs' arithmetic is dear and unevenly spread over the cells (a lattice's
+    // displacements lie in a few hundred of them), so several CTAs share a window where there are
+    // fewer than eight CTAs per SM (two where shared memory holds one CTA), each with its own copy of the
+    // window's rows.  GB300, M = 4, one CTA per window -> shared (two-cell windows with eight CTAs
+    // each): the 25 x 25 array's displacements and copy 1,472 -> 595 us (589); irregular, 8 harmonics: 60
+    // elements 329 -> 161 (263), 500 4,941 -> 4,600 (5,213), four classes 4,920 -> 4,787 (6,065); 16
+    // harmonics, 700 elements 17.8 -> 17.6 ms (27.1: narrow windows copy 17 rows for two cells).
+    if (sizeof(T) == 8) {
+      const int64_t ctas = (int64_t)fg.x * fg.y * fg.z, want = (smem <= 113 * 1024 ? 8 : 2) * (int64_t)current_sm_count();
+      b.parts = (int)std::min<int64_t>(8, std::max<int64_t>(1, (want + ctas - 1) / ctas));
+    }
     fg.x *= b.parts;
     bucket_fill_kernel<T, M, TAPS><<<fg, kBThreads, smem, s>>>(a, b);
     return cudaSuccess;
@@ -1373,14 +1384,6 @@ FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, in
     if (win < 8) win = (int)((220 * 1024) / row_bytes) - (taps - 1);
     if (win < 4) return pl;
     win = std::min(win, 64);
-    // FP64: the pairs' arithmetic is dear and unevenly spread over the cells (a lattice's
-    // displacements lie in a few hundred of them), the copy of the table rows cheap, so at least
-    // six windows per SM and eight CTAs per window.  GB300: the 25 x 25 array's displacements
-    // 1.31 -> 0.45 ms, 700 irregular elements 10.1 -> 9.0 ms, 60: 0.43 -> 0.28 ms
-    if (sizeof(T) == 8) {
-      const int cells = n_rho - taps + taps / 2;
-      win = std::min(win, std::max(2, cells / (6 * current_sm_count())));
-    }
     pl.win = win;
     pl.smem = (size_t)(win + taps - 1) * row_bytes;
   }
