@@ -1806,8 +1806,7 @@ cfft_status batch_impl(cfft_ctx* ctx, int n_items, const cfft_batch_item* items,
         int mo = 0;
         while (u < r.f1 && ftask[u].w == ftask[t].w) {
           const int i = ftask[u].x;
-          // a gridded task keeps no outputs in shared memory
-          mo = gridded ? -2 : std::max(mo, (2 * ip[i].K + 1) / (int)(ip[i].P / li[i]) + 2);
+          mo = gridded ? kNoOutputs : std::max(mo, (2 * ip[i].K + 1) / (int)(ip[i].P / li[i]) + 2);
           ++u;
         }
         r.fb.push_back(FftBucket{ftask[t].w, t, u, mo});

@@ -446,6 +446,8 @@ __host__ __device__ constexpr size_t fft_task_extra(int /*n_active_max*/, int n_
          (size_t)n_out_max * (sizeof(cpx<T>) + sizeof(T)) + 64;
 }
 
+// max_n_out of a gridded batch, whose tasks keep no outputs in shared memory (others: less two)
+constexpr int kNoOutputs = -2;
 template <class T>
 cudaError_t launch_fft_batch(const FftArgs<T>* items, const int4* tasks, int n_tasks, int* counter,
                              int log2_sub, int max_n_out, int max_active, int max_hi, int zt_arrays,

@@ -486,8 +486,9 @@ __device__ __forceinline__ T bessel_i_tail(int m, T q) {
 //    (a / 2)^m / m! instead of (2 a)^n / n!, so fewer transforms reach a tolerance.
 // use_zt: the pre-twiddled active inputs times the current weight are kept in shared
 // memory (two arrays for the Chebyshev recurrence) and advanced by the weight recurrence
-// instead of being re-read
-template <class T, int LOG2L, int NT>
+// instead of being re-read.  GRID: the gridded transform, one term with output factors (its own
+// instantiation: as a test at run time it cost the series' FFTs up to 3%)
+template <class T, int LOG2L, int NT, bool GRID>
 __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series, int k2,
                                                 unsigned char* smem_raw, int use_zt) {
   constexpr int L = 1 << LOG2L;
@@ -501,8 +502,8 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
   const int n_out = t_hi - t_lo + 1;
   const int n = a.n;
   const int na = a.n_active;
-  const bool cheb = a.expansion == 1;
-  const int n_terms = a.taylor + (cheb ? 2 : 1);
+  const bool cheb = !GRID && a.expansion == 1;
+  const int n_terms = GRID ? 1 : a.taylor + (cheb ? 2 : 1);
   const int n_hi = (n + 127) >> 7;
   const int tid = threadIdx.x;
   const int64_t P = a.fft_len;
@@ -552,9 +553,9 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
   // series, exp(a) (a/2)^m / m! for the Chebyshev series (a = H s / 2)
   const T dsh = (T)a.ds_height;
   // gridded transform: one term, each needed output used once, written as it is formed
-  const cpx<T>* of = a.out_factor;
+  const cpx<T>* of = GRID ? a.out_factor : nullptr;
   cpx<T>* out = a.grid + (size_t)series * (2 * K + 1);
-  for (int o = tid; o < n_out && !of; o += NT) {
+  for (int o = tid; o < n_out && !GRID; o += NT) {
     acc[o] = mk((T)0, (T)0);
     fac[o] = cheb ? exp((T)0.5 * dsh * (T)(k2 + D * (t_lo + o))) : (T)1;
   }
@@ -634,7 +635,7 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
         const int tt = t <= t_hi ? t : t - L;
         if (tt >= t_lo && tt <= t_hi) {
           const int o = tt - t_lo;
-          if (of) out[k2 + D * tt + K] = v * of[k2 + D * tt + K];
+          if (GRID) out[k2 + D * tt + K] = v * of[k2 + D * tt + K];
           else acc[o] = acc[o] + coef(o) * v;
         }
       };
@@ -649,12 +650,12 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
     for (int o = tid; o < n_out; o += NT) {
       int t = t_lo + o;
       int idx = t & (L - 1);  // t mod L (two's complement)
-      if (of) out[k2 + D * t + K] = buf[bidx(idx)] * of[k2 + D * t + K];
+      if (GRID) out[k2 + D * t + K] = buf[bidx(idx)] * of[k2 + D * t + K];
       else acc[o] = acc[o] + coef(o) * buf[bidx(idx)];
     }
     __syncthreads();
   }
-  if (of) return;
+  if (GRID) return;
   // ---- half-sample phase exp(-i pi k / P) and demodulation exp(+i pi k / sigma)
   const int64_t two_p = 2 * P;
   for (int o = tid; o < n_out; o += NT) {
@@ -681,14 +682,14 @@ __device__ __forceinline__ void fft_taylor_task(const FftArgs<T>& a, int series,
 template <int NT>
 constexpr int fft_min_blocks() { return NT >= 512 ? 1 : 512 / NT; }
 
-template <class T, int LOG2L, int NT>
+template <class T, int LOG2L, int NT, bool GRID>
 __global__ void __launch_bounds__(NT, fft_min_blocks<NT>()) fft_taylor_kernel(FftArgs<T> a, int use_zt) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fft_taylor_task<T, LOG2L, NT>(a, blockIdx.x, blockIdx.y, smem_raw, use_zt);
+  fft_taylor_task<T, LOG2L, NT, GRID>(a, blockIdx.x, blockIdx.y, smem_raw, use_zt);
 }
 
 // persistent form: CTAs pull (item, series, k2) tasks from a counter until none is left
-template <class T, int LOG2L, int NT>
+template <class T, int LOG2L, int NT, bool GRID>
 __global__ void __launch_bounds__(NT, fft_min_blocks<NT>()) fft_taylor_batch_kernel(const FftArgs<T>* items,
                                                               const int4* tasks, int n_tasks,
                                                               int* counter, int use_zt) {
@@ -702,7 +703,7 @@ __global__ void __launch_bounds__(NT, fft_min_blocks<NT>()) fft_taylor_batch_ker
     if (t >= n_tasks) break;
     const int4 tk = tasks[t];
     const FftArgs<T> a = items[tk.x];
-    fft_taylor_task<T, LOG2L, NT>(a, tk.y, tk.z, smem_raw, use_zt);
+    fft_taylor_task<T, LOG2L, NT, GRID>(a, tk.y, tk.z, smem_raw, use_zt);
     __syncthreads();
   }
 }
@@ -717,41 +718,55 @@ size_t fft_task_smem(int n_active, int n_out_max, int hi_max, int zt_arrays) {
 // the opt-in maximum of dynamic shared memory per block (227 KB) less the static words
 constexpr size_t kFftSmemCap = 227 * 1024 - 64;
 
-template <class T, int LOG2L>
-cudaError_t launch_l(const FftArgs<T>& a, cudaStream_t s) {
+template <class T, int LOG2L, bool GRID>
+cudaError_t launch_form(const FftArgs<T>& a, cudaStream_t s) {
   constexpr int NT = FftShape<LOG2L>::NT;
   const int D = a.n_sub;
-  const int n_out_max = a.out_factor ? 0 : (2 * a.grid_half + 1) / D + 2;
+  const int n_out_max = GRID ? 0 : (2 * a.grid_half + 1) / D + 2;
   const int hi = (a.n + 127) / 128;
   // the stored active inputs pay when at least two terms after the first read them
   const int arrays = a.expansion == 1 ? 2 : 1;
   const bool zt = a.taylor > 0 && fft_task_smem<T, LOG2L>(a.n_active, n_out_max, hi, arrays) <= kFftSmemCap;
   const size_t smem = fft_task_smem<T, LOG2L>(a.n_active, n_out_max, hi, zt ? arrays : 0);
-  cudaError_t e = cudaFuncSetAttribute(fft_taylor_kernel<T, LOG2L, NT>,
+  cudaError_t e = cudaFuncSetAttribute(fft_taylor_kernel<T, LOG2L, NT, GRID>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   dim3 grid(a.series, D);
-  fft_taylor_kernel<T, LOG2L, NT><<<grid, NT, smem, s>>>(a, zt ? 1 : 0);
+  fft_taylor_kernel<T, LOG2L, NT, GRID><<<grid, NT, smem, s>>>(a, zt ? 1 : 0);
   return cudaGetLastError();
 }
 
 template <class T, int LOG2L>
-cudaError_t launch_l_batch(const FftArgs<T>* items, const int4* tasks, int n_tasks, int* counter,
+cudaError_t launch_l(const FftArgs<T>& a, cudaStream_t s) {
+  return a.out_factor ? launch_form<T, LOG2L, true>(a, s) : launch_form<T, LOG2L, false>(a, s);
+}
+
+template <class T, int LOG2L, bool GRID>
+cudaError_t launch_form_batch(const FftArgs<T>* items, const int4* tasks, int n_tasks, int* counter,
                            int max_n_out, int max_active, int max_hi, int zt_arrays, int n_ctas,
                            cudaStream_t s) {
   constexpr int NT = FftShape<LOG2L>::NT;
   const bool zt = fft_task_smem<T, LOG2L>(max_active, max_n_out + 2, max_hi, zt_arrays) <= kFftSmemCap;
   const size_t smem = fft_task_smem<T, LOG2L>(max_active, max_n_out + 2, max_hi, zt ? zt_arrays : 0);
-  cudaError_t e = cudaFuncSetAttribute(fft_taylor_batch_kernel<T, LOG2L, NT>,
+  cudaError_t e = cudaFuncSetAttribute(fft_taylor_batch_kernel<T, LOG2L, NT, GRID>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 1;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fft_taylor_batch_kernel<T, LOG2L, NT>,
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fft_taylor_batch_kernel<T, LOG2L, NT, GRID>,
                                                     NT, smem) != cudaSuccess || per_sm < 1)
     per_sm = 1;
-  fft_taylor_batch_kernel<T, LOG2L, NT><<<n_ctas * per_sm, NT, smem, s>>>(items, tasks, n_tasks,
+  fft_taylor_batch_kernel<T, LOG2L, NT, GRID><<<n_ctas * per_sm, NT, smem, s>>>(items, tasks, n_tasks,
                                                                         counter, zt ? 1 : 0);
   return cudaGetLastError();
+}
+
+// max_n_out = kNoOutputs: every item is a gridded transform, whose tasks keep no outputs
+template <class T, int LOG2L>
+cudaError_t launch_l_batch(const FftArgs<T>* items, const int4* tasks, int n_tasks, int* counter,
+                           int max_n_out, int max_active, int max_hi, int zt_arrays, int n_ctas,
+                           cudaStream_t s) {
+  auto launch = max_n_out == kNoOutputs ? launch_form_batch<T, LOG2L, true> : launch_form_batch<T, LOG2L, false>;
+  return launch(items, tasks, n_tasks, counter, max_n_out, max_active, max_hi, zt_arrays, n_ctas, s);
 }
 
 }  // namespace
