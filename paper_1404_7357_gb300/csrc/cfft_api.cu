@@ -1118,7 +1118,7 @@ cfft_status fill_lattice(cfft_ctx* ctx, const FillArgs<double, double>& fa, bool
   const size_t groups = (size_t)c[1] * c[3];
   if (8 * groups * fa.n_cls > n * n) return CFFT_OK;
   const FillBucketPlan plan = plan_fill_bucketed<double>(std::max(c[1], c[3]), fa.n_mbf, fa.n_harm, fa.n_rho, fa.taps,
-                                                         1, 0, false);
+                                                         1, 0, false, true);
   if (!plan.ok) return CFFT_OK;
   const size_t blocks = groups * fa.n_cls * fa.n_mbf * fa.n_mbf * sizeof(cpx<double>);
   if (ctx->d_fill.ensure(plan.scratch) != cudaSuccess || ctx->d_latz.ensure(blocks + groups) != cudaSuccess) {

@@ -509,12 +509,13 @@ struct FillBucketPlan {
   int win, n_cells, nb_bits, block_rows, rows_per_wave;
   size_t n_keys_max, smem, scratch;
   bool direct;             // few pairs: no sort, a block per pair (fill only)
+  int parts;               // CTAs per window of the fill (0: by their number)
 };
 // pairs up to which fill_direct_kernel is the faster fill
 constexpr int64_t direct_pairs(bool fp64) { return fp64 ? 2048 : 6144; }
 template <class T>
 FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, int taps, int n_cls,
-                                  int block_rows, bool tc);
+                                  int block_rows, bool tc, bool lattice = false);
 template <class T>
 cudaError_t launch_fill_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& plan, void* scratch,
                                  cudaStream_t s);

@@ -495,9 +495,9 @@ __device__ __forceinline__ cpx<T> phase_power(cpx<T> e, int q) {
 // warps MBF pairs, and a warp sum ends each.  The sort, its scans and the buckets' table slices
 // are 9 launches and a serial chain of 60 us and more for any number of pairs; here a pair costs
 // its 17 KB of table rows (M = 4, 17 harmonics, 8 taps), and in FP64 its weights on the FP64 pipe.
-// GB300, M = 4, sorted -> direct per call, elements: FP32 24: 78 -> 39 us, 64: 102 -> 66,
-// 100: 106 -> 113; FP64 8: 170 -> 53 us, 48: 296 -> 271, 64: 375 -> 409: the lines between
-// (direct_pairs).
+// GB300, M = 4, sorted -> direct per call, elements: FP32 24: 79 -> 37 us, 64: 105 -> 64,
+// 100: 106 -> 113; FP64, four classes 8: 166 -> 51, 45: 274 -> 238; one class 8: 162 -> 51, 32: 164
+// -> 146, 45: 165 -> 238; M = 2 45: 125 -> 99: the lines (direct_pairs) where most forms cross.
 template <class T, int M, int TAPS>
 __global__ void __launch_bounds__(128) fill_direct_kernel(FillArgs<T, T> a, BucketArgs b) {
   constexpr int P2 = M * M, W = 4, AB = P2 < W ? 1 : P2 / W;   // MBF pairs per warp
@@ -1241,16 +1241,15 @@ cudaError_t run_bucketed(const FillArgs<T, T>& a, const FillBucketPlan& pl, void
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   return run_waves<T, TAPS>(a, pl, bucket_args(a, pl, scratch), s, [&](BucketArgs b, dim3 fg) {
-    // FP64: the pairs' arithmetic is dear and unevenly spread over the cells (a lattice's
-    // displacements lie in a few hundred of them), so several CTAs share a window where there are
-    // fewer than eight CTAs per SM (two where shared memory holds one CTA), each with its own copy of the
-    // window's rows.  GB300, M = 4, one CTA per window -> shared (two-cell windows with eight CTAs
-    // each): the 25 x 25 array's displacements and copy 1,472 -> 595 us (589); irregular, 8 harmonics: 60
-    // elements 329 -> 161 (263), 500 4,941 -> 4,600 (5,213), four classes 4,920 -> 4,787 (6,065); 16
-    // harmonics, 700 elements 17.8 -> 17.6 ms (27.1: narrow windows copy 17 rows for two cells).
+    // FP64: the pairs' arithmetic is dear and unevenly spread over the cells, so several CTAs share
+    // a window where there are fewer than eight CTAs per SM (two where shared memory holds one CTA), each
+    // with its own copy of the window's rows.  GB300, M = 4, irregular, one CTA per window ->
+    // shared (two-cell windows with eight CTAs each): 8 harmonics, 60 elements 329 -> 161 us (263),
+    // 500 4,941 -> 4,545 (5,213), four classes 4,920 -> 4,787 (6,065); 16 harmonics, 700 elements
+    // 17.8 -> 17.6 ms (27.1: narrow windows copy 17 rows for two cells).
     if (sizeof(T) == 8) {
       const int64_t ctas = (int64_t)fg.x * fg.y * fg.z, want = (smem <= 113 * 1024 ? 8 : 2) * (int64_t)current_sm_count();
-      b.parts = (int)std::min<int64_t>(8, std::max<int64_t>(1, (want + ctas - 1) / ctas));
+      b.parts = pl.parts > 0 ? pl.parts : (int)std::min<int64_t>(8, std::max<int64_t>(1, (want + ctas - 1) / ctas));
     }
     fg.x *= b.parts;
     bucket_fill_kernel<T, M, TAPS><<<fg, kBThreads, smem, s>>>(a, b);
@@ -1363,7 +1362,7 @@ cudaError_t adjoint_taps(const FillArgs<T, T>& a, const FillAdjointArgs<T>& ad, 
 // window of at least 4 stencil starts fitting in shared memory.
 template <class T>
 FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, int taps, int n_cls,
-                                  int block_rows, bool tc) {
+                                  int block_rows, bool tc, bool lattice) {
   FillBucketPlan pl{};
   pl.ok = false;
   if (!(n_mbf == 1 || n_mbf == 2 || n_mbf == 4)) return pl;
@@ -1384,6 +1383,12 @@ FillBucketPlan plan_fill_bucketed(int n_el, int n_mbf, int n_harm, int n_rho, in
     if (win < 8) win = (int)((220 * 1024) / row_bytes) - (taps - 1);
     if (win < 4) return pl;
     win = std::min(win, 64);
+    // a lattice's displacements lie in a few hundred cells: narrow windows copy no rows between
+    // them (25 x 25, M = 4, 8 harmonics, mean of ten pitches: wide windows 621 us, four cells 587)
+    if (lattice) {
+      win = std::min(win, 4);
+      pl.parts = 4;
+    }
     pl.win = win;
     pl.smem = (size_t)(win + taps - 1) * row_bytes;
   }
@@ -1441,8 +1446,8 @@ cudaError_t launch_fill_adjoint_bucketed(const FillArgs<T, T>& a, const FillAdjo
   }
 }
 
-template FillBucketPlan plan_fill_bucketed<float>(int, int, int, int, int, int, int, bool);
-template FillBucketPlan plan_fill_bucketed<double>(int, int, int, int, int, int, int, bool);
+template FillBucketPlan plan_fill_bucketed<float>(int, int, int, int, int, int, int, bool, bool);
+template FillBucketPlan plan_fill_bucketed<double>(int, int, int, int, int, int, int, bool, bool);
 template cudaError_t launch_fill_bucketed<float>(const FillArgs<float, float>&, const FillBucketPlan&, void*,
                                                  cudaStream_t);
 template cudaError_t launch_fill_bucketed<double>(const FillArgs<double, double>&, const FillBucketPlan&,
