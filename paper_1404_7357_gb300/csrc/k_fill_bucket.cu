@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(kBThreads) bucket_sort_kernel(FillArgs<T, T> a
     const BGeom<T> g = bucket_geom<T, TAPS>(a, b, m, n);
     if (g.bad) {
       if (!SCATTER) {
-        if (a.bad) a.bad[(size_t)m * a.n_el + n] = 1;
+        if (sizeof(T) == 8 && a.bad) a.bad[(size_t)m * a.n_el + n] = 1;   // a lattice's displacement
         else atomicOr(a.err, 1);
         if (a.z == nullptr) continue;   // the adjoint: no matrix
         const int M = a.n_mbf;
