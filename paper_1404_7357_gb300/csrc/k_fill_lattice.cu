@@ -10,7 +10,9 @@
 //
 // The general path is bound by the FP64 pipe (10,000 DFMA per pair of M = 4, 17 harmonics, 16 taps),
 // the copy by writing the matrix.  GB300, 25 x 25 elements (about 20,000 displacements of
-// 390,625 pairs; the differences of one pitch round to a few values each): 23 ms -> 0.63 ms.
+// 390,625 pairs; the differences of one pitch round to a few values each): 23 ms -> 0.60 ms.
+// FP64 only: the float32 fill takes 0.28 ms for 500 elements where this one's general path takes
+// 4.9, so the search, the displacements' sort and the copy (0.2 ms) would leave little.
 #include <algorithm>
 
 #include "cfft_common.cuh"
